@@ -28,7 +28,7 @@
 #include "mm_kernels.h"
 
 #ifndef MM_SHOOT_MINB
-#define MM_SHOOT_MINB 2
+#define MM_SHOOT_MINB 3
 #endif
 // streams a batch's per-map trees, expansions and second passes run on
 #define MM_BATCH_STREAMS 8
@@ -730,7 +730,7 @@ static void fill_mapdev(mm_map *h) {
   M.acc = h->acc.p;
   M.span = h->span.p;
   M.stat = h->stat.p;
-  M.bigq = reinterpret_cast<TriJob *>(h->bigq.p);
+  M.bigq = reinterpret_cast<RawTri *>(h->bigq.p);
   M.bigq_n = h->bigq_n.p;
   M.bigq_cap = h->bigq_cap;
 }
@@ -777,7 +777,7 @@ static mm_status alloc_map_buffers(mm_map *h) {
   // the queue were 17-44 % slower).  Default, for maps that fit half the L2
   // (else none): the larger triangles the autotuner's sampled runs counted,
   // with a quarter to spare, else 1 slot per 12 cells; 2^16 .. 2^27 slots
-  // (48 B each).  When that much device memory is not to be had, 2^20 slots,
+  // (32 B each).  When that much device memory is not to be had, 2^20 slots,
   // then none.  Batches that do not fit are dealt out by the first kernel.
   {
     const int64_t cells = (h->col_hi - h->col_lo) * (h->row_hi - h->row_lo);

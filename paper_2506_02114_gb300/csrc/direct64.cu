@@ -118,7 +118,7 @@ __device__ __forceinline__ Vtx load_vtx(const Vtx *verts, int64_t n0, int64_t ro
 
 // Inverse polygon mapping of stored vertices, same warp-strip decomposition
 // and triangle split as the fused FMM kernel.
-__global__ void __launch_bounds__(256) k_ipm_vertices(const MapDev *__restrict__ maps,
+__global__ void __launch_bounds__(256, 2) k_ipm_vertices(const MapDev *__restrict__ maps,
                                                       const Vtx *__restrict__ verts, int64_t n0,
                                                       int64_t row_lo, int64_t row_hi,
                                                       unsigned long long *work_counter,
@@ -126,14 +126,14 @@ __global__ void __launch_bounds__(256) k_ipm_vertices(const MapDev *__restrict__
   const int lane = threadIdx.x & 31;
   extern __shared__ __align__(16) unsigned char s_dyn[];
   WarpSmem *ws = reinterpret_cast<WarpSmem *>(s_dyn) + (threadIdx.x >> 5);
-  WarpQueue wq = {ws->quad, 0};
-  JobQueue jq = {ws->big, &ws->rows, 0};
+  WarpQueues q = {ws, 0, 0, 0};
+  LaneCount lc = {0u, 0u};
+  counts_clear(ws, lane);
   const MapDev &M = maps[0];
   const int64_t strips = (n0 - 1 + MM_STRIP - 1) / MM_STRIP;
   const int64_t rows = row_hi - row_lo;  // cell rows
   const int64_t rpi = M.rows_per_item;
   const int64_t total = strips * ((rows + rpi - 1) / rpi);
-  IpmCounters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
   while (true) {
     unsigned long long w = 0;
     if (lane == 0) w = atomicAdd(work_counter, 1ull);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256) k_ipm_vertices(const MapDev *__restrict__
     if (je > row_hi) je = row_hi;
     const bool vvalid = i < n0;
     const bool cell_col = (lane < MM_STRIP) && (i + 1 < n0);
-    RunAcc ra = {-1, 0ull};
+    RunAcc ra = MM_RUN_NONE;
     Vtx prev = load_vtx(verts, n0, row_lo, i, jb, vvalid);
     for (int64_t j = jb + 1; j <= je; j++) {
       const Vtx cur = load_vtx(verts, n0, row_lo, i, j, vvalid);
@@ -159,31 +159,15 @@ __global__ void __launch_bounds__(256) k_ipm_vertices(const MapDev *__restrict__
       prev_r.py = __shfl_down_sync(0xffffffffu, prev.py, 1);
       prev_r.fx = __shfl_down_sync(0xffffffffu, prev.fx, 1);
       prev_r.fy = __shfl_down_sync(0xffffffffu, prev.fy, 1);
-#pragma unroll 1
-      for (int tri = 0; tri < 2; tri++) {
-        TriJob job;
-        SmallTri se;
-        LineTri le;  // (unused: two-pixel triangles are apportioned in place)
-        const int code = cell_col ? ipm_triangle<false>(M, prev, tri ? cur_r : prev_r,
-                                                        tri ? cur : cur_r, ra, cnt, se, job, le)
-                                  : TRI_DONE;
-        wq_push(M, wq, code == TRI_SMALL, se, lane);
-        jq_add(jq, code == TRI_BIG, job, lane);
-        jq_share(M, jq, false, lane);
-      }
+      tri_scan(M, q, prev, prev_r, cur_r, cell_col, ra, lc, lane);
+      tri_scan(M, q, prev, cur_r, cur, cell_col, ra, lc, lane);
+      share_out(M, q, false, lc, lane);
       prev = cur;
     }
-    run_flush(M, ra);
-    wq_drain(M, wq, lane);
-    jq_share(M, jq, true, lane);
+    run_flush<MM_FIX_ONE>(M, ra);
+    share_out(M, q, true, lc, lane);
   }
-  unsigned v[MM_N_COUNTERS] = {cnt.dropped, cnt.clipped, cnt.small,  cnt.strip,
-                               cnt.big,     cnt.line,    cnt.culled, cnt.critical};
-#pragma unroll
-  for (int k = 0; k < MM_N_COUNTERS; k++) {
-    for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], d);
-    if (lane == 0 && v[k]) atomicAdd(&M.stat[k], (unsigned long long)v[k]);
-  }
+  counts_flush(M, ws, lc, lane);
 }
 
 cudaError_t launch_direct64_vertices(const double *sx, const double *sy, const double *sm,

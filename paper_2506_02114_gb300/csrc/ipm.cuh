@@ -30,18 +30,18 @@
 //     pixel): that pixel gains exactly 2^32;
 //   * it spans two pixels split by one grid line: the vertex alone on its
 //     side cuts off a similar triangle whose area fraction is a product of
-//     two edge parameters, finished here;
-//   * it spans 2 x 2 pixels: queued per warp in shared memory and
-//     apportioned 32 at a time from three quadrant areas by
-//     inclusion-exclusion;
+//     two edge parameters;
+//   * it spans 2 x 2 pixels: three quadrant areas by inclusion-exclusion;
 //   * larger (cells next to a star map to triangles up to hundreds of
-//     pixels wide; cells along a caustic to long slivers): queued per warp;
-//     the pixel rows of 32 such triangles are dealt out to the lanes, each
-//     row adds the constant 1/|area| to its run of fully covered pixels
-//     through a per-row difference array, and the partially covered pixels
-//     of those rows are then dealt out one per lane and measured from the
-//     row's edge pieces (row_pieces, piece_mean).  Work is proportional to
-//     the perimeter, not the area, and no lane loops on its own.
+//     pixels wide; cells along a caustic to long slivers): the pixel rows of
+//     32 such triangles are dealt out to the lanes, each row adds the
+//     constant 1/|area| to its run of fully covered pixels through a per-row
+//     difference array, and the partially covered pixels of those rows are
+//     then dealt out one per lane and measured from the row's edge pieces
+//     (row_pieces, piece_mean).  Work is proportional to the perimeter, not
+//     the area, and no lane loops on its own.
+// All but the first are queued per warp in shared memory and finished 32 of
+// a kind at a time.
 #pragma once
 #include <climits>
 
@@ -103,31 +103,32 @@ struct MapAcc {
   unsigned *err;
 };
 
-// Lane-private run accumulator: consecutive one-pixel triangles of a lane's
-// column usually hit the same pixel; they are summed in a register.
+// Lane-private run accumulator: consecutive one-pixel triangles (or rays) of
+// a lane's column usually hit the same pixel; they are counted in a
+// register.  UNIT is one triangle's (or ray's) fixed-point units.
 struct RunAcc {
-  long long idx;  // map index of the pixel being summed, -1 for none
-  unsigned long long val;
+  int px, py;  // the pixel being counted, px < 0 for none
+  unsigned n;
 };
+#define MM_RUN_NONE RunAcc{-1, 0, 0u}
 
+template <unsigned long long UNIT>
 __device__ __forceinline__ void run_flush(const MapDev &M, RunAcc &a) {
-  if (a.idx >= 0 && MM_INDEX_OK(M.err, a.idx, (long long)M.npix * M.npix_y))
-    atomicAdd(&M.acc[a.idx], a.val);
-  a.idx = -1;
-  a.val = 0;
+  const long long idx = (long long)a.py * M.npix + a.px;
+  if (a.px >= 0 && MM_INDEX_OK(M.err, idx, (long long)M.npix * M.npix_y))
+    atomicAdd(&M.acc[idx], a.n * UNIT);
+  a = MM_RUN_NONE;
 }
 
-// Add v to in-map pixel idx.
-__device__ __forceinline__ void run_add(const MapDev &M, RunAcc &a, long long idx,
-                                        unsigned long long v) {
-  if (idx == a.idx) {
-    a.val += v;
+// Count one in in-map pixel (px, py).
+template <unsigned long long UNIT>
+__device__ __forceinline__ void run_add(const MapDev &M, RunAcc &a, int px, int py) {
+  if (px == a.px && py == a.py) {
+    a.n++;
     return;
   }
-  if (a.idx >= 0 && MM_INDEX_OK(M.err, a.idx, (long long)M.npix * M.npix_y))
-    atomicAdd(&M.acc[a.idx], a.val);
-  a.idx = idx;
-  a.val = v;
+  run_flush<UNIT>(M, a);
+  a = RunAcc{px, py, 1u};
 }
 
 // ---------------------------------------------------------------------------
@@ -186,143 +187,151 @@ __device__ __forceinline__ float quadrant_edge(float px, float py, float qx, flo
 }
 
 // ---------------------------------------------------------------------------
-// triangles within a 2 x 2 pixel box: warp queue
+// queued triangles
 // ---------------------------------------------------------------------------
 
-// Frame pixel (ox, oy), first vertex (x0, y0) inside it, the other two
-// relative to the first.
-struct __align__(16) SmallTri {
-  int ox, oy;
-  float x0, y0, d1x, d1y, d2x, d2y;
+// A triangle waiting in a warp's queue, 32 bytes.
+//   * Within 2 x 2 pixels (the line and quad queues): (x, y) is the low
+//     corner of its pixel box, f[2 k], f[2 k + 1] vertex k's position inside
+//     its own pixel, whose offset from the corner (0 or 1 per axis) is the
+//     sign bit.
+//   * Larger (the big queue and the map's device queue): (x, y) is the first
+//     vertex's pixel and f the three vertices in its frame; the sign bit of
+//     f[0] (a fraction, >= 0) marks a box of at most MM_MED_PIXELS map pixels
+//     while the triangle is in the warp's queue.
+// The scan that finds a triangle only stores it: areas, slopes and shares
+// are formed when 32 of a kind are taken off a queue, every lane busy,
+// instead of in branches that a few lanes take on nearly every row (the
+// larger triangles' three slopes and inverse area are IEEE divisions).
+struct __align__(16) RawTri {
+  int x, y;
+  float f[6];
 };
+static_assert(sizeof(RawTri) == MM_TRIJOB_BYTES, "RawTri layout");
+
+__device__ __forceinline__ void raw_store(RawTri *e, int x, int y, float f0, float f1, float f2,
+                                          float f3, float f4, float f5) {
+  float4 *w = reinterpret_cast<float4 *>(e);
+  w[0] = make_float4(__int_as_float(x), __int_as_float(y), f0, f1);
+  w[1] = make_float4(f2, f3, f4, f5);
+}
+__device__ __forceinline__ RawTri raw_load(const RawTri *e) {
+  const float4 *w = reinterpret_cast<const float4 *>(e);
+  const float4 u = w[0], v = w[1];
+  RawTri t;
+  t.x = __float_as_int(u.x);
+  t.y = __float_as_int(u.y);
+  t.f[0] = u.z;
+  t.f[1] = u.w;
+  t.f[2] = v.x;
+  t.f[3] = v.y;
+  t.f[4] = v.z;
+  t.f[5] = v.w;
+  return t;
+}
+
+// Twice the signed area of a triangle in its frame.
+// (one rounding order for every caller, so that counts against the
+// near-critical threshold do not depend on where the area is formed)
+__device__ __forceinline__ float tri_area2(const float (&t)[6]) {
+  return fmaf(t[2] - t[0], t[5] - t[1], -__fmul_rn(t[4] - t[0], t[3] - t[1]));
+}
+
+// Vertex k's fraction with its pixel's offset from the box corner (0 or 1)
+// in the sign bit.
+__device__ __forceinline__ float with_offset(float f, int px, int lo) {
+  return __int_as_float(__float_as_int(f) | ((px - lo) << 31));
+}
+
+// A triangle within 2 x 2 pixels in the frame of its first vertex's pixel
+// (t), and that pixel's offset (ax, ay) from the box corner.
+__device__ __forceinline__ void small_frame(const RawTri &e, float (&t)[6], int &ax, int &ay) {
+  const int b0 = __float_as_int(e.f[0]), b1 = __float_as_int(e.f[1]);
+  ax = b0 < 0;
+  ay = b1 < 0;
+  const float fx = (float)ax, fy = (float)ay;
+  t[0] = fabsf(e.f[0]);
+  t[1] = fabsf(e.f[1]);
+#pragma unroll
+  for (int k = 1; k < 3; k++) {
+    // the vertex's pixel relative to the first vertex's (-1, 0 or 1), then its fraction
+    t[2 * k] = ((__float_as_int(e.f[2 * k]) < 0 ? 1.f : 0.f) - fx) + fabsf(e.f[2 * k]);
+    t[2 * k + 1] = ((__float_as_int(e.f[2 * k + 1]) < 0 ? 1.f : 0.f) - fy) + fabsf(e.f[2 * k + 1]);
+  }
+}
+
+// Counters of a lane: triangles dropped (non-finite, or without area) and
+// triangles whose local |mu| exceeds the near-critical threshold.
+struct LaneCount {
+  unsigned dropped, critical;
+};
+
+// Area test of a triangle that meets the map: false (and counted) when it
+// has none; near-critical ones are counted.
+__device__ __forceinline__ bool area_ok(const MapDev &M, float area2, LaneCount &lc) {
+  if (!(area2 != 0.f) || !isfinite(area2)) {
+    lc.dropped++;
+    return false;
+  }
+  lc.critical += fabsf(area2) < M.crit_area2;
+  return true;
+}
+
+// A triangle across one grid line u = L (u = x or y) of two pixels.  The
+// vertex alone on its side cuts off a triangle similar to the whole, of area
+// fraction d^2 / ((u_a - u_l)(u_b - u_l)) with d = L - u_l (the two edge
+// parameters at the line, multiplied).  The two shares are complements in
+// fixed point, so the pair sums to exactly one triangle.
+__device__ __forceinline__ bool line_tri_apportion(const MapDev &M, const RawTri &e,
+                                                   LaneCount &lc) {
+  float t[6];
+  int ax, ay;
+  small_frame(e, t, ax, ay);
+  if (!area_ok(M, tri_area2(t), lc)) return false;
+  // the axis whose offsets differ: 0 a vertical line, 1 a horizontal one
+  const int x0 = __float_as_int(e.f[0]), x1 = __float_as_int(e.f[2]), x2 = __float_as_int(e.f[4]);
+  const int o = ((x0 ^ x1) | (x0 ^ x2)) >= 0;
+  const float L = 1.f - (float)(o ? ay : ax);
+  const float u0 = o ? t[1] : t[0], u1 = o ? t[3] : t[2], u2 = o ? t[5] : t[4];
+  const unsigned long long vlow = low_side_fixed(u0, u1, u2, L);
+  deposit(M, e.x, e.y, vlow);
+  deposit(M, e.x + 1 - o, e.y + o, MM_FIX_ONE - vlow);
+  return true;
+}
 
 // A triangle across both grid lines of a 2 x 2 pixel block: the shares left
 // of X and below Y from the lone vertex on each line, the lower-left share
 // from the quadrant integral; the four pixel shares are differences of
 // those in fixed point and add up to exactly one triangle.
-__device__ __forceinline__ void small_tri_apportion(const MapDev &M, const SmallTri &e) {
-  const int c0 = (int)floorf(e.x0 + fminf(0.f, fminf(e.d1x, e.d2x)));
-  const int r0 = (int)floorf(e.y0 + fminf(0.f, fminf(e.d1y, e.d2y)));
+__device__ __forceinline__ bool quad_tri_apportion(const MapDev &M, const RawTri &e,
+                                                   LaneCount &lc) {
+  float t[6];
+  int ax, ay;
+  small_frame(e, t, ax, ay);
+  if (!area_ok(M, tri_area2(t), lc)) return false;
+  const float x0 = t[0], y0 = t[1];
+  const float d1x = t[2] - t[0], d1y = t[3] - t[1], d2x = t[4] - t[0], d2y = t[5] - t[1];
+  const int c0 = (int)floorf(x0 + fminf(0.f, fminf(d1x, d2x)));
+  const int r0 = (int)floorf(y0 + fminf(0.f, fminf(d1y, d2y)));
   // the grid lines, relative to the first vertex
-  const float X = (float)(c0 + 1) - e.x0, Y = (float)(r0 + 1) - e.y0;
-  const long long vL = (long long)low_side_fixed(0.f, e.d1x, e.d2x, X);
-  const long long vB = (long long)low_side_fixed(0.f, e.d1y, e.d2y, Y);
-  const float lb = quadrant_edge(0.f, 0.f, e.d1x, e.d1y, X, Y) +
-                   quadrant_edge(e.d1x, e.d1y, e.d2x, e.d2y, X, Y) +
-                   quadrant_edge(e.d2x, e.d2y, 0.f, 0.f, X, Y);
-  const float A2 = e.d1x * e.d2y - e.d2x * e.d1y;  // twice the signed area
+  const float X = (float)(c0 + 1) - x0, Y = (float)(r0 + 1) - y0;
+  const long long vL = (long long)low_side_fixed(0.f, d1x, d2x, X);
+  const long long vB = (long long)low_side_fixed(0.f, d1y, d2y, Y);
+  const float lb = quadrant_edge(0.f, 0.f, d1x, d1y, X, Y) +
+                   quadrant_edge(d1x, d1y, d2x, d2y, X, Y) +
+                   quadrant_edge(d2x, d2y, 0.f, 0.f, X, Y);
+  const float A2 = d1x * d2y - d2x * d1y;  // twice the signed area
   const long long vLB = (long long)frac_to_fixed(2.f * lb * rcp_approx_f(A2));
   const long long one = (long long)MM_FIX_ONE;
-  const int gx = e.ox + c0, gy = e.oy + r0;
+  const int gx = e.x + ax + c0, gy = e.y + ay + r0;
   deposit(M, gx, gy, (unsigned long long)vLB);
   deposit(M, gx, gy + 1, (unsigned long long)max(vL - vLB, 0ll));
   deposit(M, gx + 1, gy, (unsigned long long)max(vB - vLB, 0ll));
   deposit(M, gx + 1, gy + 1, (unsigned long long)max(one - vL - vB + vLB, 0ll));
+  return true;
 }
 
-// A triangle across one grid line of two pixels: the low pixel (gx, gy),
-// the line u = L along axis o (0: x, 1: y; the high pixel is the next one
-// along that axis) and the triangle's coordinates along that axis.
-struct __align__(16) LineTri {
-  int gx, gy;
-  float u0, u1, u2, L;
-  int o, pad;
-};
-
-// The two pixels' shares: complements in fixed point, one triangle in all.
-__device__ __forceinline__ void line_tri_apportion(const MapDev &M, const LineTri &e) {
-  const unsigned long long vlow = low_side_fixed(e.u0, e.u1, e.u2, e.L);
-  deposit(M, e.gx, e.gy, vlow);
-  deposit(M, e.gx + 1 - e.o, e.gy + e.o, MM_FIX_ONE - vlow);
-}
-
-// Per-warp queue of LineTri in shared memory (capacity 64 >= 31 + 31 + 2):
-// the two-pixel triangles are shared out 32 at a time, so the warp runs
-// their apportioning with every lane busy instead of in a branch that only
-// some lanes take (used by the single-map first pass, whose registers allow
-// it; elsewhere the triangle is apportioned where it is found).
-struct LineQueue {
-  LineTri *q;
-  int n;
-};
-
-__device__ __forceinline__ void lq_push(const MapDev &M, LineQueue &lq, bool want,
-                                        const LineTri &e, int lane) {
-  const unsigned m = __ballot_sync(0xffffffffu, want);
-  if (!m) return;
-  const int pos = lq.n + __popc(m & ((1u << lane) - 1u));
-  if (want) lq.q[pos] = e;
-  lq.n += __popc(m);
-  __syncwarp();
-  while (lq.n >= 32) {
-    const LineTri t = lq.q[lq.n - 32 + lane];
-    __syncwarp();
-    lq.n -= 32;
-    line_tri_apportion(M, t);
-  }
-}
-
-__device__ __forceinline__ void lq_drain(const MapDev &M, LineQueue &lq, int lane) {
-  if (lq.n > 0) {
-    LineTri t;
-    const bool have = lane < lq.n;
-    if (have) t = lq.q[lane];
-    __syncwarp();
-    if (have) line_tri_apportion(M, t);
-    lq.n = 0;
-  }
-  __syncwarp();
-}
-
-// Per-warp queue of SmallTri in shared memory (capacity 64 >= 31 + 31 + 2).
-struct WarpQueue {
-  SmallTri *q;
-  int n;
-};
-
-__device__ __forceinline__ void wq_push(const MapDev &M, WarpQueue &wq, bool want,
-                                        const SmallTri &e, int lane) {
-  const unsigned m = __ballot_sync(0xffffffffu, want);
-  if (!m) return;
-  const int pos = wq.n + __popc(m & ((1u << lane) - 1u));
-  if (want) wq.q[pos] = e;
-  wq.n += __popc(m);
-  __syncwarp();
-  while (wq.n >= 32) {
-    const SmallTri t = wq.q[wq.n - 32 + lane];
-    __syncwarp();
-    wq.n -= 32;
-    small_tri_apportion(M, t);
-  }
-}
-
-__device__ __forceinline__ void wq_drain(const MapDev &M, WarpQueue &wq, int lane) {
-  if (wq.n > 0) {
-    SmallTri t;
-    const bool have = lane < wq.n;
-    if (have) t = wq.q[lane];
-    __syncwarp();
-    if (have) small_tri_apportion(M, t);
-    wq.n = 0;
-  }
-  __syncwarp();
-}
-
-// ---------------------------------------------------------------------------
-// one triangle
-// ---------------------------------------------------------------------------
-
-// Per-lane triangle counters, reduced per warp into MapDev::stat:
-// [0] dropped, [1] multi-pixel (clipped) in the map, [2] within a 2 x 2 box
-// crossing both grid lines, [3] box of at most MM_MED_PIXELS pixels (pixel
-// jobs), [4] larger (row jobs), [5] two pixels split by one grid line, [6]
-// vertex rows not computed because culling proved them beyond the map.
-#define MM_N_COUNTERS 8
-struct IpmCounters {
-  unsigned dropped, clipped, small, strip, big, line, culled, critical;
-};
-
-// A triangle shared out to the whole warp: frame pixel, frame coordinates,
+// A larger triangle ready to be dealt out: frame pixel, frame coordinates,
 // 2 / signed area and the inverse slope dx/dy of each edge k -> k + 1
 // (infinite or NaN for a horizontal edge, which is never used).
 struct __align__(16) TriJob {
@@ -331,130 +340,24 @@ struct __align__(16) TriJob {
   float inv2;
   float k[3];
 };
-static_assert(sizeof(TriJob) == MM_TRIJOB_BYTES, "TriJob layout");
 
-enum { TRI_DONE = 0, TRI_SMALL = 1, TRI_BIG = 2, TRI_LINE = 3 };
-
-// Apportion one triangle (a, b, c).  Triangles within one pixel are
-// finished here, and so are those split by one grid line unless LINEQ, which
-// returns TRI_LINE (le filled) for the line queue; returns TRI_SMALL (se
-// filled) for a triangle covering 2 x 2 pixels, to be pushed on the quad
-// queue, and TRI_BIG (job filled) for a larger one, whose pixel rows and then
-// partially covered pixels the warp deals out to its lanes (warp_tri_jobs).
-template <bool LINEQ>
-__device__ __forceinline__ int ipm_triangle(const MapDev &M, const Vtx &a,
-                                            const Vtx &b, const Vtx &c, RunAcc &ra,
-                                            IpmCounters &cnt, SmallTri &se, TriJob &job,
-                                            LineTri &le) {
-  if (a.px == MM_VTX_INVALID || b.px == MM_VTX_INVALID || c.px == MM_VTX_INVALID) {
-    cnt.dropped++;
-    return TRI_DONE;
-  }
-  // the pixel box from the vertices' pixels (a vertex's pixel is the floor
-  // of its coordinate), and wholly beyond one edge of the map (most
-  // triangles of a shooting region): integer tests before any arithmetic
-  const int xlo = min(a.px, min(b.px, c.px)), xhi = max(a.px, max(b.px, c.px));
-  const int ylo = min(a.py, min(b.py, c.py)), yhi = max(a.py, max(b.py, c.py));
-  if (xhi < 0 || xlo >= M.npix || yhi < 0 || ylo >= M.npix_y) return TRI_DONE;
-  const int ox = a.px, oy = a.py;
-  float t[6];
-  t[0] = a.fx;
-  t[1] = a.fy;
-  // pixel indices stay within +-2^29, so differences fit in 32 bits
-  t[2] = (float)(b.px - ox) + b.fx;
-  t[3] = (float)(b.py - oy) + b.fy;
-  t[4] = (float)(c.px - ox) + c.fx;
-  t[5] = (float)(c.py - oy) + c.fy;
-  const float area2 = (t[2] - t[0]) * (t[5] - t[1]) - (t[4] - t[0]) * (t[3] - t[1]);
-  if (!(area2 != 0.f) || !isfinite(area2)) {
-    cnt.dropped++;
-    return TRI_DONE;
-  }
-  // near-critical: local |mu| = image area / source area above the threshold
-  cnt.critical += fabsf(area2) < M.crit_area2;
-  if (xlo == xhi && ylo == yhi) {
-    // all three vertices in one (closed) map pixel: all of the area is there
-    run_add(M, ra, (long long)oy * M.npix + ox, MM_FIX_ONE);
-    return TRI_DONE;
-  }
-  // pixel range in the frame of vertex a
-  const int cx0 = xlo - ox, cx1 = xhi - ox, cy0 = ylo - oy, cy1 = yhi - oy;
-  if ((cx1 - cx0) + (cy1 - cy0) == 1) {
-    // (two adjacent pixels that passed the test above: at least one is in
-    // the map, so the map restriction below is not needed)
-    cnt.clipped++;
-    // Two pixels split by one grid line u = L (u = x or y).  The vertex alone
-    // on its side cuts off a triangle similar to the corner it spans, of
-    // area fraction d^2 / ((u_a - u_l)(u_b - u_l)) with d = L - u_l (the two
-    // edge parameters at the line, multiplied).  The shares are complements
-    // in fixed point, so the pair sums to exactly one triangle.
-    const int o = cy1 - cy0;  // 0: vertical line, 1: horizontal line
-    const float L = (float)(o ? cy0 : cx0) + 1.f;
-    // (selects, not t[o]: a run-time index would put t in local memory)
-    const float u0 = o ? t[1] : t[0], u1 = o ? t[3] : t[2], u2 = o ? t[5] : t[4];
-    if (LINEQ) {
-      le.gx = ox + cx0;  // the low pixel (indices within +-2^29)
-      le.gy = oy + cy0;
-      le.u0 = u0;
-      le.u1 = u1;
-      le.u2 = u2;
-      le.L = L;
-      le.o = o;
-      cnt.line++;
-      return TRI_LINE;
-    }
-    const unsigned long long vlow = low_side_fixed(u0, u1, u2, L);
-    const bool b0 = u0 < L;  // vertex a on the low side
-    // the pixel holding vertex a goes through the run accumulator
-    const int glx = ox + cx0, gly = oy + cy0;  // low pixel
-    const int gax = b0 ? glx : glx + 1 - o, gay = b0 ? gly : gly + o;
-    const int gbx = b0 ? glx + 1 - o : glx, gby = b0 ? gly + o : gly;
-    const unsigned long long va = b0 ? vlow : MM_FIX_ONE - vlow;
-    if (va && gax >= 0 && gax < M.npix && gay >= 0 && gay < M.npix_y)
-      run_add(M, ra, (long long)gay * M.npix + gax, va);
-    deposit(M, gbx, gby, MM_FIX_ONE - va);
-    cnt.line++;
-    return TRI_DONE;
-  }
-  // restrict to the map: frame columns [-ox, npix-1-ox]
-  const int mcl = -ox, mch = M.npix - 1 - ox;
-  const int mrl = -oy, mrh = M.npix_y - 1 - oy;
-  const int cl = cx0 > mcl ? cx0 : mcl, ch = cx1 < mch ? cx1 : mch;
-  const int rl = cy0 > mrl ? cy0 : mrl, rh = cy1 < mrh ? cy1 : mrh;
-  if (cl > ch || rl > rh) return TRI_DONE;  // misses the map
-  cnt.clipped++;
-  if (cx1 - cx0 <= 1 && cy1 - cy0 <= 1) {
-    se.ox = ox;
-    se.oy = oy;
-    se.x0 = t[0];
-    se.y0 = t[1];
-    se.d1x = t[2] - t[0];
-    se.d1y = t[3] - t[1];
-    se.d2x = t[4] - t[0];
-    se.d2y = t[5] - t[1];
-    cnt.small++;
-    return TRI_SMALL;
-  }
-  job.ox = ox;
-  job.oy = oy;
+__device__ __forceinline__ TriJob make_job(const RawTri &e) {
+  TriJob J;
+  J.ox = e.x;
+  J.oy = e.y;
 #pragma unroll
-  for (int k = 0; k < 6; k++) job.t[k] = t[k];
-  {
-    // 2 / area from the difference of products rounded once (Kahan's FMA
-    // method): the area of a long thin triangle cancels heavily in FP32
-    const float pa = t[2] - t[0], pd = t[5] - t[1], pb = t[4] - t[0], pc = t[3] - t[1];
-    const float wbc = pb * pc;
-    const float a2 = fmaf(pa, pd, -wbc) + fmaf(-pb, pc, wbc);
-    job.inv2 = 2.0f / ((a2 != 0.f && isfinite(a2)) ? a2 : area2);
-  }
+  for (int k = 0; k < 6; k++) J.t[k] = e.f[k];
+  const float(&t)[6] = e.f;
+  // 2 / area from the difference of products rounded once (Kahan's FMA
+  // method): the area of a long thin triangle cancels heavily in FP32
+  const float pa = t[2] - t[0], pd = t[5] - t[1], pb = t[4] - t[0], pc = t[3] - t[1];
+  const float wbc = pb * pc;
+  const float a2 = fmaf(pa, pd, -wbc) + fmaf(-pb, pc, wbc);
+  J.inv2 = 2.0f / ((a2 != 0.f && isfinite(a2)) ? a2 : tri_area2(t));
 #pragma unroll
-  for (int e = 0; e < 3; e++)
-    job.k[e] = (t[(2 * e + 2) % 6] - t[2 * e]) / (t[(2 * e + 3) % 6] - t[2 * e + 1]);
-  if ((long long)(ch - cl + 1) * (rh - rl + 1) <= MM_MED_PIXELS)
-    cnt.strip++;
-  else
-    cnt.big++;
-  return TRI_BIG;
+  for (int k = 0; k < 3; k++)
+    J.k[k] = (t[(2 * k + 2) % 6] - t[2 * k]) / (t[(2 * k + 3) % 6] - t[2 * k + 1]);
+  return J;
 }
 
 // ---------------------------------------------------------------------------
@@ -702,69 +605,201 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
   __syncwarp();
 }
 
-// Per-warp queue of larger triangles in shared memory (capacity 64 >=
-// 31 + 31 + 2).  A full batch of 32 is shared out at once, so the lanes stay
-// busy and the dealing overhead is amortised.
-struct JobQueue {
-  TriJob *q;
-  RowRecs *rr;
-  int n;
-};
+// ---------------------------------------------------------------------------
+// a warp's queues
+// ---------------------------------------------------------------------------
 
-// Shared memory of one warp: the two queues and the row records.
-struct WarpSmem {
-  LineTri line[64];
-  SmallTri quad[64];
-  TriJob big[64];
-  RowRecs rows;
+// Map statistics (MapDev::stat): [0] dropped, [1] multi-pixel (clipped) in
+// the map, [2] within a 2 x 2 box crossing both grid lines, [3] box of at
+// most MM_MED_PIXELS map pixels, [4] larger, [5] two pixels split by one
+// grid line, [6] vertex rows not computed because culling proved them beyond
+// the map, [7] near-critical.
+#define MM_N_COUNTERS 8
+enum { ST_DROPPED, ST_CLIPPED, ST_QUAD, ST_BOX, ST_ROWS, ST_LINE, ST_CULLED, ST_CRITICAL };
+
+// A row of cells adds at most 62 triangles (two per cell of a warp's 31) to
+// the queues, which are emptied to fewer than 32 of a kind after each row:
+// the line and quad queues share one array from its two ends.
+#define MM_SMALL_QUEUE (31 + 31 + 62)
+#define MM_BIG_QUEUE (31 + 62)
+
+// Shared memory of one warp.  A batch of larger triangles dealt out here
+// needs the row records, which lie over the line and quad queues (emptied
+// first), and its 32 full jobs behind the at most 61 triangles then left in
+// the big queue.
+struct __align__(16) WarpSmem {
+  union {
+    RawTri small[MM_SMALL_QUEUE];
+    RowRecs rows;
+  };
+  union {
+    RawTri big[MM_BIG_QUEUE];
+    struct {
+      RawTri left[MM_BIG_QUEUE - 32];
+      TriJob job[32];
+    };
+  };
+  Vtx row[32];                    // the last vertex row, one vertex per lane
+  unsigned count[MM_N_COUNTERS];  // (dropped and critical are per lane, LaneCount)
 };
 #define MM_SHOOT_SMEM_BYTES (8 * sizeof(WarpSmem))  // 8 warps per block
 
-// A queue entry with no pixel rows (frame far below any map).
-__device__ __forceinline__ TriJob empty_job_impl() {
-  TriJob e;
-  e.ox = e.oy = -(1 << 30);
-#pragma unroll
-  for (int k = 0; k < 6; k++) e.t[k] = 0.f;
-  e.inv2 = 0.f;
-  e.k[0] = e.k[1] = e.k[2] = 0.f;
-  return e;
-}
+struct WarpQueues {
+  WarpSmem *s;
+  int line, quad, big;  // triangles waiting (warp-uniform)
+};
 
-// Queue the lanes' larger triangles (no processing).
-__device__ __forceinline__ void jq_add(JobQueue &jq, bool want, const TriJob &job, int lane) {
-  const unsigned m = __ballot_sync(0xffffffffu, want);
-  if (!m) return;
-  const int pos = jq.n + __popc(m & ((1u << lane) - 1u));
-  if (want) jq.q[pos] = job;
-  jq.n += __popc(m);
+// Apportion or queue one triangle (a, b, c) of each lane (`on`: the lane
+// has one).  A triangle inside one pixel is finished here.
+__device__ __forceinline__ void tri_scan(const MapDev &M, WarpQueues &q, const Vtx &a,
+                                         const Vtx &b, const Vtx &c, bool on, RunAcc &ra,
+                                         LaneCount &lc, int lane) {
+  // the pixel box from the vertices' pixels (a vertex's pixel is the floor
+  // of its coordinate, MM_VTX_INVALID = INT_MIN below any valid one); most
+  // triangles of a shooting region lie wholly beyond one edge of the map:
+  // integer tests before any arithmetic
+  const int xlo = min(a.px, min(b.px, c.px)), xhi = max(a.px, max(b.px, c.px));
+  const int ylo = min(a.py, min(b.py, c.py)), yhi = max(a.py, max(b.py, c.py));
+  if (on && xlo == MM_VTX_INVALID) {
+    lc.dropped++;
+    on = false;
+  }
+  on = on && xhi >= 0 && xlo < M.npix && yhi >= 0 && ylo < M.npix_y;
+  const int sx = xhi - xlo, sy = yhi - ylo;
+  const unsigned span = (unsigned)(sx | sy);
+  const bool one = on && span == 0u;
+  const bool line = on && span == 1u && !(sx & sy);
+  const bool quad = on && span == 1u && (sx & sy);
+  const bool big = on && span > 1u;
+  const unsigned ml = __ballot_sync(0xffffffffu, line), mq = __ballot_sync(0xffffffffu, quad),
+                 mb = __ballot_sync(0xffffffffu, big);
+  const unsigned below = (1u << lane) - 1u;
+  if (one) {
+    // all three vertices in one (closed) map pixel: all of the area is there
+    const float t[6] = {a.fx, a.fy, b.fx, b.fy, c.fx, c.fy};
+    if (area_ok(M, tri_area2(t), lc))
+      run_add<MM_FIX_ONE>(M, ra, a.px, a.py);
+  } else if (line || quad) {
+    const int k = line ? q.line + __popc(ml & below)
+                       : MM_SMALL_QUEUE - 1 - q.quad - __popc(mq & below);
+    raw_store(q.s->small + k, xlo, ylo, with_offset(a.fx, a.px, xlo), with_offset(a.fy, a.py, ylo),
+              with_offset(b.fx, b.px, xlo), with_offset(b.fy, b.py, ylo),
+              with_offset(c.fx, c.px, xlo), with_offset(c.fy, c.py, ylo));
+  } else if (big) {
+    // the box within the map (indices within +-2^29)
+    const int w = min(xhi, M.npix - 1) - max(xlo, 0) + 1;
+    const int h = min(yhi, M.npix_y - 1) - max(ylo, 0) + 1;
+    const bool med = (long long)w * h <= MM_MED_PIXELS;
+    // pixel indices stay within +-2^29, so differences fit in 32 bits
+    raw_store(q.s->big + q.big + __popc(mb & below), a.px, a.py, med ? -a.fx : a.fx, a.fy,
+              (float)(b.px - a.px) + b.fx, (float)(b.py - a.py) + b.fy,
+              (float)(c.px - a.px) + c.fx, (float)(c.py - a.py) + c.fy);
+  }
+  q.line += __popc(ml);
+  q.quad += __popc(mq);
+  q.big += __popc(mb);
   __syncwarp();
 }
 
-// Full batches of 32 queued triangles (with `flush` also the rest) go to
-// the map's device queue for the larger-triangle kernel (k_big_ipm), which
-// deals them out at a higher occupancy than this kernel's; a batch that
-// does not fit is dealt out here, its reserved queue slots filled with
-// empty jobs.
-__device__ __forceinline__ void jq_share(const MapDev &M, JobQueue &jq, bool flush, int lane) {
-  while (jq.n >= 32 || (flush && jq.n > 0)) {
-    const int nb = min(jq.n, 32);
-    jq.n -= nb;
+// Empty the queues down to fewer than 32 triangles of a kind (`flush`:
+// entirely).  Batches of larger triangles go to the map's device queue for
+// the larger-triangle kernel (k_big_ipm), which deals them out at a higher
+// occupancy than this kernel's; a batch that does not fit is dealt out here,
+// its reserved queue slots filled with triangles without pixel rows.
+__device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool flush,
+                                          LaneCount &lc, int lane) {
+  if (!flush && ((q.line | q.quad | q.big) & ~31) == 0) return;
+  int deal = 0;  // jobs set up to be dealt out here
+  while (true) {
+    const bool rest = flush || deal > 0;
+    while (q.line >= 32 || (rest && q.line > 0)) {
+      const int nb = min(q.line, 32);
+      q.line -= nb;
+      const bool done =
+          lane < nb && line_tri_apportion(M, raw_load(q.s->small + q.line + lane), lc);
+      const unsigned n = __popc(__ballot_sync(0xffffffffu, done));
+      if (lane == 0) q.s->count[ST_LINE] += n;
+    }
+    while (q.quad >= 32 || (rest && q.quad > 0)) {
+      const int nb = min(q.quad, 32);
+      q.quad -= nb;
+      const bool done =
+          lane < nb &&
+          quad_tri_apportion(M, raw_load(q.s->small + MM_SMALL_QUEUE - 1 - q.quad - lane), lc);
+      const unsigned n = __popc(__ballot_sync(0xffffffffu, done));
+      if (lane == 0) q.s->count[ST_QUAD] += n;
+    }
+    __syncwarp();
+    if (deal > 0) {
+      warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q.s->job, deal, &q.s->rows, lane);
+      deal = 0;
+    }
+    if (!(q.big >= 32 || (flush && q.big > 0))) break;
+    const int nb = min(q.big, 32);
+    q.big -= nb;
+    RawTri e;
+    e.x = e.y = -(1 << 30);  // no pixel rows: a frame far below any map
+#pragma unroll
+    for (int k = 0; k < 6; k++) e.f[k] = 0.f;
+    bool ok = false, med = false;
+    if (lane < nb) {
+      RawTri t = raw_load(q.s->big + q.big + lane);
+      med = __float_as_int(t.f[0]) < 0;
+      t.f[0] = fabsf(t.f[0]);
+      ok = area_ok(M, tri_area2(t.f), lc);
+      if (ok) e = t;
+    }
+    const unsigned m_ok = __ballot_sync(0xffffffffu, ok);
+    const unsigned m_med = __ballot_sync(0xffffffffu, ok && med);
+    if (lane == 0) {
+      q.s->count[ST_BOX] += __popc(m_med);
+      q.s->count[ST_ROWS] += __popc(m_ok & ~m_med);
+    }
     unsigned long long base = 0;
+    bool fits = false;
     if (M.bigq_cap > 0) {
       if (lane == 0) base = atomicAdd(M.bigq_n, (unsigned long long)nb);
       base = __shfl_sync(0xffffffffu, base, 0);
+      fits = base + nb <= (unsigned long long)M.bigq_cap;
+      if (!fits && lane < nb && base + lane < (unsigned long long)M.bigq_cap)
+        raw_store(M.bigq + base + lane, -(1 << 30), -(1 << 30), 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
     }
-    if (M.bigq_cap > 0 && base + nb <= (unsigned long long)M.bigq_cap) {
-      if (lane < nb) M.bigq[base + lane] = jq.q[jq.n + lane];
+    if (fits) {
+      if (lane < nb)
+        raw_store(M.bigq + base + lane, e.x, e.y, e.f[0], e.f[1], e.f[2], e.f[3], e.f[4], e.f[5]);
       __syncwarp();
     } else {
-      if (M.bigq_cap > 0 && lane < nb && base + lane < (unsigned long long)M.bigq_cap)
-        M.bigq[base + lane] = empty_job_impl();
-      warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, jq.q + jq.n, nb, jq.rr, lane);
+      __syncwarp();  // (the jobs overlap queue entries just read)
+      if (lane < nb) q.s->job[lane] = make_job(e);
+      deal = nb;
     }
   }
 }
 
+__device__ __forceinline__ void counts_clear(WarpSmem *s, int lane) {
+  if (lane < MM_N_COUNTERS) s->count[lane] = 0u;
+  __syncwarp();
+}
+
+// Add the warp's counters to the map's statistics and clear them.
+__device__ __forceinline__ void counts_flush(const MapDev &M, WarpSmem *s, LaneCount &lc,
+                                             int lane) {
+  const unsigned d = __reduce_add_sync(0xffffffffu, lc.dropped);
+  const unsigned c = __reduce_add_sync(0xffffffffu, lc.critical);
+  lc = LaneCount{0u, 0u};
+  __syncwarp();
+  if (lane < MM_N_COUNTERS) {
+    unsigned v = s->count[lane];
+    if (lane == ST_DROPPED) v = d;
+    if (lane == ST_CRITICAL) v = c;
+    // every multi-pixel triangle is of one of the four kinds
+    if (lane == ST_CLIPPED)
+      v = s->count[ST_QUAD] + s->count[ST_BOX] + s->count[ST_ROWS] + s->count[ST_LINE];
+    if (v) atomicAdd(&M.stat[lane], (unsigned long long)v);
+  }
+  __syncwarp();
+  if (lane < MM_N_COUNTERS) s->count[lane] = 0u;
+  __syncwarp();
+}
 
 }  // namespace mm

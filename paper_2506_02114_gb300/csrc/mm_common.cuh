@@ -70,8 +70,8 @@ struct __align__(16) Vtx {
   float fx, fy;
 };
 
-struct TriJob;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
-#define MM_TRIJOB_BYTES 48
+struct RawTri;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
+#define MM_TRIJOB_BYTES 32
 
 // Everything the deflection + mapping kernel needs about one map.
 struct MapDev {
@@ -114,7 +114,7 @@ struct MapDev {
   // statistics (per map)
   unsigned long long *stat;   // triangle counters, see IpmCounters
   // larger triangles handed to the second kernel (capacity 0: none)
-  TriJob *bigq;
+  RawTri *bigq;
   unsigned long long *bigq_n; // [0] triangles queued, [1] the second kernel's batch counter
   int64_t bigq_cap;
 };

@@ -284,35 +284,21 @@ __device__ __forceinline__ bool cell_beyond_map(const MapDev &M, const Vtx &a, c
   return x0 != MM_VTX_INVALID && (x1 < 0 || x0 >= M.npix || y1 < 0 || y0 >= M.npix_y);
 }
 
-__device__ __forceinline__ Vtx shfl_down_vtx(const Vtx &v, int d) {
-  Vtx r;
-  r.px = __shfl_down_sync(0xffffffffu, v.px, d);
-  r.py = __shfl_down_sync(0xffffffffu, v.py, d);
-  r.fx = __shfl_down_sync(0xffffffffu, v.fx, d);
-  r.fy = __shfl_down_sync(0xffffffffu, v.fy, d);
-  return r;
-}
-
-// Warp-reduce the per-lane triangle counters into the map's statistics.
-__device__ __forceinline__ void flush_counters(const MapDev &M, IpmCounters &cnt, int lane) {
-  unsigned v[MM_N_COUNTERS] = {cnt.dropped, cnt.clipped, cnt.small,  cnt.strip,
-                               cnt.big,     cnt.line,    cnt.culled, cnt.critical};
-#pragma unroll
-  for (int k = 0; k < MM_N_COUNTERS; k++) {
-    for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], d);
-    if (lane == 0 && v[k]) atomicAdd(&M.stat[k], (unsigned long long)v[k]);
-  }
-  cnt = IpmCounters{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-}
-
 // Persistent warps; each work item is a strip of 31 cell columns by
 // rows_per_item cell rows of one map.  Lane l computes vertex column
 // 31*s + l for every vertex row of the item, keeps the previous row in
 // registers and takes its right neighbour's vertices by shuffle; lanes 0..30
 // then map cells (i, j-1) as the triangles {v00, v10, v11} and
 // {v00, v11, v01} (diagonal from lower-left to upper-right).
+// Issue- and latency-bound (no pipe saturated): the kernel is shaped to run 3
+// blocks of 8 warps per SM, 80 registers a thread without spills -- the row
+// below waits in shared memory, every apportioning waits in queues emptied
+// once a row, when no vertex is live, and the counters are kept per warp.
+// 2000^2 map, 9 rays per pixel: 16.9 ms at 2 blocks with the apportioning in
+// divergent branches, 15.3 ms with the queues at 2 blocks, 13.0 ms at 3 (4
+// spill and are slower).
 #ifndef MM_SHOOT_MINB
-#define MM_SHOOT_MINB 2  // resident 256-thread blocks per SM the register budget targets
+#define MM_SHOOT_MINB 3  // resident 256-thread blocks per SM the register budget targets
 #endif
 
 // A single map (BATCH = false) arrives by value as a launch parameter, so
@@ -325,10 +311,9 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
   const int lane = threadIdx.x & 31;
   extern __shared__ __align__(16) unsigned char s_dyn[];
   WarpSmem *ws = reinterpret_cast<WarpSmem *>(s_dyn) + (threadIdx.x >> 5);
-  WarpQueue wq = {ws->quad, 0};
-  LineQueue lq = {ws->line, 0};
-  JobQueue jq = {ws->big, &ws->rows, 0};
-  IpmCounters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
+  WarpQueues q = {ws, 0, 0, 0};
+  LaneCount lc = {0u, 0u};
+  counts_clear(ws, lane);
   int last_map = -1;
   // A batch's current map, copied per warp into shared memory when the warp
   // moves to another map: its fields are then read there like a launch
@@ -355,7 +340,7 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
       mi = lo;
     }
     if (BATCH && mi != last_map) {  // warp-uniform
-      if (last_map >= 0) flush_counters(SM, cnt, lane);
+      if (last_map >= 0) counts_flush(SM, ws, lc, lane);
       __syncwarp();
       const unsigned long long *src = reinterpret_cast<const unsigned long long *>(maps + mi);
       unsigned long long *dst = reinterpret_cast<unsigned long long *>(&SM);
@@ -375,109 +360,100 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     const bool vvalid = i <= col_end;  // vertex columns [col_begin, col_end]
     const int cx = __ldg(&M.col_cell[vvalid ? i : col_end]);
     const bool cell_col = (lane < MM_STRIP) && (i < col_end);
-    RunAcc ra = {-1, 0ull};
-    Vtx prev, prev_r;  // this lane's vertex of the previous row and its right neighbour's
+    RunAcc ra = MM_RUN_NONE;
     // culling state of the previous row (warp-uniform): the map edge it is
-    // proven to lie beyond, and whether its vertices were computed
-    int prev_side = MM_CULL_NONE;
-    bool prev_exact = true;
-    {
-      const int leaf = lookup_leaf(M, cx, __ldg(&M.row_cell[jb]));
-      if (leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
-      prev = shoot_point<SQUARE, false, PRELOAD>(M, leaf, i, jb, 0.f, 0.f, vvalid);
-      prev_r = shfl_down_vtx(prev, 1);
-      int run;
-      if (M.cull) prev_side = row_cull_side<SQUARE>(M, leaf, i, jb, vvalid, run);
-    }
-    // one pass more than there are cell rows: the last one maps nothing and
-    // shares out what is left in the queue of larger triangles
+    // proven to lie beyond, and whether its vertices were computed (they are
+    // in ws->row); `side` is row j's
+    int prev_side = MM_CULL_NONE, side = MM_CULL_NONE;
+    bool prev_exact = false;
     int c_gy = INT_MIN, c_leaf = -1;  // lookup cache of this lane's column
     bool c_cull = false;              // the cached record has a culling bound
     int cull_wait = 0, cull_pause = 0;  // rows left before the next culling test
-    for (int j = jb + 1;; j++) {
+    // One pass shoots one vertex row and maps the cells between it and the
+    // row below: row jb (nothing to map), then rows j = jb + 1 .. je; a row
+    // below that culling left out is shot first (`back`).  One pass more
+    // shares out what is left in the queues.
+    bool back = false;
+    for (int j = jb;;) {
       const bool fin = j > je;  // warp-uniform
-      Vtx cur = prev, cur_r = prev_r;
-      int side = MM_CULL_NONE;
+      Vtx v00, v10, v11, v01;
+      v00.px = v10.px = v11.px = v01.px = v00.py = v10.py = v11.py = v01.py = 0;
+      v00.fx = v10.fx = v11.fx = v01.fx = v00.fy = v10.fy = v11.fy = v01.fy = 0.f;
       if (!fin) {
-        const int cy = __ldg(&M.row_cell[j]);
-        const int leaf = lookup_leaf_cached(M, cx, cy, c_gy, c_leaf, c_cull);
+        int js = j;
+        int leaf =
+            lookup_leaf_cached(M, cx, __ldg(&M.row_cell[js]), c_gy, c_leaf, c_cull);
         if (leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
         // a row is provably beyond the map only if every lane's record has a
         // culling bound; otherwise the per-vertex test cannot succeed
-        if (M.cull) {
+        if (M.cull && !back) {
           int run = 0;
+          side = MM_CULL_NONE;
           if (cull_wait > 0) {
             cull_wait--;
           } else if (!__any_sync(0xffffffffu, vvalid && !c_cull)) {
             side = row_cull_side<SQUARE>(M, leaf, i, j, vvalid, run);
             // a failed test pauses the tests of the next rows (1, 3, ... up to 8)
-            cull_pause = side == MM_CULL_NONE ? min(2 * cull_pause + 1, 8) : 0;
-            cull_wait = cull_pause;
+            if (j > jb) {
+              cull_pause = side == MM_CULL_NONE ? min(2 * cull_pause + 1, 8) : 0;
+              cull_wait = cull_pause;
+            }
           }
-          if (side != MM_CULL_NONE && side == prev_side) {
+          if (j > jb && side != MM_CULL_NONE && side == prev_side) {
             // rows j .. j + run - 1 and the one below lie beyond the same map
             // edge: the cells between them map nothing, and none of those
             // rows is computed
             const int skip = min(run, je - j + 1);
             prev_exact = false;
-            if (lane == 0) cnt.culled += (unsigned)skip;
-            j += skip - 1;
+            if (lane == 0) ws->count[ST_CULLED] += (unsigned)skip;
+            j += skip;
             continue;
           }
-          if (!prev_exact) {
-            // the row below was not computed; its cells with this row are needed
-            const int lp = lookup_leaf(M, cx, __ldg(&M.row_cell[j - 1]));
-            prev = shoot_point<SQUARE, false, PRELOAD>(M, lp, i, j - 1, 0.f, 0.f, vvalid);
-            prev_r = shfl_down_vtx(prev, 1);
-            prev_exact = true;
-          }
         }
-        cur = shoot_point<SQUARE, false, PRELOAD>(M, leaf, i, j, 0.f, 0.f, vvalid);
-        cur_r = shfl_down_vtx(cur, 1);
+        if (j > jb && !prev_exact) {
+          // the row below was not computed; its cells with this row are needed
+          js = j - 1;
+          leaf = lookup_leaf(M, cx, __ldg(&M.row_cell[js]));
+        }
+        v01 = shoot_point<SQUARE, false, PRELOAD>(M, leaf, i, js, 0.f, 0.f, vvalid);
+        // the row below waits in shared memory (not in eight registers held
+        // across the deflection), where a lane also finds its right neighbour
+        v00 = ws->row[lane];
+        v10 = ws->row[min(lane + 1, 31)];
+        __syncwarp();
+        ws->row[lane] = v01;
+        __syncwarp();
+        if (j == jb || js < j) {
+          back = js < j;
+          prev_exact = true;
+          if (j == jb) {
+            prev_side = side;
+            j++;
+          }
+          continue;
+        }
+        back = false;
+        v11 = ws->row[min(lane + 1, 31)];
+        prev_side = side;
         // a row of cells all beyond the map (and none with a non-finite
         // vertex, which must be counted) has nothing to map
-        if (__all_sync(0xffffffffu, !cell_col || cell_beyond_map(M, prev, prev_r, cur, cur_r))) {
-          prev = cur;
-          prev_r = cur_r;
-          prev_side = side;
+        if (__all_sync(0xffffffffu, !cell_col || cell_beyond_map(M, v00, v10, v01, v11))) {
+          j++;
           continue;
         }
       }
-#pragma unroll 1
-      for (int tri = 0; tri < 2; tri++) {
-        TriJob job;
-        SmallTri se;
-        LineTri le;
-        // triangle 0: (v00, v10, v11); triangle 1: (v00, v11, v01)
-        Vtx vb, vc;
-        vb.px = tri ? cur_r.px : prev_r.px;
-        vb.py = tri ? cur_r.py : prev_r.py;
-        vb.fx = tri ? cur_r.fx : prev_r.fx;
-        vb.fy = tri ? cur_r.fy : prev_r.fy;
-        vc.px = tri ? cur.px : cur_r.px;
-        vc.py = tri ? cur.py : cur_r.py;
-        vc.fx = tri ? cur.fx : cur_r.fx;
-        vc.fy = tri ? cur.fy : cur_r.fy;
-        const int code =
-            (cell_col && !fin) ? ipm_triangle<!BATCH>(M, prev, vb, vc, ra, cnt, se, job, le)
-                               : TRI_DONE;
-        // (the batch kernel, which reads its maps from memory, has no
-        // registers to spare for the line queue's state)
-        if (!BATCH) lq_push(M, lq, code == TRI_LINE, le, lane);
-        wq_push(M, wq, code == TRI_SMALL, se, lane);
-        jq_add(jq, code == TRI_BIG, job, lane);
-        jq_share(M, jq, fin && tri == 1, lane);
+      // (diagonal v00 - v11)
+      if (!fin) {
+        tri_scan(M, q, v00, v10, v11, cell_col, ra, lc, lane);
+        tri_scan(M, q, v00, v11, v01, cell_col, ra, lc, lane);
       }
+      share_out(M, q, fin, lc, lane);
       if (fin) break;
-      prev = cur;
-      prev_r = cur_r;
-      prev_side = side;
+      j++;
     }
-    run_flush(M, ra);
-    if (!BATCH) lq_drain(M, lq, lane);
-    wq_drain(M, wq, lane);
+    run_flush<MM_FIX_ONE>(M, ra);
   }
-  if (last_map >= 0) flush_counters(BATCH ? SM : M1, cnt, lane);
+  if (last_map >= 0) counts_flush(BATCH ? SM : M1, ws, lc, lane);
 }
 
 // Inverse ray shooting (Sec. 3.2; the IRS column of Table 1): every grid
@@ -498,7 +474,7 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
     k_shoot_irs(const MapDev M, int64_t total_work, unsigned long long *work_counter,
                 unsigned *err) {
   const int lane = threadIdx.x & 31;
-  IpmCounters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
+  unsigned dropped = 0, culled = 0;
   while (true) {
     unsigned long long w = 0;
     if (lane == 0) w = atomicAdd(work_counter, 1ull);
@@ -514,7 +490,7 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
     const bool vvalid = i <= col_end;
     const bool owner = vvalid && (lane < MM_STRIP || i == col_end);
     const int cx = __ldg(&M.col_cell[vvalid ? i : col_end]);
-    RunAcc ra = {-1, 0ull};
+    RunAcc ra = MM_RUN_NONE;
     int c_gy = INT_MIN, c_leaf = -1;  // lookup cache of this lane's column
     bool c_cull = false;              // the cached record has a culling bound
     int cull_wait = 0, cull_pause = 0;  // rows left before the next culling test
@@ -527,7 +503,7 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
         int run;
         if (row_cull_side<SQUARE>(M, leaf, i, j, vvalid, run) != MM_CULL_NONE) {
           const int skip = min(run, jl - j + 1);
-          if (lane == 0) cnt.culled += (unsigned)skip;
+          if (lane == 0) culled += (unsigned)skip;
           j += skip - 1;
           cull_pause = 0;
           continue;
@@ -539,20 +515,22 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
       const Vtx v = shoot_point<SQUARE, false>(M, leaf, i, j, 0.f, 0.f, vvalid);
       if (owner) {
         if (v.px == MM_VTX_INVALID)
-          cnt.dropped++;
+          dropped++;
         else if (v.px >= 0 && v.px < M.npix && v.py >= 0 && v.py < M.npix_y)
-          run_add(M, ra, (long long)v.py * M.npix + v.px, 1ull);
+          run_add<1ull>(M, ra, v.px, v.py);
       }
     }
-    run_flush(M, ra);
+    run_flush<1ull>(M, ra);
   }
-  flush_counters(M, cnt, lane);
+  dropped = __reduce_add_sync(0xffffffffu, dropped);
+  if (lane == 0 && dropped) atomicAdd(&M.stat[ST_DROPPED], (unsigned long long)dropped);
+  if (lane == 0 && culled) atomicAdd(&M.stat[ST_CULLED], (unsigned long long)culled);
 }
 
 // Second pass over the larger triangles k_shoot_ipm (or k_ipm_vertices)
 // queued for the map: each warp takes batches of 32 from the device queue
 // and deals out their pixel rows and partially covered pixels
-// (warp_tri_jobs), at 5 blocks per SM where the first kernel runs 2 (48
+// (warp_tri_jobs), at 5 blocks per SM where the first kernel runs 3 (48
 // registers allow 5 without spills: 3 % faster than 4; 6 forces spills)
 #define MM_BIG_MINB 5
 __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
@@ -569,7 +547,7 @@ __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
     const long long base = (long long)b * 32;
     if (base >= n) break;
     const int nb = (int)min(32ll, n - base);
-    if (lane < nb) q[w][lane] = M.bigq[base + lane];
+    if (lane < nb) q[w][lane] = make_job(raw_load(M.bigq + base + lane));
     __syncwarp();
     warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q[w], nb, &rr[w], lane);
   }

@@ -1,0 +1,47 @@
+"""The first pass's warp queues and the map's device queue: where a larger
+triangle is apportioned (second pass, or in the first pass when the queue is
+absent or full) must not change the map, bit for bit, whatever the width of
+the last strip of cells and however many triangles a row of cells adds."""
+import numpy as np
+import pytest
+
+import paper_2506_02114_gb300 as mm
+import synthetic
+from _metrics import MAP_P999_TOL, MEAN_TOL, band_errors
+
+pytestmark = pytest.mark.gpu
+
+# close to critical in y: nearly every triangle of a row is a larger one, so a
+# row adds up to 62 to a queue; and an ordinary model with every kind
+MODELS = {"slivers": (0.8, 0.17, 0.0, 4.0), "mixed": (0.45, 0.3, 0.4, 10.0)}
+
+
+@pytest.mark.parametrize("cols", [1, 30, 31, 32, 95])
+@pytest.mark.parametrize("model", sorted(MODELS))
+def test_queue_capacity_does_not_change_the_map(oracle_mod, model, cols):
+    import torch
+    torch.cuda.init()
+    kappa, gamma, s, rpp = MODELS[model]
+    m, pos = synthetic.star_field(11, 120, 16.0, synthetic.SALPETER_01_1)
+    rows = 700
+    half = (0.5 * cols * 0.05, 0.5 * rows * 0.02)
+    maps, counts = [], []
+    for slots in (0, -1, 1, 33, 1000):
+        h = mm.create(kappa, gamma, s, m, pos, 1.0, 40, fmm_order=25, img_half=half,
+                      ray_grid=(cols + 1, rows + 1), big_queue_slots=slots)
+        mm.run(h, 0)
+        maps.append(mm.get_map_fixed(h))
+        st = mm.get_stats(h)
+        assert st["error_bits"] == 0
+        counts.append([st[k] for k in st if k.startswith("triangles_")])
+        if slots == 0:
+            mu = mm.get_map(h)
+        mm.destroy(h)
+    assert maps[0].any()
+    for k in range(1, len(maps)):
+        assert np.array_equal(maps[0], maps[k]) and counts[0] == counts[k]
+    p = oracle_mod.derive_params(kappa, gamma, s, m, 1.0, 40, img_half=half,
+                                 ray_grid=(cols + 1, rows + 1))
+    mu_ref, _ = oracle_mod.magnification_map(p, m, pos)
+    e = band_errors(mu, mu_ref, p.mu_macro)
+    assert e["p999"] <= MAP_P999_TOL and (cols < 30 or e["mean_rel"] <= MEAN_TOL), e
