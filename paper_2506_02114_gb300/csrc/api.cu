@@ -187,7 +187,8 @@ struct mm_map {
   int64_t n_nodes = 0;
   DBuf<int64_t> d_level_off;
   DBuf<uint64_t> code;
-  DBuf<int32_t> lvl, sbeg, send, first_child, split, scan;
+  DBuf<int32_t> lvl, sbeg, send, first_child, parent, nb, split, group, top_info;
+  int top_end = 0;                 // first level not built by the top kernel
 
   // active region
   DBuf<int32_t> col_cell, row_cell, node_act, leaf_flag, leaf_scan, node_active, active_list;
@@ -361,6 +362,8 @@ static TreeDev tree_dev(const mm_map *h) {
   T.sbeg = h->sbeg.p;
   T.send = h->send.p;
   T.first_child = h->first_child.p;
+  T.parent = h->parent.p;
+  T.nb = h->nb.p;
   T.level_off = h->d_level_off.p;
   T.depth = h->depth;
   return T;
@@ -415,6 +418,23 @@ static mm_status upload_level_off(mm_map *h, cudaStream_t st) {
   return MM_OK;
 }
 
+static TreeOut tree_out(const mm_map *h) {
+  return TreeOut{h->code.p, h->lvl.p,    h->sbeg.p, h->send.p,
+                 h->first_child.p, h->parent.p, h->nb.p,   h->d_level_off.p};
+}
+
+// Room for `count` tree nodes (contents kept).
+static mm_status ensure_nodes(mm_map *h, int64_t count) {
+  CK(h->code.ensure(count, true));
+  CK(h->lvl.ensure(count, true));
+  CK(h->sbeg.ensure(count, true));
+  CK(h->send.ensure(count, true));
+  CK(h->first_child.ensure(count, true));
+  CK(h->parent.ensure(count, true));
+  CK(h->nb.ensure(9 * count, true));
+  return MM_OK;
+}
+
 // Morton sort + levels.  plan: learn and store the level counts (host reads).
 static mm_status run_tree(mm_map *h, cudaStream_t st, bool plan) {
   const int64_t N = h->N;
@@ -439,55 +459,55 @@ static mm_status run_tree(mm_map *h, cudaStream_t st, bool plan) {
   if (plan) {
     h->level_off.assign(MM_DMAX + 2, 0);
     h->level_cnt.assign(MM_DMAX + 2, 0);
-    h->level_off[0] = 0;
-    h->level_cnt[0] = 1;
-    h->level_off[1] = 1;
     CK(h->d_level_off.ensure(MM_DMAX + 2));
+    CK(h->top_info.ensure(MM_TOP_INFO));
+    CK(h->group.ensure(1));
     if (!h->pin) CK(cudaMallocHost(&h->pin, (8 + MM_DMAX + 2) * sizeof(int64_t)));
-    CKS(upload_level_off(h, st));
-    CK(h->code.ensure(5, true));
-    CK(h->lvl.ensure(5, true));
-    CK(h->sbeg.ensure(5, true));
-    CK(h->send.ensure(5, true));
-    CK(h->first_child.ensure(5, true));
+    CKS(ensure_nodes(h, MM_TOP_CAPACITY));
   }
-  LCH(launch_root_init(N, h->code.p, h->lvl.p, h->sbeg.p, h->send.p, st));
-  for (int l = 0; l <= MM_DMAX; l++) {
+  LCH(launch_tree_top(tree_dev(h), tree_out(h), h->leaf_size, h->top_info.p, st));
+  if (plan) {
+    int32_t info[MM_TOP_INFO];
+    static_assert(sizeof info <= (8 + MM_DMAX + 2) * sizeof(int64_t), "pinned scratch");
+    CK(cudaMemcpyAsync(h->pin, h->top_info.p, sizeof info, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    memcpy(info, h->pin, sizeof info);
+    h->top_end = info[0];
+    for (int l = 0; l <= std::min(info[0], MM_DMAX + 1); l++) {
+      h->level_cnt[l] = info[2 + l];
+      if (l <= MM_DMAX) h->level_off[l + 1] = h->level_off[l] + info[2 + l];
+    }
+    if (info[1]) {  // complete
+      h->depth = info[0] - 1;
+      h->n_nodes = h->level_off[info[0]];
+    } else {
+      h->depth = -1;
+    }
+  }
+  for (int l = h->top_end; l <= MM_DMAX && h->level_cnt[l] > 0; l++) {
     const int64_t n = h->level_cnt[l];
     if (plan) {
       CK(h->split.ensure(n));
-      CK(h->scan.ensure(n));
+      CK(h->group.ensure((n + MM_SPLIT_GROUP - 1) / MM_SPLIT_GROUP));
+      CK(cudaMemsetAsync(h->top_info.p, 0, sizeof(int32_t), st));
     }
-    TreeDev T = tree_dev(h);
-    LCH(launch_level_split(T, l, n, h->leaf_size, h->split.p, st));
-    CKS(cub_call(h, plan, [&](void *tmp, size_t &bytes) {
-      return cub::DeviceScan::ExclusiveSum(tmp, bytes, h->split.p, h->scan.p, (int)n, st);
-    }));
+    LCH(launch_level_split(tree_dev(h), tree_out(h), l, n, h->leaf_size, h->split.p, h->group.p,
+                           plan ? h->top_info.p : nullptr, st));
     if (plan) {
-      const int32_t *src[2] = {h->scan.p + (n - 1), h->split.p + (n - 1)};
-      int32_t ab[2];
-      CKS(read_ints(h, st, 2, src, ab));
-      const int64_t nxt = 4 * (int64_t)(ab[0] + ab[1]);
+      const int32_t *src[1] = {h->top_info.p};
+      int32_t total;
+      CKS(read_ints(h, st, 1, src, &total));
+      const int64_t nxt = 4 * (int64_t)total;
       h->level_cnt[l + 1] = nxt;
       h->level_off[l + 1] = h->level_off[l] + n;
       if (l + 2 <= MM_DMAX + 1) h->level_off[l + 2] = h->level_off[l + 1] + nxt;
-      const int64_t need = h->level_off[l + 1] + nxt;
-      CK(h->code.ensure(need, true));
-      CK(h->lvl.ensure(need, true));
-      CK(h->sbeg.ensure(need, true));
-      CK(h->send.ensure(need, true));
-      CK(h->first_child.ensure(need, true));
+      CKS(ensure_nodes(h, h->level_off[l + 1] + nxt));
       CKS(upload_level_off(h, st));
-      T = tree_dev(h);
     }
-    LCH(launch_level_children(T, l, n, h->split.p, h->scan.p, h->code.p, h->lvl.p, h->sbeg.p,
-                             h->send.p, h->first_child.p, st));
-    if (h->level_cnt[l + 1] == 0) {
-      if (plan) {
-        h->depth = l;
-        h->n_nodes = h->level_off[l + 1];
-      }
-      break;
+    LCH(launch_level_children(tree_dev(h), tree_out(h), l, n, h->split.p, h->group.p, st));
+    if (plan && h->level_cnt[l + 1] == 0) {
+      h->depth = l;
+      h->n_nodes = h->level_off[l + 1];
     }
   }
   return MM_OK;
@@ -585,8 +605,9 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   CK(cudaMemsetAsync(h->err.p, 0, sizeof(unsigned), st));
 
   // up-sweep: P2M at every leaf, then M2M level by level towards the root
-  LCH(launch_p2m(T, nn, p, h->mp.p, st));
-  for (int l = h->depth - 1; l >= 0; l--)
+  // (M2L reads multipoles of levels >= 2 only)
+  LCH(launch_p2m(T, nn, p, h->MLop.p, h->mp.p, st));
+  for (int l = h->depth - 1; l >= 2; l--)
     LCH(launch_m2m(T, l, h->level_cnt[l], p, h->MMop.p, h->mp.p, st));
   // down-sweep: levels 0 and 1 have no well-separated nodes
   CK(cudaMemsetAsync(h->loc.p, 0, (size_t)nn * P1 * sizeof(double2), st));
@@ -1718,7 +1739,8 @@ void mm_destroy(mm_map *h) {
   h->d_level_off.release();
   h->code.release();
   DBuf<int32_t> *ibs[] = {&h->lvl,       &h->sbeg,      &h->send,      &h->first_child,
-                          &h->split,     &h->scan,      &h->col_cell,  &h->row_cell,
+                          &h->parent,    &h->nb,        &h->split,     &h->group,
+                          &h->top_info,  &h->col_cell,  &h->row_cell,
                           &h->node_act,  &h->leaf_flag, &h->leaf_scan, &h->node_active,
                           &h->active_list, &h->near_cnt, &h->near_off, &h->grid};
   for (auto *b : ibs) b->release();

@@ -13,6 +13,7 @@
 //
 // The l = 0 (logarithmic) terms of the locals are not formed: the deflection
 // needs only dpsi/dz (Sec. 3.3), so c_0 never reaches a ray.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -37,6 +38,12 @@ __device__ __forceinline__ double2 cpow(double2 z, int k) {
   return r;
 }
 
+// 2^e as a double, -1022 <= e <= 1023.
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// Level, cell, centre and half-length of a node (R0 is a power of two, so
+// every step but the centre's sum is exact; no FP64 division, which takes
+// some twenty instructions of a pipe with 2 lanes per SM).
 __device__ __forceinline__ void node_geom(const TreeDev &T, int64_t node, int &level, int &cx,
                                           int &cy, double &zx, double &zy, double &L) {
   level = T.lvl[node];
@@ -44,87 +51,171 @@ __device__ __forceinline__ void node_geom(const TreeDev &T, int64_t node, int &l
   morton_decode(T.code[node], x, y);
   cx = (int)x;
   cy = (int)y;
-  const double side = 2.0 * T.R0 / (double)(1ll << level);
+  const double side = 2.0 * T.R0 * pow2(-level);
   zx = -T.R0 + ((double)cx + 0.5) * side;
   zy = -T.R0 + ((double)cy + 0.5) * side;
   L = 0.5 * side;
 }
 
-// Node id of the level-`level` cell (x, y), or -1 if that cell is not a node.
-__device__ __forceinline__ int64_t find_node(const TreeDev &T, int level, int x, int y) {
-  const int side = 1 << level;
-  if (x < 0 || y < 0 || x >= side || y >= side) return -1;
-  const uint64_t c = morton2((uint32_t)x, (uint32_t)y);
-  int64_t lo = T.level_off[level], hi = T.level_off[level + 1];
-  int64_t k = lower_bound_u64(T.code, lo, hi, c);
-  return (k < hi && T.code[k] == c) ? k : -1;
+// 1/L of a power of two L = 2^e, exactly.
+__device__ __forceinline__ double inv_pow2(double L) {
+  return pow2(1023 - (__double2hiint(L) >> 20));
+}
+
+// x / k, correctly rounded, from the rounded reciprocal of the small integer
+// k (Markstein's correction of the quotient by its exact remainder).
+__device__ __forceinline__ double div_by(double x, double k, double inv_k) {
+  const double q = x * inv_k;
+  return fma(fma(-k, q, x), inv_k, q);
+}
+
+// Squares z^2, z^4, ... for power_of.
+#define MM_POW_BITS 7  // exponents up to MM_PMAX
+__device__ __forceinline__ void powers_of_two(double2 z, int kmax, double2 *sq) {
+  sq[0] = z;
+  for (int b = 1; b < MM_POW_BITS && (1 << b) <= kmax; b++) {
+    z = cmul(z, z);
+    sq[b] = z;
+  }
+}
+// z^k (k >= 1) from the squares, multiplied in the order of the binary digits
+// from the lowest.
+__device__ __forceinline__ double2 power_of(const double2 *sq, int k) {
+  int b = __ffs(k) - 1;
+  double2 r = sq[b];
+  for (k >>= b + 1, b++; k; k >>= 1, b++)
+    if (k & 1) r = cmul(r, sq[b]);
+  return r;
 }
 
 // ---------------------------------------------------------------------------
 // P2M: a_0 = sum m_i, a_k = -(1/k) sum m_i zeta_i^k  (leaves only)
+// FP64-bound: one thread per (node, coefficient), so that the lanes stay full
+// whatever p; a star's repeated squares are formed once for all of its
+// powers.  50 000 stars, p = 25: 0.25 ms with a block per node and the
+// squares formed by every thread, 0.11 ms like this.
 // ---------------------------------------------------------------------------
-__global__ void k_p2m(TreeDev T, int64_t n_nodes, int p, double2 *mp) {
-  const int64_t node = blockIdx.x;
-  if (node >= n_nodes || T.first_child[node] >= 0) return;
-  const int k = threadIdx.x;
-  if (k > p) return;
-  int level, cx, cy;
-  double zx, zy, L;
-  node_geom(T, node, level, cx, cy, zx, zy, L);
-  const double invL = 1.0 / L;
+#define MM_P2M_THREADS 128
+#define MM_P2M_STARS 8  // stars of a node staged at a time
+__global__ void __launch_bounds__(MM_P2M_THREADS)
+    k_p2m(TreeDev T, int64_t n_nodes, int p, int per_block, const double *__restrict__ inv,
+          double2 *mp) {
+  extern __shared__ __align__(16) double2 s_p2m[];
+  const int P1 = p + 1;
+  // per node and staged star: the squares, then the mass
+  double2 *sq = s_p2m;
+  double *sm = reinterpret_cast<double *>(sq + per_block * MM_P2M_STARS * MM_POW_BITS);
+  const int64_t first = (int64_t)blockIdx.x * per_block;
+  const int local = threadIdx.x / P1, k = threadIdx.x - local * P1;
+  const int64_t node = first + local;
+  const bool mine = local < per_block && node < n_nodes && T.first_child[node] < 0;
+  const int b = mine ? T.sbeg[node] : 0, e = mine ? T.send[node] : 0;
+  // the block's longest node
+  int longest = 0;
+  for (int q = 0; q < per_block; q++) {
+    const int64_t nd = first + q;
+    if (nd < n_nodes && T.first_child[nd] < 0) longest = max(longest, T.send[nd] - T.sbeg[nd]);
+  }
   double2 s = make_double2(0.0, 0.0);
-  for (int64_t i = T.sbeg[node]; i < T.send[node]; i++) {
-    const double m = T.sm[i];
-    if (k == 0) {
-      s.x += m;
-    } else {
-      double2 zeta = make_double2((T.sx[i] - zx) * invL, (T.sy[i] - zy) * invL);
-      double2 zk = cpow(zeta, k);
-      s.x = fma(m, zk.x, s.x);
-      s.y = fma(m, zk.y, s.y);
+  for (int c = 0; c < longest; c += MM_P2M_STARS) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < per_block * MM_P2M_STARS; t += MM_P2M_THREADS) {
+      const int64_t nd = first + t / MM_P2M_STARS;
+      if (nd >= n_nodes || T.first_child[nd] >= 0) continue;
+      const int i = T.sbeg[nd] + c + t % MM_P2M_STARS;
+      if (i >= T.send[nd]) continue;
+      int level, cx, cy;
+      double zx, zy, L;
+      node_geom(T, nd, level, cx, cy, zx, zy, L);
+      const double invL = inv_pow2(L);
+      powers_of_two(make_double2((T.sx[i] - zx) * invL, (T.sy[i] - zy) * invL), p,
+                    sq + t * MM_POW_BITS);
+      sm[t] = T.sm[i];
+    }
+    __syncthreads();
+    const int cnt = min(MM_P2M_STARS, e - b - c);
+    for (int i = 0; i < cnt; i++) {
+      const int t = local * MM_P2M_STARS + i;
+      const double m = sm[t];
+      if (k == 0) {
+        s.x += m;
+      } else {
+        const double2 zk = power_of(sq + t * MM_POW_BITS, k);
+        s.x = fma(m, zk.x, s.x);
+        s.y = fma(m, zk.y, s.y);
+      }
     }
   }
-  if (k > 0) s = make_double2(-s.x / k, -s.y / k);
-  mp[node * (p + 1) + k] = s;
+  if (!mine || b == e) return;  // (a node without stars is nobody's source)
+  if (k > 0) {
+    const double dk = (double)k, ik = inv[k];
+    s = make_double2(div_by(-s.x, dk, ik), div_by(-s.y, dk, ik));
+  }
+  mp[node * P1 + k] = s;
 }
 
 // ---------------------------------------------------------------------------
 // M2M: parent b = sum over the four children of MM[q] a_child (App. C.2)
+// FP64-bound at the fine levels and a chain of latencies at the coarse ones:
+// a thread takes rows l and p + 1 - l of one child (p + 1 terms whatever l,
+// so that the triangle of binomials keeps every lane busy), and the four
+// children's sums are added up afterwards in their order.  Children without
+// stars (a quarter of the finest) add exact zeros and are left out.  Finest
+// level of 50 000 stars, p = 25: 148 us with a thread per row and the
+// children one after another, 101 us like this.
 // ---------------------------------------------------------------------------
-__global__ void k_m2m(TreeDev T, int level, int64_t n, int p, const double2 *__restrict__ MMop,
-                      double2 *mp) {
-  const int64_t node = T.level_off[level] + blockIdx.x;
-  if ((int64_t)blockIdx.x >= n) return;
-  const int fc = T.first_child[node];
-  if (fc < 0) return;
-  __shared__ double2 a[4][MM_PMAX + 1];
-  const int P1 = p + 1;
+__global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
+                      const double2 *__restrict__ MMop, double2 *mp) {
+  extern __shared__ __align__(16) double2 s_m2m[];
+  const int P1 = p + 1, half = (p + 1) / 2;
+  double2 *a = s_m2m, *t = s_m2m + per_block * 4 * P1;  // [node][child][k]
+  const int64_t first = T.level_off[level] + (int64_t)blockIdx.x * per_block;
+  const int cnt = (int)min((int64_t)per_block, n - (int64_t)blockIdx.x * per_block);
   // factored M2M: b_k = z0^-k a_k per child, then
   // c_l = sum_q (z0/2)^l (-a_0 / l + sum_{k<=l} C(l-1, k-1) b_k), c_0 = sum_q a_0
-  for (int idx = threadIdx.x; idx < 4 * P1; idx += blockDim.x) {
-    const int q = idx / P1, k = idx % P1;
+  for (int idx = threadIdx.x; idx < cnt * 4 * P1; idx += blockDim.x) {
+    const int nq = idx / P1, k = idx - nq * P1, q = nq & 3;
+    const int fc = T.first_child[first + (nq >> 2)];
+    if (fc < 0 || T.sbeg[fc + q] == T.send[fc + q]) continue;
     const double2 v = mp[(int64_t)(fc + q) * P1 + k];
-    a[q][k] = k ? cfma(MMop[(int64_t)P1 * P1 + q * 2 * P1 + k], v, make_double2(0.0, 0.0)) : v;
+    a[idx] = k ? cfma(MMop[(int64_t)P1 * P1 + q * 2 * P1 + k], v, make_double2(0.0, 0.0)) : v;
   }
   __syncthreads();
-  const int l = threadIdx.x;
-  if (l > p) return;
-  double2 s = make_double2(0.0, 0.0);
-  if (l == 0) {
-    for (int q = 0; q < 4; q++) s = make_double2(s.x + a[q][0].x, s.y + a[q][0].y);
-  } else {
-    const double2 *bl = MMop + (int64_t)l * P1;  // binomials of row l, 1/l at k = 0
-    for (int q = 0; q < 4; q++) {
-      double tx = -a[q][0].x * bl[0].x, ty = -a[q][0].y * bl[0].x;
+  const double *bt = reinterpret_cast<const double *>(MMop);  // binomials [k][l], 1/l at k = 0
+  for (int idx = threadIdx.x; idx < cnt * 4 * half; idx += blockDim.x) {
+    const int nq = idx / half, r = idx - nq * half;
+    const int fc = T.first_child[first + (nq >> 2)];
+    if (fc < 0 || T.sbeg[fc + (nq & 3)] == T.send[fc + (nq & 3)]) continue;
+    const double2 *src = a + nq * P1;
+    const int rows = 2 * (r + 1) == p + 1 ? 1 : 2;  // (the middle row of an odd p, once)
+    for (int h = 0; h < rows; h++) {
+      const int l = h ? p - r : r + 1;
+      double tx = -src[0].x * bt[l], ty = -src[0].y * bt[l];
       for (int k = 1; k <= l; k++) {
-        const double b = bl[k].x;
-        tx = fma(b, a[q][k].x, tx);
-        ty = fma(b, a[q][k].y, ty);
+        const double b = bt[k * P1 + l];
+        tx = fma(b, src[k].x, tx);
+        ty = fma(b, src[k].y, ty);
       }
-      s = cfma(MMop[(int64_t)P1 * P1 + q * 2 * P1 + P1 + l], make_double2(tx, ty), s);
+      t[nq * P1 + l] = make_double2(tx, ty);
     }
   }
-  mp[node * P1 + l] = s;
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < cnt * P1; idx += blockDim.x) {
+    const int nd = idx / P1, l = idx - nd * P1;
+    const int fc = T.first_child[first + nd];
+    if (fc < 0) continue;
+    double2 s = make_double2(0.0, 0.0);
+    for (int q = 0; q < 4; q++) {
+      if (T.sbeg[fc + q] == T.send[fc + q]) continue;
+      if (l == 0) {
+        const double2 a0 = a[(nd * 4 + q) * P1];
+        s = make_double2(s.x + a0.x, s.y + a0.y);
+      } else {
+        s = cfma(MMop[(int64_t)P1 * P1 + q * 2 * P1 + P1 + l], t[(nd * 4 + q) * P1 + l], s);
+      }
+    }
+    mp[(first + nd) * P1 + l] = s;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -132,93 +223,196 @@ __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, const double2 *__r
 //   L2L from the parent, M2L from the parent's neighbours' children that are
 //   not adjacent (<= 27), P2L from the parent's unsplit neighbours that are
 //   not adjacent (<= 5).
+// One block per node.  The sums over k of all its sources are independent:
+// thread (group g, row l) takes sources g, g + G, ... two at a time, which
+// fills the lanes for any p and gives each binomial it loads two uses; the
+// sources' results are then added up row by row in the order of the list.
+// FP64-bound at the fine levels (about 60 p instructions a source), latency
+// at the coarse ones, where the sources one after another took 100 us a level
+// whatever its size.  Sources without stars (a quarter of the finest level's)
+// add exact zeros and are left out.  50 000 stars, p = 25: 1.21 ms over all
+// levels with a warp per node, 0.62 ms like this; the finest level 477 and
+// 291 us, with the FP64 pipe 93 % busy both times.
 // ---------------------------------------------------------------------------
-__global__ void k_local(TreeDev T, int level, int64_t n, int p, const int32_t *node_act,
-                        const double2 *__restrict__ MLop, const double2 *__restrict__ LLop,
-                        const double2 *__restrict__ mp, double2 *loc, unsigned *err) {
-  if ((int64_t)blockIdx.x >= n) return;
+#define MM_LOCAL_THREADS 128
+#define MM_LOCAL_STARS 8  // P2L stars staged at a time
+struct LocalSources {
+  int n;
+  int src[32];   // first child or leaf of the source
+  int slot[32];  // M2L: offset slot; -1: P2L from the leaf's stars
+};
+
+// Shared memory: the scaled multipoles b [source][k] (then the factors of the
+// sums) and the sums t [source][l] of up to 27 sources, the L2L sum [l], the
+// parent's local and the staged stars.
+static __host__ __device__ __forceinline__ size_t local_smem(int p) {
+  const size_t P1 = (size_t)p + 1;
+  return sizeof(double2) * (2 * 27 * P1 + 2 * P1 + MM_LOCAL_STARS * (P1 + MM_POW_BITS)) +
+         sizeof(double) * MM_LOCAL_STARS * (1 + P1);
+}
+
+__global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
+    k_local(TreeDev T, int level, int64_t n, int p, const int32_t *node_act,
+            const double2 *__restrict__ MLop, const double2 *__restrict__ LLop,
+            const double2 *__restrict__ mp, double2 *loc, unsigned *err) {
+  extern __shared__ __align__(16) double2 s_loc[];
+  __shared__ LocalSources S;
   const int64_t node = T.level_off[level] + blockIdx.x;
   if (!node_act[node]) return;
-  __shared__ double2 src[MM_PMAX + 1];
-  const int P1 = p + 1;
-  const int l = threadIdx.x;
-  const bool on = l <= p && l >= 1;
+  const int P1 = p + 1, tid = threadIdx.x;
+  double2 *bs = s_loc, *ts = bs + 27 * P1, *l2l = ts + 27 * P1, *pl = l2l + P1;
+  double2 *zs = pl + P1;                   // [star][l]
+  double2 *sq = zs + MM_LOCAL_STARS * P1;  // [star][MM_POW_BITS]
+  double *sm = reinterpret_cast<double *>(sq + MM_LOCAL_STARS * MM_POW_BITS);  // [star]
+  double *fs = sm + MM_LOCAL_STARS;        // [star][l]
   int lv, nx, ny;
   double zx, zy, L;
   node_geom(T, node, lv, nx, ny, zx, zy, L);
-  const int px = nx >> 1, py = ny >> 1;
-  double2 acc = make_double2(0.0, 0.0);
+  const int64_t parent = T.parent[node];
 
-  // L2L from the parent
-  const int64_t parent = find_node(T, level - 1, px, py);
-  if (parent >= 0) {
-    for (int k = threadIdx.x; k < P1; k += blockDim.x) src[k] = loc[parent * P1 + k];
-    __syncthreads();
-    const int q = (nx & 1) | ((ny & 1) << 1);
-    const double2 *op = LLop + (int64_t)q * P1 * P1;
-    if (on)
-      for (int k = l; k <= p; k++) acc = cfma(op[k * P1 + l], src[k], acc);
-    __syncthreads();
-  }
-
-  const double invL = 1.0 / L;
-  for (int dy = -1; dy <= 1; dy++)
-    for (int dx = -1; dx <= 1; dx++) {
-      if (dx == 0 && dy == 0) continue;
-      const int qx = px + dx, qy = py + dy;
-      const int side = 1 << (level - 1);
-      if (qx < 0 || qy < 0 || qx >= side || qy >= side) continue;
-      const int64_t qid = find_node(T, level - 1, qx, qy);
+  // the sources in the order of the parent's neighbours (row-major) and their
+  // children: slot t = 4 neighbour + child
+  if (tid < 32) {
+    const int k = tid >> 2, c = tid & 3, j = k < 4 ? k : k + 1;
+    const int qx = (nx >> 1) + j % 3 - 1, qy = (ny >> 1) + j / 3 - 1, side = 1 << (level - 1);
+    bool on = false;
+    int src = 0, slot = -1;
+    if (qx >= 0 && qy >= 0 && qx < side && qy < side) {
+      const int qid = T.nb[9 * parent + j];
       if (qid < 0) {
-        if (threadIdx.x == 0) atomicOr(err, ERR_TREE_INVARIANT);
-        continue;
-      }
-      const int fc = T.first_child[qid];
-      if (fc >= 0) {
-        for (int c = 0; c < 4; c++) {
-          const int ox = 2 * qx + (c & 1) - nx, oy = 2 * qy + (c >> 1) - ny;
-          if (abs(ox) <= 1 && abs(oy) <= 1) continue;  // neighbour: near field
-          // factored M2L: b_k = (-1/z0)^k a_k, then
-          // c_l += (1/z0)^l (-a_0 / l + sum_k C(l+k-1, k-1) b_k)
-          const double2 *pw =
-              MLop + (int64_t)P1 * P1 + (int64_t)((oy + 3) * 7 + (ox + 3)) * 2 * P1;
-          for (int k = threadIdx.x; k < P1; k += blockDim.x) {
-            const double2 a = mp[(int64_t)(fc + c) * P1 + k];
-            src[k] = k ? cfma(pw[k], a, make_double2(0.0, 0.0)) : a;
-          }
-          __syncthreads();
-          if (on) {
-            const double2 *bl = MLop + (int64_t)l * P1;  // binomials of row l, 1/l at k = 0
-            double tx = -src[0].x * bl[0].x, ty = -src[0].y * bl[0].x;
-            for (int k = 1; k <= p; k++) {
-              const double b = bl[k].x;
-              tx = fma(b, src[k].x, tx);
-              ty = fma(b, src[k].y, ty);
-            }
-            acc = cfma(pw[P1 + l], make_double2(tx, ty), acc);
-          }
-          __syncthreads();
-        }
+        if (c == 0) atomicOr(err, ERR_TREE_INVARIANT);
       } else {
-        // unsplit parent-neighbour: adjacent to the node unless its 2x2
-        // level cells all lie at Chebyshev distance >= 2
-        const int x0 = 2 * qx, y0 = 2 * qy;
-        const bool adj = (x0 + 1 >= nx - 1 && x0 <= nx + 1) && (y0 + 1 >= ny - 1 && y0 <= ny + 1);
-        if (adj) continue;
-        if (on) {
-          for (int64_t i = T.sbeg[qid]; i < T.send[qid]; i++) {
-            double2 zeta = make_double2((T.sx[i] - zx) * invL, (T.sy[i] - zy) * invL);
-            const double d = zeta.x * zeta.x + zeta.y * zeta.y;
-            double2 inv = make_double2(zeta.x / d, -zeta.y / d);
-            double2 zl = cpow(inv, l);
-            const double f = -T.sm[i] / (double)l;
-            acc.x = fma(f, zl.x, acc.x);
-            acc.y = fma(f, zl.y, acc.y);
-          }
+        const int fc = T.first_child[qid];
+        if (fc >= 0) {
+          const int ox = 2 * qx + (c & 1) - nx, oy = 2 * qy + (c >> 1) - ny;
+          src = fc + c;
+          on = abs(ox) > 1 || abs(oy) > 1;  // else a neighbour: near field
+          slot = (oy + 3) * 7 + (ox + 3);
+        } else {
+          // unsplit parent-neighbour: adjacent to the node unless its 2x2
+          // level cells all lie at Chebyshev distance >= 2
+          const int x0 = 2 * qx, y0 = 2 * qy;
+          const bool adj =
+              (x0 + 1 >= nx - 1 && x0 <= nx + 1) && (y0 + 1 >= ny - 1 && y0 <= ny + 1);
+          on = c == 0 && !adj;
+          src = qid;
         }
       }
     }
-  if (l <= p) loc[node * P1 + l] = on ? acc : make_double2(0.0, 0.0);
+    on = on && T.sbeg[src] < T.send[src];
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (on) {
+      const int r = __popc(m & ((1u << tid) - 1u));
+      S.src[r] = src;
+      S.slot[r] = slot;
+    }
+    if (tid == 0) S.n = __popc(m);
+  }
+  __syncthreads();
+  const int ns = S.n;
+
+  // factored M2L: b_k = (-1/z0)^k a_k, then
+  // c_l += (1/z0)^l (-a_0 / l + sum_k C(l+k-1, k-1) b_k)
+  const double2 *pw = MLop + (int64_t)P1 * P1;  // per slot: powers of -1/z0, of 1/z0
+  for (int idx = tid; idx < ns * P1; idx += MM_LOCAL_THREADS) {
+    const int s = idx / P1, k = idx - s * P1, slot = S.slot[s];
+    if (slot < 0) continue;
+    const double2 a = mp[(int64_t)S.src[s] * P1 + k];
+    bs[idx] = k ? cfma(pw[(int64_t)slot * 2 * P1 + k], a, make_double2(0.0, 0.0)) : a;
+  }
+  for (int k = tid; k < P1; k += MM_LOCAL_THREADS) pl[k] = loc[parent * P1 + k];
+  __syncthreads();
+  // L2L from the parent, by the last threads
+  if (tid >= MM_LOCAL_THREADS - p) {
+    const int l = MM_LOCAL_THREADS - tid;
+    const int q = (nx & 1) | ((ny & 1) << 1);
+    const double2 *op = LLop + (int64_t)q * P1 * P1;
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int k = l; k <= p; k++) acc = cfma(op[k * P1 + l], pl[k], acc);
+    l2l[l] = acc;
+  }
+  const double *bt = reinterpret_cast<const double *>(MLop);  // binomials [k][l], 1/l at k = 0
+  const int G = max(1, MM_LOCAL_THREADS / p);
+  const int g = tid / p, l = tid - g * p + 1;
+  const double il = bt[l];
+  for (int s0 = g < G ? g : ns; __any_sync(0xffffffffu, s0 < ns); s0 += 2 * G) {
+    // (a P2L source's entry is not formed: its sum is not used)
+    const int s1 = s0 + G;
+    const bool on0 = s0 < ns, on1 = s1 < ns;
+    const double2 *b0 = bs + (on0 ? s0 : 0) * P1, *b1 = bs + (on1 ? s1 : 0) * P1;
+    double x0 = -b0[0].x * il, y0 = -b0[0].y * il;
+    if (__any_sync(0xffffffffu, on1)) {
+      double x1 = -b1[0].x * il, y1 = -b1[0].y * il;
+#pragma unroll 4
+      for (int k = 1; k <= p; k++) {
+        const double b = bt[k * P1 + l];
+        const double2 u = b0[k], v = b1[k];
+        x0 = fma(b, u.x, x0);
+        y0 = fma(b, u.y, y0);
+        x1 = fma(b, v.x, x1);
+        y1 = fma(b, v.y, y1);
+      }
+      if (on1) ts[s1 * P1 + l] = make_double2(x1, y1);
+    } else {
+#pragma unroll 4
+      for (int k = 1; k <= p; k++) {
+        const double b = bt[k * P1 + l];
+        const double2 u = b0[k];
+        x0 = fma(b, u.x, x0);
+        y0 = fma(b, u.y, y0);
+      }
+    }
+    if (on0) ts[s0 * P1 + l] = make_double2(x0, y0);
+  }
+  __syncthreads();
+  // the factors (1/z0)^l of the M2L sources, in place of their multipoles
+  for (int idx = tid; idx < ns * P1; idx += MM_LOCAL_THREADS) {
+    const int s = idx / P1, slot = S.slot[s];
+    if (slot >= 0) bs[idx] = pw[(int64_t)slot * 2 * P1 + P1 + (idx - s * P1)];
+  }
+  __syncthreads();
+
+  // add up row l = tid (1 .. p) in the order of the list
+  const bool on = tid >= 1 && tid <= p;
+  double2 acc = on ? l2l[tid] : make_double2(0.0, 0.0);
+  const double invL = inv_pow2(L);
+  for (int s = 0; s < ns; s++) {
+    const int slot = S.slot[s];
+    if (slot >= 0) {
+      if (on) acc = cfma(bs[s * P1 + tid], ts[s * P1 + tid], acc);
+      continue;
+    }
+    // P2L: the leaf's stars, staged; block-uniform.  Powers and weights of
+    // every (star, row) side by side, then added up star by star.
+    const int b = T.sbeg[S.src[s]], e = T.send[S.src[s]];
+    for (int c = b; c < e; c += MM_LOCAL_STARS) {
+      const int cnt = min(MM_LOCAL_STARS, e - c);
+      __syncthreads();
+      if (tid < cnt) {
+        const double2 zeta =
+            make_double2((T.sx[c + tid] - zx) * invL, (T.sy[c + tid] - zy) * invL);
+        const double d = zeta.x * zeta.x + zeta.y * zeta.y;
+        powers_of_two(make_double2(zeta.x / d, -zeta.y / d), p, sq + tid * MM_POW_BITS);
+        sm[tid] = T.sm[c + tid];
+      }
+      __syncthreads();
+      if (g < G)
+        for (int i = g; i < cnt; i += G) {
+          zs[i * P1 + l] = power_of(sq + i * MM_POW_BITS, l);
+          fs[i * P1 + l] = div_by(-sm[i], (double)l, il);
+        }
+      __syncthreads();
+      if (on)
+        for (int i = 0; i < cnt; i++) {
+          const double2 zl = zs[i * P1 + tid];
+          const double f = fs[i * P1 + tid];
+          acc.x = fma(f, zl.x, acc.x);
+          acc.y = fma(f, zl.y, acc.y);
+        }
+    }
+  }
+  if (tid <= p) loc[node * P1 + tid] = on ? acc : make_double2(0.0, 0.0);
 }
 
 // ---------------------------------------------------------------------------
@@ -236,19 +430,21 @@ __device__ __forceinline__ int for_each_near_range(const TreeDev &T, int64_t nod
     f(T.sbeg[node], T.send[node]);
     return 0;
   }
-  int64_t seen[9];
+  const int64_t parent = T.parent[node];
+  int seen[9];
   int nseen = 0;
   for (int dy = -1; dy <= 1; dy++)
     for (int dx = -1; dx <= 1; dx++) {
       const int x = nx + dx, y = ny + dy;
       const int side = 1 << level;
       if (x < 0 || y < 0 || x >= side || y >= side) continue;
-      int64_t id = find_node(T, level, x, y);
+      const int id = T.nb[9 * node + (dy + 1) * 3 + (dx + 1)];
       if (id >= 0) {
         f(T.sbeg[id], T.send[id]);
         continue;
       }
-      int64_t pid = find_node(T, level - 1, x >> 1, y >> 1);
+      const int pid =
+          T.nb[9 * parent + ((y >> 1) - (ny >> 1) + 1) * 3 + ((x >> 1) - (nx >> 1) + 1)];
       if (pid < 0) {
         atomicOr(err, ERR_TREE_INVARIANT);
         continue;
@@ -594,12 +790,14 @@ void build_operator_tables(int p, std::vector<double2> &MM, std::vector<double2>
   const int P1 = p + 1;
   auto C = binomials(2 * p + 1);
   // M2M factored like M2L below: op[k][l] = (z0/2)^l C(l-1, k-1) z0^-k for
-  // 1 <= k <= l and op[0][l] = -(z0/2)^l / l: the real binomials ([l][k],
-  // 1/l at k = 0), then per child quadrant the powers z0^-k and (z0/2)^l
+  // 1 <= k <= l and op[0][l] = -(z0/2)^l / l: the real binomials (P1 x P1
+  // doubles [k][l], 1/l at k = 0, at the head of P1 x P1 entries), then per
+  // child quadrant the powers z0^-k and (z0/2)^l
   MM.assign((size_t)P1 * P1 + (size_t)4 * 2 * P1, make_double2(0.0, 0.0));
+  double *mb = &MM[0].x;
   for (int l = 1; l <= p; l++) {
-    MM[(size_t)l * P1].x = 1.0 / l;
-    for (int k = 1; k <= l; k++) MM[(size_t)l * P1 + k].x = C[l - 1][k - 1];
+    mb[l] = 1.0 / l;
+    for (int k = 1; k <= l; k++) mb[(size_t)k * P1 + l] = C[l - 1][k - 1];
   }
   LL.assign((size_t)4 * P1 * P1, make_double2(0.0, 0.0));
   ML.assign((size_t)49 * P1 * P1, make_double2(0.0, 0.0));
@@ -628,13 +826,15 @@ void build_operator_tables(int p, std::vector<double2> &MM, std::vector<double2>
   // M2L: source centre relative to the target, z0 = 2 (dx + i dy).  The
   // operator factors as op[k][l] = (1/z0)^l C(l+k-1, k-1) (-1/z0)^k for
   // k >= 1 and op[0][l] = -(1/z0)^l / l, so the table holds the real
-  // binomials once ([l][k], with 1/l in the unused k = 0 slot) and, per
+  // binomials once (P1 x P1 doubles [k][l], with 1/l in the unused k = 0 row,
+  // at the head of P1 x P1 entries) and, per
   // offset, the powers of -1/z0 (scaling the multipoles) and of 1/z0
   // (scaling the sums): P1^2 + 49 x 2 P1 entries.
   ML.assign((size_t)P1 * P1 + (size_t)49 * 2 * P1, make_double2(0.0, 0.0));
+  double *lb = &ML[0].x;
   for (int l = 1; l <= p; l++) {
-    ML[(size_t)l * P1].x = 1.0 / l;
-    for (int k = 1; k <= p; k++) ML[(size_t)l * P1 + k].x = C[l + k - 1][k - 1];
+    lb[l] = 1.0 / l;
+    for (int k = 1; k <= p; k++) lb[(size_t)k * P1 + l] = C[l + k - 1][k - 1];
   }
   for (int dy = -3; dy <= 3; dy++)
     for (int dx = -3; dx <= 3; dx++) {
@@ -652,18 +852,30 @@ void build_operator_tables(int p, std::vector<double2> &MM, std::vector<double2>
 }
 
 static inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
-static inline int coef_threads(int p) { return 32 * ((p + 1 + 31) / 32); }
 
-cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, double2 *mp, cudaStream_t st) {
+cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *MLop, double2 *mp,
+                       cudaStream_t st) {
   if (n_nodes <= 0) return cudaSuccess;
-  k_p2m<<<(unsigned)n_nodes, coef_threads(p), 0, st>>>(T, n_nodes, p, mp);
+  const int per_block = std::min(32, MM_P2M_THREADS / (p + 1));  // (32: staged stars fit 48 KB)
+  const size_t smem = (size_t)per_block * MM_P2M_STARS *
+                      (MM_POW_BITS * sizeof(double2) + sizeof(double));
+  // (the head of MLop holds 1/k)
+  k_p2m<<<blocks_for(n_nodes, per_block), MM_P2M_THREADS, smem, st>>>(
+      T, n_nodes, p, per_block, reinterpret_cast<const double *>(MLop), mp);
   return cudaGetLastError();
 }
 
 cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const double2 *MMop,
                        double2 *mp, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_m2m<<<(unsigned)n, coef_threads(p), 0, st>>>(T, level, n, p, MMop, mp);
+  // 8 nodes a block fill its warps (4 children x p/2 rows each); fewer where
+  // their coefficients would not fit 48 KB, and where a level's nodes would
+  // leave SMs idle (a node's work is 2 us of one SM's FP64 pipe)
+  int per_block = p <= 32 ? 8 : 4;
+  while (per_block > 1 && n < 304 * (int64_t)per_block) per_block >>= 1;
+  const int threads = 32 * ((per_block * 4 * ((p + 1) / 2) + 31) / 32);
+  const size_t smem = sizeof(double2) * 2 * per_block * 4 * (size_t)(p + 1);
+  k_m2m<<<blocks_for(n, per_block), threads, smem, st>>>(T, level, n, p, per_block, MMop, mp);
   return cudaGetLastError();
 }
 
@@ -671,8 +883,14 @@ cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const in
                          const double2 *MLop, const double2 *LLop, const double2 *mp,
                          double2 *loc, unsigned *err, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_local<<<(unsigned)n, coef_threads(p), 0, st>>>(T, level, n, p, node_act, MLop, LLop, mp,
-                                                   loc, err);
+  const size_t smem = local_smem(p);
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  k_local<<<(unsigned)n, MM_LOCAL_THREADS, smem, st>>>(T, level, n, p, node_act, MLop, LLop, mp,
+                                                       loc, err);
   return cudaGetLastError();
 }
 

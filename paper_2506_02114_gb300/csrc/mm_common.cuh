@@ -125,25 +125,32 @@ __host__ __device__ __forceinline__ int coef_stride(int p_eval) {
   return p_eval <= 2 ? 2 : ((p_eval - 1 + 1) & ~1);
 }
 
+// Bit k of a 16-bit integer to bit 2k, and back.
+__host__ __device__ __forceinline__ uint32_t spread16(uint32_t v) {
+  v = (v | (v << 8)) & 0x00ff00ffu;
+  v = (v | (v << 4)) & 0x0f0f0f0fu;
+  v = (v | (v << 2)) & 0x33333333u;
+  return (v | (v << 1)) & 0x55555555u;
+}
+__host__ __device__ __forceinline__ uint32_t gather16(uint32_t v) {
+  v &= 0x55555555u;
+  v = (v | (v >> 1)) & 0x33333333u;
+  v = (v | (v >> 2)) & 0x0f0f0f0fu;
+  v = (v | (v >> 4)) & 0x00ff00ffu;
+  return (v | (v >> 8)) & 0x0000ffffu;
+}
+
 // Interleave two 21-bit integers: x in even bits, y in odd bits.
 __host__ __device__ __forceinline__ uint64_t morton2(uint32_t x, uint32_t y) {
-  uint64_t r = 0;
-#pragma unroll
-  for (int b = 0; b < MM_DMAX; b++) {
-    r |= (uint64_t)((x >> b) & 1u) << (2 * b);
-    r |= (uint64_t)((y >> b) & 1u) << (2 * b + 1);
-  }
-  return r;
+  const uint32_t lo = spread16(x & 0xffffu) | (spread16(y & 0xffffu) << 1);
+  const uint32_t hi = spread16(x >> 16) | (spread16(y >> 16) << 1);
+  return ((uint64_t)hi << 32) | lo;
 }
 
 __host__ __device__ __forceinline__ void morton_decode(uint64_t c, uint32_t &x, uint32_t &y) {
-  x = 0;
-  y = 0;
-#pragma unroll
-  for (int b = 0; b < MM_DMAX; b++) {
-    x |= (uint32_t)((c >> (2 * b)) & 1u) << b;
-    y |= (uint32_t)((c >> (2 * b + 1)) & 1u) << b;
-  }
+  const uint32_t lo = (uint32_t)c, hi = (uint32_t)(c >> 32);
+  x = gather16(lo) | (gather16(hi) << 16);
+  y = gather16(lo >> 1) | (gather16(hi >> 1) << 16);
 }
 
 // First index in [lo, hi) with a[idx] >= key (a sorted ascending).

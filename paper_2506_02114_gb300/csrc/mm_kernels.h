@@ -23,6 +23,9 @@ struct TreeDev {
   // nodes (flattened over levels)
   const uint64_t *code;
   const int32_t *lvl, *sbeg, *send, *first_child;
+  const int32_t *parent;      // -1 for the root
+  const int32_t *nb;          // per node: the nine same-level cells around it (row-major,
+                              // itself in the middle), -1 where the cell is no node
   const int64_t *level_off;   // [MM_DMAX + 2]
   int32_t depth;
 };
@@ -32,14 +35,28 @@ cudaError_t launch_star_keys(const double *pos, int64_t n, double R0, uint64_t *
 cudaError_t launch_gather_stars(const double *pos, const double *m, const int32_t *idx,
                                 int64_t n, double *sx, double *sy, double *sm,
                                 cudaStream_t st);
-cudaError_t launch_root_init(int64_t n_stars, uint64_t *code, int32_t *lvl, int32_t *sbeg,
-                             int32_t *send, cudaStream_t st);
-cudaError_t launch_level_split(const TreeDev &T, int level, int64_t n, int limit,
-                               int32_t *split, cudaStream_t st);
-cudaError_t launch_level_children(const TreeDev &T, int level, int64_t n, const int32_t *split,
-                                  const int32_t *scan, uint64_t *code, int32_t *lvl,
-                                  int32_t *sbeg, int32_t *send, int32_t *first_child,
-                                  cudaStream_t st);
+// The node arrays a level's kernels write (sizes: see TreeDev).
+struct TreeOut {
+  uint64_t *code;
+  int32_t *lvl, *sbeg, *send, *first_child, *parent, *nb;
+  int64_t *level_off;
+};
+// Levels from the root down to the first with more than MM_TOP_NODES nodes,
+// in one launch.  info[0]: the level it stopped at (not yet split); info[1]:
+// 1 when the tree is complete; info[2 + l]: nodes of level l.
+#define MM_TOP_NODES 256
+#define MM_TOP_CAPACITY ((MM_DMAX + 1) * MM_TOP_NODES + 4 * MM_TOP_NODES)
+#define MM_TOP_INFO (2 + MM_DMAX + 2)
+cudaError_t launch_tree_top(const TreeDev &T, const TreeOut &O, int limit, int32_t *info,
+                            cudaStream_t st);
+// One larger level: neighbours and split flags of its n nodes, the number of
+// split nodes per group of MM_SPLIT_GROUP, and (total not NULL) in all.
+#define MM_SPLIT_GROUP 32
+cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, int64_t n, int limit,
+                               int32_t *split, int32_t *group, int32_t *total, cudaStream_t st);
+// Its children, in Morton order.
+cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level, int64_t n,
+                                  const int32_t *split, const int32_t *group, cudaStream_t st);
 cudaError_t launch_axis_cells(double x0, double h, int64_t n, double R0, int32_t *out,
                               cudaStream_t st);
 // flags[node] = 1 for active leaves (leaf containing ray vertices); also
@@ -69,7 +86,8 @@ struct FmmConst {
   double rect_c1, rect_c2;    // > 0: rectangular star region |x| <= c1, |y| <= c2 (App. B)
 };
 
-cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, double2 *mp, cudaStream_t st);
+cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *MLop, double2 *mp,
+                       cudaStream_t st);
 cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const double2 *MMop,
                        double2 *mp, cudaStream_t st);
 cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const int32_t *node_act,

@@ -10,11 +10,18 @@
 // leaves one level up.
 //
 // Build: Morton keys of the stars (21 bits per axis), a radix sort, then one
-// level at a time: split flags from nine key-range counts per node, an
-// exclusive scan of the flags, and the children written in Morton order so
-// that each level's node array stays sorted by code.
-#include <cub/cub.cuh>
-
+// level at a time: each node's eight neighbours from its parent's (a child of
+// a neighbour of the parent, if that one is split), split flags from the nine
+// star counts, ranks of the split nodes, and the children written in Morton
+// order so that each level's node array stays sorted by code.  The levels of
+// at most MM_TOP_NODES nodes are built by one block in one launch, larger
+// ones by two launches each.  Every step is a short chain of dependent loads
+// (a binary search runs only inside an unsplit neighbour of the parent, at
+// most leaf_size stars, and over a node's own stars), so the time is latency:
+// 50 000 stars take 0.20 ms (0.09 of it the sort); 0.54 ms with counts by
+// binary search over all stars, one thread per node, and five launches a
+// level.  The one block is the faster way up to 256 nodes a level (with 1024,
+// the level of 864 took 21 us in it, 14 in two launches).
 #include "mm_kernels.h"
 
 namespace mm {
@@ -46,70 +53,211 @@ __global__ void k_gather_stars(const double *__restrict__ pos, const double *__r
   sm[t] = m[k];
 }
 
-__global__ void k_root_init(int64_t n_stars, uint64_t *code, int32_t *lvl, int32_t *sbeg,
-                            int32_t *send) {
-  code[0] = 0;
-  lvl[0] = 0;
-  sbeg[0] = 0;
-  send[0] = (int32_t)n_stars;
-}
-
-// Number of stars whose key lies in the level-`level` cell (x, y).
-__device__ __forceinline__ int64_t count_cell(const TreeDev &T, int level, int x, int y) {
-  const int sh = 2 * (MM_DMAX - level);
-  uint64_t c = morton2((uint32_t)x, (uint32_t)y);
-  uint64_t lo = c << sh, hi = (c + 1) << sh;
-  int64_t a = lower_bound_u64(T.keys, 0, T.n_stars, lo);
-  int64_t b = lower_bound_u64(T.keys, a, T.n_stars, hi);
-  return b - a;
-}
-
-__global__ void k_level_split(TreeDev T, int level, int64_t n, int limit, int32_t *split) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int64_t node = T.level_off[level] + t;
-  if (level >= MM_DMAX) {
-    split[t] = 0;
-    return;
-  }
-  uint32_t cx, cy;
-  morton_decode(T.code[node], cx, cy);
-  const int side = 1 << level;
-  int64_t count = T.send[node] - T.sbeg[node];
-  for (int dy = -1; dy <= 1; dy++)
-    for (int dx = -1; dx <= 1; dx++) {
-      if (dx == 0 && dy == 0) continue;
-      int x = (int)cx + dx, y = (int)cy + dy;
-      if (x < 0 || y < 0 || x >= side || y >= side) continue;
-      count += count_cell(T, level, x, y);
-    }
-  split[t] = count > limit ? 1 : 0;
-}
-
-__global__ void k_level_children(TreeDev T, int level, int64_t n, const int32_t *split,
-                                 const int32_t *scan, uint64_t *code, int32_t *lvl,
-                                 int32_t *sbeg, int32_t *send, int32_t *first_child) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int64_t node = T.level_off[level] + t;
-  if (!split[t]) {
-    first_child[node] = -1;
-    return;
-  }
-  const int64_t base = T.level_off[level + 1] + 4 * (int64_t)scan[t];
-  first_child[node] = (int32_t)base;
+// Neighbour s (0..7, row-major around the node without the middle) of a
+// node: the node of that cell, or -1 (no node, or outside the root), and the
+// cell's stars.
+__device__ __forceinline__ int neighbour(const TreeDev &T, int level, int64_t node, int s,
+                                         int &count) {
+  count = 0;
+  if (level == 0) return -1;
+  const int k = s < 4 ? s : s + 1;
   const uint64_t c = T.code[node];
-  const int sh = 2 * (MM_DMAX - level - 1);
-  int64_t b = T.sbeg[node];
-  const int64_t e = T.send[node];
-  for (int q = 0; q < 4; q++) {
-    uint64_t cc = (c << 2) | (uint64_t)q;
-    int64_t end = (q == 3) ? e : lower_bound_u64(T.keys, b, e, (cc + 1) << sh);
-    code[base + q] = cc;
-    lvl[base + q] = level + 1;
-    sbeg[base + q] = (int32_t)b;
-    send[base + q] = (int32_t)end;
-    b = end;
+  uint32_t cx, cy;
+  morton_decode(c, cx, cy);
+  const int x = (int)cx + k % 3 - 1, y = (int)cy + k / 3 - 1, side = 1 << level;
+  if (x < 0 || y < 0 || x >= side || y >= side) return -1;
+  // (the parent is split, so all its neighbours inside the root are nodes)
+  const int j = ((y >> 1) - (int)(cy >> 1) + 1) * 3 + ((x >> 1) - (int)(cx >> 1) + 1);
+  const int q = T.nb[9 * (int64_t)T.parent[node] + j];
+  if (q < 0) return -1;
+  const int fc = T.first_child[q];
+  if (fc >= 0) {
+    const int id = fc + ((x & 1) | ((y & 1) << 1));
+    count = T.send[id] - T.sbeg[id];
+    return id;
+  }
+  const int sh = 2 * (MM_DMAX - level);
+  const uint64_t key = morton2((uint32_t)x, (uint32_t)y);
+  const int64_t e = T.send[q];
+  const int64_t a = lower_bound_u64(T.keys, T.sbeg[q], e, key << sh);
+  count = (int)(lower_bound_u64(T.keys, a, e, (key + 1) << sh) - a);
+  return -1;
+}
+
+// Eight lanes per node (s = lane & 7): writes the node's neighbours and
+// returns whether it splits (in all eight lanes).  Call with whole warps.
+__device__ __forceinline__ bool node_split(const TreeDev &T, const TreeOut &O, int level,
+                                           int64_t node, bool valid, int s, int limit) {
+  int count = 0, own = 0;
+  if (valid) {
+    const int id = neighbour(T, level, node, s, count);
+    O.nb[9 * node + (s < 4 ? s : s + 1)] = id;
+    if (s == 0) O.nb[9 * node + 4] = (int32_t)node;
+    own = T.send[node] - T.sbeg[node];
+  }
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) count += __shfl_xor_sync(0xffffffffu, count, d);
+  return valid && level < MM_DMAX && count + own > limit;
+}
+
+__device__ __forceinline__ void write_child(const TreeDev &T, const TreeOut &O, int level,
+                                            int64_t node, int q, int64_t id, int b, int e) {
+  O.code[id] = (T.code[node] << 2) | (uint64_t)q;
+  O.lvl[id] = level + 1;
+  O.sbeg[id] = b;
+  O.send[id] = e;
+  O.parent[id] = (int32_t)node;
+}
+
+__global__ void __launch_bounds__(256) k_level_split(TreeDev T, TreeOut O, int level, int64_t n,
+                                                     int limit, int32_t *split, int32_t *group,
+                                                     int32_t *total) {
+  __shared__ int s_n[8];
+  const int64_t t = (int64_t)blockIdx.x * MM_SPLIT_GROUP + (threadIdx.x >> 3);
+  const int s = threadIdx.x & 7;
+  const bool f = node_split(T, O, level, T.level_off[level] + t, t < n, s, limit);
+  if (s == 0 && t < n) split[t] = f;
+  const unsigned m = __ballot_sync(0xffffffffu, f && s == 0);
+  if ((threadIdx.x & 31) == 0) s_n[threadIdx.x >> 5] = __popc(m);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int c = 0;
+    for (int k = 0; k < 8; k++) c += s_n[k];
+    group[blockIdx.x] = c;
+    if (total && c) atomicAdd(total, c);
+  }
+}
+
+// Four lanes per node, 64 nodes (two groups) per block.
+__global__ void __launch_bounds__(256) k_level_children(TreeDev T, TreeOut O, int level, int64_t n,
+                                                        const int32_t *split,
+                                                        const int32_t *group) {
+  __shared__ int s_w[8], s_base;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = threadIdx.x & 3;
+  // split nodes of the groups before this block's
+  int before = 0;
+  for (int64_t k = threadIdx.x; k < 2 * (int64_t)blockIdx.x; k += 256) before += group[k];
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (threadIdx.x == 0) s_base = 0;
+  __syncthreads();
+  if (lane == 0 && before) atomicAdd(&s_base, before);
+  const int64_t t = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2);
+  const int64_t node = T.level_off[level] + t;
+  const bool f = t < n && split[t];
+  const unsigned m = __ballot_sync(0xffffffffu, f && q == 0);
+  if (lane == 0) s_w[w] = __popc(m);
+  int b = 0, e = 0, end = 0;
+  if (f) {
+    b = T.sbeg[node];
+    e = T.send[node];
+    const int sh = 2 * (MM_DMAX - level - 1);
+    end = q == 3 ? e
+                 : (int)lower_bound_u64(T.keys, b, e, ((T.code[node] << 2) + (uint64_t)q + 1) << sh);
+  }
+  const int up = __shfl_up_sync(0xffffffffu, end, 1);
+  __syncthreads();
+  if (!f) {
+    if (q == 0 && t < n) O.first_child[node] = -1;
+    return;
+  }
+  int rank = s_base + __popc(m & ((1u << (lane & ~3)) - 1u));
+  for (int k = 0; k < w; k++) rank += s_w[k];
+  const int64_t base = T.level_off[level + 1] + 4 * (int64_t)rank;
+  if (q == 0) O.first_child[node] = (int32_t)base;
+  write_child(T, O, level, node, q, base + q, q ? up : b, end);
+}
+
+// First index in [lo, hi) with a[idx] >= key, by a whole warp: 32 probes a
+// step.
+__device__ __forceinline__ int64_t warp_lower_bound(const uint64_t *a, int64_t lo, int64_t hi,
+                                                    uint64_t key, int lane) {
+  while (hi - lo > 32) {
+    const int64_t step = (hi - lo + 32) / 33;
+    const int64_t p = lo + (lane + 1) * step;
+    const int c = __popc(__ballot_sync(0xffffffffu, p < hi && a[p] < key));
+    // a[lo + c step] < key <= a[lo + (c + 1) step]
+    const int64_t end = lo + (c + 1) * step;
+    if (c) lo += c * step + 1;
+    if (end < hi) hi = end;
+  }
+  return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && a[lo + lane] < key));
+}
+
+// The levels of at most MM_TOP_NODES nodes, one block.
+__global__ void __launch_bounds__(1024) k_tree_top(TreeDev T, TreeOut O, int limit,
+                                                   int32_t *info) {
+  static_assert(MM_TOP_NODES <= 1024, "one thread per node");
+  __shared__ int s_flag[MM_TOP_NODES], s_w[32], s_end[3 * MM_TOP_NODES];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) {
+    O.code[0] = 0;
+    O.lvl[0] = 0;
+    O.sbeg[0] = 0;
+    O.send[0] = (int32_t)T.n_stars;
+    O.parent[0] = -1;
+    O.level_off[0] = 0;
+    O.level_off[1] = 1;
+  }
+  if (tid < MM_TOP_INFO) info[tid] = 0;
+  __syncthreads();
+  int n = 1, level = 0, done = 0;
+  int64_t off = 0;
+  while (n <= MM_TOP_NODES) {
+    if (tid == 0) info[2 + level] = n;
+    for (int b = 0; b < 8 * n; b += 1024) {
+      const int t = (b + tid) >> 3;
+      const bool f = node_split(T, O, level, off + t, t < n, tid & 7, limit);
+      if ((tid & 7) == 0 && t < n) s_flag[t] = f;
+    }
+    __syncthreads();
+    // rank of each split node, and the split nodes in all
+    const int f = tid < n && s_flag[tid];
+    const unsigned m = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) s_w[w] = __popc(m);
+    // the ends of the first three children of the split nodes: a warp per
+    // search while there are few and long ones, else a thread per search
+    const int sh = 2 * (MM_DMAX - level - 1);
+    const bool by_warp = n <= 32;
+    for (int k = by_warp ? w : tid; k < 3 * n; k += by_warp ? 32 : 1024) {
+      const int t = k / 3;
+      if (!s_flag[t]) continue;
+      const int64_t b = T.sbeg[off + t], e = T.send[off + t];
+      const uint64_t key = ((T.code[off + t] << 2) + (uint64_t)(k - 3 * t) + 1) << sh;
+      const int64_t r = by_warp ? warp_lower_bound(T.keys, b, e, key, lane)
+                                : lower_bound_u64(T.keys, b, e, key);
+      if (!by_warp || lane == 0) s_end[k] = (int)r;
+    }
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int k = 0; k < 32; k++) {
+      if (k < w) before += s_w[k];
+      total += s_w[k];
+    }
+    if (tid < n) {
+      const int64_t node = off + tid;
+      const int64_t base = off + n + 4 * (int64_t)(before + __popc(m & ((1u << lane) - 1u)));
+      O.first_child[node] = f ? (int32_t)base : -1;
+      if (f) {
+        int b = T.sbeg[node];
+        for (int q = 0; q < 4; q++) {
+          const int e = q == 3 ? T.send[node] : s_end[3 * tid + q];
+          write_child(T, O, level, node, q, base + q, b, e);
+          b = e;
+        }
+      }
+    }
+    off += n;
+    if (tid == 0 && level + 2 <= MM_DMAX + 1) O.level_off[level + 2] = off + 4 * (int64_t)total;
+    n = 4 * total;
+    level++;
+    done = total == 0;
+    __syncthreads();
+    if (done) break;
+  }
+  if (tid == 0) {
+    info[0] = level;
+    info[1] = done;
+    if (level <= MM_DMAX + 1) info[2 + level] = n;
   }
 }
 
@@ -195,26 +343,24 @@ cudaError_t launch_gather_stars(const double *pos, const double *m, const int32_
   return cudaGetLastError();
 }
 
-cudaError_t launch_root_init(int64_t n_stars, uint64_t *code, int32_t *lvl, int32_t *sbeg,
-                             int32_t *send, cudaStream_t st) {
-  k_root_init<<<1, 1, 0, st>>>(n_stars, code, lvl, sbeg, send);
+cudaError_t launch_tree_top(const TreeDev &T, const TreeOut &O, int limit, int32_t *info,
+                            cudaStream_t st) {
+  k_tree_top<<<1, 1024, 0, st>>>(T, O, limit, info);
   return cudaGetLastError();
 }
 
-cudaError_t launch_level_split(const TreeDev &T, int level, int64_t n, int limit,
-                               int32_t *split, cudaStream_t st) {
+cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, int64_t n, int limit,
+                               int32_t *split, int32_t *group, int32_t *total, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_level_split<<<blocks_for(n, 128), 128, 0, st>>>(T, level, n, limit, split);
+  k_level_split<<<blocks_for(n, MM_SPLIT_GROUP), 256, 0, st>>>(T, O, level, n, limit, split, group,
+                                                               total);
   return cudaGetLastError();
 }
 
-cudaError_t launch_level_children(const TreeDev &T, int level, int64_t n, const int32_t *split,
-                                  const int32_t *scan, uint64_t *code, int32_t *lvl,
-                                  int32_t *sbeg, int32_t *send, int32_t *first_child,
-                                  cudaStream_t st) {
+cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level, int64_t n,
+                                  const int32_t *split, const int32_t *group, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_level_children<<<blocks_for(n, 128), 128, 0, st>>>(T, level, n, split, scan, code, lvl,
-                                                       sbeg, send, first_child);
+  k_level_children<<<blocks_for(n, 64), 256, 0, st>>>(T, O, level, n, split, group);
   return cudaGetLastError();
 }
 
