@@ -198,7 +198,9 @@ struct mm_map {
 
   // expansions
   DBuf<double2> MMop, MLop, LLop, mp, loc;
-  DBuf<int32_t> near_cnt, near_off;
+  DBuf<double2> sub_up;            // tables of the re-centring (k_sub_tables)
+  DBuf<float2> sub_fp;
+  DBuf<float> sub_bin;
   int64_t n_near = 0;
   DBuf<LeafRec> leaf;
   DBuf<NearPos> near_pos;
@@ -597,12 +599,15 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
                        cudaMemcpyHostToDevice, st));  // (the cached tables outlive the copies)
     CK(h->mp.ensure((size_t)nn * (h->p + 1)));
     CK(h->loc.ensure((size_t)nn * (h->p + 1)));
-    CK(h->near_cnt.ensure(h->n_active << (2 * h->sub)));
-    CK(h->near_off.ensure(h->n_active << (2 * h->sub)));
-    CK(h->err.ensure(1));
+    const size_t P1 = (size_t)h->p + 1;
+    CK(h->sub_up.ensure(P1 << (2 * h->sub)));
+    CK(h->sub_fp.ensure(P1 << (2 * h->sub)));
+    CK(h->sub_bin.ensure(P1 * P1));
+    LCH(launch_sub_tables(h->sub, h->p, h->sub_up.p, h->sub_fp.p, h->sub_bin.p, st));
   }
   const int p = h->p, P1 = p + 1;
-  CK(cudaMemsetAsync(h->err.p, 0, sizeof(unsigned), st));
+  // the error word, and the direct stars' slots reserved so far
+  CK(cudaMemsetAsync(h->err.p, 0, 2 * sizeof(unsigned), st));
 
   // up-sweep: P2M at every leaf, then M2M level by level towards the root
   // (M2L reads multipoles of levels >= 2 only)
@@ -630,6 +635,8 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   C.y0 = P.x0[1];
   C.hx = P.h[0];
   C.hy = P.h[1];
+  C.inv_hx = 1.0 / P.h[0];
+  C.inv_hy = 1.0 / P.h[1];
   C.lox = P.center_y[0] - P.half_length;
   C.loy = P.center_y[1] - P.half_length_y;
   C.delta = P.delta;
@@ -638,24 +645,23 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   C.rect_c1 = h->opt.star_rect[0];
   C.rect_c2 = h->opt.star_rect[1];
   const int64_t n_rec = h->n_active << (2 * h->sub);
-  LCH(launch_near_count(T, C, h->n_active, h->active_list.p, h->near_cnt.p, h->err.p, st));
-  CKS(cub_call(h, plan, [&](void *tmp, size_t &bytes) {
-    return cub::DeviceScan::ExclusiveSum(tmp, bytes, h->near_cnt.p, h->near_off.p, (int)n_rec,
-                                         st);
-  }));
   if (plan) {
-    const int32_t *src[2] = {h->near_off.p + (n_rec - 1), h->near_cnt.p + (n_rec - 1)};
-    int32_t ab[2];
-    CKS(read_ints(h, st, 2, src, ab));
-    h->n_near = (int64_t)ab[0] + ab[1];
+    unsigned *count = h->err.p + 1;
+    LCH(launch_near_count(T, C, h->n_active, h->active_list.p, count, h->err.p, st));
+    const int32_t *src[1] = {reinterpret_cast<const int32_t *>(count)};
+    int32_t total;
+    CKS(read_ints(h, st, 1, src, &total));
+    h->n_near = total;
     CK(h->leaf.ensure(n_rec));
     CK(h->near_pos.ensure(h->n_near));
     CK(h->near_m.ensure(h->n_near));
     CK(h->coef.ensure((size_t)n_rec * coef_stride(h->p_eval)));
+    CK(cudaMemsetAsync(count, 0, sizeof(unsigned), st));
   }
-  LCH(launch_leaf_finalize(T, C, h->n_active, h->active_list.p, h->near_off.p, h->near_cnt.p,
-                          h->loc.p, h->leaf.p, h->near_pos.p, h->near_m.p, h->coef.p,
-                          h->err.p, st));
+  const SubTables tb = {h->sub_up.p, h->sub_fp.p, h->sub_bin.p};
+  LCH(launch_leaf_finalize(T, C, h->n_active, h->active_list.p, tb, h->loc.p, h->leaf.p,
+                           h->near_pos.p, h->near_m.p, h->coef.p, h->err.p + 1,
+                           (unsigned)h->n_near, h->err.p, st));
 
   if (plan) {
     // lookup grid over the active cell rectangle, as deep as 4M entries allow
@@ -839,8 +845,8 @@ static mm_status alloc_map_buffers(mm_map *h) {
       for (size_t k = have; k < h->seg_ev.size(); k++) CK(cudaEventCreate(&h->seg_ev[k]));
     }
   }
-  CK(h->err.ensure(1));
-  CK(cudaMemset(h->err.p, 0, sizeof(unsigned)));  // read after the plan in every mode
+  CK(h->err.ensure(2));
+  CK(cudaMemset(h->err.p, 0, 2 * sizeof(unsigned)));  // read after the plan in every mode
   CK(h->d_md.ensure(1));
   return MM_OK;
 }
@@ -1742,13 +1748,16 @@ void mm_destroy(mm_map *h) {
                           &h->parent,    &h->nb,        &h->split,     &h->group,
                           &h->top_info,  &h->col_cell,  &h->row_cell,
                           &h->node_act,  &h->leaf_flag, &h->leaf_scan, &h->node_active,
-                          &h->active_list, &h->near_cnt, &h->near_off, &h->grid};
+                          &h->active_list, &h->grid};
   for (auto *b : ibs) b->release();
   DBuf<double2> *cbs[] = {&h->MMop, &h->MLop, &h->LLop, &h->mp, &h->loc};
   for (auto *b : cbs) b->release();
   h->leaf.release();
   h->near_pos.release();
   h->near_m.release();
+  h->sub_up.release();
+  h->sub_fp.release();
+  h->sub_bin.release();
   h->coef.release();
   h->acc.release();
   h->span.release();

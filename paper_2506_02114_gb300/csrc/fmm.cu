@@ -416,63 +416,82 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
 }
 
 // ---------------------------------------------------------------------------
-// Near field of an active leaf: the leaf, its same-level neighbour cells that
-// are nodes (with all their descendants), and the unsplit nodes one level up
-// covering the missing neighbour cells.
+// Leaf records.  A block of 128 threads forms 16 consecutive sub-cell records
+// (one leaf's with the default 4 x 4 sub-cells), eight lanes a record.
 // ---------------------------------------------------------------------------
-template <class F>
-__device__ __forceinline__ int for_each_near_range(const TreeDev &T, int64_t node, F &&f,
-                                                   unsigned *err) {
-  int level, nx, ny;
-  double zx, zy, L;
-  node_geom(T, node, level, nx, ny, zx, zy, L);
-  if (level == 0) {
-    f(T.sbeg[node], T.send[node]);
-    return 0;
-  }
-  const int64_t parent = T.parent[node];
-  int seen[9];
-  int nseen = 0;
-  for (int dy = -1; dy <= 1; dy++)
-    for (int dx = -1; dx <= 1; dx++) {
-      const int x = nx + dx, y = ny + dy;
-      const int side = 1 << level;
-      if (x < 0 || y < 0 || x >= side || y >= side) continue;
-      const int id = T.nb[9 * node + (dy + 1) * 3 + (dx + 1)];
-      if (id >= 0) {
-        f(T.sbeg[id], T.send[id]);
-        continue;
+#define MM_REC 16  // records per block
+#define MM_REC_THREADS (8 * MM_REC)
+
+// The near field of the block's leaves: the leaf, its same-level neighbour
+// cells that are nodes (with all their descendants), and the unsplit nodes one
+// level up covering the missing neighbour cells, in row-major order and each
+// once.  Star i of leaf q is off[q][k] + i for the first k with i < end[q][k].
+struct NearRanges {
+  int off[MM_REC][9], end[MM_REC][9];
+};
+
+__device__ __forceinline__ void near_ranges(const TreeDev &T, const int32_t *active_list,
+                                            int64_t first_leaf, int n_leaf, NearRanges &N,
+                                            unsigned *err) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x & 15;
+  for (int q0 = 0; q0 < n_leaf; q0 += MM_REC_THREADS / 16) {
+    const int q = q0 + (threadIdx.x >> 4);
+    int src = -1, key = -2 - lane;
+    bool up = false;
+    if (q < n_leaf && k < 9) {
+      const int64_t node = active_list[first_leaf + q];
+      const int level = T.lvl[node], side = 1 << level;
+      uint32_t nx, ny;
+      morton_decode(T.code[node], nx, ny);
+      const int x = (int)nx + k % 3 - 1, y = (int)ny + k / 3 - 1;
+      if (x >= 0 && y >= 0 && x < side && y < side) {
+        src = T.nb[9 * node + k];
+        if (src < 0) {
+          up = true;
+          src = T.nb[9 * (int64_t)T.parent[node] + ((y >> 1) - (int)(ny >> 1) + 1) * 3 +
+                     ((x >> 1) - (int)(nx >> 1) + 1)];
+          if (src < 0) atomicOr(err, ERR_TREE_INVARIANT);
+          if (src >= 0) key = src;
+        }
       }
-      const int pid =
-          T.nb[9 * parent + ((y >> 1) - (ny >> 1) + 1) * 3 + ((x >> 1) - (nx >> 1) + 1)];
-      if (pid < 0) {
-        atomicOr(err, ERR_TREE_INVARIANT);
-        continue;
-      }
-      bool dup = false;
-      for (int s = 0; s < nseen; s++) dup |= (seen[s] == pid);
-      if (dup) continue;
-      seen[nseen++] = pid;
-      f(T.sbeg[pid], T.send[pid]);
     }
-  return 0;
+    // a coarser node covers several cells: taken at the first
+    const unsigned same = __match_any_sync(0xffffffffu, key) & (0xffffu << (lane & 16));
+    if (up && (same & ((1u << lane) - 1u))) src = -1;
+    const int b = src >= 0 ? T.sbeg[src] : 0, cnt = src >= 0 ? T.send[src] - b : 0;
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, d, 16);
+      if (k >= d) incl += u;
+    }
+    if (q < n_leaf && k < 9) {
+      N.off[q][k] = b - (incl - cnt);
+      N.end[q][k] = incl;
+    }
+  }
 }
 
-// Sub-cell q of active leaf t (records are numbered g = 4^s t + q, q
-// row-major with y major): its centre and half-length.
-__device__ __forceinline__ void sub_cell_geom(const TreeDev &T, const FmmConst &C,
-                                              const int32_t *active_list, int64_t g,
-                                              int64_t &node, double &zx, double &zy,
-                                              double &L, double &cx, double &cy, double &Lq) {
-  const int ns = 1 << C.sub, NS = ns * ns;
-  const int64_t t = g / NS;
-  const int q = (int)(g % NS), qx = q & (ns - 1), qy = q >> C.sub;
-  node = active_list[t];
+__device__ __forceinline__ int near_star(const NearRanges &N, int q, int i) {
+  int k = 0;
+  while (k < 8 && i >= N.end[q][k]) k++;
+  return N.off[q][k] + i;
+}
+
+// Sub-cell record g (records are numbered 4^s t + q for active leaf t, q
+// row-major with y major): its leaf's node and, along axis ax, the leaf's and
+// the sub-cell's centre.
+__device__ __forceinline__ void sub_cell_axis(const TreeDev &T, const FmmConst &C, int64_t node,
+                                              int64_t g, int ax, double &z, double &L, double &c,
+                                              double &Lq) {
+  const int ns = 1 << C.sub, q = (int)(g & (ns * ns - 1));
+  const int qa = ax ? q >> C.sub : q & (ns - 1);
   int level, nx, ny;
+  double zx, zy;
   node_geom(T, node, level, nx, ny, zx, zy, L);
-  Lq = L / ns;
-  cx = zx + (double)(2 * qx + 1 - ns) * Lq;
-  cy = zy + (double)(2 * qy + 1 - ns) * Lq;
+  z = ax ? zy : zx;
+  Lq = L * pow2(-C.sub);
+  c = z + (double)(2 * qa + 1 - ns) * Lq;
 }
 
 // Whether a star of the leaf's near field stays in the sub-cell's direct
@@ -488,153 +507,327 @@ __device__ __forceinline__ bool stays_direct(const FmmConst &C, double dx, doubl
   return fabs(dx) < hw && fabs(dy) < hw;
 }
 
-// Direct-sum stars per sub-cell record.
-__global__ void k_near_count(TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list,
-                             int32_t *near_cnt, unsigned *err) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_rec) return;
-  int64_t node;
-  double zx, zy, L, cx, cy, Lq;
-  sub_cell_geom(T, C, active_list, g, node, zx, zy, L, cx, cy, Lq);
-  int64_t total = 0;
-  for_each_near_range(
-      T, node,
-      [&](int64_t b, int64_t e) {
-        for (int64_t i = b; i < e; i++) total += stays_direct(C, T.sx[i] - cx, T.sy[i] - cy, Lq);
-      },
-      err);
-  near_cnt[g] = (int32_t)total;
+// Direct-sum stars of the block's record `rec` (all eight lanes).
+__device__ __forceinline__ int count_direct(const TreeDev &T, const FmmConst &C,
+                                            const NearRanges &N, int q, int total, int longest,
+                                            double cx, double cy, double Lq) {
+  const int j = threadIdx.x & 7, sh = threadIdx.x & 24;
+  if (C.sub == 0) return total;
+  int cnt = 0;
+  for (int c = 0; c < longest; c += 8) {
+    bool d = false;
+    if (c + j < total) {
+      const int i = near_star(N, q, c + j);
+      d = stays_direct(C, T.sx[i] - cx, T.sy[i] - cy, Lq);
+    }
+    cnt += __popc((__ballot_sync(0xffffffffu, d) >> sh) & 0xffu);
+  }
+  return cnt;
 }
 
-// One thread per sub-cell record g (active leaf t, sub-cell q).  The leaf's
-// local expansion psi = sum_l c_l zeta^l, zeta = (z - z_c)/L, is re-centred
-// exactly on the sub-cell centre z_q (an L2L translation to a descendant of
-// the leaf, which receives no further M2L terms: its far field is the
-// leaf's):
+// Direct-sum stars of all records, added to *total (the plan sizes their
+// arrays with it).
+__global__ void __launch_bounds__(MM_REC_THREADS)
+    k_near_count(TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list,
+                 unsigned *total, unsigned *err) {
+  __shared__ NearRanges N;
+  const int n_leaf_max = MM_REC >> (2 * C.sub);
+  const int64_t g0 = (int64_t)blockIdx.x * MM_REC, first_leaf = g0 >> (2 * C.sub);
+  const int n_leaf = (int)min((int64_t)n_leaf_max, (n_rec >> (2 * C.sub)) - first_leaf);
+  near_ranges(T, active_list, first_leaf, n_leaf, N, err);
+  __syncthreads();
+  const int rec = threadIdx.x >> 3, q = rec >> (2 * C.sub);
+  const bool valid = g0 + rec < n_rec;
+  double cx = 0.0, cy = 0.0, z, L, Lq = 0.0;
+  if (valid) {
+    const int64_t node = active_list[first_leaf + q];
+    sub_cell_axis(T, C, node, g0 + rec, 0, z, L, cx, Lq);
+    sub_cell_axis(T, C, node, g0 + rec, 1, z, L, cy, Lq);
+  }
+  const int mine = valid ? N.end[q][8] : 0;
+  const int longest = __reduce_max_sync(0xffffffffu, mine);
+  const int cnt = count_direct(T, C, N, valid ? q : 0, mine, longest, cx, cy, Lq);
+  if ((threadIdx.x & 7) == 0 && cnt) atomicAdd(total, (unsigned)cnt);
+}
+
+// Complex product a b in FP32 with a fixed order of rounding (a sum of two
+// products could be contracted either way).
+__device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+
+// Powers u^k of the sub-cells' positions u = (z_q - z_c)/L in their leaf, in
+// FP64 and FP32, [k][q], and the binomials C(n + m, n) in FP32, [n][m]: what
+// every re-centring of a plan shares.
+__global__ void k_sub_tables(int sub, int p, double2 *up, float2 *fp, float *bin) {
+  const int ns = 1 << sub, NS = ns * ns, t = threadIdx.x;
+  if (t < NS) {
+    const double ux = (double)(2 * (t & (ns - 1)) + 1 - ns) / ns;
+    const double uy = (double)(2 * (t >> sub) + 1 - ns) / ns;
+    const double2 u = make_double2(ux, uy);
+    const float2 fu = make_float2((float)ux, (float)uy);
+    double2 w = make_double2(1.0, 0.0);
+    float2 fw = make_float2(1.f, 0.f);
+    for (int k = 0; k <= p; k++) {
+      up[k * NS + t] = w;
+      fp[k * NS + t] = fw;
+      w = cmul(w, u);
+      fw = cmul32(fw, fu);
+    }
+  }
+  for (int n = t; n <= p; n += blockDim.x) {
+    float binom = 1.f;
+    for (int l = n; l <= p; l++) {
+      bin[n * (p + 1) + l - n] = binom;
+      binom = binom * (float)(l + 1) / (float)(l + 1 - n);
+    }
+  }
+}
+
+// 1/x: hardware approximation refined by two Newton-Raphson steps.
+__device__ __forceinline__ double rcp_near(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  y = fma(y, e, y);
+  e = fma(-x, y, 1.0);
+  return fma(y, e, y);
+}
+// a / x from y ~ 1/x: the quotient corrected by its exact remainder.
+__device__ __forceinline__ double div_near(double a, double x, double y) {
+  const double q = a * y;
+  return fma(fma(-x, q, a), y, q);
+}
+
+// x / n for a small integer n, correctly rounded (Markstein's correction).
+__device__ __forceinline__ float div_by_f(float x, float n, float inv_n) {
+  const float q = x * inv_n;
+  return fmaf(fmaf(-n, q, x), inv_n, q);
+}
+
+// Shared memory of k_leaf_finalize<NB>.
+template <int NB>
+struct RecSmem {
+  NearRanges N;
+  double c[2][MM_REC], r[2][MM_REC], Lq[MM_REC], d1[2][MM_REC];
+  float fs[MM_REC];                         // 1 / (L_q delta)
+  double star[MM_REC][8][3];                // far stars of a round: mass, 1/w
+  float2 v[MM_REC][8 * (NB - 1) + 2];       // their terms m w^-n / n
+  float F[MM_REC], md[MM_REC];
+  int cnt[MM_REC];
+  unsigned base;
+  double2 lg[MM_REC][4];                    // corner logarithms (rectangular region)
+};
+
+// The leaf's local expansion psi = sum_l c_l zeta^l, zeta = (z - z_c)/L, is
+// re-centred exactly on each sub-cell's centre z_q (an L2L translation to a
+// descendant of the leaf, which receives no further M2L terms: its far field
+// is the leaf's):
 //   d_n = (L_q/L)^n sum_{l>=n} C(l, n) c_l u^(l-n),  u = (z_q - z_c)/L;
 // the leaf's near-field stars that leave the direct sum (stays_direct) add
 // their own expansion about z_q (P2L): m log(z - z_i) contributes
 //   d_n += -m / (n w^n),  w = (z_i - z_q)/L_q,  n >= 1,
 // and the result is kept to n <= p_eval.  A record's coefficients
 // e_n = n d_n / (L_q delta), n = 2..p_eval, take coef_stride(p_eval) slots
-// (an even count, zero-padded) so the kernel loads them in pairs; its
-// direct stars are stored in its own grid frame.
-// NB >= p_eval bounds the coefficients at compile time, so they stay in
-// registers.
+// (an even count, zero-padded) so the kernel loads them in pairs; its direct
+// stars are stored in its own grid frame.  d_1 sets the FP64 image of the
+// centre and is formed in FP64; d_2..d_pe are stored as FP32 coefficients,
+// scaled to the sub-cell (terms decay like the convergence ratio), and are
+// formed in FP32 from FP32 copies of the leaf's coefficients (GB300's FP64
+// rate is 1/64 of its FP32 rate).
+//
+// Bound by the FP64 pipe where there are many records (two lanes an SM: the
+// stars' positions and 1/w, the centre's image) and by the length of a
+// record's chain of steps where there are few.  Eight lanes a record: a lane
+// sums every eighth n of d_n, the stars' FP64 work and powers go one to a
+// lane, eight at a time, and their terms are then added up n by n in the
+// stars' order; the direct stars of a record are only noted in that pass and
+// put into its frame together; powers and binomials come from the plan's
+// tables; 32 threads form the 16 records' centres, d_1 and images, one axis
+// each.  Records reserve their direct stars' slots themselves.  67 000 records
+// of 50 000 stars: 307 us with a thread a record (after a count and a scan of
+// 32 us), 188 us like this; a 48^2 map's 848 records 160 and 30 us.
+// NB >= p_eval.
 template <int NB>
-__global__ void __launch_bounds__(64) k_leaf_finalize(TreeDev T, FmmConst C, int64_t n_rec,
-                                const int32_t *active_list, const int32_t *near_off,
-                                const int32_t *near_cnt, const double2 *__restrict__ loc,
-                                LeafRec *leaf, NearPos *near_pos, float *near_m, float2 *coef,
-                                unsigned *err) {
-  __shared__ float2 s_cf[64][MM_PMAX + 1];  // per thread: FP32 copy of the leaf's coefficients
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_rec) return;
-  int64_t node;
-  double zx, zy, L, cx, cy, Lq;
-  sub_cell_geom(T, C, active_list, g, node, zx, zy, L, cx, cy, Lq);
+__global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
+    TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list, SubTables tb,
+    const double2 *__restrict__ loc, LeafRec *leaf, NearPos *near_pos, float *near_m,
+    float2 *coef, unsigned *near_total, unsigned near_cap, unsigned *err) {
+  extern __shared__ __align__(16) unsigned char s_rec[];
+  RecSmem<NB> &S = *reinterpret_cast<RecSmem<NB> *>(s_rec);
   const int p = C.p, P1 = p + 1, pe = min(C.p_eval, NB), cs = coef_stride(pe);
+  const int sub2 = 2 * C.sub, NS = 1 << sub2, bs = P1 | 1;
+  float2 *cf = reinterpret_cast<float2 *>(&S + 1);  // [leaf][l]
+  float2 *fp = cf + (MM_REC >> sub2) * P1;          // [k][q]
+  float *bin = reinterpret_cast<float *>(fp + P1 * NS);  // [n][m], stride bs
+  const int tid = threadIdx.x, rec = tid >> 3, j = tid & 7, sh = tid & 24;
+  const int64_t g0 = (int64_t)blockIdx.x * MM_REC, g = g0 + rec;
+  const int64_t first_leaf = g0 >> sub2;
+  const int n_leaf = (int)min((int64_t)(MM_REC >> sub2), (n_rec >> sub2) - first_leaf);
+  const int n_here = n_leaf << sub2;  // records of this block
+  const bool valid = rec < n_here;
+  const int q = valid ? rec >> sub2 : 0, sq = rec & (NS - 1);
 
-  // the grid vertex nearest the sub-cell centre
-  const double gi = rint((cx - C.x0) / C.hx), gj = rint((cy - C.y0) / C.hy);
-  const double xr = C.x0 + gi * C.hx, yr = C.y0 + gj * C.hy;
-  LeafRec R;
-  R.i_ref = (int32_t)gi;
-  R.j_ref = (int32_t)gj;
-  R.fcx = (float)((cx - xr) / C.hx);
-  R.fcy = (float)((cy - yr) / C.hy);
-  R.cull_side = MM_CULL_NONE;
-  R.cull_r2 = -1.f;
+  near_ranges(T, active_list, first_leaf, n_leaf, S.N, err);
+  for (int i = tid; i < n_leaf * P1; i += MM_REC_THREADS) {
+    const int lf = i / P1;
+    const double2 c = loc[(int64_t)active_list[first_leaf + lf] * P1 + (i - lf * P1)];
+    cf[i] = make_float2((float)c.x, (float)c.y);
+  }
+  for (int i = tid; i < P1 * NS; i += MM_REC_THREADS) fp[i] = tb.fp[i];
+  for (int i = tid; i < (pe + 1) * P1; i += MM_REC_THREADS)
+    bin[(i / P1) * bs + i % P1] = tb.bin[i];
 
-  // re-centred leaf expansion.  d_1 sets the FP64 image of the centre and is
-  // formed in FP64; d_2..d_pe are stored as FP32 coefficients, scaled to the
-  // sub-cell (terms decay like the convergence ratio), and are formed in
-  // FP32 from FP32 copies of the leaf's coefficients (GB300's FP64 rate is
-  // 1/64 of its FP32 rate).
-  const double2 *c = loc + node * P1;
-  const double ux = (cx - zx) / L, uy = (cy - zy) / L, r = Lq / L;
-  double2 d1 = make_double2(0.0, 0.0);
-  if (pe >= 1) {
-    double sx = 0.0, sy = 0.0, px = 1.0, py = 0.0;  // u^(l-1); C(l, 1) = l
+  // threads 0..31: record tid / 2, axis tid % 2
+  const int rec2 = tid >> 1, ax = tid & 1;
+  int ref = 0;
+  float fc = 0.f;
+  double ctr = 0.0, Lq2 = 1.0;
+  int node2 = 0;
+  if (tid < 32 && rec2 < n_here) {
+    node2 = active_list[first_leaf + (rec2 >> sub2)];
+    double z, L;
+    sub_cell_axis(T, C, node2, g0 + rec2, ax, z, L, ctr, Lq2);
+    // the grid vertex nearest the sub-cell centre
+    const double h = ax ? C.hy : C.hx, x0 = ax ? C.y0 : C.x0;
+    const double gi = rint((ctr - x0) / h), xr = x0 + gi * h;
+    ref = (int)gi;
+    fc = (float)((ctr - xr) / h);
+    S.c[ax][rec2] = ctr;
+    S.r[ax][rec2] = xr;
+    if (!ax) {
+      S.Lq[rec2] = Lq2;
+      S.fs[rec2] = (float)(1.0 / (Lq2 * C.delta));
+    }
+    // d_1 of the leaf's expansion (pe >= 1: p >= 1)
+    const double2 *c = loc + (int64_t)node2 * P1;
+    double sum = 0.0;
     for (int l = 1; l <= p; l++) {
-      const double2 cl = c[l];
-      sx += l * (cl.x * px - cl.y * py);
-      sy += l * (cl.x * py + cl.y * px);
-      const double npx = px * ux - py * uy;
-      py = px * uy + py * ux;
-      px = npx;
+      const double2 cl = c[l], u = tb.up[(l - 1) * NS + (rec2 & (NS - 1))];
+      const double u1 = ax ? u.y : u.x, u2 = ax ? u.x : -u.y;
+      sum = fma((double)l, fma(cl.x, u1, cl.y * u2), sum);
     }
-    d1 = make_double2(sx * r, sy * r);
+    S.d1[ax][rec2] = sum * pow2(-C.sub);
   }
-  float2 *cf = s_cf[threadIdx.x];
-  for (int l = 0; l <= p; l++) cf[l] = make_float2((float)c[l].x, (float)c[l].y);
-  const float fux = (float)ux, fuy = (float)uy, fr = (float)r;
-  float2 d[NB + 1];
-  float rn = fr;
+  __syncthreads();
+
+  // re-centred coefficients: lane j holds n = 2 + j, 10 + j, ...
+  constexpr int NPL = (NB - 1 + 7) / 8;
+  float2 d[NPL];
+  {
+    const float2 *c = cf + q * P1;
 #pragma unroll
-  for (int n = 2; n <= NB; n++) {
-    d[n] = make_float2(0.f, 0.f);
-    if (n > pe) continue;
-    rn *= fr;
-    float sx = 0.f, sy = 0.f, px = 1.f, py = 0.f, binom = 1.f;  // u^(l-n), C(l, n)
-#pragma unroll 1
-    for (int l = n; l <= p; l++) {
-      const float2 cl = cf[l];
-      sx = fmaf(binom, cl.x * px - cl.y * py, sx);
-      sy = fmaf(binom, cl.x * py + cl.y * px, sy);
-      const float npx = px * fux - py * fuy;
-      py = px * fuy + py * fux;
-      px = npx;
-      binom = binom * (float)(l + 1) / (float)(l + 1 - n);
+    for (int i = 0; i < NPL; i++) {
+      const int n = 2 + j + 8 * i;
+      float sx = 0.f, sy = 0.f;
+      if (n <= pe) {
+        for (int m = 0; n + m <= p; m++) {
+          const float2 t = cmul32(c[n + m], fp[m * NS + sq]);
+          const float b = bin[n * bs + m];
+          sx = fmaf(b, t.x, sx);
+          sy = fmaf(b, t.y, sy);
+        }
+      }
+      const float rn = __int_as_float((127 - C.sub * n) << 23);  // (L_q/L)^n = 2^(-s n)
+      d[i] = make_float2(sx * rn, sy * rn);
     }
-    d[n] = make_float2(sx * rn, sy * rn);
   }
 
-  // near-field stars: direct (in this record's frame) or into the expansion;
-  // the direct ones never exceed the slots k_near_count reserved
-  int64_t k = near_off[g];
-  const int64_t kend = k + near_cnt[g];
-  double m_direct = 0.0;
-  for_each_near_range(
-      T, node,
-      [&](int64_t b, int64_t e) {
-        for (int64_t i = b; i < e; i++) {
-          const double dxs = T.sx[i] - cx, dys = T.sy[i] - cy;
-          if (stays_direct(C, dxs, dys, Lq) && k < kend) {
-            const double sxg = (T.sx[i] - xr) / C.hx, syg = (T.sy[i] - yr) / C.hy;
-            const double Kx = rint(sxg), Ky = rint(syg);
-            NearPos np;
-            np.Kx = (float)Kx;
-            np.fx = (float)(sxg - Kx);
-            np.Ky = (float)Ky;
-            np.fy = (float)(syg - Ky);
-            near_pos[k] = np;
-            near_m[k] = (float)T.sm[i];
-            m_direct += T.sm[i];
-            k++;
-          } else {
-            // 1/w = L_q / (z_i - z_q); d_1 in FP64, the rest in FP32
-            const double den = dxs * dxs + dys * dys;
-            const double ix = Lq * dxs / den, iy = -Lq * dys / den;
-            const double m = T.sm[i];
-            d1.x -= m * ix;
-            d1.y -= m * iy;
-            const float fix = (float)ix, fiy = (float)iy, fm = (float)m;
-            float tx = fix * fix - fiy * fiy, ty = 2.f * fix * fiy;  // w^-2
+  // slots of the direct stars
+  const double cx = S.c[0][valid ? rec : 0], cy = S.c[1][valid ? rec : 0];
+  const double Lq = S.Lq[valid ? rec : 0];
+  const int total = valid ? S.N.end[q][8] : 0;
+  const int longest = __reduce_max_sync(0xffffffffu, total);
+  const int n_dir = count_direct(T, C, S.N, q, total, longest, cx, cy, Lq);
+  if (j == 0) S.cnt[rec] = n_dir;
+  __syncthreads();
+  if (tid == 0) {
+    int sum = 0;
+    for (int r = 0; r < MM_REC; r++) {
+      const int c = S.cnt[r];
+      S.cnt[r] = sum;
+      sum += c;
+    }
+    S.base = atomicAdd(near_total, (unsigned)sum);
+  }
+  __syncthreads();
+  const unsigned off = S.base + (unsigned)S.cnt[rec];
+  // (never exceeded: the plan counted the same stars)
+  const bool room = off + (unsigned)n_dir <= near_cap;
+
+  // near-field stars, eight at a time: into the expansion, or noted as direct
+  double d1 = j < 2 ? S.d1[j][rec] : 0.0;
+  int k = 0;
+  for (int c = 0; c < longest; c += 8) {
+    const bool on = c + j < total;
+    bool dir = false;
+    int i = 0;
+    if (on) {
+      i = near_star(S.N, q, c + j);
+      const double dx = T.sx[i] - cx, dy = T.sy[i] - cy;
+      dir = stays_direct(C, dx, dy, Lq);
+      if (!dir) {
+        // 1/w = L_q / (z_i - z_q); d_1 in FP64, the rest in FP32
+        const double den = fma(dx, dx, dy * dy), rc = rcp_near(den);
+        const double ix = div_near(Lq * dx, den, rc), iy = div_near(-Lq * dy, den, rc);
+        const double m = T.sm[i];
+        S.star[rec][j][0] = m;
+        S.star[rec][j][1] = ix;
+        S.star[rec][j][2] = iy;
+        const float2 iw = make_float2((float)ix, (float)iy);
+        const float fm = (float)m;
+        float2 t = make_float2(fmaf(iw.x, iw.x, -__fmul_rn(iw.y, iw.y)), 2.f * iw.x * iw.y);  // w^-2
+        float2 *v = &S.v[rec][j * (NB - 1)];
 #pragma unroll
-            for (int n = 2; n <= NB; n++) {
-              if (n <= pe) {
-                d[n].x -= fm * tx / n;
-                d[n].y -= fm * ty / n;
-              }
-              const float ntx = tx * fix - ty * fiy;
-              ty = tx * fiy + ty * fix;
-              tx = ntx;
-            }
-          }
+        for (int n = 2; n <= NB; n++) {
+          v[n - 2] = make_float2(div_by_f(fm * t.x, (float)n, 1.f / n),
+                                 div_by_f(fm * t.y, (float)n, 1.f / n));
+          t = cmul32(t, iw);
         }
-      },
-      err);
+      }
+    }
+    const unsigned md = (__ballot_sync(0xffffffffu, on && dir) >> sh) & 0xffu;
+    unsigned mf = (__ballot_sync(0xffffffffu, on && !dir) >> sh) & 0xffu;
+    if (on && dir && room) near_m[off + k + __popc(md & ((1u << j) - 1u))] = __int_as_float(i);
+    k += __popc(md);
+    __syncwarp();
+    for (; mf; mf &= mf - 1) {
+      const int t = __ffs(mf) - 1;
+      if (j < 2) d1 -= S.star[rec][t][0] * S.star[rec][t][1 + j];
+#pragma unroll
+      for (int e = 0; e < NPL; e++) {
+        const int n = 2 + j + 8 * e;
+        if (n <= pe) {
+          const float2 v = S.v[rec][t * (NB - 1) + n - 2];
+          d[e].x -= v.x;
+          d[e].y -= v.y;
+        }
+      }
+    }
+    __syncwarp();
+  }
+  // the direct stars in the record's grid frame, and their mass (for the
+  // culling bound alone)
+  float md = 0.f;
+  if (room) {
+    const double xr = S.r[0][rec], yr = S.r[1][rec];
+    for (int t = j; t < n_dir; t += 8) {
+      const int i = __float_as_int(near_m[off + t]);
+      const double sxg = div_near(T.sx[i] - xr, C.hx, C.inv_hx);
+      const double syg = div_near(T.sy[i] - yr, C.hy, C.inv_hy);
+      const double Kx = rint(sxg), Ky = rint(syg);
+      NearPos np;
+      np.Kx = (float)Kx;
+      np.fx = (float)(sxg - Kx);
+      np.Ky = (float)Ky;
+      np.fy = (float)(syg - Ky);
+      near_pos[off + t] = np;
+      const float m = (float)T.sm[i];
+      near_m[off + t] = m;
+      md += m;
+    }
+  }
+  for (int b = 1; b < 8; b <<= 1) md += __shfl_xor_sync(0xffffffffu, md, b);
 
   // Rectangular star region: the sheet's part beyond -kappa_star z is the
   // conjugate of At, analytic inside the rectangle, so its potential joins
@@ -644,117 +837,164 @@ __global__ void __launch_bounds__(64) k_leaf_finalize(TreeDev T, FmmConst C, int
   // i.e. d_n += (kappa_star i / pi) L_q^2 sum_a s_a r_a^(n-2) / (n (n-1) (n-2))
   // for n >= 3, r_a = L_q / (a - z_q).  No per-ray cost.
   if (C.rect_c1 > 0.0) {
-    const double2 t0 = rect_sheet_At(C.kappa_star, C.rect_c1, C.rect_c2, cx, cy);
-    d1.x += t0.x * Lq;
-    d1.y += t0.y * Lq;
-    const double f = C.kappa_star / 3.14159265358979323846;
-    double lx = 0.0, ly = 0.0, rx[4], ry[4], px[4], py[4], sg[4], dmin2 = 1e300;
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      double ax, ay;
-      rect_corner(C.rect_c1, C.rect_c2, k, ax, ay, sg[k]);
-      const double dx = ax - cx, dy = ay - cy, q = Lq / (dx * dx + dy * dy);
-      dmin2 = fmin(dmin2, dx * dx + dy * dy);
-      const double2 l = clog64(dx, dy);
-      lx -= sg[k] * l.x;
-      ly -= sg[k] * l.y;
-      rx[k] = dx * q;   // L_q / (a - z_q)
-      ry[k] = -dy * q;
-      px[k] = 1.0;      // r_a^(n-2)
-      py[k] = 0.0;
+    __syncthreads();
+    if (tid < 4 * MM_REC && (tid >> 2) < n_here) {
+      double ax_, ay_, sg;
+      rect_corner(C.rect_c1, C.rect_c2, tid & 3, ax_, ay_, sg);
+      S.lg[tid >> 2][tid & 3] = clog64(ax_ - S.c[0][tid >> 2], ay_ - S.c[1][tid >> 2]);
     }
-    // the series converges like sqrt(2) L_q / (distance to the nearest
-    // corner) over the record; beyond 1/2 its truncation is not negligible
-    // (only sub-cells meeting the ray grid are ever evaluated)
-    const bool on_grid = cx + Lq >= C.x0 && cx - Lq <= C.x1 && cy + Lq >= C.y0 && cy - Lq <= C.y1;
-    if (on_grid && 2.0 * Lq * Lq > 0.25 * dmin2) atomicOr(err, ERR_RECT_CORNER);
-    const double l2 = Lq * Lq;
-    if (pe >= 2) {
-      d[2].x += (float)((-f * ly - C.kappa_star) * l2 * 0.5);
-      d[2].y += (float)(f * lx * l2 * 0.5);
-    }
+    __syncthreads();
+    if (tid < n_here) {
+      const double zx = S.c[0][tid], zy = S.c[1][tid], lq = S.Lq[tid];
+      const double f = C.kappa_star / 3.14159265358979323846;
+      double gx = 0.0, gy = 0.0, lx = 0.0, ly = 0.0, rx[4], ry[4], px[4], py[4], sg[4];
+      double dmin2 = 1e300;
 #pragma unroll
-    for (int n = 3; n <= NB; n++) {
-      double sx = 0.0, sy = 0.0;
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const double t = px[k] * rx[k] - py[k] * ry[k];
-        py[k] = px[k] * ry[k] + py[k] * rx[k];
-        px[k] = t;
-        sx += sg[k] * px[k];
-        sy += sg[k] * py[k];
+      for (int a = 0; a < 4; a++) {
+        double ax_, ay_;
+        rect_corner(C.rect_c1, C.rect_c2, a, ax_, ay_, sg[a]);
+        const double dx = ax_ - zx, dy = ay_ - zy, w = lq / (dx * dx + dy * dy);
+        dmin2 = fmin(dmin2, dx * dx + dy * dy);
+        const double2 l = S.lg[tid][a];
+        gx += sg[a] * (dx * l.x - dy * l.y);
+        gy += sg[a] * (dx * l.y + dy * l.x);
+        lx -= sg[a] * l.x;
+        ly -= sg[a] * l.y;
+        rx[a] = dx * w;   // L_q / (a - z_q)
+        ry[a] = -dy * w;
+        px[a] = 1.0;      // r_a^(n-2)
+        py[a] = 0.0;
       }
-      if (n <= pe) {
+      // At(z_q) (see rect_sheet_At)
+      S.star[tid][0][0] = -f * gy - C.kappa_star * (2.0 * C.rect_c1 + zx);
+      S.star[tid][0][1] = f * gx - C.kappa_star * zy;
+      // the series converges like sqrt(2) L_q / (distance to the nearest
+      // corner) over the record; beyond 1/2 its truncation is not negligible
+      // (only sub-cells meeting the ray grid are ever evaluated)
+      const bool on_grid = zx + lq >= C.x0 && zx - lq <= C.x1 && zy + lq >= C.y0 &&
+                           zy - lq <= C.y1;
+      if (on_grid && 2.0 * lq * lq > 0.25 * dmin2) atomicOr(err, ERR_RECT_CORNER);
+      const double l2 = lq * lq;
+      float2 *v = S.v[tid];
+      v[0] = make_float2((float)((-f * ly - C.kappa_star) * l2 * 0.5), (float)(f * lx * l2 * 0.5));
+      for (int n = 3; n <= pe; n++) {
+        double sx = 0.0, sy = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+          const double t = px[a] * rx[a] - py[a] * ry[a];
+          py[a] = px[a] * ry[a] + py[a] * rx[a];
+          px[a] = t;
+          sx += sg[a] * px[a];
+          sy += sg[a] * py[a];
+        }
         const double w = f * l2 / ((double)n * (n - 1) * (n - 2));  // times i
-        d[n].x += (float)(-w * sy);
-        d[n].y += (float)(w * sx);
+        v[n - 2] = make_float2((float)(-w * sy), (float)(w * sx));
+      }
+    }
+    __syncthreads();
+    if (valid) {
+      if (j < 2) d1 = fma(S.star[rec][0][j], Lq, d1);
+#pragma unroll
+      for (int e = 0; e < NPL; e++) {
+        const int n = 2 + j + 8 * e;
+        if (n <= pe) {
+          d[e].x += S.v[rec][n - 2].x;
+          d[e].y += S.v[rec][n - 2].y;
+        }
       }
     }
   }
-  R.near_off = near_off[g];
-  R.near_cnt = (int32_t)(k - R.near_off);
 
-  const double s = 1.0 / (Lq * C.delta);
-  const float fs = (float)s;
+  // coefficients, and the bound of the evaluated series over the sub-cell:
+  // sum_n |e_n| zeta_max^(n-1)
+  const float fs = S.fs[valid ? rec : 0];
+  const float hmax = (float)fmax(C.hx, C.hy), fLq = (float)Lq;
+  const float zmax = 1.4142137f * (fLq + hmax) / fLq;
+  float F = 0.f;
 #pragma unroll
-  for (int n = 2; n <= NB; n++)
-    if (n <= pe) coef[g * cs + (n - 2)] = make_float2(n * d[n].x * fs, n * d[n].y * fs);
-  for (int kk = pe - 1; kk < cs; kk++) coef[g * cs + kk] = make_float2(0.f, 0.f);
+  for (int e = 0; e < NPL; e++) {
+    const int n = 2 + j + 8 * e;
+    if (n <= pe) {
+      const float2 v = make_float2(n * d[e].x * fs, n * d[e].y * fs);
+      if (valid) coef[g * cs + (n - 2)] = v;
+      F = fmaf(sqrtf(fmaf(v.x, v.x, v.y * v.y)), powf(zmax, (float)(n - 1)), F);
+    }
+  }
+  for (int b = 1; b < 8; b <<= 1) F += __shfl_xor_sync(0xffffffffu, F, b);
+  if (valid && j == 0) {
+    for (int kk = pe - 1; kk < cs; kk++) coef[g * cs + kk] = make_float2(0.f, 0.f);
+    S.F[rec] = F;
+    S.md[rec] = md;
+    S.cnt[rec] = room ? n_dir : 0;
+    S.star[rec][1][2] = __hiloint2double(0, (int)off);
+  }
+  if (valid && j < 2) S.d1[j][rec] = d1;
+  __syncthreads();
+  if (tid >= 32) return;
 
   // FP64 image of the sub-cell centre: macro model + sheet - far field there
-  const double ak = 1.0 - C.kappa + C.kappa_star;
-  const double Wx = (ak + C.gamma) * cx - d1.x / Lq;
-  const double Wy = (ak - C.gamma) * cy + d1.y / Lq;  // - conj(d1/L_q)
-  double U = (Wx - C.lox) / C.delta, V = (Wy - C.loy) / C.delta;
-  // |Ui|, |Vi| < 2^28 keeps vertex pixel indices within +-2^29
+  const bool here = rec2 < n_here;
+  const int r2 = here ? rec2 : 0;
+  const double ak = 1.0 - C.kappa + C.kappa_star, a = ax ? ak - C.gamma : ak + C.gamma;
+  const double iLq = inv_pow2(Lq2), dq = S.d1[ax][r2] * iLq;
+  const double W = ax ? a * ctr + dq : a * ctr - dq;  // - conj(d1/L_q)
+  double U = (W - (ax ? C.loy : C.lox)) / C.delta;
+  // |Ui| < 2^28 keeps vertex pixel indices within +-2^29
   U = fmin(fmax(U, -2.0e8), 2.0e8);
-  V = fmin(fmax(V, -2.0e8), 2.0e8);
-  const double Ui = floor(U), Vi = floor(V);
-  R.Ui = (int32_t)Ui;
-  R.Vi = (int32_t)Vi;
-  R.Uf = (float)(U - Ui);
-  R.Vf = (float)(V - Vi);
-  R.zsx = (float)(C.hx / Lq);
-  R.zsy = (float)(C.hy / Lq);
-  R.coef_off = (int32_t)(g * cs);
-  R.node = (int32_t)node;
+  const double Ui = floor(U);
+  const int iU = (int)Ui;
+  const float fU = (float)(U - Ui), zs = (float)((ax ? C.hy : C.hx) * iLq);
 
   // Culling bounds.  A vertex of this sub-cell (grid offset within
   // L_s + h of its centre) lands at the centre's image plus the macro term,
   // the evaluated far-field series and the direct stars' deflection, all in
   // pixels.  The first two stay within a box of half-widths B about (U, V):
   // |macro| <= |1 - kappa + kappa_* +- gamma| (L_s + h)/delta and
-  // |series| <= sum_n |e_n| zeta_max^(n-1) over the stored coefficients.  If
-  // that box lies D pixels beyond a map edge, a vertex whose direct stars
-  // are all farther than M_direct / (delta (D - margin)) is deflected by
-  // them less than D - margin, so it lands beyond that edge too.
-  if (C.cull) {
-    const double ak = 1.0 - C.kappa + C.kappa_star;
-    const double hmax = fmax(C.hx, C.hy);
-    const double zmax = sqrt(2.0) * (Lq + hmax) / Lq;
-    double F = 0.0, zp = 1.0;
-#pragma unroll
-    for (int n = 2; n <= NB; n++) {
-      zp *= zmax;  // zeta_max^(n-1)
-      if (n <= pe) F += hypot((double)(n * d[n].x * fs), (double)(n * d[n].y * fs)) * zp;
-    }
-    F *= 1.01;
-    const double Bu = fabs(ak + C.gamma) * (Lq + hmax) / C.delta + F;
-    const double Bv = fabs(ak - C.gamma) * (Lq + hmax) / C.delta + F;
-    const double Uc = U, Vc = V, n = (double)C.npix, ny = (double)C.npix_y, margin = 2.0;
-    const double Dl = -(Uc + Bu), Dr = (Uc - Bu) - n, Db = -(Vc + Bv), Dt = (Vc - Bv) - ny;
-    double D = Dl;
-    int side = MM_CULL_LEFT;
-    if (Dr > D) D = Dr, side = MM_CULL_RIGHT;
-    if (Db > D) D = Db, side = MM_CULL_BOTTOM;
-    if (Dt > D) D = Dt, side = MM_CULL_TOP;
-    if (D > 2.0 * margin && U > -1.9e8 && U < 1.9e8 && V > -1.9e8 && V < 1.9e8) {
-      const double rc = m_direct / (C.delta * (D - margin) * C.hx);  // grid units of h_x
-      R.cull_side = side;
-      R.cull_r2 = (float)(rc * rc * 1.01);
-    }
+  // |series| <= F.  If that box lies D pixels beyond a map edge, a vertex
+  // whose direct stars are all farther than M_direct / (delta (D - margin))
+  // is deflected by them less than D - margin, so it lands beyond that edge
+  // too.  (F and M_direct are FP32 sums: 1 % covers their rounding.)
+  const double margin = 2.0;
+  const double B = fabs(a) * (Lq2 + fmax(C.hx, C.hy)) / C.delta + 1.01 * (double)S.F[r2];
+  const double Dlo = -(U + B), Dhi = (U - B) - (double)(ax ? C.npix_y : C.npix);
+  double D = Dlo;
+  int side = ax ? MM_CULL_BOTTOM : MM_CULL_LEFT;
+  if (Dhi > D) D = Dhi, side = ax ? MM_CULL_TOP : MM_CULL_RIGHT;
+  const bool in = U > -1.9e8 && U < 1.9e8;
+  // axis 1's numbers to axis 0's thread, which writes the record
+  const double D1 = __shfl_down_sync(0xffffffffu, D, 1);
+  const int side1 = __shfl_down_sync(0xffffffffu, side, 1);
+  const int in1 = __shfl_down_sync(0xffffffffu, (int)in, 1);
+  const int ref1 = __shfl_down_sync(0xffffffffu, ref, 1);
+  const int iU1 = __shfl_down_sync(0xffffffffu, iU, 1);
+  const float fc1 = __shfl_down_sync(0xffffffffu, fc, 1);
+  const float fU1 = __shfl_down_sync(0xffffffffu, fU, 1);
+  const float zs1 = __shfl_down_sync(0xffffffffu, zs, 1);
+  if (ax || !here) return;
+  if (D1 > D) D = D1, side = side1;
+  LeafRec R;
+  R.i_ref = ref;
+  R.j_ref = ref1;
+  R.fcx = fc;
+  R.fcy = fc1;
+  R.Ui = iU;
+  R.Vi = iU1;
+  R.Uf = fU;
+  R.Vf = fU1;
+  R.zsx = zs;
+  R.zsy = zs1;
+  R.near_off = __double2loint(S.star[rec2][1][2]);
+  R.near_cnt = S.cnt[rec2];
+  R.coef_off = (int32_t)((g0 + rec2) * cs);
+  R.node = node2;
+  R.cull_side = MM_CULL_NONE;
+  R.cull_r2 = -1.f;
+  if (C.cull && D > 2.0 * margin && in && in1) {
+    const double rc = 1.001 * (double)S.md[rec2] / (C.delta * (D - margin) * C.hx);  // of h_x
+    R.cull_side = side;
+    R.cull_r2 = (float)(rc * rc * 1.01);
   }
-  leaf[g] = R;
+  leaf[g0 + rec2] = R;
 }
 
 // ---------------------------------------------------------------------------
@@ -895,32 +1135,55 @@ cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const in
 }
 
 cudaError_t launch_near_count(const TreeDev &T, const FmmConst &C, int64_t n_active,
-                              const int32_t *active_list, int32_t *near_cnt, unsigned *err,
+                              const int32_t *active_list, unsigned *total, unsigned *err,
                               cudaStream_t st) {
   if (n_active <= 0) return cudaSuccess;
   const int64_t n = n_active << (2 * C.sub);
-  k_near_count<<<blocks_for(n, 128), 128, 0, st>>>(T, C, n, active_list, near_cnt, err);
+  k_near_count<<<blocks_for(n, MM_REC), MM_REC_THREADS, 0, st>>>(T, C, n, active_list, total, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sub_tables(int sub, int p, double2 *up, float2 *fp, float *bin,
+                              cudaStream_t st) {
+  k_sub_tables<<<1, 128, 0, st>>>(sub, p, up, fp, bin);
+  return cudaGetLastError();
+}
+
+template <int NB>
+static cudaError_t launch_finalize_t(const TreeDev &T, const FmmConst &C, int64_t n,
+                                     const int32_t *active_list, const SubTables &tb,
+                                     const double2 *loc, LeafRec *leaf, NearPos *near_pos,
+                                     float *near_m, float2 *coef, unsigned *near_total,
+                                     unsigned near_cap, unsigned *err, cudaStream_t st) {
+  const size_t P1 = (size_t)C.p + 1;
+  const size_t smem = sizeof(RecSmem<NB>) +
+                      sizeof(float2) * ((MM_REC >> (2 * C.sub)) * P1 + (P1 << (2 * C.sub))) +
+                      sizeof(float) * (std::min(C.p_eval, NB) + 1) * (P1 | 1);
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k_leaf_finalize<NB>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  k_leaf_finalize<NB><<<blocks_for(n, MM_REC), MM_REC_THREADS, smem, st>>>(
+      T, C, n, active_list, tb, loc, leaf, near_pos, near_m, coef, near_total, near_cap, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_leaf_finalize(const TreeDev &T, const FmmConst &C, int64_t n_active,
-                                 const int32_t *active_list, const int32_t *near_off,
-                                 const int32_t *near_cnt, const double2 *loc, LeafRec *leaf,
-                                 NearPos *near_pos, float *near_m, float2 *coef, unsigned *err,
-                                 cudaStream_t st) {
+                                 const int32_t *active_list, const SubTables &tb,
+                                 const double2 *loc, LeafRec *leaf, NearPos *near_pos,
+                                 float *near_m, float2 *coef, unsigned *near_total,
+                                 unsigned near_cap, unsigned *err, cudaStream_t st) {
   if (n_active <= 0) return cudaSuccess;
   const int64_t n = n_active << (2 * C.sub);
-  const unsigned nb = blocks_for(n, 64);
   if (C.p_eval <= 16)
-    k_leaf_finalize<16><<<nb, 64, 0, st>>>(T, C, n, active_list, near_off, near_cnt, loc, leaf,
-                                           near_pos, near_m, coef, err);
-  else if (C.p_eval <= 32)
-    k_leaf_finalize<32><<<nb, 64, 0, st>>>(T, C, n, active_list, near_off, near_cnt, loc, leaf,
-                                           near_pos, near_m, coef, err);
-  else
-    k_leaf_finalize<MM_PMAX><<<nb, 64, 0, st>>>(T, C, n, active_list, near_off, near_cnt, loc,
-                                                leaf, near_pos, near_m, coef, err);
-  return cudaGetLastError();
+    return launch_finalize_t<16>(T, C, n, active_list, tb, loc, leaf, near_pos, near_m, coef,
+                                 near_total, near_cap, err, st);
+  if (C.p_eval <= 32)
+    return launch_finalize_t<32>(T, C, n, active_list, tb, loc, leaf, near_pos, near_m, coef,
+                                 near_total, near_cap, err, st);
+  return launch_finalize_t<MM_PMAX>(T, C, n, active_list, tb, loc, leaf, near_pos, near_m, coef,
+                                    near_total, near_cap, err, st);
 }
 
 }  // namespace mm

@@ -81,6 +81,7 @@ struct FmmConst {
   int cull;                   // 1: compute the culling bounds
   double kappa, gamma, kappa_star;
   double x0, y0, hx, hy;      // ray grid
+  double inv_hx, inv_hy;      // 1 / hx, 1 / hy
   double x1, y1;              // the grid's last vertex
   double lox, loy, delta;     // map lower-left corner and pixel side
   double rect_c1, rect_c2;    // > 0: rectangular star region |x| <= c1, |y| <= c2 (App. B)
@@ -93,14 +94,25 @@ cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const doub
 cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const int32_t *node_act,
                          const double2 *MLop, const double2 *LLop, const double2 *mp,
                          double2 *loc, unsigned *err, cudaStream_t st);
+// *total += direct-sum stars of all records (the plan sizes their arrays)
 cudaError_t launch_near_count(const TreeDev &T, const FmmConst &C, int64_t n_active,
-                              const int32_t *active_list, int32_t *near_cnt, unsigned *err,
+                              const int32_t *active_list, unsigned *total, unsigned *err,
                               cudaStream_t st);
+// What every re-centring of a plan shares (k_sub_tables): powers of the
+// sub-cells' positions [k][q], k = 0 .. p, and binomials [n][m], n, m <= p.
+struct SubTables {
+  const double2 *up;
+  const float2 *fp;
+  const float *bin;
+};
+cudaError_t launch_sub_tables(int sub, int p, double2 *up, float2 *fp, float *bin,
+                              cudaStream_t st);
+// near_total: slots reserved so far (0 before the call), of near_cap
 cudaError_t launch_leaf_finalize(const TreeDev &T, const FmmConst &C, int64_t n_active,
-                                 const int32_t *active_list, const int32_t *near_off,
-                                 const int32_t *near_cnt,
+                                 const int32_t *active_list, const SubTables &tb,
                                  const double2 *loc, LeafRec *leaf, NearPos *near_pos,
-                                 float *near_m, float2 *coef, unsigned *err, cudaStream_t st);
+                                 float *near_m, float2 *coef, unsigned *near_total,
+                                 unsigned near_cap, unsigned *err, cudaStream_t st);
 void build_operator_tables(int p, std::vector<double2> &MM, std::vector<double2> &ML,
                            std::vector<double2> &LL);
 

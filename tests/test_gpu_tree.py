@@ -76,16 +76,18 @@ def test_tree_follows_the_split_rule(name):
 
 @pytest.mark.parametrize("p", [1, 2, 3, 20, 31, 32, 33, 40, 63, 64])
 @pytest.mark.parametrize("leaf", [4, 100])
-def test_deflection_at_every_dealing_of_the_order(oracle_mod, p, leaf):
+@pytest.mark.parametrize("sub", [-1, 1, 2])
+def test_deflection_at_every_dealing_of_the_order(oracle_mod, p, leaf, sub):
     """Worst case of the truncated translations: a source's multipole at the
     nearest well-separated cell converges like r = sqrt(2) / (4 - sqrt(2)), so
     the deflection's error is at most a few times r^p of the deflection (the
     leading coefficient 1 / (1 - r) = 2.2 for the potential, times p + 1 for
-    its derivative), on top of the FP32 evaluation."""
+    its derivative), on top of the FP32 evaluation.  The sub-cells' series are
+    cut where their own bound, (sqrt(2) / 3)^p, is below that."""
     m, pos = synthetic.star_field(17, 700, 30.0, synthetic.SALPETER_01_1)
     kappa, gamma, s = 0.4, 0.3, 0.2
     grid = dict(img_half=(6.0, 6.0), ray_grid=(241, 241))
-    h = mm.create(kappa, gamma, s, m, pos, 1.0, 16, fmm_order=p, leaf_size=leaf, sub_levels=-1,
+    h = mm.create(kappa, gamma, s, m, pos, 1.0, 16, fmm_order=p, leaf_size=leaf, sub_levels=sub,
                   **grid)
     z = 12.0 * np.stack([synthetic.uniform(8, 0, 2000), synthetic.uniform(8, 1, 2000)], 1) - 6.0
     w = mm.shoot_points(h, z)
