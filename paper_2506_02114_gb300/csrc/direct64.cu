@@ -159,8 +159,9 @@ __global__ void __launch_bounds__(256, 2) k_ipm_vertices(const MapDev *__restric
       prev_r.py = __shfl_down_sync(0xffffffffu, prev.py, 1);
       prev_r.fx = __shfl_down_sync(0xffffffffu, prev.fx, 1);
       prev_r.fy = __shfl_down_sync(0xffffffffu, prev.fy, 1);
-      tri_scan(M, q, prev, prev_r, cur_r, cell_col, ra, lc, lane);
-      tri_scan(M, q, prev, cur_r, cur, cell_col, ra, lc, lane);
+      const unsigned o = outcode(M, prev) & outcode(M, cur_r);
+      tri_scan(M, q, prev, prev_r, cur_r, cell_col && !(o & outcode(M, prev_r)), ra, lc, lane);
+      tri_scan(M, q, prev, cur_r, cur, cell_col && !(o & outcode(M, cur)), ra, lc, lane);
       share_out(M, q, false, lc, lane);
       prev = cur;
     }

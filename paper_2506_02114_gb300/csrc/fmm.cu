@@ -605,6 +605,10 @@ __device__ __forceinline__ float div_by_f(float x, float n, float inv_n) {
   return fmaf(fmaf(-n, q, x), inv_n, q);
 }
 
+// Place of coefficient k's real part in its record's floats (the imaginary
+// part two further): pairs are stored real parts first.
+__device__ __forceinline__ int coef_slot(int k) { return 4 * (k >> 1) + (k & 1); }
+
 // Shared memory of k_leaf_finalize<NB>.
 template <int NB>
 struct RecSmem {
@@ -916,13 +920,20 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     const int n = 2 + j + 8 * e;
     if (n <= pe) {
       const float2 v = make_float2(n * d[e].x * fs, n * d[e].y * fs);
-      if (valid) coef[g * cs + (n - 2)] = v;
+      if (valid) {
+        float *out = reinterpret_cast<float *>(coef + g * cs) + coef_slot(n - 2);
+        out[0] = v.x;
+        out[2] = v.y;
+      }
       F = fmaf(sqrtf(fmaf(v.x, v.x, v.y * v.y)), powf(zmax, (float)(n - 1)), F);
     }
   }
   for (int b = 1; b < 8; b <<= 1) F += __shfl_xor_sync(0xffffffffu, F, b);
   if (valid && j == 0) {
-    for (int kk = pe - 1; kk < cs; kk++) coef[g * cs + kk] = make_float2(0.f, 0.f);
+    for (int kk = pe - 1; kk < cs; kk++) {
+      float *out = reinterpret_cast<float *>(coef + g * cs) + coef_slot(kk);
+      out[0] = out[2] = 0.f;
+    }
     S.F[rec] = F;
     S.md[rec] = md;
     S.cnt[rec] = room ? n_dir : 0;

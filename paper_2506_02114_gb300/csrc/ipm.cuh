@@ -51,6 +51,7 @@ namespace mm {
 
 #define MM_VTX_INVALID INT_MIN
 #define MM_FIX_ONE 4294967296ull  // one whole triangle in fixed-point units
+#define MM_U24_ONE 16777216u      // and in 2^-24 triangles
 
 __device__ __forceinline__ float rcp_approx_f(float x) {
   float y;
@@ -67,6 +68,14 @@ __device__ __forceinline__ unsigned frac_to_u24(float f) {  // in 2^-24 triangle
 }
 __device__ __forceinline__ unsigned long long frac_to_fixed(float f) {
   return (unsigned long long)frac_to_u24(f) << 8;
+}
+
+// The map edges a vertex lies beyond, one bit each (0 when non-finite): a
+// triangle lies wholly beyond one edge when its vertices share a bit.
+__device__ __forceinline__ unsigned outcode(const MapDev &M, const Vtx &v) {
+  const unsigned c = (v.px < 0 ? 1u : 0u) | (v.px >= M.npix ? 2u : 0u) | (v.py < 0 ? 4u : 0u) |
+                     (v.py >= M.npix_y ? 8u : 0u);
+  return v.px == MM_VTX_INVALID ? 0u : c;
 }
 
 // ---------------------------------------------------------------------------
@@ -88,13 +97,10 @@ __device__ __forceinline__ bool mm_index_ok(unsigned *err, long long idx, long l
 #define MM_INDEX_OK(err, idx, n) true
 #endif
 
-// Add v fixed-point units to map pixel (gx, gy) if it lies in the map
-// (pixel indices stay within +-2^30: vertices are clamped to +-2^28 pixels
-// about their sub-cell's centre image, and boxes to +-1e9 of a vertex).
-__device__ __forceinline__ void deposit(const MapDev &M, int gx, int gy, unsigned long long v) {
-  if (v && gx >= 0 && gx < M.npix && gy >= 0 && gy < M.npix_y &&
-      MM_INDEX_OK(M.err, (long long)gy * M.npix + gx, (long long)M.npix * M.npix_y))
-    atomicAdd(&M.acc[(long long)gy * M.npix + gx], v);
+// Add u (in 2^-24 triangles) to map pixel idx if `in` the map.
+__device__ __forceinline__ void deposit(const MapDev &M, bool in, long long idx, unsigned u) {
+  if (in && u && MM_INDEX_OK(M.err, idx, (long long)M.npix * M.npix_y))
+    atomicAdd(&M.acc[idx], (unsigned long long)u << 8);
 }
 
 // The map's accumulators alone, passed as scalars to the out-of-line row
@@ -161,18 +167,17 @@ __device__ __forceinline__ float lone_vertex_share(float u0, float u1, float u2,
   return d * d * rcp_approx_f((ua - ul) * (ub - ul));
 }
 
-// Fixed-point share of T on the low side u < L of one grid line it crosses.
-// The line is chosen from the vertices' integer pixels, and a vertex's FP32
-// coordinate in a neighbouring pixel's frame can round onto the line (k + f
-// with f within 2^-24 of 1), leaving no vertex strictly below it: then
-// nothing of T lies below the line (and all of it when none lies above).
-__device__ __forceinline__ unsigned long long low_side_fixed(float u0, float u1, float u2,
-                                                             float L) {
+// Share of T (in 2^-24 triangles) on the low side u < L of one grid line it
+// crosses.  The line is chosen from the vertices' integer pixels, and a
+// vertex's FP32 coordinate in a neighbouring pixel's frame can round onto the
+// line (k + f with f within 2^-24 of 1), leaving no vertex strictly below it:
+// then nothing of T lies below the line (and all of it when none lies above).
+__device__ __forceinline__ unsigned low_side_u24(float u0, float u1, float u2, float L) {
   const int nlow = (u0 < L) + (u1 < L) + (u2 < L);
   bool lone_low;
   const float v = lone_vertex_share(u0, u1, u2, L, lone_low);
   const float low = nlow == 0 ? 0.f : (nlow == 3 ? 1.f : (lone_low ? v : 1.f - v));
-  return frac_to_fixed(low);
+  return frac_to_u24(low);
 }
 
 // Contribution of edge P -> Q to the signed area of T n {x < X, y < Y}
@@ -296,9 +301,13 @@ __device__ __forceinline__ bool line_tri_apportion(const MapDev &M, const RawTri
   const int o = ((x0 ^ x1) | (x0 ^ x2)) >= 0;
   const float L = 1.f - (float)(o ? ay : ax);
   const float u0 = o ? t[1] : t[0], u1 = o ? t[3] : t[2], u2 = o ? t[5] : t[4];
-  const unsigned long long vlow = low_side_fixed(u0, u1, u2, L);
-  deposit(M, e.x, e.y, vlow);
-  deposit(M, e.x + 1 - o, e.y + o, MM_FIX_ONE - vlow);
+  const unsigned low = low_side_u24(u0, u1, u2, L);
+  // (pixel indices stay within +-2^29)
+  const int hx = e.x + 1 - o, hy = e.y + o;
+  const long long idx = (long long)e.y * M.npix + e.x;
+  deposit(M, (unsigned)e.x < (unsigned)M.npix && (unsigned)e.y < (unsigned)M.npix_y, idx, low);
+  deposit(M, (unsigned)hx < (unsigned)M.npix && (unsigned)hy < (unsigned)M.npix_y,
+          idx + (o ? M.npix : 1), MM_U24_ONE - low);
   return true;
 }
 
@@ -318,19 +327,21 @@ __device__ __forceinline__ bool quad_tri_apportion(const MapDev &M, const RawTri
   const int r0 = (int)floorf(y0 + fminf(0.f, fminf(d1y, d2y)));
   // the grid lines, relative to the first vertex
   const float X = (float)(c0 + 1) - x0, Y = (float)(r0 + 1) - y0;
-  const long long vL = (long long)low_side_fixed(0.f, d1x, d2x, X);
-  const long long vB = (long long)low_side_fixed(0.f, d1y, d2y, Y);
+  const int vL = (int)low_side_u24(0.f, d1x, d2x, X);
+  const int vB = (int)low_side_u24(0.f, d1y, d2y, Y);
   const float lb = quadrant_edge(0.f, 0.f, d1x, d1y, X, Y) +
                    quadrant_edge(d1x, d1y, d2x, d2y, X, Y) +
                    quadrant_edge(d2x, d2y, 0.f, 0.f, X, Y);
   const float A2 = d1x * d2y - d2x * d1y;  // twice the signed area
-  const long long vLB = (long long)frac_to_fixed(2.f * lb * rcp_approx_f(A2));
-  const long long one = (long long)MM_FIX_ONE;
+  const int vLB = (int)frac_to_u24(2.f * lb * rcp_approx_f(A2));
   const int gx = e.x + ax + c0, gy = e.y + ay + r0;
-  deposit(M, gx, gy, (unsigned long long)vLB);
-  deposit(M, gx, gy + 1, (unsigned long long)max(vL - vLB, 0ll));
-  deposit(M, gx + 1, gy, (unsigned long long)max(vB - vLB, 0ll));
-  deposit(M, gx + 1, gy + 1, (unsigned long long)max(one - vL - vB + vLB, 0ll));
+  const bool x0in = (unsigned)gx < (unsigned)M.npix, x1in = (unsigned)(gx + 1) < (unsigned)M.npix;
+  const bool y0in = (unsigned)gy < (unsigned)M.npix_y, y1in = (unsigned)(gy + 1) < (unsigned)M.npix_y;
+  const long long idx = (long long)gy * M.npix + gx;
+  deposit(M, x0in && y0in, idx, (unsigned)vLB);
+  deposit(M, x0in && y1in, idx + M.npix, (unsigned)max(vL - vLB, 0));
+  deposit(M, x1in && y0in, idx + 1, (unsigned)max(vB - vLB, 0));
+  deposit(M, x1in && y1in, idx + M.npix + 1, (unsigned)max((int)MM_U24_ONE - vL - vB + vLB, 0));
   return true;
 }
 
@@ -382,36 +393,6 @@ __device__ __forceinline__ float edge_x_at(float y, float px, float py, float qx
                                           float k) {
   const float d1 = y - py, d2 = y - qy;
   return fabsf(d1) <= fabsf(d2) ? fmaf(d1, k, px) : fmaf(d2, k, qx);
-}
-
-// Packed FP32 pairs (sm_100 and later): one instruction, each half rounded
-// like the scalar operation.
-struct F2 {
-  float x, y;
-};
-__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
-  F2 r;
-  asm("{.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-      "mov.b64 c, {%6, %7};\n\tfma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;}"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return r;
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-  F2 r;
-  asm("{.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;}"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-  F2 r;
-  asm("{.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-      "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;}"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
 }
 
 // Mean of clamp(x, 0, 1) over x in [a, b] (a piece shifted to its pixel),
@@ -612,6 +593,7 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
   }
   __syncwarp();
   int row_first = 0;
+#pragma unroll 1
   for (int base = 0; base < total; base += 32) {
     const int task = base + lane;
     const int o = deal_owner_slot(nrows, excl, base, lane, row_first);
@@ -671,6 +653,7 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
     }
     __syncwarp();
     int px_first = 0;
+#pragma unroll 1
     for (int pbase = 0; pbase < ptotal; pbase += 32)
       pixel_task(M, rr, deal_owner_slot(np, pexcl, pbase, lane, px_first), pbase + lane, ptotal);
   }
@@ -712,6 +695,7 @@ struct __align__(16) WarpSmem {
     };
   };
   Vtx row[32];                    // the last vertex row, one vertex per lane
+  Vtx next[32];                   // the next one, where it was shot with it
   unsigned count[MM_N_COUNTERS];  // (dropped and critical are per lane, LaneCount)
 };
 #define MM_SHOOT_SMEM_BYTES (8 * sizeof(WarpSmem))  // 8 warps per block
@@ -722,21 +706,19 @@ struct WarpQueues {
 };
 
 // Apportion or queue one triangle (a, b, c) of each lane (`on`: the lane
-// has one).  A triangle inside one pixel is finished here.
+// has one, not wholly beyond one edge of the map).  A triangle inside one
+// pixel is finished here.
 __device__ __forceinline__ void tri_scan(const MapDev &M, WarpQueues &q, const Vtx &a,
                                          const Vtx &b, const Vtx &c, bool on, RunAcc &ra,
                                          LaneCount &lc, int lane) {
   // the pixel box from the vertices' pixels (a vertex's pixel is the floor
-  // of its coordinate, MM_VTX_INVALID = INT_MIN below any valid one); most
-  // triangles of a shooting region lie wholly beyond one edge of the map:
-  // integer tests before any arithmetic
+  // of its coordinate, MM_VTX_INVALID = INT_MIN below any valid one)
   const int xlo = min(a.px, min(b.px, c.px)), xhi = max(a.px, max(b.px, c.px));
   const int ylo = min(a.py, min(b.py, c.py)), yhi = max(a.py, max(b.py, c.py));
   if (on && xlo == MM_VTX_INVALID) {
     lc.dropped++;
     on = false;
   }
-  on = on && xhi >= 0 && xlo < M.npix && yhi >= 0 && ylo < M.npix_y;
   const int sx = xhi - xlo, sy = yhi - ylo;
   const unsigned span = (unsigned)(sx | sy);
   const bool one = on && span == 0u;
@@ -782,8 +764,10 @@ __device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool f
                                           LaneCount &lc, int lane) {
   if (!flush && ((q.line | q.quad | q.big) & ~31) == 0) return;
   int deal = 0;  // jobs set up to be dealt out here
+#pragma unroll 1
   while (true) {
     const bool rest = flush || deal > 0;
+#pragma unroll 1
     while (q.line >= 32 || (rest && q.line > 0)) {
       const int nb = min(q.line, 32);
       q.line -= nb;
@@ -792,6 +776,7 @@ __device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool f
       const unsigned n = __popc(__ballot_sync(0xffffffffu, done));
       if (lane == 0) q.s->count[ST_LINE] += n;
     }
+#pragma unroll 1
     while (q.quad >= 32 || (rest && q.quad > 0)) {
       const int nb = min(q.quad, 32);
       q.quad -= nb;

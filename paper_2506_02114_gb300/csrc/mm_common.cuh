@@ -120,7 +120,8 @@ struct MapDev {
 };
 
 // Far-field coefficient slots per sub-cell record: the p_eval - 1
-// coefficients rounded up to an even count (>= 2), loaded as float4 pairs.
+// coefficients rounded up to an even count (>= 2), loaded as float4 pairs
+// (re e_2j, re e_2j+1, im e_2j, im e_2j+1), the operands of packed arithmetic.
 __host__ __device__ __forceinline__ int coef_stride(int p_eval) {
   return p_eval <= 2 ? 2 : ((p_eval - 1 + 1) & ~1);
 }
@@ -138,6 +139,36 @@ __host__ __device__ __forceinline__ uint32_t gather16(uint32_t v) {
   v = (v | (v >> 2)) & 0x0f0f0f0fu;
   v = (v | (v >> 4)) & 0x00ff00ffu;
   return (v | (v >> 8)) & 0x0000ffffu;
+}
+
+// Packed FP32 pairs (sm_100 and later): one instruction, each half rounded
+// like the scalar operation.
+struct F2 {
+  float x, y;
+};
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("{.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mov.b64 c, {%6, %7};\n\tfma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("{.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("{.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
 }
 
 // Interleave two 21-bit integers: x in even bits, y in odd bits.

@@ -33,6 +33,7 @@ __device__ __forceinline__ int lookup_leaf(const MapDev &M, int cx, int cy) {
   int e = __ldg(&M.grid[(int64_t)gy * M.gw + gx]);
   if (e >= 0) return e;
   int node = -e - 1;
+#pragma unroll 1
   for (int lvl = M.glevel + 1; lvl <= MM_DMAX; lvl++) {
     int fc = __ldg(&M.first_child[node]);
     if (fc < 0) break;
@@ -46,55 +47,109 @@ __device__ __forceinline__ int lookup_leaf(const MapDev &M, int cx, int cy) {
   return (a << (2 * M.sub)) + (((cy >> sh) & mask) << M.sub) + ((cx >> sh) & mask);
 }
 
-// lookup_leaf with a per-lane cache keyed by the lookup-grid row: a grid
-// entry that names a record directly holds for every finest-level row of
-// that grid row (the lane's column is fixed), so consecutive vertex rows
-// skip the grid read until they leave it
-__device__ __forceinline__ int lookup_leaf_cached(const MapDev &M, int cx, int cy, int &c_gy,
-                                                  int &c_leaf, bool &c_cull) {
-  const int gy = (cy >> M.gshift) - M.gy0;
-  if (gy == c_gy) return c_leaf;
-  const int gx = (cx >> M.gshift) - M.gx0;
+// The records of vertex row j in every lane's column (lookup_leaf), whether
+// the lane's record can prove a vertex beyond the map at all, and the first
+// row after j that may lie in other records: a grid entry that names a record
+// holds for every row of its grid row (the lanes' columns are fixed), so the
+// rows up to `j_same` need no lookup.  Rows up to je.
+__device__ __forceinline__ int lookup_rows(const MapDev &M, int cx, int j, int je, int lane,
+                                           bool vvalid, int &j_same, bool &c_cull) {
+  const int cy = __ldg(&M.row_cell[j]);
+  const int gy = (cy >> M.gshift) - M.gy0, gx = (cx >> M.gshift) - M.gx0;
+  const int ahead = __ldg(&M.row_cell[min(j + 1 + lane, je)]);
   int e = -1;
-  if (gx >= 0 && gy >= 0 && gx < M.gw && gy < M.gh) {
-    e = __ldg(&M.grid[(int64_t)gy * M.gw + gx]);
-    if (e >= 0) {
-      c_gy = gy;
-      c_leaf = e;
-    } else {
-      c_gy = INT_MIN;  // a tree walk: not cached
-      e = lookup_leaf(M, cx, cy);
-    }
-  } else {
-    c_gy = INT_MIN;
-  }
-  // whether the record can prove a vertex beyond the map at all
+  if (gx >= 0 && gy >= 0 && gx < M.gw && gy < M.gh) e = __ldg(&M.grid[(int64_t)gy * M.gw + gx]);
+  const bool direct = e >= 0;
+  if (!direct) e = lookup_leaf(M, cx, cy);
   c_cull = e >= 0 && __ldg(&M.leaf[e].cull_side) != MM_CULL_NONE;
+  j_same = j + 1;
+  if (__all_sync(0xffffffffu, direct || !vvalid)) {
+    const unsigned other = __ballot_sync(0xffffffffu, (ahead >> M.gshift) - M.gy0 != gy);
+    j_same += other ? __ffs(other) - 1 : 32;
+  }
   return e;
 }
 
-// One Horner step of the two far-field chains: E <- E w + (c.x, c.y) and
-// O <- O w + (c.z, c.w) in complex arithmetic, w = (wx, wy).
-__device__ __forceinline__ void horner_pair(const float4 c, float wx, float wy, float &Er,
-                                            float &Ei, float &Or, float &Oi) {
-  const float er = fmaf(Er, wx, fmaf(-Ei, wy, c.x));
-  const float ei = fmaf(Er, wy, fmaf(Ei, wx, c.y));
-  const float orr = fmaf(Or, wx, fmaf(-Oi, wy, c.z));
-  const float oi = fmaf(Or, wy, fmaf(Oi, wx, c.w));
-  Er = er;
-  Ei = ei;
-  Or = orr;
-  Oi = oi;
+// Far field f = sum_{k>=0} e_k zeta^(k+1), e_k = (k+2) c_(k+2) / (L delta), as
+// zeta E(w) + w O(w), w = zeta^2, E and O the even and odd k: two independent
+// Horner chains as one chain of packed pairs, one (e_2j, e_2j+1) pair per
+// 16-byte load.  State of the chains at one point.
+struct FarField {
+  float zx, zy, wx, wy;
+  F2 re, im;  // (E, O)
+};
+__device__ __forceinline__ void far_start(FarField &f, float zx, float zy, float4 c) {
+  f.zx = zx;
+  f.zy = zy;
+  f.wx = fmaf(zx, zx, -zy * zy);
+  f.wy = 2.f * zx * zy;
+  f.re = F2{c.x, c.y};
+  f.im = F2{c.z, c.w};
+}
+// (E, O) <- (E, O) w + c in complex arithmetic.
+__device__ __forceinline__ void far_step(FarField &f, float4 c) {
+  const F2 wx = {f.wx, f.wx}, wy = {f.wy, f.wy}, nwy = {-f.wy, -f.wy};
+  const F2 re = f2_fma(f.re, wx, f2_fma(f.im, nwy, F2{c.x, c.y}));
+  f.im = f2_fma(f.re, wy, f2_fma(f.im, wx, F2{c.z, c.w}));
+  f.re = re;
+}
+__device__ __forceinline__ void far_end(const FarField &f, float &fr, float &fi) {
+  const float Er = f.re.x, Or = f.re.y, Ei = f.im.x, Oi = f.im.y;
+  fr = fmaf(f.zx, Er, fmaf(-f.zy, Ei, fmaf(f.wx, Or, -f.wy * Oi)));
+  fi = fmaf(f.zx, Ei, fmaf(f.zy, Er, fmaf(f.wx, Oi, f.wy * Or)));
+}
+
+// The coefficient pairs after the last, highest first, each applied to N
+// points; loaded G at a time, so that their latencies overlap (the usual 15
+// terms have six after the first pair).  G = 3 in the polygon-mapping kernel,
+// which has no registers for more and whose loop has to fit the instruction
+// cache; 6 in k_shoot_irs (2.64 ms against 2.72 with 3, 1537^2 map).
+template <int G, int N>
+__device__ __forceinline__ void far_chain(FarField (&f)[N], const float4 *e, int npair) {
+  int j = npair - 2;
+#pragma unroll 1
+  for (; j >= G - 1; j -= G) {
+    float4 cc[G];
+#pragma unroll
+    for (int q = 0; q < G; q++) cc[q] = __ldg(e + j - q);
+#pragma unroll
+    for (int q = 0; q < G; q++)
+#pragma unroll
+      for (int k = 0; k < N; k++) far_step(f[k], cc[q]);
+  }
+#pragma unroll 1
+  for (; j >= 0; j--) {
+    const float4 c = __ldg(e + j);
+#pragma unroll
+    for (int k = 0; k < N; k++) far_step(f[k], c);
+  }
+}
+
+// A source position (u, v) in pixels relative to pixel (Ui, Vi) in canonical
+// form.
+__device__ __forceinline__ Vtx pixel_form(bool ok, float u, float v, int Ui, int Vi) {
+  Vtx out;
+  if (!ok || !isfinite(u) || !isfinite(v)) {
+    out.px = MM_VTX_INVALID;
+    out.py = MM_VTX_INVALID;
+    out.fx = 0.f;
+    out.fy = 0.f;
+    return out;
+  }
+  const float lim = 268435456.0f;  // 2^28 pixels: far outside any map
+  u = fminf(fmaxf(u, -lim), lim);
+  v = fminf(fmaxf(v, -lim), lim);
+  float flu = floorf(u), flv = floorf(v);
+  out.px = Ui + (int)flu;
+  out.py = Vi + (int)flv;
+  out.fx = u - flu;
+  out.fy = v - flv;
+  return out;
 }
 
 // Source-plane position of grid point (i + ti, j + tj) in pixel units:
 // returns the integer pixel and the fraction.  ti = tj = 0 for ray vertices.
-// PRELOAD: the far-field coefficient pairs are loaded ahead of the Horner
-// steps (all six of the usual 15-term case at once, other orders four at a
-// time); else each where it is used, which holds fewer registers across the
-// steps (better in the polygon-mapping kernel of a map without a
-// second-pass queue, which deals every larger triangle itself).
-template <bool SQUARE, bool FRAC, bool PRELOAD = true>
+template <bool SQUARE, bool FRAC, int G = 3>
 __device__ __forceinline__ Vtx shoot_point(const MapDev &M, int leaf, int i, int j,
                                            float ti, float tj, bool valid) {
   const int4 *rp = reinterpret_cast<const int4 *>(M.leaf + (leaf < 0 ? 0 : leaf));
@@ -126,6 +181,7 @@ __device__ __forceinline__ Vtx shoot_point(const MapDev &M, int leaf, int i, int
   // contribution is selected away after the reciprocal (a stand-in on a
   // vertex would otherwise give 0 x 1/0 = NaN there)
   int k = 0;
+#pragma unroll 1
   for (; k + 1 < maxcnt; k += 2) {
     const bool a0 = k < near_cnt, a1 = k + 1 < near_cnt;
     const float4 s0 = a0 ? __ldg(np_ + k) : make_float4(0.f, 1.f, 0.f, 0.f);
@@ -163,64 +219,84 @@ __device__ __forceinline__ Vtx shoot_point(const MapDev &M, int leaf, int i, int
   Sx += Sx2;
   Sy += Sy2;
 
-  // far field: f = sum_{k>=0} e_k zeta^(k+1), e_k = (k+2) c_(k+2) / (L delta),
-  // as zeta E(w) + w O(w), w = zeta^2, E and O the even and odd k: two
-  // independent Horner chains, one (e_2j, e_2j+1) pair per 16-byte load
   float fr = 0.f, fim = 0.f;
   const int npair = M.p >> 1;
   if (npair >= 1 && leaf >= 0) {
-    const float zx = gx * zsx, zy = gy * zsy;
-    const float wx = fmaf(zx, zx, -zy * zy), wy = 2.f * zx * zy;
     const float4 *e = reinterpret_cast<const float4 *>(M.coef + coef_off);
-    const float4 c = __ldg(e + (npair - 1));
-    float Er = c.x, Ei = c.y, Or = c.z, Oi = c.w;
-    if (!PRELOAD) {
-      for (int j = npair - 2; j >= 0; j--) horner_pair(__ldg(e + j), wx, wy, Er, Ei, Or, Oi);
-    } else if (npair == 7) {
-      // the usual case (15 terms): the other six pairs are all loaded before
-      // the chains start, so their latencies overlap (a loop that loads each
-      // pair where it is used waits on every load in turn)
-      float4 cc[6];
-#pragma unroll
-      for (int j = 0; j < 6; j++) cc[j] = __ldg(e + j);
-#pragma unroll
-      for (int j = 5; j >= 0; j--) horner_pair(cc[j], wx, wy, Er, Ei, Or, Oi);
-    } else {
-      // other orders: four pairs loaded at a time
-      int j = npair - 2;
-      for (; j >= 3; j -= 4) {
-        const float4 c0 = __ldg(e + j), c1 = __ldg(e + j - 1), c2 = __ldg(e + j - 2),
-                     c3 = __ldg(e + j - 3);
-        horner_pair(c0, wx, wy, Er, Ei, Or, Oi);
-        horner_pair(c1, wx, wy, Er, Ei, Or, Oi);
-        horner_pair(c2, wx, wy, Er, Ei, Or, Oi);
-        horner_pair(c3, wx, wy, Er, Ei, Or, Oi);
-      }
-      for (; j >= 0; j--) horner_pair(__ldg(e + j), wx, wy, Er, Ei, Or, Oi);
-    }
-    fr = fmaf(zx, Er, fmaf(-zy, Ei, fmaf(wx, Or, -wy * Oi)));
-    fim = fmaf(zx, Ei, fmaf(zy, Er, fmaf(wx, Oi, wy * Or)));
+    FarField f[1];
+    far_start(f[0], gx * zsx, gy * zsy, __ldg(e + (npair - 1)));
+    far_chain<G>(f, e, npair);
+    far_end(f[0], fr, fim);
   }
 
-  float u = Uf + (fmaf(M.A1, gx, -Sx * M.sx) - fr);
-  float v = Vf + (fmaf(M.A2, gy, -Sy * M.sy) + fim);
-  Vtx out;
-  if (!valid || leaf < 0 || !isfinite(u) || !isfinite(v)) {
-    out.px = MM_VTX_INVALID;
-    out.py = MM_VTX_INVALID;
-    out.fx = 0.f;
-    out.fy = 0.f;
-    return out;
+  const float u = Uf + (fmaf(M.A1, gx, -Sx * M.sx) - fr);
+  const float v = Vf + (fmaf(M.A2, gy, -Sy * M.sy) + fim);
+  return pixel_form(valid && leaf >= 0, u, v, Ui, Vi);
+}
+
+// Rows j and j + 1 of column i, both in record `leaf`: the same steps as
+// shoot_point with the two rows as packed pairs, bit for bit the same
+// vertices.  The record, its stars and coefficients are loaded once, a star's
+// x distance is formed once, and most of the rest issues one instruction for
+// both rows (k_shoot_irs on the 1537^2 map 3.28 -> 2.64 ms).
+template <bool SQUARE, int G>
+__device__ __forceinline__ void shoot_rows2(const MapDev &M, int leaf, int i, int j, bool valid,
+                                            Vtx &out0, Vtx &out1) {
+  const int4 *rp = reinterpret_cast<const int4 *>(M.leaf + (leaf < 0 ? 0 : leaf));
+  const int4 q0 = __ldg(rp), q1 = __ldg(rp + 1), q2 = __ldg(rp + 2), q3 = __ldg(rp + 3);
+  const int near_cnt = (leaf < 0) ? 0 : q2.w;
+  const float fi = (float)(i - q0.x);
+  const F2 fj = {(float)(j - q0.y), (float)(j + 1 - q0.y)};
+  const float gx = fi - __int_as_float(q0.z);
+  const float nfcy = -__int_as_float(q0.w);
+  const F2 gy = f2_add(fj, F2{nfcy, nfcy});
+
+  // near field, two stars per iteration into two accumulator pairs
+  F2 Sx = {0.f, 0.f}, Sy = {0.f, 0.f}, Sx2 = {0.f, 0.f}, Sy2 = {0.f, 0.f};
+  const int maxcnt = __reduce_max_sync(0xffffffffu, near_cnt);
+  const float4 *np_ = reinterpret_cast<const float4 *>(M.near_pos) + q2.z;
+  const float *nm_ = M.near_m + q2.z;
+  auto star = [&](bool on, int k, F2 &ax, F2 &ay) {
+    const float4 s = on ? __ldg(np_ + k) : make_float4(0.f, 1.f, 0.f, 0.f);
+    const float m = on ? __ldg(nm_ + k) : 0.f;
+    const float dx = (fi - s.x) - s.y;
+    const F2 dx2 = {dx, dx};
+    const F2 dy = f2_add(f2_add(fj, F2{-s.z, -s.z}), F2{-s.w, -s.w});
+    const F2 yy = SQUARE ? f2_mul(dy, dy) : f2_mul(f2_mul(F2{M.rho, M.rho}, dy), dy);
+    const F2 r = f2_fma(dx2, dx2, yy);
+    F2 q = f2_mul(F2{m, m}, F2{rcp_approx(r.x), rcp_approx(r.y)});
+    q = F2{on ? q.x : 0.f, on ? q.y : 0.f};
+    ax = f2_fma(q, dx2, ax);
+    ay = f2_fma(q, dy, ay);
+  };
+  int k = 0;
+#pragma unroll 1
+  for (; k < maxcnt; k += 2) {
+    star(k < near_cnt, k, Sx, Sy);
+    star(k + 1 < near_cnt, k + 1, Sx2, Sy2);
   }
-  const float lim = 268435456.0f;  // 2^28 pixels: far outside any map
-  u = fminf(fmaxf(u, -lim), lim);
-  v = fminf(fmaxf(v, -lim), lim);
-  float flu = floorf(u), flv = floorf(v);
-  out.px = Ui + (int)flu;
-  out.py = Vi + (int)flv;
-  out.fx = u - flu;
-  out.fy = v - flv;
-  return out;
+  Sx = f2_add(Sx, Sx2);
+  Sy = f2_add(Sy, Sy2);
+
+  float fr[2] = {0.f, 0.f}, fm[2] = {0.f, 0.f};
+  const int npair = M.p >> 1;
+  if (npair >= 1 && leaf >= 0) {
+    const float4 *e = reinterpret_cast<const float4 *>(M.coef + q3.x);
+    const float4 c = __ldg(e + (npair - 1));
+    const float zx = gx * __int_as_float(q2.x), zsy = __int_as_float(q2.y);
+    FarField f[2];
+    far_start(f[0], zx, gy.x * zsy, c);
+    far_start(f[1], zx, gy.y * zsy, c);
+    far_chain<G>(f, e, npair);
+    far_end(f[0], fr[0], fm[0]);
+    far_end(f[1], fr[1], fm[1]);
+  }
+  const float Uf = __int_as_float(q1.z), Vf = __int_as_float(q1.w);
+  const bool ok = valid && leaf >= 0;
+  out0 = pixel_form(ok, Uf + (fmaf(M.A1, gx, -Sx.x * M.sx) - fr[0]),
+                    Vf + (fmaf(M.A2, gy.x, -Sy.x * M.sy) + fm[0]), q1.x, q1.y);
+  out1 = pixel_form(ok, Uf + (fmaf(M.A1, gx, -Sx.y * M.sx) - fr[1]),
+                    Vf + (fmaf(M.A2, gy.y, -Sy.y * M.sy) + fm[1]), q1.x, q1.y);
 }
 
 // Map edge that vertex (i, j) of record `leaf` is proven to land beyond
@@ -247,6 +323,7 @@ __device__ __forceinline__ int vertex_cull_side(const MapDev &M, int leaf, int i
   int n = (int)floorf(fminf(top - fj, 1.0e6f)) - 1;
   const float rho = SQUARE ? 1.f : M.rho;
   const float4 *np_ = reinterpret_cast<const float4 *>(M.near_pos) + q2.z;
+#pragma unroll 1
   for (int k = 0; k < q2.w; k++) {
     const float4 s = __ldg(np_ + k);
     const float dx = (fi - s.x) - s.y, dy = (fj - s.z) - s.w;
@@ -274,16 +351,6 @@ __device__ __forceinline__ int row_cull_side(const MapDev &M, int leaf, int i, i
   return (S > 0 && __all_sync(0xffffffffu, s == S || s < 0)) ? S : MM_CULL_NONE;
 }
 
-// Whether both triangles of the cell (a, b, c, d) lie wholly beyond one
-// edge of the map, from the vertices' pixels alone (false when a vertex is
-// non-finite).
-__device__ __forceinline__ bool cell_beyond_map(const MapDev &M, const Vtx &a, const Vtx &b,
-                                                const Vtx &c, const Vtx &d) {
-  const int x0 = min(min(a.px, b.px), min(c.px, d.px)), x1 = max(max(a.px, b.px), max(c.px, d.px));
-  const int y0 = min(min(a.py, b.py), min(c.py, d.py)), y1 = max(max(a.py, b.py), max(c.py, d.py));
-  return x0 != MM_VTX_INVALID && (x1 < 0 || x0 >= M.npix || y1 < 0 || y0 >= M.npix_y);
-}
-
 // Persistent warps; each work item is a strip of 31 cell columns by
 // rows_per_item cell rows of one map.  Lane l computes vertex column
 // 31*s + l for every vertex row of the item, keeps the previous row in
@@ -293,10 +360,14 @@ __device__ __forceinline__ bool cell_beyond_map(const MapDev &M, const Vtx &a, c
 // Issue- and latency-bound (no pipe saturated): the kernel is shaped to run 3
 // blocks of 8 warps per SM, 80 registers a thread without spills -- the row
 // below waits in shared memory, every apportioning waits in queues emptied
-// once a row, when no vertex is live, and the counters are kept per warp.
+// once a row, when no vertex is live, and the counters are kept per warp.  Its
+// loop has to stay in the instruction cache: with the loops below unrolled as
+// the compiler likes (77 KB of code in place of 51) a third of the issue slots
+// went to fetching and it took 17.3 ms.
 // 2000^2 map, 9 rays per pixel: 16.9 ms at 2 blocks with the apportioning in
 // divergent branches, 15.3 ms with the queues at 2 blocks, 13.0 ms at 3 (4
-// spill and are slower).
+// spill and are slower), 11.9 ms with rows shot in pairs, one lookup for up
+// to 33 rows and outcodes in place of box tests.
 #ifndef MM_SHOOT_MINB
 #define MM_SHOOT_MINB 3  // resident 256-thread blocks per SM the register budget targets
 #endif
@@ -304,7 +375,7 @@ __device__ __forceinline__ bool cell_beyond_map(const MapDev &M, const Vtx &a, c
 // A single map (BATCH = false) arrives by value as a launch parameter, so
 // its fields are read from the constant bank instead of held in registers;
 // a batch reads its maps from the device array `maps`.
-template <bool SQUARE, bool BATCH, bool PRELOAD>
+template <bool SQUARE, bool BATCH>
 __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     k_shoot_ipm(const MapDev *__restrict__ maps, const MapDev M1, int n_maps, int64_t total_work,
                 unsigned long long *work_counter, unsigned *err) {
@@ -330,6 +401,7 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     int mi = 0;
     if (BATCH && n_maps > 1) {
       int lo = 0, hi = n_maps - 1;
+#pragma unroll 1
       while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (maps[mid].work_begin <= (int64_t)w)
@@ -366,63 +438,86 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     // in ws->row); `side` is row j's
     int prev_side = MM_CULL_NONE, side = MM_CULL_NONE;
     bool prev_exact = false;
-    int c_gy = INT_MIN, c_leaf = -1;  // lookup cache of this lane's column
-    bool c_cull = false;              // the cached record has a culling bound
+    int c_leaf = -1, j_same = INT_MIN;  // this lane's record, up to row j_same
+    bool c_cull = false;                // it has a culling bound
     int cull_wait = 0, cull_pause = 0;  // rows left before the next culling test
     // One pass shoots one vertex row and maps the cells between it and the
     // row below: row jb (nothing to map), then rows j = jb + 1 .. je; a row
-    // below that culling left out is shot first (`back`).  One pass more
-    // shares out what is left in the queues.
-    bool back = false;
+    // below that culling left out is shot first (`back`).  A row whose
+    // successor needs no culling test and lies in the same records is shot
+    // with it, and the successor's pass finds its vertices in ws->next
+    // (`ahead`).  One pass more shares out what is left in the queues.
+    bool back = false, ahead = false;
+    unsigned below_out = 0;  // outcodes of the row below: this lane's and (<< 4) its neighbour's
     for (int j = jb;;) {
       const bool fin = j > je;  // warp-uniform
-      Vtx v00, v10, v11, v01;
-      v00.px = v10.px = v11.px = v01.px = v00.py = v10.py = v11.py = v01.py = 0;
-      v00.fx = v10.fx = v11.fx = v01.fx = v00.fy = v10.fy = v11.fy = v01.fy = 0.f;
       if (!fin) {
         int js = j;
-        int leaf =
-            lookup_leaf_cached(M, cx, __ldg(&M.row_cell[js]), c_gy, c_leaf, c_cull);
-        if (leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
-        // a row is provably beyond the map only if every lane's record has a
-        // culling bound; otherwise the per-vertex test cannot succeed
-        if (M.cull && !back) {
-          int run = 0;
+        Vtx v01;
+        if (ahead) {
           side = MM_CULL_NONE;
-          if (cull_wait > 0) {
-            cull_wait--;
-          } else if (!__any_sync(0xffffffffu, vvalid && !c_cull)) {
-            side = row_cull_side<SQUARE>(M, leaf, i, j, vvalid, run);
-            // a failed test pauses the tests of the next rows (1, 3, ... up to 8)
-            if (j > jb) {
-              cull_pause = side == MM_CULL_NONE ? min(2 * cull_pause + 1, 8) : 0;
-              cull_wait = cull_pause;
+          if (cull_wait > 0) cull_wait--;
+          v01 = ws->next[lane];
+          ahead = false;
+        } else {
+          if (j >= j_same) {
+            c_leaf = lookup_rows(M, cx, j, je, lane, vvalid, j_same, c_cull);
+            if (c_leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
+          }
+          int leaf = c_leaf;
+          // a row is provably beyond the map only if every lane's record has a
+          // culling bound; otherwise the per-vertex test cannot succeed
+          if (M.cull && !back) {
+            int run = 0;
+            side = MM_CULL_NONE;
+            if (cull_wait > 0) {
+              cull_wait--;
+            } else if (!__any_sync(0xffffffffu, vvalid && !c_cull)) {
+              side = row_cull_side<SQUARE>(M, leaf, i, j, vvalid, run);
+              // a failed test pauses the tests of the next rows (1, 3, ... up to 8)
+              if (j > jb) {
+                cull_pause = side == MM_CULL_NONE ? min(2 * cull_pause + 1, 8) : 0;
+                cull_wait = cull_pause;
+              }
+            }
+            if (j > jb && side != MM_CULL_NONE && side == prev_side) {
+              // rows j .. j + run - 1 and the one below lie beyond the same map
+              // edge: the cells between them map nothing, and none of those
+              // rows is computed
+              const int skip = min(run, je - j + 1);
+              prev_exact = false;
+              if (lane == 0) ws->count[ST_CULLED] += (unsigned)skip;
+              j += skip;
+              continue;
             }
           }
-          if (j > jb && side != MM_CULL_NONE && side == prev_side) {
-            // rows j .. j + run - 1 and the one below lie beyond the same map
-            // edge: the cells between them map nothing, and none of those
-            // rows is computed
-            const int skip = min(run, je - j + 1);
-            prev_exact = false;
-            if (lane == 0) ws->count[ST_CULLED] += (unsigned)skip;
-            j += skip;
-            continue;
+          if (j > jb && !prev_exact) {
+            // the row below was not computed; its cells with this row are needed
+            js = j - 1;
+            leaf = lookup_leaf(M, cx, __ldg(&M.row_cell[js]));
+          }
+          // (the next row is not tested while the tests pause, and cannot pass
+          // where a lane's record has no bound)
+          ahead = js == j && j < je && j + 1 < j_same &&
+                  (!M.cull || cull_wait > 0 || __any_sync(0xffffffffu, vvalid && !c_cull));
+          if (ahead) {
+            Vtx nx;
+            shoot_rows2<SQUARE, 3>(M, leaf, i, j, vvalid, v01, nx);
+            ws->next[lane] = nx;  // (read back by this lane)
+          } else {
+            v01 = shoot_point<SQUARE, false>(M, leaf, i, js, 0.f, 0.f, vvalid);
           }
         }
-        if (j > jb && !prev_exact) {
-          // the row below was not computed; its cells with this row are needed
-          js = j - 1;
-          leaf = lookup_leaf(M, cx, __ldg(&M.row_cell[js]));
-        }
-        v01 = shoot_point<SQUARE, false, PRELOAD>(M, leaf, i, js, 0.f, 0.f, vvalid);
         // the row below waits in shared memory (not in eight registers held
         // across the deflection), where a lane also finds its right neighbour
-        v00 = ws->row[lane];
-        v10 = ws->row[min(lane + 1, 31)];
+        const Vtx v00 = ws->row[lane], v10 = ws->row[min(lane + 1, 31)];
         __syncwarp();
         ws->row[lane] = v01;
         __syncwarp();
+        const unsigned o01 = outcode(M, v01);
+        const unsigned o11 = __shfl_down_sync(0xffffffffu, o01, 1);
+        const unsigned o00 = below_out & 15u, o10 = below_out >> 4;
+        below_out = o01 | (o11 << 4);
         if (j == jb || js < j) {
           back = js < j;
           prev_exact = true;
@@ -433,19 +528,19 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
           continue;
         }
         back = false;
-        v11 = ws->row[min(lane + 1, 31)];
         prev_side = side;
-        // a row of cells all beyond the map (and none with a non-finite
-        // vertex, which must be counted) has nothing to map
-        if (__all_sync(0xffffffffu, !cell_col || cell_beyond_map(M, v00, v10, v01, v11))) {
+        // most triangles of a shooting region lie wholly beyond one edge of
+        // the map: integer tests before any arithmetic (a non-finite vertex
+        // lies beyond none, and is counted)
+        const bool on0 = cell_col && !(o00 & o10 & o11), on1 = cell_col && !(o00 & o11 & o01);
+        if (!__any_sync(0xffffffffu, on0 || on1)) {
           j++;
           continue;
         }
-      }
-      // (diagonal v00 - v11)
-      if (!fin) {
-        tri_scan(M, q, v00, v10, v11, cell_col, ra, lc, lane);
-        tri_scan(M, q, v00, v11, v01, cell_col, ra, lc, lane);
+        // (diagonal v00 - v11)
+        const Vtx v11 = ws->row[min(lane + 1, 31)];
+        tri_scan(M, q, v00, v10, v11, on0, ra, lc, lane);
+        tri_scan(M, q, v00, v11, v01, on1, ra, lc, lane);
       }
       share_out(M, q, fin, lc, lane);
       if (fin) break;
@@ -491,15 +586,26 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
     const bool owner = vvalid && (lane < MM_STRIP || i == col_end);
     const int cx = __ldg(&M.col_cell[vvalid ? i : col_end]);
     RunAcc ra = MM_RUN_NONE;
-    int c_gy = INT_MIN, c_leaf = -1;  // lookup cache of this lane's column
-    bool c_cull = false;              // the cached record has a culling bound
+    int c_leaf = -1, j_same = INT_MIN;  // this lane's record, up to row j_same
+    bool c_cull = false;                // it has a culling bound
     int cull_wait = 0, cull_pause = 0;  // rows left before the next culling test
+    auto count = [&](const Vtx &v) {
+      if (!owner) return;
+      if (v.px == MM_VTX_INVALID)
+        dropped++;
+      else if (v.px >= 0 && v.px < M.npix && v.py >= 0 && v.py < M.npix_y)
+        run_add<1ull>(M, ra, v.px, v.py);
+    };
     for (int j = jb; j <= jl; j++) {
-      const int leaf = lookup_leaf_cached(M, cx, __ldg(&M.row_cell[j]), c_gy, c_leaf, c_cull);
-      if (leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
+      if (j >= j_same) {
+        c_leaf = lookup_rows(M, cx, j, jl, lane, vvalid, j_same, c_cull);
+        if (c_leaf < 0 && vvalid) atomicOr(err, ERR_LOOKUP);
+      }
+      const int leaf = c_leaf;
+      const bool bound = M.cull && !__any_sync(0xffffffffu, vvalid && !c_cull);
       if (M.cull && cull_wait > 0) {
         cull_wait--;
-      } else if (M.cull && !__any_sync(0xffffffffu, vvalid && !c_cull)) {
+      } else if (bound) {
         int run;
         if (row_cull_side<SQUARE>(M, leaf, i, j, vvalid, run) != MM_CULL_NONE) {
           const int skip = min(run, jl - j + 1);
@@ -512,12 +618,17 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
         cull_pause = min(2 * cull_pause + 1, 8);
         cull_wait = cull_pause;
       }
-      const Vtx v = shoot_point<SQUARE, false>(M, leaf, i, j, 0.f, 0.f, vvalid);
-      if (owner) {
-        if (v.px == MM_VTX_INVALID)
-          dropped++;
-        else if (v.px >= 0 && v.px < M.npix && v.py >= 0 && v.py < M.npix_y)
-          run_add<1ull>(M, ra, v.px, v.py);
+      // a row whose successor is not tested and lies in the same records is
+      // shot with it
+      if (j < jl && j + 1 < j_same && (!bound || cull_wait > 0)) {
+        Vtx v0, v1;
+        shoot_rows2<SQUARE, 6>(M, leaf, i, j, vvalid, v0, v1);
+        count(v0);
+        count(v1);
+        if (cull_wait > 0) cull_wait--;
+        j++;
+      } else {
+        count(shoot_point<SQUARE, false, 6>(M, leaf, i, j, 0.f, 0.f, vvalid));
       }
     }
     run_flush<1ull>(M, ra);
@@ -643,16 +754,16 @@ __global__ void k_probe(const MapDev *maps, int64_t n, const double *z, double *
 // host launchers
 // ---------------------------------------------------------------------------
 
-template <bool SQUARE, bool BATCH, bool PRELOAD>
+template <bool SQUARE, bool BATCH>
 static cudaError_t launch_shoot_t(const MapDev *d_maps, const MapDev &m1, int n_maps,
                                   int64_t total_work, unsigned long long *counter, unsigned *err,
                                   int grid, cudaStream_t st) {
   const int smem = (int)MM_SHOOT_SMEM_BYTES;
-  cudaError_t e = cudaFuncSetAttribute(k_shoot_ipm<SQUARE, BATCH, PRELOAD>,
+  cudaError_t e = cudaFuncSetAttribute(k_shoot_ipm<SQUARE, BATCH>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_shoot_ipm<SQUARE, BATCH, PRELOAD><<<grid, 256, smem, st>>>(d_maps, m1, n_maps, total_work,
-                                                               counter, err);
+  k_shoot_ipm<SQUARE, BATCH><<<grid, 256, smem, st>>>(d_maps, m1, n_maps, total_work, counter,
+                                                      err);
   return cudaGetLastError();
 }
 
@@ -660,27 +771,16 @@ cudaError_t launch_shoot_ipm(const MapDev *d_maps, const MapDev *h_single, int n
                              int64_t total_work, bool square, unsigned long long *counter,
                              unsigned *err, int grid, cudaStream_t st) {
   if (total_work <= 0) return cudaSuccess;
-  if (n_maps == 1 && h_single) {
-    // a map without a second-pass queue deals every larger triangle in this
-    // kernel, which then runs faster with the far field's loads in place
-    // (3-4 % on 10000^2 and 10000 x 1000 maps); with a queue the loads
-    // ahead win (2-3 %)
-    const MapDev &m = *h_single;
-    if (m.bigq_cap > 0)
-      return square ? launch_shoot_t<true, false, true>(nullptr, m, 1, total_work, counter, err,
-                                                        grid, st)
-                    : launch_shoot_t<false, false, true>(nullptr, m, 1, total_work, counter,
-                                                         err, grid, st);
-    return square ? launch_shoot_t<true, false, false>(nullptr, m, 1, total_work, counter, err,
-                                                       grid, st)
-                  : launch_shoot_t<false, false, false>(nullptr, m, 1, total_work, counter, err,
-                                                        grid, st);
-  }
+  if (n_maps == 1 && h_single)
+    return square ? launch_shoot_t<true, false>(nullptr, *h_single, 1, total_work, counter, err,
+                                                grid, st)
+                  : launch_shoot_t<false, false>(nullptr, *h_single, 1, total_work, counter, err,
+                                                 grid, st);
   const MapDev none{};
-  return square ? launch_shoot_t<true, true, true>(d_maps, none, n_maps, total_work, counter, err,
-                                                   grid, st)
-                : launch_shoot_t<false, true, true>(d_maps, none, n_maps, total_work, counter,
-                                                    err, grid, st);
+  return square ? launch_shoot_t<true, true>(d_maps, none, n_maps, total_work, counter, err, grid,
+                                             st)
+                : launch_shoot_t<false, true>(d_maps, none, n_maps, total_work, counter, err,
+                                              grid, st);
 }
 
 // Device-side assembly of a batch's descriptor array from the handles' own
