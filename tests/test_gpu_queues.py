@@ -45,3 +45,26 @@ def test_queue_capacity_does_not_change_the_map(oracle_mod, model, cols):
     mu_ref, _ = oracle_mod.magnification_map(p, m, pos)
     e = band_errors(mu, mu_ref, p.mu_macro)
     assert e["p999"] <= MAP_P999_TOL and (cols < 30 or e["mean_rel"] <= MEAN_TOL), e
+
+
+@pytest.mark.parametrize("cols,rows", [(1, 1), (1, 700), (31, 5), (62, 63), (95, 2000)])
+def test_stored_vertices_map_like_the_oracle(oracle_mod, cols, rows):
+    """The plain FP64 path's mapping kernel: work items of 2 to 64 rows, the
+    last strip and the last item of any width, queues kept from item to item."""
+    import torch
+    torch.cuda.init()
+    kappa, gamma, s, _ = MODELS["mixed"]
+    m, pos = synthetic.star_field(12, 60, 12.0, synthetic.SALPETER_01_1)
+    half = (0.02 * cols + 0.01, 0.005 * rows + 0.01)
+    grid = dict(img_half=half, ray_grid=(cols + 1, rows + 1))
+    h = mm.create(kappa, gamma, s, m, pos, 2.0, 40, mode=mm.MM_PLAIN_FP64, **grid)
+    mm.run(h, 0)
+    mu, st = mm.get_map(h), mm.get_stats(h)
+    mm.destroy(h)
+    p = oracle_mod.derive_params(kappa, gamma, s, m, 2.0, 40, **grid)
+    mu_ref, info = oracle_mod.magnification_map(p, m, pos)
+    assert st["triangles_dropped"] == info["dropped"]
+    e = band_errors(mu, mu_ref, p.mu_macro)
+    assert e["p999"] <= MAP_P999_TOL, e
+    # (a mean over a few cells is their outline's, to FP32)
+    assert cols * rows < 1000 or e["mean_rel"] <= MEAN_TOL, e
