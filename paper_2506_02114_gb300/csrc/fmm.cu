@@ -62,6 +62,17 @@ __device__ __forceinline__ double inv_pow2(double L) {
   return pow2(1023 - (__double2hiint(L) >> 20));
 }
 
+// x with its sign flipped if `neg`, by an integer operation.
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
+
+// Real part (im = false) or imaginary part of a b + c, c that part of the
+// addend: the two halves of cfma, in two FP64 instructions either way.
+__device__ __forceinline__ double cfma_part(double2 a, double2 b, double c, bool im) {
+  return fma(a.x, im ? b.y : b.x, fma(flip(a.y, !im), im ? b.x : b.y, c));
+}
+
 // x / k, correctly rounded, from the rounded reciprocal of the small integer
 // k (Markstein's correction of the quotient by its exact remainder).
 __device__ __forceinline__ double div_by(double x, double k, double inv_k) {
@@ -162,7 +173,7 @@ __global__ void __launch_bounds__(MM_P2M_THREADS)
 // children's sums are added up afterwards in their order.  Children without
 // stars (a quarter of the finest) add exact zeros and are left out.  Finest
 // level of 50 000 stars, p = 25: 148 us with a thread per row and the
-// children one after another, 101 us like this.
+// children one after another, 70 us like this.
 // ---------------------------------------------------------------------------
 __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
                       const double2 *__restrict__ MMop, double2 *mp) {
@@ -187,16 +198,23 @@ __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
     const int fc = T.first_child[first + (nq >> 2)];
     if (fc < 0 || T.sbeg[fc + (nq & 3)] == T.send[fc + (nq & 3)]) continue;
     const double2 *src = a + nq * P1;
-    const int rows = 2 * (r + 1) == p + 1 ? 1 : 2;  // (the middle row of an odd p, once)
-    for (int h = 0; h < rows; h++) {
-      const int l = h ? p - r : r + 1;
-      double tx = -src[0].x * bt[l], ty = -src[0].y * bt[l];
-      for (int k = 1; k <= l; k++) {
-        const double b = bt[k * P1 + l];
-        tx = fma(b, src[k].x, tx);
-        ty = fma(b, src[k].y, ty);
+    // rows r + 1 and p - r one after the other (the middle row of an odd p
+    // once), each from its k = 0 term on
+    int l = r + 1, k = 0;
+    const int steps = 2 * l == p + 1 ? l + 1 : p + 3;
+    double tx = 0.0, ty = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < steps; i++) {
+      const double b = bt[k * P1 + l];
+      const double2 u = src[k];
+      // (-a_0 / l first: a product rounded once, as the first of its sum)
+      tx = fma(b, flip(u.x, k == 0), k ? tx : 0.0);
+      ty = fma(b, flip(u.y, k == 0), k ? ty : 0.0);
+      if (++k > l) {
+        t[nq * P1 + l] = make_double2(tx, ty);
+        l = p - r;
+        k = 0;
       }
-      t[nq * P1 + l] = make_double2(tx, ty);
     }
   }
   __syncthreads();
@@ -223,7 +241,9 @@ __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
 //   L2L from the parent, M2L from the parent's neighbours' children that are
 //   not adjacent (<= 27), P2L from the parent's unsplit neighbours that are
 //   not adjacent (<= 5).
-// One block per node.  The sums over k of all its sources are independent:
+// One block per node and part of its rows l (one part where a level has
+// nodes enough; a node's work is 11 us of one SM's FP64 pipe, so small levels
+// share it out over SMs).  The sums over k of all its sources are independent:
 // thread (group g, row l) takes sources g, g + G, ... two at a time, which
 // fills the lanes for any p and gives each binomial it loads two uses; the
 // sources' results are then added up row by row in the order of the list.
@@ -231,8 +251,8 @@ __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
 // at the coarse ones, where the sources one after another took 100 us a level
 // whatever its size.  Sources without stars (a quarter of the finest level's)
 // add exact zeros and are left out.  50 000 stars, p = 25: 1.21 ms over all
-// levels with a warp per node, 0.62 ms like this; the finest level 477 and
-// 291 us, with the FP64 pipe 93 % busy both times.
+// levels with a warp per node, 0.56 ms like this; the finest level 477 and
+// 283 us, with the FP64 pipe 93 % busy both times.
 // ---------------------------------------------------------------------------
 #define MM_LOCAL_THREADS 128
 #define MM_LOCAL_STARS 8  // P2L stars staged at a time
@@ -260,6 +280,10 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
   const int64_t node = T.level_off[level] + blockIdx.x;
   if (!node_act[node]) return;
   const int P1 = p + 1, tid = threadIdx.x;
+  // this block's rows: r0 + 1 .. r0 + nr
+  const int per = (p + (int)gridDim.y - 1) / (int)gridDim.y, r0 = (int)blockIdx.y * per;
+  const int nr = min(per, p - r0);
+  if (nr <= 0) return;
   double2 *bs = s_loc, *ts = bs + 27 * P1, *l2l = ts + 27 * P1, *pl = l2l + P1;
   double2 *zs = pl + P1;                   // [star][l]
   double2 *sq = zs + MM_LOCAL_STARS * P1;  // [star][MM_POW_BITS]
@@ -322,19 +346,22 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
   }
   for (int k = tid; k < P1; k += MM_LOCAL_THREADS) pl[k] = loc[parent * P1 + k];
   __syncthreads();
-  // L2L from the parent, by the last threads
-  if (tid >= MM_LOCAL_THREADS - p) {
-    const int l = MM_LOCAL_THREADS - tid;
+  // L2L from the parent: real parts by the last two warps' threads, imaginary
+  // parts by the first two's (an FP64 instruction takes 64 cycles of a warp's
+  // quarter of the SM, so the two halves of a complex sum go to two quarters)
+  const int half = MM_LOCAL_THREADS / 2, hr = tid & (half - 1), im = tid < half;
+  if (hr >= half - nr) {
+    const int l = r0 + half - hr;
     const int q = (nx & 1) | ((ny & 1) << 1);
     const double2 *op = LLop + (int64_t)q * P1 * P1;
-    double2 acc = make_double2(0.0, 0.0);
+    double acc = 0.0;
 #pragma unroll 4
-    for (int k = l; k <= p; k++) acc = cfma(op[k * P1 + l], pl[k], acc);
-    l2l[l] = acc;
+    for (int k = l; k <= p; k++) acc = cfma_part(op[k * P1 + l], pl[k], acc, im);
+    (im ? &l2l[l].y : &l2l[l].x)[0] = acc;
   }
   const double *bt = reinterpret_cast<const double *>(MLop);  // binomials [k][l], 1/l at k = 0
-  const int G = max(1, MM_LOCAL_THREADS / p);
-  const int g = tid / p, l = tid - g * p + 1;
+  const int G = MM_LOCAL_THREADS / nr;  // (nr <= MM_PMAX < MM_LOCAL_THREADS)
+  const int g = tid / nr, l = r0 + tid - g * nr + 1;
   const double il = bt[l];
   for (int s0 = g < G ? g : ns; __any_sync(0xffffffffu, s0 < ns); s0 += 2 * G) {
     // (a P2L source's entry is not formed: its sum is not used)
@@ -367,20 +394,21 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
   }
   __syncthreads();
   // the factors (1/z0)^l of the M2L sources, in place of their multipoles
-  for (int idx = tid; idx < ns * P1; idx += MM_LOCAL_THREADS) {
-    const int s = idx / P1, slot = S.slot[s];
-    if (slot >= 0) bs[idx] = pw[(int64_t)slot * 2 * P1 + P1 + (idx - s * P1)];
+  for (int idx = tid; idx < ns * nr; idx += MM_LOCAL_THREADS) {
+    const int s = idx / nr, k = r0 + idx - s * nr + 1, slot = S.slot[s];
+    if (slot >= 0) bs[s * P1 + k] = pw[(int64_t)slot * 2 * P1 + P1 + k];
   }
   __syncthreads();
 
-  // add up row l = tid (1 .. p) in the order of the list
-  const bool on = tid >= 1 && tid <= p;
-  double2 acc = on ? l2l[tid] : make_double2(0.0, 0.0);
+  // add up row `row` in the order of the list, real and imaginary parts apart
+  const bool on = hr < nr;
+  const int row = r0 + hr + 1;
+  double acc = on ? (im ? l2l[row].y : l2l[row].x) : 0.0;
   const double invL = inv_pow2(L);
   for (int s = 0; s < ns; s++) {
     const int slot = S.slot[s];
     if (slot >= 0) {
-      if (on) acc = cfma(bs[s * P1 + tid], ts[s * P1 + tid], acc);
+      if (on) acc = cfma_part(bs[s * P1 + row], ts[s * P1 + row], acc, im);
       continue;
     }
     // P2L: the leaf's stars, staged; block-uniform.  Powers and weights of
@@ -405,14 +433,12 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
       __syncthreads();
       if (on)
         for (int i = 0; i < cnt; i++) {
-          const double2 zl = zs[i * P1 + tid];
-          const double f = fs[i * P1 + tid];
-          acc.x = fma(f, zl.x, acc.x);
-          acc.y = fma(f, zl.y, acc.y);
+          const double2 zl = zs[i * P1 + row];
+          acc = fma(fs[i * P1 + row], im ? zl.y : zl.x, acc);
         }
     }
   }
-  if (tid <= p) loc[node * P1 + tid] = on ? acc : make_double2(0.0, 0.0);
+  if (on) (im ? &loc[node * P1 + row].y : &loc[node * P1 + row].x)[0] = acc;  // (c_0 stays zero)
 }
 
 // ---------------------------------------------------------------------------
@@ -609,6 +635,12 @@ __device__ __forceinline__ float div_by_f(float x, float n, float inv_n) {
 // part two further): pairs are stored real parts first.
 __device__ __forceinline__ int coef_slot(int k) { return 4 * (k >> 1) + (k & 1); }
 
+// 0, 1, ..., MM_PMAX (a conversion is an FP64 instruction too).
+__constant__ double c_int[MM_PMAX + 1] = {
+    0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21,
+    22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38, 39, 40, 41, 42, 43,
+    44, 45, 46, 47, 48, 49, 50, 51, 52, 53, 54, 55, 56, 57, 58, 59, 60, 61, 62, 63, 64};
+
 // Shared memory of k_leaf_finalize<NB>.
 template <int NB>
 struct RecSmem {
@@ -706,10 +738,10 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     // d_1 of the leaf's expansion (pe >= 1: p >= 1)
     const double2 *c = loc + (int64_t)node2 * P1;
     double sum = 0.0;
+#pragma unroll 4
     for (int l = 1; l <= p; l++) {
       const double2 cl = c[l], u = tb.up[(l - 1) * NS + (rec2 & (NS - 1))];
-      const double u1 = ax ? u.y : u.x, u2 = ax ? u.x : -u.y;
-      sum = fma((double)l, fma(cl.x, u1, cl.y * u2), sum);
+      sum = fma(c_int[l], fma(cl.x, ax ? u.y : u.x, cl.y * flip(ax ? u.x : u.y, !ax)), sum);
     }
     S.d1[ax][rec2] = sum * pow2(-C.sub);
   }
@@ -1140,7 +1172,12 @@ cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const in
                                          (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_local<<<(unsigned)n, MM_LOCAL_THREADS, smem, st>>>(T, level, n, p, node_act, MLop, LLop, mp,
+  // parts per node where a level's nodes (most of them inactive when the grid
+  // is a small part of the star region) leave SMs idle: the levels of 16 and 64
+  // nodes took 24 and 36 us in one part, 14 and 22 in four; above 3000 nodes
+  // the pipe is busy anyway and a part costs 6 % more of it
+  const unsigned parts = n <= 304 ? 4 : n <= 3000 ? 2 : 1;
+  k_local<<<dim3((unsigned)n, parts), MM_LOCAL_THREADS, smem, st>>>(T, level, n, p, node_act, MLop, LLop, mp,
                                                        loc, err);
   return cudaGetLastError();
 }
