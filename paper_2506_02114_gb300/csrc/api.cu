@@ -191,7 +191,7 @@ struct mm_map {
   int top_end = 0;                 // first level not built by the top kernel
 
   // active region
-  DBuf<int32_t> col_cell, row_cell, node_act, leaf_flag, leaf_scan, node_active, active_list;
+  DBuf<int32_t> col_cell, row_cell, node_act, leaf_flag, leaf_group, node_active, active_list;
   int64_t n_active = 0;
   double min_leaf_L = 0.0;
   int max_leaf_level = 0;
@@ -211,10 +211,13 @@ struct mm_map {
   int glevel = 0, gshift = 0, gx0 = 0, gy0 = 0, gw = 1, gh = 1;
   DBuf<int32_t> grid;
 
-  // map
-  DBuf<unsigned long long> acc, span, stat, counter, fixed_out;
+  // map: what every run starts from zero lies in one allocation -- the
+  // accumulator, the row-difference array, the statistics [8], the work
+  // counter [1] and the queue's counters [2] (queued, batches taken)
+  DBuf<unsigned long long> zeroed, fixed_out;
+  unsigned long long *acc = nullptr, *span = nullptr, *stat = nullptr, *counter = nullptr;
+  unsigned long long *bigq_n = nullptr;
   DBuf<char> bigq;                     // larger triangles for the second IPM pass
-  DBuf<unsigned long long> bigq_n;     // [0] queued, [1] batches taken
   int64_t bigq_cap = 0;
   DBuf<unsigned> err;
   DBuf<float> map;
@@ -543,26 +546,23 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
     CK(h->row_cell.ensure(P.n[1]));
     CK(h->node_act.ensure(nn));
     CK(h->leaf_flag.ensure(nn));
-    CK(h->leaf_scan.ensure(nn));
+    CK(h->leaf_group.ensure((nn + MM_ACTIVE_GROUP - 1) / MM_ACTIVE_GROUP));
+    CK(h->active_list.ensure(nn));
     CK(h->node_active.ensure(nn));
   }
-  LCH(launch_axis_cells(P.x0[0], P.h[0], P.n[0], h->R0, h->col_cell.p, st));
-  LCH(launch_axis_cells(P.x0[1], P.h[1], P.n[1], h->R0, h->row_cell.p, st));
+  LCH(launch_axis_cells(P.x0[0], P.x0[1], P.h[0], P.h[1], P.n[0], P.n[1], h->R0, h->col_cell.p,
+                        h->row_cell.p, st));
   LCH(launch_active_flags(T, nn, h->col_cell.p, h->col_lo, h->col_hi, h->row_cell.p, h->row_lo,
-                          h->row_hi, h->node_act.p, h->leaf_flag.p, st));
-  CKS(cub_call(h, plan, [&](void *tmp, size_t &bytes) {
-    return cub::DeviceScan::ExclusiveSum(tmp, bytes, h->leaf_flag.p, h->leaf_scan.p, (int)nn, st);
-  }));
+                          h->row_hi, h->node_act.p, h->leaf_flag.p, h->leaf_group.p, st));
+  LCH(launch_compact_leaves(nn, h->leaf_flag.p, h->leaf_group.p, h->node_active.p,
+                            h->active_list.p, h->top_info.p, st));
   if (plan) {
-    const int32_t *src[2] = {h->leaf_scan.p + (nn - 1), h->leaf_flag.p + (nn - 1)};
-    int32_t ab[2];
-    CKS(read_ints(h, st, 2, src, ab));
-    h->n_active = (int64_t)ab[0] + ab[1];
+    const int32_t *src[1] = {h->top_info.p};
+    int32_t total;
+    CKS(read_ints(h, st, 1, src, &total));
+    h->n_active = total;
     if (h->n_active <= 0) return fail(MM_ECUDA, "internal: no active leaf");
-    CK(h->active_list.ensure(h->n_active));
   }
-  LCH(launch_compact_leaves(nn, h->leaf_flag.p, h->leaf_scan.p, h->node_active.p,
-                           h->active_list.p, st));
 
   if (plan) {
     // smallest active leaf and the deepest active level (plan-time analysis)
@@ -614,8 +614,9 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   LCH(launch_p2m(T, nn, p, h->MLop.p, h->mp.p, st));
   for (int l = h->depth - 1; l >= 2; l--)
     LCH(launch_m2m(T, l, h->level_cnt[l], p, h->MMop.p, h->mp.p, st));
-  // down-sweep: levels 0 and 1 have no well-separated nodes
-  CK(cudaMemsetAsync(h->loc.p, 0, (size_t)nn * P1 * sizeof(double2), st));
+  // down-sweep: levels 0 and 1 have no well-separated nodes, so their locals
+  // (at most five) are zero; every active node below gets its own
+  CK(cudaMemsetAsync(h->loc.p, 0, (size_t)std::min<int64_t>(nn, 5) * P1 * sizeof(double2), st));
   for (int l = 2; l <= h->depth; l++)
     LCH(launch_local(T, l, h->level_cnt[l], p, h->node_act.p, h->MLop.p, h->LLop.p, h->mp.p,
                     h->loc.p, h->err.p, st));
@@ -754,22 +755,16 @@ static void fill_mapdev(mm_map *h) {
   M.npix = P.npix;
   M.npix_y = P.npix_y;
   M.err = h->err.p;
-  M.acc = h->acc.p;
-  M.span = h->span.p;
-  M.stat = h->stat.p;
+  M.acc = h->acc;
+  M.span = h->span;
+  M.stat = h->stat;
   M.bigq = reinterpret_cast<RawTri *>(h->bigq.p);
-  M.bigq_n = h->bigq_n.p;
+  M.bigq_n = h->bigq_n;
   M.bigq_cap = h->bigq_cap;
 }
 
 static mm_status clear_map(mm_map *h, cudaStream_t st) {
-  const size_t np = (size_t)h->P.npix * h->P.npix_y;
-  CK(cudaMemsetAsync(h->acc.p, 0, np * sizeof(unsigned long long), st));
-  CK(cudaMemsetAsync(h->span.p, 0, (size_t)h->P.npix_y * (h->P.npix + 1) * sizeof(unsigned long long),
-                     st));
-  CK(cudaMemsetAsync(h->stat.p, 0, 8 * sizeof(unsigned long long), st));
-  CK(cudaMemsetAsync(h->counter.p, 0, sizeof(unsigned long long), st));
-  CK(cudaMemsetAsync(h->bigq_n.p, 0, 2 * sizeof(unsigned long long), st));
+  CK(cudaMemsetAsync(h->zeroed.p, 0, h->zeroed.n * sizeof(unsigned long long), st));
   return MM_OK;
 }
 
@@ -790,11 +785,14 @@ static int64_t est_jobs(const mm_map *h, int64_t cells) {
 
 static mm_status alloc_map_buffers(mm_map *h) {
   const size_t np = (size_t)h->P.npix * h->P.npix_y;
-  CK(h->acc.ensure(np));
-  CK(h->span.ensure((size_t)h->P.npix_y * (h->P.npix + 1)));
+  const size_t nspan = (size_t)h->P.npix_y * (h->P.npix + 1);
+  CK(h->zeroed.ensure(np + nspan + 8 + 1 + 2));
+  h->acc = h->zeroed.p;
+  h->span = h->acc + np;
+  h->stat = h->span + nspan;
+  h->counter = h->stat + 8;
+  h->bigq_n = h->counter + 1;
   CK(h->map.ensure(np));
-  CK(h->stat.ensure(8));
-  CK(h->counter.ensure(1));
   // Queue for the second IPM pass.  It pays while the map's accumulators
   // (acc + row-difference array, 16 B per pixel) stay in L2: the second pass
   // then finds their lines there.  A larger map's lines are gone by the time
@@ -833,7 +831,6 @@ static mm_status alloc_map_buffers(mm_map *h) {
       }
       CK(e);
     }
-    CK(h->bigq_n.ensure(2));
     // a map that fits: the first pass runs in segments so that each
     // segment's larger triangles fit the queue
     h->segments = 1;
@@ -918,7 +915,7 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
     C.rect_c2 = h->opt.star_rect[1];
     LCH(launch_direct64_vertices(h->sx.p, h->sy.p, h->sm.p, h->N, C, R.c0, R.c1 - R.c0 + 1,
                                  R.r0, R.r1, h->verts.p, st));
-    LCH(launch_ipm_vertices(h->d_md.p, h->verts.p, R.c1 - R.c0 + 1, R.r0, R.r1, h->counter.p,
+    LCH(launch_ipm_vertices(h->d_md.p, h->verts.p, R.c1 - R.c0 + 1, R.r0, R.r1, h->counter,
                             h->err.p, shoot_grid(), st));
     CKS(record(h, 5, st));
     LCH(launch_big_ipm(h->md, st));
@@ -936,11 +933,11 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
     const int64_t work =
         (int64_t)base.strips * ((base.row_blocks + base.item_stride - 1) / base.item_stride);
     if (h->mode == MM_FMM_IRS) {
-      LCH(launch_shoot_irs(base, work, base.square_cells != 0, h->counter.p, h->err.p, st));
+      LCH(launch_shoot_irs(base, work, base.square_cells != 0, h->counter, h->err.p, st));
       h->last_segments = 0;
       CKS(record(h, 5, st));
       CKS(record(h, 3, st));
-      LCH(launch_normalize(h->acc.p, h->span.p, P.npix, P.npix_y, map_scale(h), h->map.p, st));
+      LCH(launch_normalize(h->acc, h->span, P.npix, P.npix_y, map_scale(h), h->map.p, st));
       CKS(record(h, 4, st));
       h->ev_recorded = h->opt.time_stages != 0;
       h->last_stream = st;
@@ -953,13 +950,12 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
     int64_t k = 0;
     for (int64_t w0 = 0; w0 < work; w0 += per, k++) {
       if (w0 > 0) {  // the previous segment's second pass has drained the queue
-        CK(cudaMemsetAsync(h->counter.p, 0, sizeof(unsigned long long), st));
-        CK(cudaMemsetAsync(h->bigq_n.p, 0, 2 * sizeof(unsigned long long), st));
+        CK(cudaMemsetAsync(h->counter, 0, 3 * sizeof(unsigned long long), st));
       }
       MapDev ms = base;
       ms.work_begin = -w0;  // this launch's item w is item w0 + w of the map
       LCH(launch_shoot_ipm(h->d_md.p, &ms, 1, std::min(per, work - w0), base.square_cells != 0,
-                          h->counter.p, h->err.p, shoot_grid(), st));
+                          h->counter, h->err.p, shoot_grid(), st));
       if (h->opt.time_stages) CK(cudaEventRecord(h->seg_ev[2 * k], st));
       LCH(launch_big_ipm(ms, st));
       if (h->opt.time_stages) CK(cudaEventRecord(h->seg_ev[2 * k + 1], st));
@@ -968,7 +964,7 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
     CKS(record(h, 5, st));
   }
   CKS(record(h, 3, st));
-  LCH(launch_normalize(h->acc.p, h->span.p, P.npix, P.npix_y, map_scale(h), h->map.p, st));
+  LCH(launch_normalize(h->acc, h->span, P.npix, P.npix_y, map_scale(h), h->map.p, st));
   CKS(record(h, 4, st));
   h->ev_recorded = h->opt.time_stages != 0;
   h->last_stream = st;
@@ -1332,7 +1328,7 @@ static mm_status autotune(const CreateArgs &a, mm_options &o, int32_t &leaf_size
             // the larger triangles of the sampled run (statistics 3 and 4),
             // scaled to the whole grid, per 2^20 cells
             unsigned long long st[8] = {};
-            ce = cudaMemcpy(st, t->stat.p, sizeof st, cudaMemcpyDeviceToHost);
+            ce = cudaMemcpy(st, t->stat, sizeof st, cudaMemcpyDeviceToHost);
             if (ce != cudaSuccess) {
               s = fail(MM_ECUDA, "autotune: %s", cudaGetErrorString(ce));
               break;
@@ -1504,7 +1500,7 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
   int gl = 0;
   CK(launch_batch_gather(src.data(), wb.data(), n, lead->batch_md.p, gl, st));
   lead->launches += gl;
-  CK(launch_shoot_ipm(lead->batch_md.p, nullptr, n, work, all_square, lead->counter.p, lead->err.p,
+  CK(launch_shoot_ipm(lead->batch_md.p, nullptr, n, work, all_square, lead->counter, lead->err.p,
                       shoot_grid(), st));
   lead->launches++;
   if (lead->opt.time_stages) {
@@ -1521,7 +1517,7 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     CKS(record(h, 5, si));
     LCH(launch_big_ipm(h->md, si));
     CKS(record(h, 3, si));
-    LCH(launch_normalize(h->acc.p, h->span.p, h->P.npix, h->P.npix_y, map_scale(h), h->map.p, si));
+    LCH(launch_normalize(h->acc, h->span, h->P.npix, h->P.npix_y, map_scale(h), h->map.p, si));
     CKS(record(h, 4, si));
     h->ev_recorded = h->opt.time_stages != 0;
     h->last_stream = st;
@@ -1556,7 +1552,7 @@ mm_status mm_get_map_fixed(const mm_map *hc, uint64_t *out, int32_t on_device) {
   CK(cudaSetDevice(h->device));
   const size_t np = (size_t)h->P.npix * h->P.npix_y;
   CK(h->fixed_out.ensure(np));
-  LCH(launch_fold_span(h->acc.p, h->span.p, h->P.npix, h->P.npix_y, h->fixed_out.p,
+  LCH(launch_fold_span(h->acc, h->span, h->P.npix, h->P.npix_y, h->fixed_out.p,
                        h->last_stream));
   if (on_device) {
     CK(cudaMemcpyAsync(out, h->fixed_out.p, np * 8, cudaMemcpyDeviceToDevice, h->last_stream));
@@ -1673,7 +1669,7 @@ mm_status mm_get_stats(const mm_map *hc, mm_stats *out) {
   }
   if (h->ran) {
     unsigned long long st[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    CK(cudaMemcpy(st, h->stat.p, sizeof st, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(st, h->stat, sizeof st, cudaMemcpyDeviceToHost));
     out->triangles_dropped = (int64_t)st[0];
     out->triangles_clipped = (int64_t)st[1];
     out->triangles_quad = (int64_t)st[2];
@@ -1738,7 +1734,7 @@ void mm_destroy(mm_map *h) {
   h->keys_in.release();
   h->keys.release();
   h->bigq.release();
-  h->bigq_n.release();
+  h->zeroed.release();
   h->idx_in.release();
   h->idx.release();
   h->cub_tmp.release();
@@ -1747,7 +1743,7 @@ void mm_destroy(mm_map *h) {
   DBuf<int32_t> *ibs[] = {&h->lvl,       &h->sbeg,      &h->send,      &h->first_child,
                           &h->parent,    &h->nb,        &h->split,     &h->group,
                           &h->top_info,  &h->col_cell,  &h->row_cell,
-                          &h->node_act,  &h->leaf_flag, &h->leaf_scan, &h->node_active,
+                          &h->node_act,  &h->leaf_flag, &h->leaf_group, &h->node_active,
                           &h->active_list, &h->grid};
   for (auto *b : ibs) b->release();
   DBuf<double2> *cbs[] = {&h->MMop, &h->MLop, &h->LLop, &h->mp, &h->loc};
@@ -1759,10 +1755,6 @@ void mm_destroy(mm_map *h) {
   h->sub_fp.release();
   h->sub_bin.release();
   h->coef.release();
-  h->acc.release();
-  h->span.release();
-  h->stat.release();
-  h->counter.release();
   h->fixed_out.release();
   h->err.release();
   h->map.release();

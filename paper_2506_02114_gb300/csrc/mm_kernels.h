@@ -57,17 +57,19 @@ cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, in
 // Its children, in Morton order.
 cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level, int64_t n,
                                   const int32_t *split, const int32_t *group, cudaStream_t st);
-cudaError_t launch_axis_cells(double x0, double h, int64_t n, double R0, int32_t *out,
-                              cudaStream_t st);
-// flags[node] = 1 for active leaves (leaf containing ray vertices); also
-// node_act[node] = 1 for every active node
+cudaError_t launch_axis_cells(double x0, double y0, double hx, double hy, int64_t n0, int64_t n1,
+                              double R0, int32_t *col, int32_t *row, cudaStream_t st);
+// flags[node] = 1 for active leaves (leaf containing ray vertices) and their
+// number per group of MM_ACTIVE_GROUP nodes; also node_act[node] = 1 for every
+// active node
+#define MM_ACTIVE_GROUP 256
 cudaError_t launch_active_flags(const TreeDev &T, int64_t n_nodes, const int32_t *col_cell,
                                 int64_t col_lo, int64_t col_hi, const int32_t *row_cell,
                                 int64_t row_lo, int64_t row_hi, int32_t *node_act,
-                                int32_t *leaf_flag, cudaStream_t st);
-cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag,
-                                  const int32_t *leaf_scan, int32_t *node_active,
-                                  int32_t *active_list, cudaStream_t st);
+                                int32_t *leaf_flag, int32_t *group, cudaStream_t st);
+cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag, const int32_t *group,
+                                  int32_t *node_active, int32_t *active_list, int32_t *total,
+                                  cudaStream_t st);
 cudaError_t launch_lookup_grid(const TreeDev &T, const int32_t *node_active, int glevel,
                                int sub, int gx0, int gy0, int gw, int gh, int32_t *grid,
                                cudaStream_t st);

@@ -261,19 +261,23 @@ __global__ void __launch_bounds__(1024) k_tree_top(TreeDev T, TreeOut O, int lim
   }
 }
 
-__global__ void k_axis_cells(double x0, double h, int64_t n, double R0, int32_t *out) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  double x = __dadd_rn(x0, __dmul_rn((double)t, h));
-  out[t] = cell_of(x, R0);
+// Finest-level cells of the vertex columns (first n0 threads) and rows.
+__global__ void k_axis_cells(double x0, double y0, double hx, double hy, int64_t n0, int64_t n1,
+                             double R0, int32_t *col, int32_t *row) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < n0)
+    col[t] = cell_of(__dadd_rn(x0, __dmul_rn((double)t, hx)), R0);
+  else if (t < n0 + n1)
+    row[t - n0] = cell_of(__dadd_rn(y0, __dmul_rn((double)(t - n0), hy)), R0);
 }
 
 __global__ void k_active_flags(TreeDev T, int64_t n_nodes, const int32_t *col_cell,
                                int64_t col_lo, int64_t col_hi, const int32_t *row_cell,
                                int64_t row_lo, int64_t row_hi, int32_t *node_act,
-                               int32_t *leaf_flag) {
+                               int32_t *leaf_flag, int32_t *group) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_nodes) return;
+  const bool valid = t < n_nodes;
+  if (!valid) t = n_nodes - 1;
   const int CX0 = col_cell[col_lo], CX1 = col_cell[col_hi];
   const int CY0 = row_cell[row_lo], CY1 = row_cell[row_hi];
   uint32_t cx, cy;
@@ -282,21 +286,39 @@ __global__ void k_active_flags(TreeDev T, int64_t n_nodes, const int32_t *col_ce
   const int64_t x0 = (int64_t)cx << sh, x1 = (((int64_t)cx + 1) << sh) - 1;
   const int64_t y0 = (int64_t)cy << sh, y1 = (((int64_t)cy + 1) << sh) - 1;
   const int act = (x1 >= CX0 && x0 <= CX1 && y1 >= CY0 && y0 <= CY1) ? 1 : 0;
-  node_act[t] = act;
-  leaf_flag[t] = (act && T.first_child[t] < 0) ? 1 : 0;
+  const int leaf = valid && act && T.first_child[t] < 0;
+  if (valid) {
+    node_act[t] = act;
+    leaf_flag[t] = leaf;
+  }
+  const int n = __syncthreads_count(leaf);
+  if (threadIdx.x == 0) group[blockIdx.x] = n;
 }
 
-__global__ void k_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag,
-                                 const int32_t *leaf_scan, int32_t *node_active,
-                                 int32_t *active_list) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_nodes) return;
-  if (leaf_flag[t]) {
-    node_active[t] = leaf_scan[t];
-    active_list[leaf_scan[t]] = (int32_t)t;
-  } else {
-    node_active[t] = -1;
-  }
+// Numbers the active leaves in the order of their nodes, block by block of
+// k_active_flags; the last block stores how many there are.
+__global__ void __launch_bounds__(256) k_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag,
+                                                        const int32_t *group,
+                                                        int32_t *node_active,
+                                                        int32_t *active_list, int32_t *total) {
+  __shared__ int s_w[8], s_base;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int before = 0;
+  for (int64_t k = threadIdx.x; k < blockIdx.x; k += 256) before += group[k];
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (threadIdx.x == 0) s_base = 0;
+  __syncthreads();
+  if (lane == 0 && before) atomicAdd(&s_base, before);
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const bool f = t < n_nodes && leaf_flag[t];
+  const unsigned m = __ballot_sync(0xffffffffu, f);
+  if (lane == 0) s_w[w] = __popc(m);
+  __syncthreads();
+  int rank = s_base + __popc(m & ((1u << lane) - 1u));
+  for (int k = 0; k < w; k++) rank += s_w[k];
+  if (t < n_nodes) node_active[t] = f ? rank : -1;
+  if (f) active_list[rank] = (int32_t)t;
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) *total = s_base + group[blockIdx.x];
 }
 
 // Lookup grid over the active region at level glevel: the active leaf
@@ -364,30 +386,30 @@ cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level,
   return cudaGetLastError();
 }
 
-cudaError_t launch_axis_cells(double x0, double h, int64_t n, double R0, int32_t *out,
-                              cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  k_axis_cells<<<blocks_for(n, 256), 256, 0, st>>>(x0, h, n, R0, out);
+cudaError_t launch_axis_cells(double x0, double y0, double hx, double hy, int64_t n0, int64_t n1,
+                              double R0, int32_t *col, int32_t *row, cudaStream_t st) {
+  if (n0 + n1 <= 0) return cudaSuccess;
+  k_axis_cells<<<blocks_for(n0 + n1, 256), 256, 0, st>>>(x0, y0, hx, hy, n0, n1, R0, col, row);
   return cudaGetLastError();
 }
 
 cudaError_t launch_active_flags(const TreeDev &T, int64_t n_nodes, const int32_t *col_cell,
                                 int64_t col_lo, int64_t col_hi, const int32_t *row_cell,
                                 int64_t row_lo, int64_t row_hi, int32_t *node_act,
-                                int32_t *leaf_flag, cudaStream_t st) {
+                                int32_t *leaf_flag, int32_t *group, cudaStream_t st) {
   if (n_nodes <= 0) return cudaSuccess;
-  k_active_flags<<<blocks_for(n_nodes, 256), 256, 0, st>>>(T, n_nodes, col_cell, col_lo, col_hi,
-                                                           row_cell, row_lo, row_hi, node_act,
-                                                           leaf_flag);
+  k_active_flags<<<blocks_for(n_nodes, MM_ACTIVE_GROUP), MM_ACTIVE_GROUP, 0, st>>>(
+      T, n_nodes, col_cell, col_lo, col_hi, row_cell, row_lo, row_hi, node_act, leaf_flag, group);
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag,
-                                  const int32_t *leaf_scan, int32_t *node_active,
-                                  int32_t *active_list, cudaStream_t st) {
+cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag, const int32_t *group,
+                                  int32_t *node_active, int32_t *active_list, int32_t *total,
+                                  cudaStream_t st) {
+  static_assert(MM_ACTIVE_GROUP == 256, "one thread per node of a group");
   if (n_nodes <= 0) return cudaSuccess;
-  k_compact_leaves<<<blocks_for(n_nodes, 256), 256, 0, st>>>(n_nodes, leaf_flag, leaf_scan,
-                                                             node_active, active_list);
+  k_compact_leaves<<<blocks_for(n_nodes, 256), 256, 0, st>>>(n_nodes, leaf_flag, group,
+                                                             node_active, active_list, total);
   return cudaGetLastError();
 }
 
