@@ -97,3 +97,19 @@ def test_deflection_at_every_dealing_of_the_order(oracle_mod, p, leaf, sub):
     r = math.sqrt(2.0) / (4.0 - math.sqrt(2.0))
     err = deflection_rel_error(par, z, w, w_ref).max()
     assert err <= DEFLECTION_TOL + 2.2 * (p + 1) * r ** p, err
+
+
+def test_probe_buffer_of_any_size():
+    """Source positions do not depend on the calls before: small, large (given
+    back) and small again, on both paths."""
+    m, pos = synthetic.star_field(17, 100, 12.0, synthetic.EQUAL)
+    n = (1 << 20) + 3
+    z = 4.0 * np.stack([synthetic.uniform(9, 0, n), synthetic.uniform(9, 1, n)], 1) - 2.0
+    for mode in (mm.MM_FMM_FP32, mm.MM_PLAIN_FP64):
+        h = mm.create(0.4, 0.3, 0.0, m, pos, 1.0, 16, fmm_order=20, mode=mode, img_half=(2.0, 2.0),
+                      ray_grid=(101, 101))
+        few = mm.shoot_points(h, z[:7])
+        whole = mm.shoot_points(h, z)
+        assert np.array_equal(whole[:7], few) and np.isfinite(whole).all()
+        assert np.array_equal(mm.shoot_points(h, z[-5:]), whole[-5:])
+        mm.destroy(h)
