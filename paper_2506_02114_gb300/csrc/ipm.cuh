@@ -355,6 +355,16 @@ struct __align__(16) TriJob {
   float k[3];
 };
 
+static_assert(sizeof(TriJob) == 48, "TriJob layout");
+__device__ __forceinline__ TriJob job_load(const TriJob *p) {
+  TriJob J;
+  const float4 *w = reinterpret_cast<const float4 *>(p);
+  float4 *d = reinterpret_cast<float4 *>(&J);
+#pragma unroll
+  for (int k = 0; k < 3; k++) d[k] = w[k];
+  return J;
+}
+
 __device__ __forceinline__ TriJob make_job(const RawTri &e) {
   TriJob J;
   J.ox = e.x;
@@ -420,8 +430,8 @@ __device__ __forceinline__ F2 piece_mean2(F2 a, F2 b) {
 // Frame row r of J: each edge's piece inside the band r <= y <= r + 1
 // (x-range [a, b] and signed height h, all zero when it misses the band),
 // the columns [c0, c1] the band meets (widened by a small margin; extra
-// columns get zero area) and the fully covered run [fa, fb] (empty when
-// fa > fb).  A pixel of the row is fully covered when the band lies within
+// columns get zero area) and the fully covered run [fa, fb) (empty when
+// fa >= fb).  A pixel of the row is fully covered when the band lies within
 // T's height and the pixel between T's two sides; the sides are the pieces
 // that fall and those that rise when T is traversed anticlockwise, and each
 // (T convex) comes closest to the other side at an end of a piece.
@@ -452,15 +462,13 @@ __device__ __forceinline__ void row_pieces(const TriJob &J, int r, float (&a)[3]
   }
   const float ymin = fminf(J.t[1], fminf(J.t[3], J.t[5]));
   const float ymax = fmaxf(J.t[1], fmaxf(J.t[3], J.t[5]));
-  const float eps = 1e-3f, lim = 1.0e9f;
-  c0 = (int)floorf(fminf(fmaxf(lo - eps, -lim), lim));
-  c1 = (int)floorf(fminf(fmaxf(hi + eps, -lim), lim));
-  fa = 1;
-  fb = 0;
-  if (ymin <= y0 && ymax >= y1) {
-    fa = (int)ceilf(fminf(fmaxf(left + eps, -lim), lim));
-    fb = (int)floorf(fminf(fmaxf(right - eps, -lim), lim)) - 1;
-  }
+  // (conversions saturate: the caller clamps to the map before any arithmetic)
+  const float eps = 1e-3f;
+  c0 = __float2int_rd(lo - eps);
+  c1 = __float2int_rd(hi + eps);
+  const bool full = ymin <= y0 && ymax >= y1;
+  fa = full ? __float2int_ru(left + eps) : 1;
+  fb = full ? __float2int_rd(right - eps) : 1;
 }
 
 // Dealing tasks from a warp's lanes: lane j owns n_j tasks, numbered
@@ -510,7 +518,7 @@ struct __align__(16) RowRec {
 static_assert(sizeof(RowRec) == 80, "RowRec layout");
 struct RowRecs {
   RowRec r[32];
-  int tk[32], trl[32], tex[32];  // triangles with rows: lane, first row, first row task
+  int2 tri[32];  // triangles with rows: lane, first row less first row task
 };
 
 // Add v to the 64-bit word at global address `at` (an address kept as an
@@ -585,42 +593,40 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
   const int excl = incl - nrows;
   const int total = __shfl_sync(0xffffffffu, incl, 31);
   const unsigned with_rows = __ballot_sync(0xffffffffu, nrows > 0);
-  if (nrows > 0) {
-    const int slot = __popc(with_rows & ((1u << lane) - 1u));
-    rr->tk[slot] = lane;
-    rr->trl[slot] = rl;
-    rr->tex[slot] = excl;
-  }
+  if (nrows > 0) rr->tri[__popc(with_rows & ((1u << lane) - 1u))] = make_int2(lane, rl - excl);
   __syncwarp();
   int row_first = 0;
 #pragma unroll 1
   for (int base = 0; base < total; base += 32) {
     const int task = base + lane;
     const int o = deal_owner_slot(nrows, excl, base, lane, row_first);
-    int np = 0, r = 0, c0 = 0, fa = 1, fb = 0, k = 0;
-    float pa[3], pb[3], ph[3];
+    int np = 0, c0 = 0, gx = 0, gy = 0, run = INT_MAX, run_len = 0;
+    float pa[3], pb[3], ph[3], inv2 = 0.f;
     if (task < total) {
-      k = rr->tk[o];
-      r = rr->trl[o] + task - rr->tex[o];
-      const TriJob &J = q[k];
-      int c1;
-      row_pieces(J, r, pa, pb, ph, c0, c1, fa, fb);
+      const int2 t = rr->tri[o];
+      const TriJob J = job_load(q + t.x);
+      int c1, fa, fb;
+      row_pieces(J, t.y + task, pa, pb, ph, c0, c1, fa, fb);
+      inv2 = J.inv2;
+      gy = J.oy + t.y + task;
       c0 = max(c0, -J.ox);
       c1 = min(c1, M.npix - 1 - J.ox);
       fa = max(fa, c0);
-      fb = min(fb, c1);
+      fb = min(fb, c1 + 1);
+      gx = J.ox + c0;
       if (c0 <= c1) {
         np = c1 - c0 + 1;
-        if (fa <= fb) {
-          np -= fb - fa + 1;
+        if (fa < fb) {
+          run = fa - c0;
+          run_len = fb - fa;
+          np -= run_len;
           // a fully covered pixel holds 1/|area| of the triangle (< 1 when any does)
-          const unsigned long long full = frac_to_fixed(fabsf(J.inv2));
-          const long long row = (long long)(J.oy + r) * (M.npix + 1);
+          const unsigned long long full = frac_to_fixed(fabsf(inv2));
+          const long long at = (long long)gy * (M.npix + 1) + (gx + run);
           const long long sn = (long long)M.npix_y * (M.npix + 1);
-          if (MM_INDEX_OK(M.err, row + J.ox + fa, sn) &&
-              MM_INDEX_OK(M.err, row + J.ox + fb + 1, sn)) {
-            atomicAdd(&M.span[row + J.ox + fa], full);
-            atomicAdd(&M.span[row + J.ox + fb + 1], 0ull - full);
+          if (MM_INDEX_OK(M.err, at, sn) && MM_INDEX_OK(M.err, at + run_len, sn)) {
+            atomicAdd(&M.span[at], full);
+            atomicAdd(&M.span[at + run_len], 0ull - full);
           }
         }
       }
@@ -632,24 +638,22 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
     const int slot = __popc(__ballot_sync(0xffffffffu, np > 0) & ((1u << lane) - 1u));
     __syncwarp();  // the previous round's readers are done with the records
     if (np > 0) {
-      const TriJob &J = q[k];
       const float fc0 = (float)c0;
 #pragma unroll
       for (int e = 0; e < 3; e++) {
         // x relative to column c0 (zero-height pieces stay zero)
         pa[e] = ph[e] != 0.f ? pa[e] - fc0 : 0.f;
         pb[e] = ph[e] != 0.f ? pb[e] - fc0 : 0.f;
-        ph[e] *= J.inv2;
+        ph[e] *= inv2;
       }
       RowRec &R = rr->r[slot];
       const unsigned long long at =
-          __cvta_generic_to_global(M.acc + ((long long)(J.oy + r) * M.npix + (J.ox + c0)));
+          __cvta_generic_to_global(M.acc + ((long long)gy * M.npix + gx));
       *reinterpret_cast<float4 *>(&R.a0) = make_float4(pa[0], pa[1], pb[0], pb[1]);
       *reinterpret_cast<float4 *>(&R.h0) = make_float4(ph[0], ph[1], pa[2], pb[2]);
       *reinterpret_cast<int4 *>(&R.h2) =
-          make_int4(__float_as_int(ph[2]), fa <= fb ? fa - c0 : INT_MAX, (int)(unsigned)at,
-                    (int)(unsigned)(at >> 32));
-      *reinterpret_cast<int2 *>(&R.run_len) = make_int2(fb - fa + 1, pexcl);
+          make_int4(__float_as_int(ph[2]), run, (int)(unsigned)at, (int)(unsigned)(at >> 32));
+      *reinterpret_cast<int2 *>(&R.run_len) = make_int2(run_len, pexcl);
     }
     __syncwarp();
     int px_first = 0;
