@@ -786,7 +786,7 @@ def run_native(args):
                    "sub_levels": sorted({st["sub_levels"] for st in stats}),
                    "rows_per_item": sorted({st["rows_per_item"] for st in stats}),
                    "tuned_from_cache": tuned.count(2), "tuned_by_timing": tuned.count(1),
-                   "queue_gb": sum(st["queue_slots"] for st in stats) * 48 / 1e9,
+                   "queue_gb": sum(st["queue_slots"] for st in stats) * 32 / 1e9,
                    "mapping": "irs" if args.irs else "ipm",
                    "band_rows": list(band[:2]) if band else None,
                    "l2": "flushed before every step (256 MiB write)",

@@ -103,18 +103,20 @@ typedef struct {
                                as the row below (the map is unchanged: such
                                cells lie wholly outside it) */
   int32_t big_queue_slots;  /* queue for the second mapping pass, in triangles:
-                               0 -> when the map's accumulators (16 B per
-                               pixel) fit half the GPU's L2, the larger
-                               triangles the autotuner counted (its
-                               jobs_per_mcell, scaled to the grid) plus a
+                               0 -> the larger triangles the autotuner counted
+                               (its jobs_per_mcell, scaled to the grid) plus a
                                quarter, else 1 per 12 cells, within 2^16 ..
                                2^27 (2^20, then none, when the device has not
-                               that much memory free); else none.  -1 -> none
-                               (the first pass deals every larger triangle);
-                               n > 0 -> n.  With a queue and a map that fits,
-                               the first pass runs in consecutive segments of
-                               work items, each followed by the second pass,
-                               so that the expected larger triangles fit.
+                               that much memory free).  A map whose
+                               accumulators (16 B per pixel) exceed half the
+                               GPU's L2: else 2 per cell, at most 64 per pixel;
+                               none below 2^22 or beyond 1/8 of the memory free.
+                               -1 -> none (the first pass deals every larger
+                               triangle); n > 0 -> n.  When the expected larger
+                               triangles exceed it the first pass runs in
+                               segments, each followed by the second pass;
+                               above half the L2 that wants 2^22 slots, and the
+                               second pass goes by bands of map rows.
                                Batches that still do not fit are dealt by the
                                first pass (same map). */
   int32_t autotune;         /* FMM mode, 1: mm_create first times candidate

@@ -213,12 +213,13 @@ struct mm_map {
 
   // map: what every run starts from zero lies in one allocation -- the
   // accumulator, the row-difference array, the statistics [8], the work
-  // counter [1] and the queue's counters [2] (queued, batches taken)
+  // counter [1] and the queue's counters (MapDev::bigq_n)
   DBuf<unsigned long long> zeroed, fixed_out;
   unsigned long long *acc = nullptr, *span = nullptr, *stat = nullptr, *counter = nullptr;
   unsigned long long *bigq_n = nullptr;
   DBuf<char> bigq;                     // larger triangles for the second IPM pass
   int64_t bigq_cap = 0;
+  int band_shift = -1;                 // second pass by bands of 2^band_shift rows (MapDev)
   DBuf<unsigned> err;
   DBuf<float> map;
   DBuf<MapDev> d_md;
@@ -246,9 +247,11 @@ struct mm_map {
   double ms_tune = 0.0;
   int32_t jobs_pm = -1;
 
-  // The first mapping pass runs in `segments` launches over consecutive work
-  // items, each followed by the second pass, so that the queue of larger
-  // triangles (est_jobs) fits its capacity.  Per segment k,
+  // The first mapping pass runs in `segments` launches, each followed by the
+  // second pass, so that the queue of larger triangles (est_jobs) fits its
+  // capacity: launches over equal, consecutive runs of work items, or, on a
+  // map taken by bands, launches that stop taking work items when the queue is
+  // nearly full (MapDev::bigq_limit).  Per segment k,
   // seg_ev[2k] marks the end of its first pass and seg_ev[2k + 1] the end of
   // its second (time_stages only).
   int64_t segments = 1, last_segments = 0;
@@ -762,10 +765,23 @@ static void fill_mapdev(mm_map *h) {
   M.bigq = reinterpret_cast<RawTri *>(h->bigq.p);
   M.bigq_n = h->bigq_n;
   M.bigq_cap = h->bigq_cap;
+  M.bigq_limit = INT64_MAX;
+  // (one allocation: the slots, their order, their bands)
+  M.band_shift = h->bigq_cap > 0 ? h->band_shift : -1;
+  M.bigq_order = reinterpret_cast<uint32_t *>(h->bigq.p + h->bigq_cap * MM_TRIJOB_BYTES);
+  M.bigq_band = reinterpret_cast<uchar2 *>(M.bigq_order + MM_BAND_ENTRIES * h->bigq_cap);
 }
 
 static mm_status clear_map(mm_map *h, cudaStream_t st) {
   CK(cudaMemsetAsync(h->zeroed.p, 0, h->zeroed.n * sizeof(unsigned long long), st));
+  return MM_OK;
+}
+
+// The second mapping pass of a run's (or segment's) queued triangles.
+static mm_status second_pass(mm_map *h, const MapDev &m, cudaStream_t st) {
+  int n = 0;
+  CK(launch_big_ipm(m, n, st));
+  h->launches += n;
   return MM_OK;
 }
 
@@ -778,52 +794,99 @@ static double map_scale(const mm_map *h) {
 }
 
 // Larger triangles (queued for the second pass) expected from `cells` cells:
-// the autotuner's count scaled to them, else one per 12 cells.
+// the autotuner's count scaled to them, else one per 12 cells.  On a map taken
+// by bands all of them, at most 64 a pixel (measured 4.5 to 47): a triangle
+// that finds no slot is dealt out where its lines miss the L2, and a segment
+// too many costs 0.03 ms.
 static int64_t est_jobs(const mm_map *h, int64_t cells) {
   if (h->jobs_pm >= 0) return (int64_t)std::ceil((double)cells * h->jobs_pm / 1048576.0);
+  if (h->band_shift >= 0) return std::min(2 * cells, 64 * (int64_t)h->P.npix * h->P.npix_y);
   return cells / 12;
+}
+
+// A map taken by bands: queued triangles beyond which a segment takes no new
+// work item.  What the items then in work still add (one for each resident
+// warp, counted with a triangle a cell) must find room; what does not is dealt
+// out in place.
+static int64_t segment_limit(const mm_map *h) {
+  const int64_t rows = h->opt.rows_per_item > 0 ? h->rows_per_item : 256;
+  return h->bigq_cap - std::min(h->bigq_cap / 2, 8 * (int64_t)shoot_grid() * MM_STRIP * rows);
+}
+
+// First-pass segments that `cells` cells may need (maps with a queue that
+// adapts, polygon mapping only).  By bands a quarter and one to spare: launches
+// beyond the last work item find nothing to do.
+static int64_t segments_for(const mm_map *h, int64_t cells) {
+  const int64_t est = est_jobs(h, cells);
+  if (est <= h->bigq_cap) return 1;
+  if (h->band_shift < 0) return (est + h->bigq_cap - 1) / h->bigq_cap;
+  return (est + est / 4) / segment_limit(h) + 2;
 }
 
 static mm_status alloc_map_buffers(mm_map *h) {
   const size_t np = (size_t)h->P.npix * h->P.npix_y;
   const size_t nspan = (size_t)h->P.npix_y * (h->P.npix + 1);
-  CK(h->zeroed.ensure(np + nspan + 8 + 1 + 2));
+  CK(h->zeroed.ensure(np + nspan + 8 + 1 + MM_BIGQ_COUNTERS));
   h->acc = h->zeroed.p;
   h->span = h->acc + np;
   h->stat = h->span + nspan;
   h->counter = h->stat + 8;
   h->bigq_n = h->counter + 1;
   CK(h->map.ensure(np));
-  // Queue for the second IPM pass.  It pays while the map's accumulators
-  // (acc + row-difference array, 16 B per pixel) stay in L2: the second pass
-  // then finds their lines there.  A larger map's lines are gone by the time
-  // the second pass reaches a triangle, whereas the first pass deals it where
-  // the lines are hot (measured on 5000^2 and 10000^2 maps: no queue was 18 %
-  // and 8 % faster than a queue, and first passes split into segments to fit
-  // the queue were 17-44 % slower).  Default, for maps that fit half the L2
-  // (else none): the larger triangles the autotuner's sampled runs counted,
-  // with a quarter to spare, else 1 slot per 12 cells; 2^16 .. 2^27 slots
-  // (32 B each).  When that much device memory is not to be had, 2^20 slots,
-  // then none.  Batches that do not fit are dealt out by the first kernel.
+  // Queue for the second IPM pass.  While the map's accumulators (acc +
+  // row-difference array, 16 B per pixel) stay in L2 the second pass finds
+  // their lines there in any order.  A larger map's second pass goes band by
+  // band: 2^band_shift rows of about 16 MB (8 and 32 measured the same), at
+  // most MM_BANDS bands and a band at most a quarter of the L2, so that the few
+  // bands in work stay there; and at least 32 rows, else most triangles would
+  // lie in several.  A map that cannot be cut so has no queue: the first pass
+  // deals every larger triangle where it finds it.  Default size: the larger
+  // triangles the autotuner's sampled runs counted, with a quarter to spare,
+  // else est_jobs' share of the cells; 2^16 .. 2^27 slots (32 B each, and 10 B
+  // more with bands).  When that much device memory is not to be had, 2^20
+  // slots, then none (with bands none, also when it would take more than an
+  // eighth of the free memory).  Batches that do not fit are dealt out by the
+  // first kernel.  A queue of less than 2^22 slots is not taken by bands: a
+  // segment's launches and its last items would cost more than the order gains.
+  // Measured, no queue -> by bands: 3001^2 near the critical line 128 -> 96 ms,
+  // 5000^2 456 -> 172, 5000^2 far from it 128 -> 116, 2060^2 30.7 -> 24.5, a
+  // quarter of the rays 33 -> 24 (3000^2); with 6 cells a pixel 51 -> 32 and, the
+  // only loss found, 9.4 -> 10.8.  2^26 / 2^27 / 2^28 slots: 99 / 97 / 96 ms and,
+  // on the second 5000^2 map, 141 / 130 / 127 (before triangles were cut at the
+  // bands).
   {
     const int64_t cells = (h->col_hi - h->col_lo) * (h->row_hi - h->row_lo);
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
-    const bool fits_l2 = 16.0 * (double)h->P.npix * (double)h->P.npix_y <= 0.5 * (double)l2;
+    const double row_bytes = 16.0 * (double)h->P.npix;
+    const bool fits_l2 = row_bytes * (double)h->P.npix_y <= 0.5 * (double)l2;
+    int shift = 5;
+    while (((h->P.npix_y - 1) >> shift) >= MM_BANDS) shift++;
+    while (shift < 30 && std::ldexp(row_bytes, shift + 1) <= 16.0 * (1 << 20)) shift++;
+    h->band_shift = !fits_l2 && std::ldexp(row_bytes, shift) <= 0.25 * (double)l2 ? shift : -1;
     const int32_t want = h->mode == MM_FMM_IRS ? -1 : h->opt.big_queue_slots;
     const int64_t est = est_jobs(h, cells);
-    const int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;
-    h->bigq_cap = want < 0 ? 0
-                  : want > 0 ? (int64_t)want
-                  : fits_l2  ? std::min<int64_t>(int64_t(1) << 27,
-                                                 std::max<int64_t>(int64_t(1) << 16, slots))
-                             : 0;
+    int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;
+    slots = want > 0 ? want
+                     : std::min<int64_t>(int64_t(1) << 27,
+                                         std::max<int64_t>(int64_t(1) << 16, slots));
+    size_t slot_bytes = MM_TRIJOB_BYTES, mem_free = 0, mem_total = 0;
+    if (slots < (1 << 22)) h->band_shift = -1;
+    if (h->band_shift >= 0) {
+      slot_bytes += MM_BAND_ENTRIES * sizeof(uint32_t) + sizeof(uchar2);
+      // (many large maps' handles leave memory for one another's maps)
+      if (want == 0 && (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess ||
+                        (size_t)slots * slot_bytes > mem_free / 8))
+        h->band_shift = -1;
+    }
+    const bool banded = h->band_shift >= 0;
+    h->bigq_cap = want < 0 || (want == 0 && !fits_l2 && !banded) ? 0 : slots;
     if (h->bigq_cap > 0) {
-      cudaError_t e = h->bigq.ensure((size_t)h->bigq_cap * MM_TRIJOB_BYTES);
+      cudaError_t e = h->bigq.ensure((size_t)h->bigq_cap * slot_bytes);
       if (e == cudaErrorMemoryAllocation && want == 0) {
         cudaGetLastError();  // (clears the failed allocation's error)
-        h->bigq_cap = std::min<int64_t>(h->bigq_cap, int64_t(1) << 20);
-        e = h->bigq.ensure((size_t)h->bigq_cap * MM_TRIJOB_BYTES);
+        h->bigq_cap = banded ? 0 : std::min<int64_t>(h->bigq_cap, int64_t(1) << 20);
+        e = h->bigq.ensure((size_t)h->bigq_cap * slot_bytes);
         if (e == cudaErrorMemoryAllocation) {
           cudaGetLastError();
           h->bigq_cap = 0;
@@ -832,11 +895,10 @@ static mm_status alloc_map_buffers(mm_map *h) {
       }
       CK(e);
     }
-    // a map that fits: the first pass runs in segments so that each
-    // segment's larger triangles fit the queue
+    // (a map that neither fits nor is taken by bands runs one first pass)
     h->segments = 1;
-    if (h->bigq_cap > 0 && h->mode == MM_FMM_FP32 && fits_l2)
-      h->segments = std::max<int64_t>(1, (est + h->bigq_cap - 1) / h->bigq_cap);
+    if (h->bigq_cap > 0 && h->mode == MM_FMM_FP32 && (fits_l2 || banded))
+      h->segments = segments_for(h, cells);
     if (h->opt.time_stages && (int64_t)h->seg_ev.size() < 2 * h->segments) {
       const size_t have = h->seg_ev.size();
       h->seg_ev.resize(2 * h->segments, nullptr);
@@ -881,13 +943,6 @@ static MapDev restrict_mapdev(const mm_map *h, const CellRect &r) {
   return m;
 }
 
-// First-pass segments for `cells` cells: their larger triangles must fit
-// the queue (maps that fit L2, polygon mapping only).
-static int64_t segments_for(const mm_map *h, int64_t cells) {
-  if (h->segments <= 1 || h->bigq_cap <= 0) return 1;
-  return std::max<int64_t>(1, (est_jobs(h, cells) + h->bigq_cap - 1) / h->bigq_cap);
-}
-
 // One run of the handle's map over its cells, or over the rectangle `rect`
 // of them (NULL: all).
 static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = nullptr) {
@@ -919,7 +974,7 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
     LCH(launch_ipm_vertices(h->d_md.p, h->verts.p, R.c1 - R.c0 + 1, R.r0, R.r1, h->counter,
                             h->err.p, shoot_grid(), st));
     CKS(record(h, 5, st));
-    LCH(launch_big_ipm(h->md, st));
+    CKS(second_pass(h, h->md, st));
   } else {
     // The plan of mm_create ran the whole tree and expansion pipeline on the
     // same stars; the first run uses that result instead of repeating it.
@@ -945,20 +1000,27 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
       h->ran = true;
       return MM_OK;
     }
-    const int64_t segs = rect ? segments_for(h, (R.r1 - R.r0) * (R.c1 - R.c0)) : h->segments;
+    const int64_t segs =
+        rect && h->segments > 1
+            ? std::min(h->segments, segments_for(h, (R.r1 - R.r0) * (R.c1 - R.c0)))
+            : h->segments;
     const int64_t nseg = std::max<int64_t>(1, std::min(segs, work));
-    const int64_t per = (work + nseg - 1) / nseg;
+    const bool banded = h->band_shift >= 0;
+    const int64_t per = banded ? work : (work + nseg - 1) / nseg;  // items of a launch
     int64_t k = 0;
-    for (int64_t w0 = 0; w0 < work; w0 += per, k++) {
-      if (w0 > 0) {  // the previous segment's second pass has drained the queue
-        CK(cudaMemsetAsync(h->counter, 0, 3 * sizeof(unsigned long long), st));
-      }
+    for (int64_t w0 = 0; banded ? k < nseg : w0 < work; k++, w0 += per) {
+      // the previous segment's second pass has drained the queue; launches
+      // over runs of items begin anew, by bands each goes on with the next item
+      if (k > 0 && !banded) CK(cudaMemsetAsync(h->counter, 0, sizeof(unsigned long long), st));
+      if (k > 0)
+        CK(cudaMemsetAsync(h->bigq_n, 0, MM_BIGQ_COUNTERS * sizeof(unsigned long long), st));
       MapDev ms = base;
-      ms.work_begin = -w0;  // this launch's item w is item w0 + w of the map
-      LCH(launch_shoot_ipm(h->d_md.p, &ms, 1, std::min(per, work - w0), base.square_cells != 0,
-                          h->counter, h->err.p, shoot_grid(), st));
+      if (!banded) ms.work_begin = -w0;  // this launch's item w is item w0 + w of the map
+      if (banded && k + 1 < nseg) ms.bigq_limit = segment_limit(h);
+      LCH(launch_shoot_ipm(h->d_md.p, &ms, 1, banded ? work : std::min(per, work - w0),
+                          base.square_cells != 0, h->counter, h->err.p, shoot_grid(), st));
       if (h->opt.time_stages) CK(cudaEventRecord(h->seg_ev[2 * k], st));
-      LCH(launch_big_ipm(ms, st));
+      CKS(second_pass(h, ms, st));
       if (h->opt.time_stages) CK(cudaEventRecord(h->seg_ev[2 * k + 1], st));
     }
     h->last_segments = k;
@@ -1516,7 +1578,7 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     cudaStream_t si = lead->fan[i % nfan];
     h->last_segments = 0;  // one first pass for the whole batch
     CKS(record(h, 5, si));
-    LCH(launch_big_ipm(h->md, si));
+    CKS(second_pass(h, h->md, si));
     CKS(record(h, 3, si));
     LCH(launch_normalize(h->acc, h->span, h->P.npix, h->P.npix_y, map_scale(h), h->map.p, si));
     CKS(record(h, 4, si));

@@ -577,15 +577,15 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
                                                   unsigned long long *span, int npix,
                                                   int npix_y, unsigned *err,
                                                   const TriJob *q, int nb, RowRecs *rr,
-                                                  int lane) {
+                                                  int lane, int row_lo, int row_hi) {
   const MapAcc M = {acc, span, npix, npix_y, err};
   int rl = 0, nrows = 0;
   if (lane < nb) {
     const TriJob &J = q[lane];
     const float ymin = fminf(J.t[1], fminf(J.t[3], J.t[5]));
     const float ymax = fmaxf(J.t[1], fmaxf(J.t[3], J.t[5]));
-    const int r0 = max((int)floorf(fmaxf(ymin, -1.0e9f)), -J.oy);
-    const int r1 = min((int)floorf(fminf(ymax, 1.0e9f)), M.npix_y - 1 - J.oy);
+    const int r0 = max((int)floorf(fmaxf(ymin, -1.0e9f)), row_lo - J.oy);
+    const int r1 = min((int)floorf(fminf(ymax, 1.0e9f)), row_hi - 1 - J.oy);
     rl = r0;
     nrows = r1 >= r0 ? r1 - r0 + 1 : 0;
   }
@@ -792,7 +792,8 @@ __device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool f
     }
     __syncwarp();
     if (deal > 0) {
-      warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q.s->job, deal, &q.s->rows, lane);
+      warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q.s->job, deal, &q.s->rows, lane, 0,
+                    M.npix_y);
       deal = 0;
     }
     if (!(q.big >= 32 || (flush && q.big > 0))) break;

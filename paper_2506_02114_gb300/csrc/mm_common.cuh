@@ -72,6 +72,9 @@ struct __align__(16) Vtx {
 
 struct RawTri;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
 #define MM_TRIJOB_BYTES 32
+#define MM_BANDS 64           // row bands of the second pass at most
+#define MM_BIGQ_COUNTERS (2 + 2 * MM_BANDS)
+#define MM_BAND_ENTRIES 2     // room in bigq_order for so many entries a slot
 
 // Everything the deflection + mapping kernel needs about one map.
 struct MapDev {
@@ -115,8 +118,15 @@ struct MapDev {
   unsigned long long *stat;   // triangle counters, see IpmCounters
   // larger triangles handed to the second kernel (capacity 0: none)
   RawTri *bigq;
-  unsigned long long *bigq_n; // [0] triangles queued, [1] the second kernel's batch counter
+  unsigned long long *bigq_n; // [0] triangles queued, [1] the second kernel's batch counter,
+                              // then per band its entries and the places taken of them
   int64_t bigq_cap;
+  int64_t bigq_limit;         // the first pass takes no new work item beyond so many queued
+  // a map too large for the L2: the second pass takes the queue by bands of
+  // 2^band_shift map rows (-1: in queue order)
+  uchar2 *bigq_band;          // per slot: the first and the last band of its rows
+  uint32_t *bigq_order;       // slots in the order of their bands, one entry for each band
+  int32_t band_shift, pad;
 };
 
 // Far-field coefficient slots per sub-cell record: the p_eval - 1

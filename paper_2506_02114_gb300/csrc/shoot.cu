@@ -394,8 +394,12 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
   __shared__ MapDev s_md[8];
   MapDev &SM = s_md[threadIdx.x >> 5];
   while (true) {
-    unsigned long long w = 0;
-    if (lane == 0) w = atomicAdd(work_counter, 1ull);
+    // (a single map whose larger triangles may exceed its queue stops at the
+    // limit; its next launch goes on where this one stopped)
+    unsigned long long w = (unsigned long long)total_work;
+    if (lane == 0 && (BATCH || M1.bigq_limit == INT64_MAX ||
+                      (int64_t)__ldcg(M1.bigq_n) < M1.bigq_limit))
+      w = atomicAdd(work_counter, 1ull);
     w = __shfl_sync(0xffffffffu, w, 0);
     if ((int64_t)w >= total_work) break;
     int mi = 0;
@@ -643,14 +647,51 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
 // and deals out their pixel rows and partially covered pixels
 // (warp_tri_jobs), at 5 blocks per SM where the first kernel runs 3 (48
 // registers allow 5 without spills: 3 % faster than 4; 6 forces spills)
+//
+// BANDED: a map too large for the L2 is taken band by band (the entries in the
+// order k_band_scatter puts them), so that the lines of the rows being worked
+// on stay in the L2.  A triangle reaching into several bands has an entry in
+// each and is dealt there within that band's rows: triangles near a star are
+// large (a height above L for 1/L of them), and whole they would touch lines
+// far from the band.  3001^2 map near the critical line, 4.3e8 triangles: 173 ms
+// in queue order, 73 ms by bands; 5000^2 map, 2.6e8 triangles: 51 ms by bands
+// with whole triangles (10 GB written in 1.3e8), 39 ms cut (the map once).
 #define MM_BIG_MINB 5
+
+// Queued triangles that found a slot.
+__device__ __forceinline__ long long queued(const MapDev &M) {
+  const unsigned long long cap = (unsigned long long)M.bigq_cap, qn = *M.bigq_n;
+  return (long long)(qn < cap ? qn : cap);
+}
+// The bands of a triangle's rows within the map; x > y: none.
+__device__ __forceinline__ int2 band_range(const MapDev &M, const RawTri &t) {
+  const float ymin = fminf(t.f[1], fminf(t.f[3], t.f[5]));
+  const float ymax = fmaxf(t.f[1], fmaxf(t.f[3], t.f[5]));
+  const int r0 = max(t.y + __float2int_rd(fminf(fmaxf(ymin, -1.0e9f), 1.0e9f)), 0);
+  const int r1 = min(t.y + __float2int_rd(fminf(fmaxf(ymax, -1.0e9f), 1.0e9f)), M.npix_y - 1);
+  if (r0 > r1) return make_int2(1, 0);
+  return make_int2(r0 >> M.band_shift, r1 >> M.band_shift);
+}
+// s_end[k]: entries of bands 0 .. k.  False: more than there is room for (then
+// the queue is taken in its own order).  Call with all threads of the block.
+__device__ __forceinline__ bool band_ends(const MapDev &M, unsigned long long *s_end) {
+  if (threadIdx.x < MM_BANDS) {
+    unsigned long long n = 0;
+    for (int k = 0; k <= threadIdx.x; k++) n += M.bigq_n[2 + k];
+    s_end[threadIdx.x] = n;
+  }
+  __syncthreads();
+  return s_end[MM_BANDS - 1] <= MM_BAND_ENTRIES * (unsigned long long)M.bigq_cap;
+}
+
+template <bool BANDED>
 __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
   __shared__ TriJob q[8][32];
   __shared__ RowRecs rr[8];
+  __shared__ unsigned long long s_end[BANDED ? MM_BANDS : 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const unsigned long long cap = (unsigned long long)M.bigq_cap;
-  const unsigned long long qn = *M.bigq_n;
-  const long long n = (long long)(qn < cap ? qn : cap);
+  const bool sorted = BANDED && band_ends(M, s_end);
+  const long long n = sorted ? (long long)s_end[BANDED ? MM_BANDS - 1 : 0] : queued(M);
   while (true) {
     unsigned long long b = 0;
     if (lane == 0) b = atomicAdd(M.bigq_n + 1, 1ull);
@@ -658,9 +699,102 @@ __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
     const long long base = (long long)b * 32;
     if (base >= n) break;
     const int nb = (int)min(32ll, n - base);
-    if (lane < nb) q[w][lane] = make_job(raw_load(M.bigq + base + lane));
+    int row_lo = 0, row_hi = M.npix_y;
+    if (lane < nb) {
+      const long long slot = sorted ? (long long)M.bigq_order[base + lane] : base + lane;
+      const RawTri t = raw_load(M.bigq + slot);
+      q[w][lane] = make_job(t);
+      if (sorted) {
+        int band = 0;  // the first band that ends beyond this entry
+#pragma unroll
+        for (int step = MM_BANDS / 2; step > 0; step >>= 1)
+          if (s_end[band + step - 1] <= (unsigned long long)(base + lane)) band += step;
+        const int2 r = band_range(M, t);
+        // (the outer bands take what rounding puts beyond them)
+        if (band > r.x) row_lo = band << M.band_shift;
+        if (band < r.y) row_hi = (band + 1) << M.band_shift;
+      }
+    }
     __syncwarp();
-    warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q[w], nb, &rr[w], lane);
+    warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q[w], nb, &rr[w], lane, row_lo, row_hi);
+  }
+}
+
+// The bands of each queued triangle, and the entries per band (bigq_n[2 +
+// band]; a warp's lanes of one first band count together).  Here and not where
+// the triangle is queued: one more pass over the queue (0.2 ms a 1.3e8 slots)
+// against spills in the first pass's batch kernel (5 % slower).
+#define MM_BAND_CHUNK 4096  // slots per block of the two kernels below
+__device__ __forceinline__ void band_tally(unsigned *s_n, int2 r, int lane) {
+  const int first = r.x <= r.y ? r.x : -1;
+  const unsigned m = __match_any_sync(0xffffffffu, first);
+  if (first >= 0 && lane == __ffs(m) - 1) atomicAdd(&s_n[first], (unsigned)__popc(m));
+  for (int k = r.x + 1; k <= r.y; k++) atomicAdd(&s_n[k], 1u);
+}
+__global__ void __launch_bounds__(256) k_band_count(const MapDev M) {
+  __shared__ unsigned s_n[MM_BANDS];
+  if (threadIdx.x < MM_BANDS) s_n[threadIdx.x] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const long long n = queued(M);
+  for (long long c = (long long)blockIdx.x * MM_BAND_CHUNK; c < n;
+       c += (long long)gridDim.x * MM_BAND_CHUNK) {
+    const long long e = min(n, c + MM_BAND_CHUNK);
+    for (long long k = c + threadIdx.x; k - lane < e; k += 256) {
+      int2 r = make_int2(1, 0);
+      if (k < e) {
+        r = band_range(M, raw_load(M.bigq + k));
+        M.bigq_band[k] = make_uchar2((unsigned char)r.x, (unsigned char)r.y);
+      }
+      band_tally(s_n, r, lane);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < MM_BANDS && s_n[threadIdx.x])
+    atomicAdd(M.bigq_n + 2 + threadIdx.x, (unsigned long long)s_n[threadIdx.x]);
+}
+
+// The slots in the order of their bands (any order within one): each chunk
+// counts its entries per band, reserves their places, and writes them.
+__global__ void __launch_bounds__(256) k_band_scatter(const MapDev M) {
+  __shared__ unsigned s_n[MM_BANDS];
+  __shared__ unsigned long long s_end[MM_BANDS], s_at[MM_BANDS];
+  if (!band_ends(M, s_end)) return;
+  const int lane = threadIdx.x & 31;
+  const long long n = queued(M);
+  for (long long c = (long long)blockIdx.x * MM_BAND_CHUNK; c < n;
+       c += (long long)gridDim.x * MM_BAND_CHUNK) {
+    const long long e = min(n, c + MM_BAND_CHUNK);
+    __syncthreads();
+    if (threadIdx.x < MM_BANDS) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    for (long long k = c + threadIdx.x; k - lane < e; k += 256) {
+      const uchar2 r = k < e ? M.bigq_band[k] : make_uchar2(1, 0);
+      band_tally(s_n, make_int2(r.x, r.y), lane);
+    }
+    __syncthreads();
+    if (threadIdx.x < MM_BANDS) {
+      const unsigned cnt = s_n[threadIdx.x];
+      if (cnt)
+        s_at[threadIdx.x] =
+            (threadIdx.x ? s_end[threadIdx.x - 1] : 0ull) +
+            atomicAdd(M.bigq_n + 2 + MM_BANDS + threadIdx.x, (unsigned long long)cnt);
+      s_n[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    for (long long k = c + threadIdx.x; k - lane < e; k += 256) {
+      const uchar2 r = k < e ? M.bigq_band[k] : make_uchar2(1, 0);
+      const int band = r.x <= r.y ? r.x : -1;
+      const unsigned m = __match_any_sync(0xffffffffu, band);
+      const int first = __ffs(m) - 1;
+      unsigned at = 0;
+      if (band >= 0 && lane == first) at = atomicAdd(&s_n[band], (unsigned)__popc(m));
+      at = __shfl_sync(0xffffffffu, at, first);
+      if (band >= 0)
+        M.bigq_order[s_at[band] + at + __popc(m & ((1u << lane) - 1u))] = (uint32_t)k;
+      for (int o = r.x + 1; o <= r.y; o++)
+        M.bigq_order[s_at[o] + atomicAdd(&s_n[o], 1u)] = (uint32_t)k;
+    }
   }
 }
 
@@ -835,12 +969,20 @@ cudaError_t launch_shoot_irs(const MapDev &m, int64_t total_work, bool square,
   return cudaGetLastError();
 }
 
-cudaError_t launch_big_ipm(const MapDev &m, cudaStream_t st) {
+cudaError_t launch_big_ipm(const MapDev &m, int &launches, cudaStream_t st) {
   if (m.bigq_cap <= 0) return cudaSuccess;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  k_big_ipm<<<sms * MM_BIG_MINB, 256, 0, st>>>(m);
+  if (m.band_shift >= 0) {
+    k_band_count<<<sms * 8, 256, 0, st>>>(m);
+    k_band_scatter<<<sms * 8, 256, 0, st>>>(m);
+    k_big_ipm<true><<<sms * MM_BIG_MINB, 256, 0, st>>>(m);
+    launches += 3;
+  } else {
+    k_big_ipm<false><<<sms * MM_BIG_MINB, 256, 0, st>>>(m);
+    launches++;
+  }
   return cudaGetLastError();
 }
 

@@ -68,3 +68,64 @@ def test_stored_vertices_map_like_the_oracle(oracle_mod, cols, rows):
     assert e["p999"] <= MAP_P999_TOL, e
     # (a mean over a few cells is their outline's, to FP32)
     assert cols * rows < 1000 or e["mean_rel"] <= MEAN_TOL, e
+
+
+@pytest.mark.parametrize("shape,grid,gamma,slots", [
+    ((2200, 2200), (350, 300), 0.3, (0, 1000, 1 << 22)),  # too few cells for a queue by default
+    ((2200, 2200), (3400, 3300), 0.3, (0, 1 << 22)),      # 2^22 slots: several first passes
+    ((60, 110000), (200, 900), 0.3, (1 << 22,)),          # 64 bands at most, of tall strips
+    ((30000, 300), (900, 200), 0.3, (1 << 22,)),          # 32 rows a band, triangles over many
+    ((2200, 2200), (2500000, 3), -0.3, (1 << 22,)),       # more bands a triangle than there is room
+])
+@pytest.mark.parametrize("mode", [mm.MM_FMM_FP32, mm.MM_PLAIN_FP64])
+def test_bands_of_a_large_map_do_not_change_it(shape, grid, gamma, slots, mode):
+    """A map above half the L2: its second pass takes a queue of 2^22 slots or
+    more by bands of rows.  Queue or none, one first pass or several, whole, in
+    two rectangles of cells or in a batch: one map, bit for bit, and the same
+    counts."""
+    import torch
+    torch.cuda.init()
+    if mode == mm.MM_PLAIN_FP64 and grid[0] * grid[1] > 1000000:
+        pytest.skip("the segments are the FMM path's")
+    kappa, s = 0.45, 0.4
+    m, pos = synthetic.star_field(13, 40, 14.0, synthetic.SALPETER_01_1)
+    half = 2.0 * shape[0] / max(shape)
+    opts = dict(fmm_order=20, img_half=(7.0, 3.0), ray_grid=(grid[0] + 1, grid[1] + 1),
+                npix_y=shape[1], mode=mode)
+
+    def result(h):
+        st = mm.get_stats(h)
+        assert st["error_bits"] == 0
+        return mm.get_map_fixed(h), [st[k] for k in st if k.startswith("triangles_")], st
+
+    def make(n):
+        return mm.create(kappa, gamma, s, m, pos, half, shape[0], big_queue_slots=n, **opts)
+
+    h = make(-1)
+    mm.run(h, 0)
+    ref, counts, st0 = result(h)
+    mm.destroy(h)
+    assert ref.any() and st0["triangles_box"] + st0["triangles_rows"] > 500
+    for n in slots:
+        h = make(n)
+        for rep in range(2):
+            mm.run(h, 0)
+            got, c, st = result(h)
+            assert np.array_equal(ref, got) and c == counts
+        few = grid[0] * grid[1] < 1 << 21
+        assert (st["queue_slots"] > 0) == (n > 0 or not few)
+        if n == 1 << 22 and not few:
+            assert st["kernel_launches"] > st0["kernel_launches"] + 6
+        cut = grid[1] // 3
+        mm.run_cells(h, 0, cut, 0, grid[0], 0)
+        tot = mm.get_map_fixed(h)
+        mm.run_cells(h, cut, grid[1], 0, grid[0], 0)
+        assert np.array_equal(ref, tot + mm.get_map_fixed(h))
+        if mode == mm.MM_FMM_FP32:
+            other = make(n)
+            mm.run_batch([h, other], 0)
+            for one in (h, other):
+                got, c, _ = result(one)
+                assert np.array_equal(ref, got) and c == counts
+            mm.destroy(other)
+        mm.destroy(h)
