@@ -72,7 +72,7 @@ __device__ __forceinline__ unsigned long long frac_to_fixed(float f) {
 
 // The map edges a vertex lies beyond, one bit each (0 when non-finite): a
 // triangle lies wholly beyond one edge when its vertices share a bit.
-__device__ __forceinline__ unsigned outcode(const MapDev &M, const Vtx &v) {
+__device__ __forceinline__ unsigned outcode(const MapCore &M, const Vtx &v) {
   const unsigned c = (v.px < 0 ? 1u : 0u) | (v.px >= M.npix ? 2u : 0u) | (v.py < 0 ? 4u : 0u) |
                      (v.py >= M.npix_y ? 8u : 0u);
   return v.px == MM_VTX_INVALID ? 0u : c;
@@ -98,7 +98,7 @@ __device__ __forceinline__ bool mm_index_ok(unsigned *err, long long idx, long l
 #endif
 
 // Add u (in 2^-24 triangles) to map pixel idx if `in` the map.
-__device__ __forceinline__ void deposit(const MapDev &M, bool in, long long idx, unsigned u) {
+__device__ __forceinline__ void deposit(const MapCore &M, bool in, long long idx, unsigned u) {
   if (in && u && MM_INDEX_OK(M.err, idx, (long long)M.npix * M.npix_y))
     atomicAdd(&M.acc[idx], (unsigned long long)u << 8);
 }
@@ -122,7 +122,7 @@ struct RunAcc {
 #define MM_RUN_NONE RunAcc{-1, 0, 0u}
 
 template <unsigned long long UNIT>
-__device__ __forceinline__ void run_flush(const MapDev &M, RunAcc &a) {
+__device__ __forceinline__ void run_flush(const MapCore &M, RunAcc &a) {
   const long long idx = (long long)a.py * M.npix + a.px;
   if (a.px >= 0 && MM_INDEX_OK(M.err, idx, (long long)M.npix * M.npix_y))
     atomicAdd(&M.acc[idx], a.n * UNIT);
@@ -131,7 +131,7 @@ __device__ __forceinline__ void run_flush(const MapDev &M, RunAcc &a) {
 
 // Count one in in-map pixel (px, py).
 template <unsigned long long UNIT>
-__device__ __forceinline__ void run_add(const MapDev &M, RunAcc &a, int px, int py) {
+__device__ __forceinline__ void run_add(const MapCore &M, RunAcc &a, int px, int py) {
   if (px == a.px && py == a.py) {
     a.n++;
     return;
@@ -276,7 +276,7 @@ struct LaneCount {
 
 // Area test of a triangle that meets the map: false (and counted) when it
 // has none; near-critical ones are counted.
-__device__ __forceinline__ bool area_ok(const MapDev &M, float area2, LaneCount &lc) {
+__device__ __forceinline__ bool area_ok(const MapCore &M, float area2, LaneCount &lc) {
   if (!(area2 != 0.f) || !isfinite(area2)) {
     lc.dropped++;
     return false;
@@ -290,7 +290,7 @@ __device__ __forceinline__ bool area_ok(const MapDev &M, float area2, LaneCount 
 // fraction d^2 / ((u_a - u_l)(u_b - u_l)) with d = L - u_l (the two edge
 // parameters at the line, multiplied).  The two shares are complements in
 // fixed point, so the pair sums to exactly one triangle.
-__device__ __forceinline__ bool line_tri_apportion(const MapDev &M, const RawTri &e,
+__device__ __forceinline__ bool line_tri_apportion(const MapCore &M, const RawTri &e,
                                                    LaneCount &lc) {
   float t[6];
   int ax, ay;
@@ -315,7 +315,7 @@ __device__ __forceinline__ bool line_tri_apportion(const MapDev &M, const RawTri
 // of X and below Y from the lone vertex on each line, the lower-left share
 // from the quadrant integral; the four pixel shares are differences of
 // those in fixed point and add up to exactly one triangle.
-__device__ __forceinline__ bool quad_tri_apportion(const MapDev &M, const RawTri &e,
+__device__ __forceinline__ bool quad_tri_apportion(const MapCore &M, const RawTri &e,
                                                    LaneCount &lc) {
   float t[6];
   int ax, ay;
@@ -504,21 +504,14 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 // the weighted sum of piece means is the pixel's share.  Then the
 // first column of the fully covered run relative to c0 (INT_MAX: none) and
 // its length, the address of the map's pixel (c0, row), and the row's first
-// pixel task.  Stored as 16-byte words for 16-byte loads, with one of padding
-// so that eight consecutive records fall on distinct banks.
-struct __align__(16) RowRec {
-  float a0, a1, b0, b1;
-  float h0, h1, a2, b2;
-  float h2;
-  int run;
-  unsigned long long px;
-  int run_len, first;
-  int pad[6];
-};
-static_assert(sizeof(RowRec) == 80, "RowRec layout");
+// pixel task.  One array per 16-byte word: consecutive slots fall on distinct
+// banks without padding.
 struct RowRecs {
-  RowRec r[32];
-  int2 tri[32];  // triangles with rows: lane, first row less first row task
+  float4 piece[32];   // a0, a1, b0, b1
+  float4 height[32];  // h0, h1, a2, b2
+  int4 pixel[32];     // h2, run, address
+  int2 task[32];      // run length, first task
+  int2 tri[32];       // triangles with rows: lane, first row less first row task
 };
 
 // Add v to the 64-bit word at global address `at` (an address kept as an
@@ -533,11 +526,9 @@ __device__ __forceinline__ void red_add(unsigned long long at, unsigned long lon
 __device__ __forceinline__ void pixel_task(const MapAcc &M, const RowRecs *rr, int o, int task,
                                            int ptotal) {
   if (task < ptotal) {
-    const RowRec &R = rr->r[o];
-    const float4 p0 = *reinterpret_cast<const float4 *>(&R.a0);
-    const float4 p1 = *reinterpret_cast<const float4 *>(&R.h0);
-    const int4 p2 = *reinterpret_cast<const int4 *>(&R.h2);
-    const int2 p3 = *reinterpret_cast<const int2 *>(&R.run_len);
+    const float4 p0 = rr->piece[o], p1 = rr->height[o];
+    const int4 p2 = rr->pixel[o];
+    const int2 p3 = rr->task[o];
     int c = task - p3.y;
     if (c >= p2.y) c += p3.x;
     const float nc = -(float)c;
@@ -646,14 +637,13 @@ __device__ __forceinline__ void warp_tri_jobs(unsigned long long *acc,
         pb[e] = ph[e] != 0.f ? pb[e] - fc0 : 0.f;
         ph[e] *= inv2;
       }
-      RowRec &R = rr->r[slot];
       const unsigned long long at =
           __cvta_generic_to_global(M.acc + ((long long)gy * M.npix + gx));
-      *reinterpret_cast<float4 *>(&R.a0) = make_float4(pa[0], pa[1], pb[0], pb[1]);
-      *reinterpret_cast<float4 *>(&R.h0) = make_float4(ph[0], ph[1], pa[2], pb[2]);
-      *reinterpret_cast<int4 *>(&R.h2) =
-          make_int4(__float_as_int(ph[2]), run, (int)(unsigned)at, (int)(unsigned)(at >> 32));
-      *reinterpret_cast<int2 *>(&R.run_len) = make_int2(run_len, pexcl);
+      rr->piece[slot] = make_float4(pa[0], pa[1], pb[0], pb[1]);
+      rr->height[slot] = make_float4(ph[0], ph[1], pa[2], pb[2]);
+      rr->pixel[slot] = make_int4(__float_as_int(ph[2]), run, (int)(unsigned)at,
+                                  (int)(unsigned)(at >> 32));
+      rr->task[slot] = make_int2(run_len, pexcl);
     }
     __syncwarp();
     int px_first = 0;
@@ -682,22 +672,21 @@ enum { ST_DROPPED, ST_CLIPPED, ST_QUAD, ST_BOX, ST_ROWS, ST_LINE, ST_CULLED, ST_
 #define MM_SMALL_QUEUE (31 + 31 + 62)
 #define MM_BIG_QUEUE (31 + 62)
 
-// Shared memory of one warp.  A batch of larger triangles dealt out here
-// needs the row records, which lie over the line and quad queues (emptied
-// first), and its 32 full jobs behind the at most 61 triangles then left in
-// the big queue.
+// Shared memory of one warp.  A batch of larger triangles dealt out here has
+// its row records and jobs over the line and quad queues (emptied first).
+// 8000 bytes: three blocks of the shooting kernel then leave the L1 60 KB in
+// place of 28 (shared memory is taken in steps, 196 and 228 KB the last), and
+// 85 % of the records' sectors hit it in place of 60 %: first pass of the
+// 2000^2 map 11.97 -> 11.48 ms, 12 maps in a batch 35.1 -> 32.3 ms.
 struct __align__(16) WarpSmem {
   union {
     RawTri small[MM_SMALL_QUEUE];
-    RowRecs rows;
-  };
-  union {
-    RawTri big[MM_BIG_QUEUE];
     struct {
-      RawTri left[MM_BIG_QUEUE - 32];
+      RowRecs rows;
       TriJob job[32];
     };
   };
+  RawTri big[MM_BIG_QUEUE];
   Vtx row[32];                    // the last vertex row, one vertex per lane
   Vtx next[32];                   // the next one, where it was shot with it
   unsigned count[MM_N_COUNTERS];  // (dropped and critical are per lane, LaneCount)
@@ -712,7 +701,7 @@ struct WarpQueues {
 // Apportion or queue one triangle (a, b, c) of each lane (`on`: the lane
 // has one, not wholly beyond one edge of the map).  A triangle inside one
 // pixel is finished here.
-__device__ __forceinline__ void tri_scan(const MapDev &M, WarpQueues &q, const Vtx &a,
+__device__ __forceinline__ void tri_scan(const MapCore &M, WarpQueues &q, const Vtx &a,
                                          const Vtx &b, const Vtx &c, bool on, RunAcc &ra,
                                          LaneCount &lc, int lane) {
   // the pixel box from the vertices' pixels (a vertex's pixel is the floor
@@ -764,7 +753,7 @@ __device__ __forceinline__ void tri_scan(const MapDev &M, WarpQueues &q, const V
 // the larger-triangle kernel (k_big_ipm), which deals them out at a higher
 // occupancy than this kernel's; a batch that does not fit is dealt out here,
 // its reserved queue slots filled with triangles without pixel rows.
-__device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool flush,
+__device__ __forceinline__ void share_out(const MapCore &M, WarpQueues &q, bool flush,
                                           LaneCount &lc, int lane) {
   if (!flush && ((q.line | q.quad | q.big) & ~31) == 0) return;
   int deal = 0;  // jobs set up to be dealt out here
@@ -792,6 +781,8 @@ __device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool f
     }
     __syncwarp();
     if (deal > 0) {
+      if (lane < deal) q.s->job[lane] = make_job(raw_load(q.s->big + q.big + lane));
+      __syncwarp();
       warp_tri_jobs(M.acc, M.span, M.npix, M.npix_y, M.err, q.s->job, deal, &q.s->rows, lane, 0,
                     M.npix_y);
       deal = 0;
@@ -831,8 +822,10 @@ __device__ __forceinline__ void share_out(const MapDev &M, WarpQueues &q, bool f
         raw_store(M.bigq + base + lane, e.x, e.y, e.f[0], e.f[1], e.f[2], e.f[3], e.f[4], e.f[5]);
       __syncwarp();
     } else {
-      __syncwarp();  // (the jobs overlap queue entries just read)
-      if (lane < nb) q.s->job[lane] = make_job(e);
+      // (back to its place above the queue's end until the others are empty)
+      if (lane < nb)
+        raw_store(q.s->big + q.big + lane, e.x, e.y, e.f[0], e.f[1], e.f[2], e.f[3], e.f[4],
+                  e.f[5]);
       deal = nb;
     }
   }
@@ -844,7 +837,7 @@ __device__ __forceinline__ void counts_clear(WarpSmem *s, int lane) {
 }
 
 // Add the warp's counters to the map's statistics and clear them.
-__device__ __forceinline__ void counts_flush(const MapDev &M, WarpSmem *s, LaneCount &lc,
+__device__ __forceinline__ void counts_flush(const MapCore &M, WarpSmem *s, LaneCount &lc,
                                              int lane) {
   const unsigned d = __reduce_add_sync(0xffffffffu, lc.dropped);
   const unsigned c = __reduce_add_sync(0xffffffffu, lc.critical);

@@ -76,8 +76,9 @@ struct RawTri;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
 #define MM_BIGQ_COUNTERS (2 + 2 * MM_BANDS)
 #define MM_BAND_ENTRIES 2     // room in bigq_order for so many entries a slot
 
-// Everything the deflection + mapping kernel needs about one map.
-struct MapDev {
+// Everything the deflection + mapping kernel needs about one map: what a work
+// item's bounds come from,
+struct MapItems {
   // ray grid
   int64_t n0, n1;             // vertices per axis
   int64_t row_begin, row_end; // cell rows [row_begin, row_end)
@@ -87,6 +88,11 @@ struct MapDev {
   int64_t item_stride;        // >= 1: work item k covers row block k * item_stride
                               // (> 1 only for the autotuner's sampled runs)
   int64_t work_begin;         // first global work item of this map
+};
+
+// what is read for every ray or triangle (in a batch each warp keeps its map's
+// in shared memory),
+struct MapCore {
   // leaf lookup
   const int32_t *col_cell, *row_cell;   // finest-level cell index per vertex column / row
   const int32_t *grid;                  // lookup grid: sub-cell record id, or -(node+1)
@@ -121,6 +127,10 @@ struct MapDev {
   unsigned long long *bigq_n; // [0] triangles queued, [1] the second kernel's batch counter,
                               // then per band its entries and the places taken of them
   int64_t bigq_cap;
+};
+
+// and the second pass's order.
+struct MapDev : MapItems, MapCore {
   int64_t bigq_limit;         // the first pass takes no new work item beyond so many queued
   // a map too large for the L2: the second pass takes the queue by bands of
   // 2^band_shift map rows (-1: in queue order)

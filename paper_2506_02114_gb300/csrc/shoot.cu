@@ -27,7 +27,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // Record of the sub-cell of the active leaf containing finest-level cell
 // (cx, cy); -1 if none.
-__device__ __forceinline__ int lookup_leaf(const MapDev &M, int cx, int cy) {
+__device__ __forceinline__ int lookup_leaf(const MapCore &M, int cx, int cy) {
   int gx = (cx >> M.gshift) - M.gx0, gy = (cy >> M.gshift) - M.gy0;
   if (gx < 0 || gy < 0 || gx >= M.gw || gy >= M.gh) return -1;
   int e = __ldg(&M.grid[(int64_t)gy * M.gw + gx]);
@@ -52,7 +52,7 @@ __device__ __forceinline__ int lookup_leaf(const MapDev &M, int cx, int cy) {
 // row after j that may lie in other records: a grid entry that names a record
 // holds for every row of its grid row (the lanes' columns are fixed), so the
 // rows up to `j_same` need no lookup.  Rows up to je.
-__device__ __forceinline__ int lookup_rows(const MapDev &M, int cx, int j, int je, int lane,
+__device__ __forceinline__ int lookup_rows(const MapCore &M, int cx, int j, int je, int lane,
                                            bool vvalid, int &j_same, bool &c_cull) {
   const int cy = __ldg(&M.row_cell[j]);
   const int gy = (cy >> M.gshift) - M.gy0, gx = (cx >> M.gshift) - M.gx0;
@@ -150,7 +150,7 @@ __device__ __forceinline__ Vtx pixel_form(bool ok, float u, float v, int Ui, int
 // Source-plane position of grid point (i + ti, j + tj) in pixel units:
 // returns the integer pixel and the fraction.  ti = tj = 0 for ray vertices.
 template <bool SQUARE, bool FRAC, int G = 3>
-__device__ __forceinline__ Vtx shoot_point(const MapDev &M, int leaf, int i, int j,
+__device__ __forceinline__ Vtx shoot_point(const MapCore &M, int leaf, int i, int j,
                                            float ti, float tj, bool valid) {
   const int4 *rp = reinterpret_cast<const int4 *>(M.leaf + (leaf < 0 ? 0 : leaf));
   int4 q0 = __ldg(rp), q1 = __ldg(rp + 1), q2 = __ldg(rp + 2), q3 = __ldg(rp + 3);
@@ -240,7 +240,7 @@ __device__ __forceinline__ Vtx shoot_point(const MapDev &M, int leaf, int i, int
 // x distance is formed once, and most of the rest issues one instruction for
 // both rows (k_shoot_irs on the 1537^2 map 3.28 -> 2.64 ms).
 template <bool SQUARE, int G>
-__device__ __forceinline__ void shoot_rows2(const MapDev &M, int leaf, int i, int j, bool valid,
+__device__ __forceinline__ void shoot_rows2(const MapCore &M, int leaf, int i, int j, bool valid,
                                             Vtx &out0, Vtx &out1) {
   const int4 *rp = reinterpret_cast<const int4 *>(M.leaf + (leaf < 0 ? 0 : leaf));
   const int4 q0 = __ldg(rp), q1 = __ldg(rp + 1), q2 = __ldg(rp + 2), q3 = __ldg(rp + 3);
@@ -308,7 +308,7 @@ __device__ __forceinline__ void shoot_rows2(const MapDev &M, int leaf, int i, in
 // culling radius of every direct star (a star above is approached by one
 // row per row; one below or level only recedes).
 template <bool SQUARE>
-__device__ __forceinline__ int vertex_cull_side(const MapDev &M, int leaf, int i, int j,
+__device__ __forceinline__ int vertex_cull_side(const MapCore &M, int leaf, int i, int j,
                                                 int &run) {
   run = 0;
   if (leaf < 0) return MM_CULL_NONE;
@@ -342,7 +342,7 @@ __device__ __forceinline__ int vertex_cull_side(const MapDev &M, int leaf, int i
 // (lanes without a vertex agree with anything), and the rows from j on the
 // proof holds for in every lane; MM_CULL_NONE otherwise.
 template <bool SQUARE>
-__device__ __forceinline__ int row_cull_side(const MapDev &M, int leaf, int i, int j,
+__device__ __forceinline__ int row_cull_side(const MapCore &M, int leaf, int i, int j,
                                              bool vvalid, int &run) {
   int r = 1 << 30;
   const int s = vvalid ? vertex_cull_side<SQUARE>(M, leaf, i, j, r) : -1;
@@ -353,9 +353,8 @@ __device__ __forceinline__ int row_cull_side(const MapDev &M, int leaf, int i, i
 
 // Persistent warps; each work item is a strip of 31 cell columns by
 // rows_per_item cell rows of one map.  Lane l computes vertex column
-// 31*s + l for every vertex row of the item, keeps the previous row in
-// registers and takes its right neighbour's vertices by shuffle; lanes 0..30
-// then map cells (i, j-1) as the triangles {v00, v10, v11} and
+// 31*s + l for every vertex row of the item; the row below and the right
+// neighbour's vertices wait in shared memory; lanes 0..30 then map cells (i, j-1) as the triangles {v00, v10, v11} and
 // {v00, v11, v01} (diagonal from lower-left to upper-right).
 // Issue- and latency-bound (no pipe saturated): the kernel is shaped to run 3
 // blocks of 8 warps per SM, 80 registers a thread without spills -- the row
@@ -367,7 +366,8 @@ __device__ __forceinline__ int row_cull_side(const MapDev &M, int leaf, int i, i
 // 2000^2 map, 9 rays per pixel: 16.9 ms at 2 blocks with the apportioning in
 // divergent branches, 15.3 ms with the queues at 2 blocks, 13.0 ms at 3 (4
 // spill and are slower), 11.9 ms with rows shot in pairs, one lookup for up
-// to 33 rows and outcodes in place of box tests.
+// to 33 rows and outcodes in place of box tests, 11.5 with a larger L1
+// (WarpSmem).
 #ifndef MM_SHOOT_MINB
 #define MM_SHOOT_MINB 3  // resident 256-thread blocks per SM the register budget targets
 #endif
@@ -391,8 +391,11 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
   // parameter's, which leaves the registers to the per-ray work (reading
   // them from the descriptor array in global memory costs registers, and
   // spills, that the single-map kernel never pays).
-  __shared__ MapDev s_md[8];
-  MapDev &SM = s_md[threadIdx.x >> 5];
+  static_assert(MM_SHOOT_MINB != 3 ||
+                    3 * (MM_SHOOT_SMEM_BYTES + 8 * sizeof(MapCore) + 64 + 1024) <= 196 * 1024,
+                "a step of shared memory taken from the L1");
+  __shared__ MapCore s_md[BATCH ? 8 : 1];
+  MapCore &SM = s_md[BATCH ? threadIdx.x >> 5 : 0];
   while (true) {
     // (a single map whose larger triangles may exceed its queue stops at the
     // limit; its next launch goes on where this one stopped)
@@ -418,21 +421,23 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     if (BATCH && mi != last_map) {  // warp-uniform
       if (last_map >= 0) counts_flush(SM, ws, lc, lane);
       __syncwarp();
-      const unsigned long long *src = reinterpret_cast<const unsigned long long *>(maps + mi);
+      const unsigned long long *src = reinterpret_cast<const unsigned long long *>(
+          static_cast<const MapCore *>(maps + mi));
       unsigned long long *dst = reinterpret_cast<unsigned long long *>(&SM);
-      for (int k = lane; k < (int)(sizeof(MapDev) / 8); k += 32) dst[k] = src[k];
+      if (lane < (int)(sizeof(MapCore) / 8)) dst[lane] = src[lane];
       __syncwarp();
       last_map = mi;
     }
     if (!BATCH) last_map = 0;
-    const MapDev &M = BATCH ? SM : M1;
-    const int64_t local = (int64_t)w - M.work_begin;
-    const int64_t s = local % M.strips, b = (local / M.strips) * M.item_stride;
+    const MapCore &M = BATCH ? SM : static_cast<const MapCore &>(M1);
+    const MapItems &I = BATCH ? maps[mi] : M1;
+    const int64_t local = (int64_t)w - I.work_begin;
+    const int64_t s = local % I.strips, b = (local / I.strips) * I.item_stride;
     // grid indices fit 32 bits (at most 2^31 - 1 rays per axis)
-    const int i = (int)(M.col_begin + s * MM_STRIP) + lane;
-    const int jb = (int)(M.row_begin + b * M.rows_per_item);
-    const int je = (int)min((int64_t)jb + M.rows_per_item, M.row_end);
-    const int col_end = (int)M.col_end;
+    const int i = (int)(I.col_begin + s * MM_STRIP) + lane;
+    const int jb = (int)(I.row_begin + b * I.rows_per_item);
+    const int je = (int)min((int64_t)jb + I.rows_per_item, I.row_end);
+    const int col_end = (int)I.col_end;
     const bool vvalid = i <= col_end;  // vertex columns [col_begin, col_end]
     const int cx = __ldg(&M.col_cell[vvalid ? i : col_end]);
     const bool cell_col = (lane < MM_STRIP) && (i < col_end);
@@ -552,7 +557,7 @@ __global__ void __launch_bounds__(256, MM_SHOOT_MINB)
     }
     run_flush<MM_FIX_ONE>(M, ra);
   }
-  if (last_map >= 0) counts_flush(BATCH ? SM : M1, ws, lc, lane);
+  if (last_map >= 0) counts_flush(BATCH ? SM : static_cast<const MapCore &>(M1), ws, lc, lane);
 }
 
 // Inverse ray shooting (Sec. 3.2; the IRS column of Table 1): every grid
@@ -659,7 +664,7 @@ __global__ void __launch_bounds__(256, MM_IRS_MINB)
 #define MM_BIG_MINB 5
 
 // Queued triangles that found a slot.
-__device__ __forceinline__ long long queued(const MapDev &M) {
+__device__ __forceinline__ long long queued(const MapCore &M) {
   const unsigned long long cap = (unsigned long long)M.bigq_cap, qn = *M.bigq_n;
   return (long long)(qn < cap ? qn : cap);
 }
@@ -674,7 +679,7 @@ __device__ __forceinline__ int2 band_range(const MapDev &M, const RawTri &t) {
 }
 // s_end[k]: entries of bands 0 .. k.  False: more than there is room for (then
 // the queue is taken in its own order).  Call with all threads of the block.
-__device__ __forceinline__ bool band_ends(const MapDev &M, unsigned long long *s_end) {
+__device__ __forceinline__ bool band_ends(const MapCore &M, unsigned long long *s_end) {
   if (threadIdx.x < MM_BANDS) {
     unsigned long long n = 0;
     for (int k = 0; k <= threadIdx.x; k++) n += M.bigq_n[2 + k];
@@ -926,7 +931,8 @@ struct BatchGather {
   int64_t work_begin[MM_GATHER_MAX];
   int n;
 };
-static_assert(sizeof(MapDev) % 8 == 0, "MapDev copied in 8-byte words");
+static_assert(sizeof(MapDev) % 8 == 0 && sizeof(MapCore) % 8 == 0 && sizeof(MapCore) <= 256,
+              "copied in 8-byte words, the core's one a lane");
 
 __global__ void k_batch_gather(const BatchGather g, MapDev *dst) {
   const int i = blockIdx.x;
