@@ -842,8 +842,11 @@ static mm_status alloc_map_buffers(mm_map *h) {
   // lie in several.  A map that cannot be cut so has no queue: the first pass
   // deals every larger triangle where it finds it.  Default size: the larger
   // triangles the autotuner's sampled runs counted, with a quarter to spare,
-  // else est_jobs' share of the cells; 2^16 .. 2^27 slots (32 B each, and 10 B
-  // more with bands).  When that much device memory is not to be had, 2^20
+  // else est_jobs' share of the cells and at least two a cell or 32 a pixel,
+  // whichever is less (0.5 to 47 a pixel measured; with few rays per pixel one
+  // cell in 12 is too few: 400^2 map, 14 % of the cells, 0.71 + 0.20 ms for the
+  // two passes with one in 12, 0.20 + 0.34 with these); 2^16 .. 2^27 slots (32 B
+  // each, and 10 B more with bands).  When that much device memory is not to be had, 2^20
   // slots, then none (with bands none, also when it would take more than an
   // eighth of the free memory).  Batches that do not fit are dealt out by the
   // first kernel.  A queue of less than 2^22 slots is not taken by bands: a
@@ -867,6 +870,8 @@ static mm_status alloc_map_buffers(mm_map *h) {
     const int32_t want = h->mode == MM_FMM_IRS ? -1 : h->opt.big_queue_slots;
     const int64_t est = est_jobs(h, cells);
     int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;
+    if (h->jobs_pm < 0)
+      slots = std::max(slots, std::min(2 * cells, 32 * (int64_t)h->P.npix * h->P.npix_y));
     slots = want > 0 ? want
                      : std::min<int64_t>(int64_t(1) << 27,
                                          std::max<int64_t>(int64_t(1) << 16, slots));
