@@ -689,7 +689,10 @@ __device__ __forceinline__ bool band_ends(const MapCore &M, unsigned long long *
   return s_end[MM_BANDS - 1] <= MM_BAND_ENTRIES * (unsigned long long)M.bigq_cap;
 }
 
-template <bool BANDED>
+// SMALL: a queue that gives its warps less than two batches of 32 is dealt in
+// batches of 16 .. 4: a batch's rows are a chain of rounds (48^2 map, 13 000
+// triangles: 23 -> 12 us).
+template <bool BANDED, bool SMALL>
 __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
   __shared__ TriJob q[8][32];
   __shared__ RowRecs rr[8];
@@ -697,13 +700,16 @@ __global__ void __launch_bounds__(256, MM_BIG_MINB) k_big_ipm(const MapDev M) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool sorted = BANDED && band_ends(M, s_end);
   const long long n = sorted ? (long long)s_end[BANDED ? MM_BANDS - 1 : 0] : queued(M);
+  int log_size = 5;
+  if (SMALL)
+    while (log_size > 2 && (n >> (log_size + 1)) < gridDim.x * 8) log_size--;
   while (true) {
     unsigned long long b = 0;
     if (lane == 0) b = atomicAdd(M.bigq_n + 1, 1ull);
     b = __shfl_sync(0xffffffffu, b, 0);
-    const long long base = (long long)b * 32;
+    const long long base = (long long)b << log_size;
     if (base >= n) break;
-    const int nb = (int)min(32ll, n - base);
+    const int nb = (int)min(1ll << log_size, n - base);
     int row_lo = 0, row_hi = M.npix_y;
     if (lane < nb) {
       const long long slot = sorted ? (long long)M.bigq_order[base + lane] : base + lane;
@@ -980,13 +986,17 @@ cudaError_t launch_big_ipm(const MapDev &m, int &launches, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int grid = sms * MM_BIG_MINB;
   if (m.band_shift >= 0) {
     k_band_count<<<sms * 8, 256, 0, st>>>(m);
     k_band_scatter<<<sms * 8, 256, 0, st>>>(m);
-    k_big_ipm<true><<<sms * MM_BIG_MINB, 256, 0, st>>>(m);
+    k_big_ipm<true, false><<<grid, 256, 0, st>>>(m);
     launches += 3;
+  } else if (m.bigq_cap < 64 * 8 * (int64_t)grid) {
+    k_big_ipm<false, true><<<grid, 256, 0, st>>>(m);
+    launches++;
   } else {
-    k_big_ipm<false><<<sms * MM_BIG_MINB, 256, 0, st>>>(m);
+    k_big_ipm<false, false><<<grid, 256, 0, st>>>(m);
     launches++;
   }
   return cudaGetLastError();

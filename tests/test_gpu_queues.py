@@ -129,3 +129,29 @@ def test_bands_of_a_large_map_do_not_change_it(shape, grid, gamma, slots, mode):
                 assert np.array_equal(ref, got) and c == counts
             mm.destroy(other)
         mm.destroy(h)
+
+
+@pytest.mark.parametrize("cols,rows", [(1, 3), (60, 200), (300, 900), (700, 2400), (1200, 4000),
+                                       (1200, 9000)])
+@pytest.mark.parametrize("model", sorted(MODELS))
+def test_short_items_and_small_batches_leave_the_map_unchanged(model, cols, rows):
+    """Small grids: work items of 8 to 64 rows, a second pass in batches of 4 to
+    32 triangles, and with few rays per pixel a queue sized by the pixels: the
+    map of long items without a queue, bit for bit."""
+    import torch
+    torch.cuda.init()
+    kappa, gamma, s, _ = MODELS[model]
+    m, pos = synthetic.star_field(14, 60, 14.0, synthetic.SALPETER_01_1)
+    maps, counts = [], []
+    for opts in (dict(rows_per_item=256, big_queue_slots=-1), dict(), dict(big_queue_slots=5000)):
+        h = mm.create(kappa, gamma, s, m, pos, 1.5, 150, fmm_order=20, img_half=(6.0, 3.0),
+                      ray_grid=(cols + 1, rows + 1), **opts)
+        mm.run(h, 0)
+        st = mm.get_stats(h)
+        assert st["error_bits"] == 0
+        maps.append(mm.get_map_fixed(h))
+        counts.append([st[k] for k in st if k.startswith("triangles_")])
+        mm.destroy(h)
+    assert maps[0].any()
+    for k in (1, 2):
+        assert np.array_equal(maps[0], maps[k]) and counts[0] == counts[k]
