@@ -40,6 +40,7 @@ using namespace mm;
 // ---------------------------------------------------------------------------
 
 static thread_local std::string g_err;
+thread_local int LaunchApart::depth = 0;
 
 static mm_status fail(mm_status s, const char *fmt, ...) {
   char buf[512];
@@ -1068,6 +1069,7 @@ static mm_status create_impl(mm_map *h, double kappa_tot, double shear, double s
                              int64_t n_stars, const double *masses, const double *pos_xy,
                              double half_length, int32_t npix, double rays_per_pixel,
                              int32_t fmm_order, int32_t leaf_size) {
+  const LaunchApart apart;
   mm_params &P = h->P;
   CKS(derive(kappa_tot, shear, smooth_fraction, n_stars, masses, half_length, npix,
              rays_per_pixel, h->opt, P));
@@ -1517,6 +1519,7 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     if (hs[i]->timed_out) return fail(MM_ESTATE, "handle %d timed out earlier", i);
   }
   CK(cudaSetDevice(hs[0]->device));
+  const LaunchApart apart;
   mm_map *lead = hs[0];
   // the lead's fan-out streams (created by its first batch call)
   const int nfan = std::min<int>(n, MM_BATCH_STREAMS);

@@ -111,6 +111,7 @@ __device__ __forceinline__ double2 power_of(const double2 *sq, int k) {
 __global__ void __launch_bounds__(MM_P2M_THREADS)
     k_p2m(TreeDev T, int64_t n_nodes, int p, int per_block, const double *__restrict__ inv,
           double2 *mp) {
+  grid_begin();
   extern __shared__ __align__(16) double2 s_p2m[];
   const int P1 = p + 1;
   // per node and staged star: the squares, then the mass
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(MM_P2M_THREADS)
 // ---------------------------------------------------------------------------
 __global__ void k_m2m(TreeDev T, int level, int64_t n, int p, int per_block,
                       const double2 *__restrict__ MMop, double2 *mp) {
+  grid_begin();
   extern __shared__ __align__(16) double2 s_m2m[];
   const int P1 = p + 1, half = (p + 1) / 2;
   double2 *a = s_m2m, *t = s_m2m + per_block * 4 * P1;  // [node][child][k]
@@ -275,6 +277,7 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
     k_local(TreeDev T, int level, int64_t n, int p, const int32_t *node_act,
             const double2 *__restrict__ MLop, const double2 *__restrict__ LLop,
             const double2 *__restrict__ mp, double2 *loc, unsigned *err) {
+  grid_begin();
   extern __shared__ __align__(16) double2 s_loc[];
   __shared__ LocalSources S;
   const int64_t node = T.level_off[level] + blockIdx.x;
@@ -556,6 +559,7 @@ __device__ __forceinline__ int count_direct(const TreeDev &T, const FmmConst &C,
 __global__ void __launch_bounds__(MM_REC_THREADS)
     k_near_count(TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list,
                  unsigned *total, unsigned *err) {
+  grid_begin();
   __shared__ NearRanges N;
   const int n_leaf_max = MM_REC >> (2 * C.sub);
   const int64_t g0 = (int64_t)blockIdx.x * MM_REC, first_leaf = g0 >> (2 * C.sub);
@@ -586,6 +590,7 @@ __device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
 // FP64 and FP32, [k][q], and the binomials C(n + m, n) in FP32, [n][m]: what
 // every re-centring of a plan shares.
 __global__ void k_sub_tables(int sub, int p, double2 *up, float2 *fp, float *bin) {
+  grid_begin();
   const int ns = 1 << sub, NS = ns * ns, t = threadIdx.x;
   if (t < NS) {
     const double ux = (double)(2 * (t & (ns - 1)) + 1 - ns) / ns;
@@ -689,6 +694,7 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list, SubTables tb,
     const double2 *__restrict__ loc, LeafRec *leaf, NearPos *near_pos, float *near_m,
     float2 *coef, unsigned *near_total, unsigned near_cap, unsigned *err) {
+  grid_begin();
   extern __shared__ __align__(16) unsigned char s_rec[];
   RecSmem<NB> &S = *reinterpret_cast<RecSmem<NB> *>(s_rec);
   const int p = C.p, P1 = p + 1, pe = min(C.p_eval, NB), cs = coef_stride(pe);
@@ -1143,7 +1149,7 @@ cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *
   const size_t smem = (size_t)per_block * MM_P2M_STARS *
                       (MM_POW_BITS * sizeof(double2) + sizeof(double));
   // (the head of MLop holds 1/k)
-  k_p2m<<<blocks_for(n_nodes, per_block), MM_P2M_THREADS, smem, st>>>(
+  launch_next(k_p2m, blocks_for(n_nodes, per_block), MM_P2M_THREADS, smem, st,
       T, n_nodes, p, per_block, reinterpret_cast<const double *>(MLop), mp);
   return cudaGetLastError();
 }
@@ -1158,7 +1164,7 @@ cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const doub
   while (per_block > 1 && n < 304 * (int64_t)per_block) per_block >>= 1;
   const int threads = 32 * ((per_block * 4 * ((p + 1) / 2) + 31) / 32);
   const size_t smem = sizeof(double2) * 2 * per_block * 4 * (size_t)(p + 1);
-  k_m2m<<<blocks_for(n, per_block), threads, smem, st>>>(T, level, n, p, per_block, MMop, mp);
+  launch_next(k_m2m, blocks_for(n, per_block), threads, smem, st, T, level, n, p, per_block, MMop, mp);
   return cudaGetLastError();
 }
 
@@ -1177,7 +1183,7 @@ cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const in
   // nodes took 24 and 36 us in one part, 14 and 22 in four; above 3000 nodes
   // the pipe is busy anyway and a part costs 6 % more of it
   const unsigned parts = n <= 304 ? 4 : n <= 3000 ? 2 : 1;
-  k_local<<<dim3((unsigned)n, parts), MM_LOCAL_THREADS, smem, st>>>(T, level, n, p, node_act, MLop, LLop, mp,
+  launch_next(k_local, dim3((unsigned)n, parts), MM_LOCAL_THREADS, smem, st, T, level, n, p, node_act, MLop, LLop, mp,
                                                        loc, err);
   return cudaGetLastError();
 }
@@ -1187,13 +1193,13 @@ cudaError_t launch_near_count(const TreeDev &T, const FmmConst &C, int64_t n_act
                               cudaStream_t st) {
   if (n_active <= 0) return cudaSuccess;
   const int64_t n = n_active << (2 * C.sub);
-  k_near_count<<<blocks_for(n, MM_REC), MM_REC_THREADS, 0, st>>>(T, C, n, active_list, total, err);
+  launch_next(k_near_count, blocks_for(n, MM_REC), MM_REC_THREADS, 0, st, T, C, n, active_list, total, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sub_tables(int sub, int p, double2 *up, float2 *fp, float *bin,
                               cudaStream_t st) {
-  k_sub_tables<<<1, 128, 0, st>>>(sub, p, up, fp, bin);
+  launch_next(k_sub_tables, 1, 128, 0, st, sub, p, up, fp, bin);
   return cudaGetLastError();
 }
 
@@ -1212,7 +1218,7 @@ static cudaError_t launch_finalize_t(const TreeDev &T, const FmmConst &C, int64_
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_leaf_finalize<NB><<<blocks_for(n, MM_REC), MM_REC_THREADS, smem, st>>>(
+  launch_next(k_leaf_finalize<NB>, blocks_for(n, MM_REC), MM_REC_THREADS, smem, st,
       T, C, n, active_list, tb, loc, leaf, near_pos, near_m, coef, near_total, near_cap, err);
   return cudaGetLastError();
 }

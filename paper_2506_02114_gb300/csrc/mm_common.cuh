@@ -22,6 +22,14 @@
 
 namespace mm {
 
+// First thing in a kernel that launch_next launches: the stream's next kernel
+// may be set up from now on, and this one begins when the kernels before it
+// are complete and their writes visible.
+__device__ __forceinline__ void grid_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Error word bits written by kernels (read back by the host).
 enum : unsigned int {
   ERR_TREE_INVARIANT = 1u,    // a split node lacks a same-level neighbour

@@ -35,6 +35,7 @@ __device__ __forceinline__ int cell_of(double x, double R0) {
 
 __global__ void k_star_keys(const double *__restrict__ pos, int64_t n, double R0,
                             uint64_t *keys, int32_t *idx) {
+  grid_begin();
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   int cx = cell_of(pos[2 * t], R0), cy = cell_of(pos[2 * t + 1], R0);
@@ -45,6 +46,7 @@ __global__ void k_star_keys(const double *__restrict__ pos, int64_t n, double R0
 __global__ void k_gather_stars(const double *__restrict__ pos, const double *__restrict__ m,
                                const int32_t *__restrict__ idx, int64_t n, double *sx,
                                double *sy, double *sm) {
+  grid_begin();
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   int32_t k = idx[t];
@@ -112,6 +114,7 @@ __device__ __forceinline__ void write_child(const TreeDev &T, const TreeOut &O, 
 __global__ void __launch_bounds__(256) k_level_split(TreeDev T, TreeOut O, int level, int64_t n,
                                                      int limit, int32_t *split, int32_t *group,
                                                      int32_t *total) {
+  grid_begin();
   __shared__ int s_n[8];
   const int64_t t = (int64_t)blockIdx.x * MM_SPLIT_GROUP + (threadIdx.x >> 3);
   const int s = threadIdx.x & 7;
@@ -132,6 +135,7 @@ __global__ void __launch_bounds__(256) k_level_split(TreeDev T, TreeOut O, int l
 __global__ void __launch_bounds__(256) k_level_children(TreeDev T, TreeOut O, int level, int64_t n,
                                                         const int32_t *split,
                                                         const int32_t *group) {
+  grid_begin();
   __shared__ int s_w[8], s_base;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = threadIdx.x & 3;
   // split nodes of the groups before this block's
@@ -186,6 +190,7 @@ __device__ __forceinline__ int64_t warp_lower_bound(const uint64_t *a, int64_t l
 // The levels of at most MM_TOP_NODES nodes, one block.
 __global__ void __launch_bounds__(1024) k_tree_top(TreeDev T, TreeOut O, int limit,
                                                    int32_t *info) {
+  grid_begin();
   static_assert(MM_TOP_NODES <= 1024, "one thread per node");
   __shared__ int s_flag[MM_TOP_NODES], s_w[32], s_end[3 * MM_TOP_NODES];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -264,6 +269,7 @@ __global__ void __launch_bounds__(1024) k_tree_top(TreeDev T, TreeOut O, int lim
 // Finest-level cells of the vertex columns (first n0 threads) and rows.
 __global__ void k_axis_cells(double x0, double y0, double hx, double hy, int64_t n0, int64_t n1,
                              double R0, int32_t *col, int32_t *row) {
+  grid_begin();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n0)
     col[t] = cell_of(__dadd_rn(x0, __dmul_rn((double)t, hx)), R0);
@@ -275,6 +281,7 @@ __global__ void k_active_flags(TreeDev T, int64_t n_nodes, const int32_t *col_ce
                                int64_t col_lo, int64_t col_hi, const int32_t *row_cell,
                                int64_t row_lo, int64_t row_hi, int32_t *node_act,
                                int32_t *leaf_flag, int32_t *group) {
+  grid_begin();
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = t < n_nodes;
   if (!valid) t = n_nodes - 1;
@@ -301,6 +308,7 @@ __global__ void __launch_bounds__(256) k_compact_leaves(int64_t n_nodes, const i
                                                         const int32_t *group,
                                                         int32_t *node_active,
                                                         int32_t *active_list, int32_t *total) {
+  grid_begin();
   __shared__ int s_w[8], s_base;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int before = 0;
@@ -329,6 +337,7 @@ __global__ void __launch_bounds__(256) k_compact_leaves(int64_t n_nodes, const i
 // continues.
 __global__ void k_lookup_grid(TreeDev T, const int32_t *node_active, int glevel, int sub,
                               int gx0, int gy0, int gw, int gh, int32_t *grid) {
+  grid_begin();
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)gw * gh) return;
   const int gx = gx0 + (int)(t % gw), gy = gy0 + (int)(t / gw);
@@ -353,7 +362,7 @@ static inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b -
 cudaError_t launch_star_keys(const double *pos, int64_t n, double R0, uint64_t *keys,
                              int32_t *idx, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_star_keys<<<blocks_for(n, 256), 256, 0, st>>>(pos, n, R0, keys, idx);
+  launch_next(k_star_keys, blocks_for(n, 256), 256, 0, st, pos, n, R0, keys, idx);
   return cudaGetLastError();
 }
 
@@ -361,20 +370,20 @@ cudaError_t launch_gather_stars(const double *pos, const double *m, const int32_
                                 int64_t n, double *sx, double *sy, double *sm,
                                 cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_gather_stars<<<blocks_for(n, 256), 256, 0, st>>>(pos, m, idx, n, sx, sy, sm);
+  launch_next(k_gather_stars, blocks_for(n, 256), 256, 0, st, pos, m, idx, n, sx, sy, sm);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tree_top(const TreeDev &T, const TreeOut &O, int limit, int32_t *info,
                             cudaStream_t st) {
-  k_tree_top<<<1, 1024, 0, st>>>(T, O, limit, info);
+  launch_next(k_tree_top, 1, 1024, 0, st, T, O, limit, info);
   return cudaGetLastError();
 }
 
 cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, int64_t n, int limit,
                                int32_t *split, int32_t *group, int32_t *total, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_level_split<<<blocks_for(n, MM_SPLIT_GROUP), 256, 0, st>>>(T, O, level, n, limit, split, group,
+  launch_next(k_level_split, blocks_for(n, MM_SPLIT_GROUP), 256, 0, st, T, O, level, n, limit, split, group,
                                                                total);
   return cudaGetLastError();
 }
@@ -382,14 +391,14 @@ cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, in
 cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level, int64_t n,
                                   const int32_t *split, const int32_t *group, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_level_children<<<blocks_for(n, 64), 256, 0, st>>>(T, O, level, n, split, group);
+  launch_next(k_level_children, blocks_for(n, 64), 256, 0, st, T, O, level, n, split, group);
   return cudaGetLastError();
 }
 
 cudaError_t launch_axis_cells(double x0, double y0, double hx, double hy, int64_t n0, int64_t n1,
                               double R0, int32_t *col, int32_t *row, cudaStream_t st) {
   if (n0 + n1 <= 0) return cudaSuccess;
-  k_axis_cells<<<blocks_for(n0 + n1, 256), 256, 0, st>>>(x0, y0, hx, hy, n0, n1, R0, col, row);
+  launch_next(k_axis_cells, blocks_for(n0 + n1, 256), 256, 0, st, x0, y0, hx, hy, n0, n1, R0, col, row);
   return cudaGetLastError();
 }
 
@@ -398,7 +407,7 @@ cudaError_t launch_active_flags(const TreeDev &T, int64_t n_nodes, const int32_t
                                 int64_t row_lo, int64_t row_hi, int32_t *node_act,
                                 int32_t *leaf_flag, int32_t *group, cudaStream_t st) {
   if (n_nodes <= 0) return cudaSuccess;
-  k_active_flags<<<blocks_for(n_nodes, MM_ACTIVE_GROUP), MM_ACTIVE_GROUP, 0, st>>>(
+  launch_next(k_active_flags, blocks_for(n_nodes, MM_ACTIVE_GROUP), MM_ACTIVE_GROUP, 0, st,
       T, n_nodes, col_cell, col_lo, col_hi, row_cell, row_lo, row_hi, node_act, leaf_flag, group);
   return cudaGetLastError();
 }
@@ -408,7 +417,7 @@ cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag, con
                                   cudaStream_t st) {
   static_assert(MM_ACTIVE_GROUP == 256, "one thread per node of a group");
   if (n_nodes <= 0) return cudaSuccess;
-  k_compact_leaves<<<blocks_for(n_nodes, 256), 256, 0, st>>>(n_nodes, leaf_flag, group,
+  launch_next(k_compact_leaves, blocks_for(n_nodes, 256), 256, 0, st, n_nodes, leaf_flag, group,
                                                              node_active, active_list, total);
   return cudaGetLastError();
 }
@@ -418,7 +427,7 @@ cudaError_t launch_lookup_grid(const TreeDev &T, const int32_t *node_active, int
                                cudaStream_t st) {
   int64_t n = (int64_t)gw * gh;
   if (n <= 0) return cudaSuccess;
-  k_lookup_grid<<<blocks_for(n, 256), 256, 0, st>>>(T, node_active, glevel, sub, gx0, gy0, gw,
+  launch_next(k_lookup_grid, blocks_for(n, 256), 256, 0, st, T, node_active, glevel, sub, gx0, gy0, gw,
                                                     gh, grid);
   return cudaGetLastError();
 }
