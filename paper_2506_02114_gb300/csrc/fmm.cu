@@ -73,6 +73,12 @@ __device__ __forceinline__ double cfma_part(double2 a, double2 b, double c, bool
   return fma(a.x, im ? b.y : b.x, fma(flip(a.y, !im), im ? b.x : b.y, c));
 }
 
+// 0, 1, ..., MM_PMAX (a conversion is an FP64 instruction too).
+__constant__ double c_int[MM_PMAX + 1] = {
+    0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21,
+    22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38, 39, 40, 41, 42, 43,
+    44, 45, 46, 47, 48, 49, 50, 51, 52, 53, 54, 55, 56, 57, 58, 59, 60, 61, 62, 63, 64};
+
 // x / k, correctly rounded, from the rounded reciprocal of the small integer
 // k (Markstein's correction of the quotient by its exact remainder).
 __device__ __forceinline__ double div_by(double x, double k, double inv_k) {
@@ -101,66 +107,110 @@ __device__ __forceinline__ double2 power_of(const double2 *sq, int k) {
 
 // ---------------------------------------------------------------------------
 // P2M: a_0 = sum m_i, a_k = -(1/k) sum m_i zeta_i^k  (leaves only)
-// FP64-bound: one thread per (node, coefficient), so that the lanes stay full
-// whatever p; a star's repeated squares are formed once for all of its
-// powers.  50 000 stars, p = 25: 0.25 ms with a block per node and the
-// squares formed by every thread, 0.11 ms like this.
+// FP64-bound, a thread per (node, coefficient) and four lanes per star for its
+// powers: z^k is z^(k - 2^b) times the square z^(2^b), b the top digit of k,
+// one product a power and formed once for the node.  Stars staged side by side,
+// so that the four lanes of few stars fill warps, and nodes without stars take
+// no threads.  50 000 stars, p = 25: 0.25 ms with a block per node, 0.11 ms
+// with the powers formed by each (node, coefficient) from the squares, 0.06 ms
+// like this (64 us in blocks of 256 threads, 73 of 128, 61 of 512; two lanes a
+// star: 58, but 84 in place of 76 where most leaves hold none or one).
 // ---------------------------------------------------------------------------
-#define MM_P2M_THREADS 128
-#define MM_P2M_STARS 8  // stars of a node staged at a time
+#define MM_P2M_THREADS 256
+#define MM_P2M_STARS 4  // stars of a node staged at a time
+#define MM_P2M_LANES 4  // lanes that share a star's powers
 __global__ void __launch_bounds__(MM_P2M_THREADS)
     k_p2m(TreeDev T, int64_t n_nodes, int p, int per_block, const double *__restrict__ inv,
           double2 *mp) {
   grid_begin();
   extern __shared__ __align__(16) double2 s_p2m[];
   const int P1 = p + 1;
-  // per node and staged star: the squares, then the mass
-  double2 *sq = s_p2m;
-  double *sm = reinterpret_cast<double *>(sq + per_block * MM_P2M_STARS * MM_POW_BITS);
+  // per staged star: z^0 (unused) .. z^p, then the masses
+  double2 *zs = s_p2m;
+  double *sm = reinterpret_cast<double *>(zs + per_block * MM_P2M_STARS * P1);
+  __shared__ int s_node[32], s_beg[32], s_cnt[32], s_off[33];  // the block's nodes with stars
   const int64_t first = (int64_t)blockIdx.x * per_block;
-  const int local = threadIdx.x / P1, k = threadIdx.x - local * P1;
-  const int64_t node = first + local;
-  const bool mine = local < per_block && node < n_nodes && T.first_child[node] < 0;
-  const int b = mine ? T.sbeg[node] : 0, e = mine ? T.send[node] : 0;
-  // the block's longest node
-  int longest = 0;
-  for (int q = 0; q < per_block; q++) {
-    const int64_t nd = first + q;
-    if (nd < n_nodes && T.first_child[nd] < 0) longest = max(longest, T.send[nd] - T.sbeg[nd]);
+  if (threadIdx.x < 32) {
+    const int64_t nd = first + threadIdx.x;
+    const bool leaf = threadIdx.x < per_block && nd < n_nodes && T.first_child[nd] < 0;
+    const int beg = leaf ? T.sbeg[nd] : 0, cnt = leaf ? T.send[nd] - beg : 0;
+    const unsigned with = __ballot_sync(0xffffffffu, cnt > 0);
+    s_cnt[threadIdx.x] = 0;
+    __syncwarp();
+    if (cnt > 0) {
+      const int o = __popc(with & ((1u << threadIdx.x) - 1u));
+      s_node[o] = threadIdx.x;
+      s_beg[o] = beg;
+      s_cnt[o] = cnt;
+    }
   }
+  __syncthreads();
+  const int local = threadIdx.x / P1, k = threadIdx.x - local * P1;
+  const bool mine = local < per_block && s_cnt[local] > 0;
+  const int64_t node = first + (mine ? s_node[local] : 0);
   double2 s = make_double2(0.0, 0.0);
-  for (int c = 0; c < longest; c += MM_P2M_STARS) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < per_block * MM_P2M_STARS; t += MM_P2M_THREADS) {
-      const int64_t nd = first + t / MM_P2M_STARS;
-      if (nd >= n_nodes || T.first_child[nd] >= 0) continue;
-      const int i = T.sbeg[nd] + c + t % MM_P2M_STARS;
-      if (i >= T.send[nd]) continue;
-      int level, cx, cy;
-      double zx, zy, L;
-      node_geom(T, nd, level, cx, cy, zx, zy, L);
-      const double invL = inv_pow2(L);
-      powers_of_two(make_double2((T.sx[i] - zx) * invL, (T.sy[i] - zy) * invL), p,
-                    sq + t * MM_POW_BITS);
-      sm[t] = T.sm[i];
+  for (int c = 0;; c += MM_P2M_STARS) {
+    // the next stars of each node, the nodes' one after another
+    if (threadIdx.x < 32) {
+      int n = min(max(s_cnt[threadIdx.x] - c, 0), MM_P2M_STARS);
+      for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, n, d);
+        if (threadIdx.x >= d) n += u;
+      }
+      if (threadIdx.x == 0) s_off[0] = 0;
+      s_off[threadIdx.x + 1] = n;
     }
     __syncthreads();
-    const int cnt = min(MM_P2M_STARS, e - b - c);
-    for (int i = 0; i < cnt; i++) {
-      const int t = local * MM_P2M_STARS + i;
-      const double m = sm[t];
+    const int staged = s_off[32];
+    if (staged == 0) break;
+    const int r = threadIdx.x % MM_P2M_LANES;
+    for (int base = 0; base < staged; base += MM_P2M_THREADS / MM_P2M_LANES) {
+      const int t = base + threadIdx.x / MM_P2M_LANES;
+      if (base + (int)(threadIdx.x & ~31u) / MM_P2M_LANES >= staged) break;  // (warp-uniform)
+      double2 sq = make_double2(0.0, 0.0);
+      if (t < staged) {
+        int q = 0;
+        for (int step = 16; step > 0; step >>= 1)
+          if (s_off[q + step] <= t) q += step;
+        const int i = s_beg[q] + c + t - s_off[q];
+        int level, cx, cy;
+        double zx, zy, L;
+        node_geom(T, first + s_node[q], level, cx, cy, zx, zy, L);
+        const double invL = inv_pow2(L);
+        sq = make_double2((T.sx[i] - zx) * invL, (T.sy[i] - zy) * invL);
+        if (r == 0) {
+          if (p > 0) zs[t * P1 + 1] = sq;
+          sm[t] = T.sm[i];
+        }
+      }
+      for (int top = 2; top <= p; top *= 2) {
+        __syncwarp();
+        sq = cmul(sq, sq);
+        if (t < staged) {
+          if (r == 0) zs[t * P1 + top] = sq;
+          for (int j = 1 + r; j < top && top + j <= p; j += MM_P2M_LANES)
+            zs[t * P1 + top + j] = cmul(zs[t * P1 + j], sq);
+        }
+      }
+    }
+    __syncthreads();
+    const int cnt = mine ? min(MM_P2M_STARS, s_cnt[local] - c) : 0;
+    const int at = mine ? s_off[local] : 0;
+    for (int i = at; i < at + cnt; i++) {
+      const double m = sm[i];
       if (k == 0) {
         s.x += m;
       } else {
-        const double2 zk = power_of(sq + t * MM_POW_BITS, k);
+        const double2 zk = zs[i * P1 + k];
         s.x = fma(m, zk.x, s.x);
         s.y = fma(m, zk.y, s.y);
       }
     }
+    __syncthreads();  // (the next stars take these places)
   }
-  if (!mine || b == e) return;  // (a node without stars is nobody's source)
+  if (!mine) return;  // (a node without stars is nobody's source)
   if (k > 0) {
-    const double dk = (double)k, ik = inv[k];
+    const double dk = c_int[k], ik = inv[k];
     s = make_double2(div_by(-s.x, dk, ik), div_by(-s.y, dk, ik));
   }
   mp[node * P1 + k] = s;
@@ -640,11 +690,6 @@ __device__ __forceinline__ float div_by_f(float x, float n, float inv_n) {
 // part two further): pairs are stored real parts first.
 __device__ __forceinline__ int coef_slot(int k) { return 4 * (k >> 1) + (k & 1); }
 
-// 0, 1, ..., MM_PMAX (a conversion is an FP64 instruction too).
-__constant__ double c_int[MM_PMAX + 1] = {
-    0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21,
-    22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38, 39, 40, 41, 42, 43,
-    44, 45, 46, 47, 48, 49, 50, 51, 52, 53, 54, 55, 56, 57, 58, 59, 60, 61, 62, 63, 64};
 
 // Shared memory of k_leaf_finalize<NB>.
 template <int NB>
@@ -1145,9 +1190,9 @@ static inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b -
 cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *MLop, double2 *mp,
                        cudaStream_t st) {
   if (n_nodes <= 0) return cudaSuccess;
-  const int per_block = std::min(32, MM_P2M_THREADS / (p + 1));  // (32: staged stars fit 48 KB)
+  const int per_block = std::min(32, MM_P2M_THREADS / (p + 1));
   const size_t smem = (size_t)per_block * MM_P2M_STARS *
-                      (MM_POW_BITS * sizeof(double2) + sizeof(double));
+                      ((p + 1) * sizeof(double2) + sizeof(double));
   // (the head of MLop holds 1/k)
   launch_next(k_p2m, blocks_for(n_nodes, per_block), MM_P2M_THREADS, smem, st,
       T, n_nodes, p, per_block, reinterpret_cast<const double *>(MLop), mp);
