@@ -110,8 +110,10 @@ typedef struct {
                                2^16 .. 2^27 (2^20, then none, when the device has not
                                that much memory free).  A map whose
                                accumulators (16 B per pixel) exceed half the
-                               GPU's L2: else 2 per cell, at most 64 per pixel;
-                               none below 2^22 or beyond 1/8 of the memory free.
+                               GPU's L2: else 2 per cell, at most the most of 1
+                               per 5 cells and 64 per pixel; none below 2^22 or
+                               beyond 1/8 of the memory free, or with
+                               kappa_star < 0.001.
                                -1 -> none (the first pass deals every larger
                                triangle); n > 0 -> n.  When the expected larger
                                triangles exceed it the first pass runs in

@@ -801,12 +801,13 @@ static double map_scale(const mm_map *h) {
 
 // Larger triangles (queued for the second pass) expected from `cells` cells:
 // the autotuner's count scaled to them, else one per 12 cells.  On a map taken
-// by bands all of them, at most 64 a pixel (measured 4.5 to 47): a triangle
-// that finds no slot is dealt out where its lines miss the L2, and a segment
-// too many costs 0.03 ms.
+// by bands the most of one per 5 cells (near the critical line) and 64 a pixel
+// (few rays a pixel), no more than there are: a triangle that finds no slot is
+// dealt out where its lines miss the L2, and a segment too many costs 0.03 ms.
 static int64_t est_jobs(const mm_map *h, int64_t cells) {
   if (h->jobs_pm >= 0) return (int64_t)std::ceil((double)cells * h->jobs_pm / 1048576.0);
-  if (h->band_shift >= 0) return std::min(2 * cells, 64 * (int64_t)h->P.npix * h->P.npix_y);
+  if (h->band_shift >= 0)
+    return std::min(2 * cells, std::max(cells / 5, 64 * (int64_t)h->P.npix * h->P.npix_y));
   return cells / 12;
 }
 
@@ -858,11 +859,14 @@ static mm_status alloc_map_buffers(mm_map *h) {
   // first kernel.  A queue of less than 2^22 slots is not taken by bands: a
   // segment's launches and its last items would cost more than the order gains.
   // Measured, no queue -> by bands: 3001^2 near the critical line 128 -> 96 ms,
-  // 5000^2 456 -> 172, 5000^2 far from it 128 -> 116, 2060^2 30.7 -> 24.5, a
-  // quarter of the rays 33 -> 24 (3000^2); with 6 cells a pixel 51 -> 32 and, the
-  // only loss found, 9.4 -> 10.8.  2^26 / 2^27 / 2^28 slots: 99 / 97 / 96 ms and,
-  // on the second 5000^2 map, 141 / 130 / 127 (before triangles were cut at the
-  // bands).
+  // 5000^2 1557 -> 665 (1500 cells a pixel), 5000^2 and 10000^2 far from it
+  // 128 -> 110 and 656 -> 470, 2060^2 30.7 -> 24.5, a quarter of the rays 33 ->
+  // 24 (3000^2), 6 cells a pixel 51 -> 32 and 9.4 -> 10.8; by kappa_star (4000^2)
+  // 168 -> 119 at 0.25, 71 -> 58 at 0.05, 52 -> 44 at 0.01.  Next to no stars
+  // (3e-5, 10000 x 1000): 70 -> 125 ms, the macro model maps neighbours onto the
+  // same few pixels and every triangle is a larger one, so below 1e-3 no bands.
+  // 2^26 / 2^27 / 2^28 slots: 99 / 97 / 96 ms and, on the second 5000^2 map,
+  // 141 / 130 / 127 (before triangles were cut at the bands).
   {
     const int64_t cells = (h->col_hi - h->col_lo) * (h->row_hi - h->row_lo);
     int l2 = 0;
@@ -872,7 +876,10 @@ static mm_status alloc_map_buffers(mm_map *h) {
     int shift = 5;
     while (((h->P.npix_y - 1) >> shift) >= MM_BANDS) shift++;
     while (shift < 30 && std::ldexp(row_bytes, shift + 1) <= 16.0 * (1 << 20)) shift++;
-    h->band_shift = !fits_l2 && std::ldexp(row_bytes, shift) <= 0.25 * (double)l2 ? shift : -1;
+    h->band_shift = !fits_l2 && std::ldexp(row_bytes, shift) <= 0.25 * (double)l2 &&
+                            h->P.kappa_star >= 1e-3
+                        ? shift
+                        : -1;
     const int32_t want = h->mode == MM_FMM_IRS ? -1 : h->opt.big_queue_slots;
     const int64_t est = est_jobs(h, cells);
     int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;

@@ -80,7 +80,7 @@ struct __align__(16) Vtx {
 
 struct RawTri;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
 #define MM_TRIJOB_BYTES 32
-#define MM_BANDS 64           // row bands of the second pass at most
+#define MM_BANDS 128          // row bands of the second pass at most
 #define MM_BIGQ_COUNTERS (2 + 2 * MM_BANDS)
 #define MM_BAND_ENTRIES 2     // room in bigq_order for so many entries a slot
 

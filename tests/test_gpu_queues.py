@@ -73,7 +73,7 @@ def test_stored_vertices_map_like_the_oracle(oracle_mod, cols, rows):
 @pytest.mark.parametrize("shape,grid,gamma,slots", [
     ((2200, 2200), (350, 300), 0.3, (0, 1000, 1 << 22)),  # too few cells for a queue by default
     ((2200, 2200), (3400, 3300), 0.3, (0, 1 << 22)),      # 2^22 slots: several first passes
-    ((60, 110000), (200, 900), 0.3, (1 << 22,)),          # 64 bands at most, of tall strips
+    ((60, 110000), (200, 900), 0.3, (1 << 22,)),          # over a hundred bands of a narrow map
     ((30000, 300), (900, 200), 0.3, (1 << 22,)),          # 32 rows a band, triangles over many
     ((2200, 2200), (2500000, 3), -0.3, (1 << 22,)),       # more bands a triangle than there is room
 ])
