@@ -64,13 +64,13 @@ TUNE_CACHE = os.path.join(ROOT, "paper_2506_02114_gb300", "tune", "sm_103.jsonl"
 # (profiles/counters_fmm_fp32_salpeter_2000_rpp1.md): valid only for the kernel
 # sources they were taken on (hash below), reported beside the live roofline.
 NCU_COUNTERS = {
-    "sources_sha1": "5517307e56512defd1c015340608c52b0e4ab670",
+    "sources_sha1": "80cfb1b8280ba260da4a0304e21ea6bba0d63497",
     "case": "fmm_fp32_salpeter_2000 at 1 ray per pixel (1.64e8 rays), ncu --clock-control none",
-    "k_shoot_ipm": {"issue_active": 0.633, "warps_active": 0.194, "alu_active": 0.505,
-                    "fma_active": 0.191, "l2_red_requests_per_s": 4.10e10},
-    "k_big_ipm": {"issue_active": 0.803, "warps_active": 0.548, "alu_active": 0.630,
-                  "fma_active": 0.299, "l2_red_requests_per_s": 9.63e10},
-    "k_direct64_vertices": {"fp64_pipe_active": 0.907},
+    "k_shoot_ipm": {"issue_active": 0.641, "warps_active": 0.370, "alu_active": 0.470,
+                    "fma_active": 0.268, "l2_red_requests_per_s": 3.41e10},
+    "k_big_ipm": {"issue_active": 0.835, "warps_active": 0.573, "alu_active": 0.581,
+                  "fma_active": 0.393, "l2_red_requests_per_s": 1.27e11},
+    "k_direct64_vertices": {"fp64_pipe_active": 0.914},
 }
 
 
@@ -731,17 +731,17 @@ def run_native(args):
             mm.destroy(h)
         hs = []
         ppr = pairs_per_ray(specs, [st["rays"] for st in stats])
-        # the direct sum's inner loop issues 11 FP64 instructions per star-ray
-        # pair (2 subtractions, a multiply and an FMA for |d|^2, the two
-        # Newton-Raphson steps of the reciprocal (4 FMA), the mass multiply and
-        # 2 FMA into the sum): its FP64-pipe load against the FMA-chain probe's
+        # the direct sum's inner loop issues 10 FP64 instructions per star-ray
+        # pair (2 subtractions, a multiply and an FMA for |d|^2, the refinement
+        # of the reciprocal (3 FMA), the mass multiply and 2 FMA into the sum):
+        # its FP64-pipe load against the FMA-chain probe's
         # instruction rate (peak TFLOP/s / 2 flops per FMA)
-        dp_rate = 11.0 * pps
+        dp_rate = 10.0 * pps
         dp_peak = peaks["fp64_tflops"] * 1e12 / 2.0
         fp64_plain = {"value": pps / ppr, "unit": UNIT, "pairs_per_s": pps,
                       "pairs_per_ray": ppr, "bands": bands,
                       "speedup_fmm_fp32": value / world / (pps / ppr),
-                      "fp64_pipe": {"dp_inst_per_pair": 11, "achieved_ginst_s": dp_rate / 1e9,
+                      "fp64_pipe": {"dp_inst_per_pair": 10, "achieved_ginst_s": dp_rate / 1e9,
                                     "probe_ginst_s": dp_peak / 1e9, "frac": dp_rate / dp_peak}}
         map_error = {"p999": worst[0], "mean_rel": worst[1], "tol_p999": MAP_P999_TOL,
                      "tol_mean": MEAN_TOL,
