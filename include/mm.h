@@ -106,14 +106,14 @@ typedef struct {
                                0 -> the larger triangles the autotuner counted
                                (its jobs_per_mcell, scaled to the grid) plus a
                                quarter, else the most of 1 per 12 cells and
-                               (kappa_star >= 0.001) the less of 2 per cell and
-                               32 per pixel, within 2^16 .. 2^27 (2^20, then
-                               none, when the device has not that much memory
-                               free).  A map whose
+                               (kappa_star >= 0.001, and at most 1/32 of the
+                               memory to be had) the less of 2 per cell and 32
+                               per pixel, within 2^16 .. 2^27 (2^20, then none,
+                               when the device has not that much memory free).  A map whose
                                accumulators (16 B per pixel) exceed half the
                                GPU's L2: else 2 per cell, at most the most of 1
                                per 5 cells and 64 per pixel; none below 2^22 or
-                               beyond 1/8 of the memory free, or with
+                               beyond 1/32 of the memory to be had, or with
                                kappa_star < 0.001.
                                -1 -> none (the first pass deals every larger
                                triangle); n > 0 -> n.  When the expected larger

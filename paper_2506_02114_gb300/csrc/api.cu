@@ -830,6 +830,21 @@ static int64_t segments_for(const mm_map *h, int64_t cells) {
   return (est + est / 4) / segment_limit(h) + 2;
 }
 
+// Whether a default queue of so many bytes takes at most 1/32 of the device
+// memory to be had (free, or held unused by the pool), so that many handles
+// alive at once leave one another room for their maps.
+static bool leaves_room(int device, int64_t bytes) {
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+  cudaMemPool_t pool;
+  uint64_t held = 0, used = 0;
+  if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+    free_b += held - used;
+  return (uint64_t)bytes <= free_b / 32;
+}
+
 static mm_status alloc_map_buffers(mm_map *h) {
   const size_t np = (size_t)h->P.npix * h->P.npix_y;
   const size_t nspan = (size_t)h->P.npix_y * (h->P.npix + 1);
@@ -853,12 +868,13 @@ static mm_status alloc_map_buffers(mm_map *h) {
   // whichever is less (0.5 to 47 a pixel measured; with few rays per pixel one
   // cell in 12 is too few: 400^2 map, 14 % of the cells, 0.71 + 0.20 ms for the
   // two passes with one in 12, 0.20 + 0.34 with these; next to no stars one in
-  // 12 is 5 % faster, see below); 2^16 .. 2^27 slots (32 B
-  // each, and 10 B more with bands).  When that much device memory is not to be had, 2^20
-  // slots, then none (with bands none, also when it would take more than an
-  // eighth of the free memory).  Batches that do not fit are dealt out by the
-  // first kernel.  A queue of less than 2^22 slots is not taken by bands: a
-  // segment's launches and its last items would cost more than the order gains.
+  // 12 is 5 % faster, see below); 2^16 .. 2^27 slots (32 B each, and 10 B more
+  // with bands).  When that much device memory is not to be had, 2^20 slots, then
+  // none (with bands none).  What a default takes beyond one slot per 12 cells
+  // has to leave room for others (leaves_room).  Batches that do not fit are
+  // dealt out by the first kernel.  A queue of less than 2^22 slots is not taken
+  // by bands: a segment's launches and its last items would cost more than the
+  // order gains.
   // Measured, no queue -> by bands: 3001^2 near the critical line 128 -> 96 ms,
   // 5000^2 1557 -> 665 (1500 cells a pixel), 5000^2 and 10000^2 far from it
   // 128 -> 110 and 656 -> 470, 2060^2 30.7 -> 24.5, a quarter of the rays 33 ->
@@ -884,19 +900,18 @@ static mm_status alloc_map_buffers(mm_map *h) {
     const int32_t want = h->mode == MM_FMM_IRS ? -1 : h->opt.big_queue_slots;
     const int64_t est = est_jobs(h, cells);
     int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;
-    if (h->jobs_pm < 0 && h->P.kappa_star >= 1e-3)
-      slots = std::max(slots, std::min(2 * cells, 32 * (int64_t)h->P.npix * h->P.npix_y));
+    const int64_t ample = std::min(2 * cells, 32 * (int64_t)h->P.npix * h->P.npix_y);
+    if (want == 0 && h->jobs_pm < 0 && h->P.kappa_star >= 1e-3 && slots < ample &&
+        leaves_room(h->device, std::min(ample, int64_t(1) << 27) * MM_TRIJOB_BYTES))
+      slots = ample;
     slots = want > 0 ? want
                      : std::min<int64_t>(int64_t(1) << 27,
                                          std::max<int64_t>(int64_t(1) << 16, slots));
-    size_t slot_bytes = MM_TRIJOB_BYTES, mem_free = 0, mem_total = 0;
+    size_t slot_bytes = MM_TRIJOB_BYTES;
     if (slots < (1 << 22)) h->band_shift = -1;
     if (h->band_shift >= 0) {
       slot_bytes += MM_BAND_ENTRIES * sizeof(uint32_t) + sizeof(uchar2);
-      // (many large maps' handles leave memory for one another's maps)
-      if (want == 0 && (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess ||
-                        (size_t)slots * slot_bytes > mem_free / 8))
-        h->band_shift = -1;
+      if (want == 0 && !leaves_room(h->device, slots * (int64_t)slot_bytes)) h->band_shift = -1;
     }
     const bool banded = h->band_shift >= 0;
     h->bigq_cap = want < 0 || (want == 0 && !fits_l2 && !banded) ? 0 : slots;
