@@ -646,6 +646,7 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   C.lox = P.center_y[0] - P.half_length;
   C.loy = P.center_y[1] - P.half_length_y;
   C.delta = P.delta;
+  C.inv_delta = 1.0 / P.delta;
   C.x1 = P.x0[0] + (double)(P.n[0] - 1) * P.h[0];
   C.y1 = P.x0[1] + (double)(P.n[1] - 1) * P.h[1];
   C.rect_c1 = h->opt.star_rect[0];

@@ -589,15 +589,18 @@ __device__ __forceinline__ bool stays_direct(const FmmConst &C, double dx, doubl
 // Direct-sum stars of the block's record `rec` (all eight lanes).
 __device__ __forceinline__ int count_direct(const TreeDev &T, const FmmConst &C,
                                             const NearRanges &N, int q, int total, int longest,
-                                            double cx, double cy, double Lq) {
+                                            double cx, double cy, double Lq, unsigned &mine) {
   const int j = threadIdx.x & 7, sh = threadIdx.x & 24;
+  mine = ~0u;
   if (C.sub == 0) return total;
+  mine = 0u;
   int cnt = 0;
   for (int c = 0; c < longest; c += 8) {
     bool d = false;
     if (c + j < total) {
       const int i = near_star(N, q, c + j);
       d = stays_direct(C, T.sx[i] - cx, T.sy[i] - cy, Lq);
+      if (d && c < 256) mine |= 1u << (c >> 3);
     }
     cnt += __popc((__ballot_sync(0xffffffffu, d) >> sh) & 0xffu);
   }
@@ -626,7 +629,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS)
   }
   const int mine = valid ? N.end[q][8] : 0;
   const int longest = __reduce_max_sync(0xffffffffu, mine);
-  const int cnt = count_direct(T, C, N, valid ? q : 0, mine, longest, cx, cy, Lq);
+  unsigned direct;
+  const int cnt = count_direct(T, C, N, valid ? q : 0, mine, longest, cx, cy, Lq, direct);
   if ((threadIdx.x & 7) == 0 && cnt) atomicAdd(total, (unsigned)cnt);
 }
 
@@ -732,7 +736,8 @@ struct RecSmem {
 // tables; 32 threads form the 16 records' centres, d_1 and images, one axis
 // each.  Records reserve their direct stars' slots themselves.  67 000 records
 // of 50 000 stars: 307 us with a thread a record (after a count and a scan of
-// 32 us), 188 us like this; a 48^2 map's 848 records 160 and 30 us.
+// 32 us), 162 us like this (171 with IEEE divisions by the grid steps and the
+// pixel, and the near stars tested twice); a 48^2 map's 848 records 160 and 24 us.
 // NB >= p_eval.
 template <int NB>
 __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
@@ -776,15 +781,15 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     double z, L;
     sub_cell_axis(T, C, node2, g0 + rec2, ax, z, L, ctr, Lq2);
     // the grid vertex nearest the sub-cell centre
-    const double h = ax ? C.hy : C.hx, x0 = ax ? C.y0 : C.x0;
-    const double gi = rint((ctr - x0) / h), xr = x0 + gi * h;
+    const double h = ax ? C.hy : C.hx, ih = ax ? C.inv_hy : C.inv_hx, x0 = ax ? C.y0 : C.x0;
+    const double gi = rint(div_near(ctr - x0, h, ih)), xr = x0 + gi * h;
     ref = (int)gi;
-    fc = (float)((ctr - xr) / h);
+    fc = (float)div_near(ctr - xr, h, ih);
     S.c[ax][rec2] = ctr;
     S.r[ax][rec2] = xr;
     if (!ax) {
       S.Lq[rec2] = Lq2;
-      S.fs[rec2] = (float)(1.0 / (Lq2 * C.delta));
+      S.fs[rec2] = (float)(C.inv_delta * inv_pow2(Lq2));
     }
     // d_1 of the leaf's expansion (pe >= 1: p >= 1)
     const double2 *c = loc + (int64_t)node2 * P1;
@@ -825,7 +830,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   const double Lq = S.Lq[valid ? rec : 0];
   const int total = valid ? S.N.end[q][8] : 0;
   const int longest = __reduce_max_sync(0xffffffffu, total);
-  const int n_dir = count_direct(T, C, S.N, q, total, longest, cx, cy, Lq);
+  unsigned direct;  // the lane's direct stars among the first 256
+  const int n_dir = count_direct(T, C, S.N, q, total, longest, cx, cy, Lq, direct);
   if (j == 0) S.cnt[rec] = n_dir;
   __syncthreads();
   if (tid == 0) {
@@ -851,9 +857,10 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     int i = 0;
     if (on) {
       i = near_star(S.N, q, c + j);
-      const double dx = T.sx[i] - cx, dy = T.sy[i] - cy;
-      dir = stays_direct(C, dx, dy, Lq);
+      dir = c < 256 ? direct >> (c >> 3) & 1u
+                    : stays_direct(C, T.sx[i] - cx, T.sy[i] - cy, Lq);
       if (!dir) {
+        const double dx = T.sx[i] - cx, dy = T.sy[i] - cy;
         // 1/w = L_q / (z_i - z_q); d_1 in FP64, the rest in FP32
         const double den = fma(dx, dx, dy * dy), rc = rcp_near(den);
         const double ix = div_near(Lq * dx, den, rc), iy = div_near(-Lq * dy, den, rc);
@@ -1032,7 +1039,7 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   const double ak = 1.0 - C.kappa + C.kappa_star, a = ax ? ak - C.gamma : ak + C.gamma;
   const double iLq = inv_pow2(Lq2), dq = S.d1[ax][r2] * iLq;
   const double W = ax ? a * ctr + dq : a * ctr - dq;  // - conj(d1/L_q)
-  double U = (W - (ax ? C.loy : C.lox)) / C.delta;
+  double U = div_near(W - (ax ? C.loy : C.lox), C.delta, C.inv_delta);
   // |Ui| < 2^28 keeps vertex pixel indices within +-2^29
   U = fmin(fmax(U, -2.0e8), 2.0e8);
   const double Ui = floor(U);
@@ -1049,7 +1056,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   // is deflected by them less than D - margin, so it lands beyond that edge
   // too.  (F and M_direct are FP32 sums: 1 % covers their rounding.)
   const double margin = 2.0;
-  const double B = fabs(a) * (Lq2 + fmax(C.hx, C.hy)) / C.delta + 1.01 * (double)S.F[r2];
+  const double B = div_near(fabs(a) * (Lq2 + fmax(C.hx, C.hy)), C.delta, C.inv_delta) +
+                   1.01 * (double)S.F[r2];
   const double Dlo = -(U + B), Dhi = (U - B) - (double)(ax ? C.npix_y : C.npix);
   double D = Dlo;
   int side = ax ? MM_CULL_BOTTOM : MM_CULL_LEFT;

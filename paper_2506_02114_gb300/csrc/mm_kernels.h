@@ -115,7 +115,7 @@ struct FmmConst {
   int cull;                   // 1: compute the culling bounds
   double kappa, gamma, kappa_star;
   double x0, y0, hx, hy;      // ray grid
-  double inv_hx, inv_hy;      // 1 / hx, 1 / hy
+  double inv_hx, inv_hy, inv_delta;  // 1 / hx, 1 / hy, 1 / delta
   double x1, y1;              // the grid's last vertex
   double lox, loy, delta;     // map lower-left corner and pixel side
   double rect_c1, rect_c2;    // > 0: rectangular star region |x| <= c1, |y| <= c2 (App. B)
