@@ -1038,7 +1038,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   const int r2 = here ? rec2 : 0;
   const double ak = 1.0 - C.kappa + C.kappa_star, a = ax ? ak - C.gamma : ak + C.gamma;
   const double iLq = inv_pow2(Lq2), dq = S.d1[ax][r2] * iLq;
-  const double W = ax ? a * ctr + dq : a * ctr - dq;  // - conj(d1/L_q)
+  // - conj(d1/L_q)
+  const double W = ax ? fma(a, ctr, dq) : __dsub_rn(__dmul_rn(a, ctr), dq);
   double U = div_near(W - (ax ? C.loy : C.lox), C.delta, C.inv_delta);
   // |Ui| < 2^28 keeps vertex pixel indices within +-2^29
   U = fmin(fmax(U, -2.0e8), 2.0e8);
