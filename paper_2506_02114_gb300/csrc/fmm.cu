@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
         dmin2 = fmin(dmin2, dx * dx + dy * dy);
         const double2 l = S.lg[tid][a];
         gx += sg[a] * (dx * l.x - dy * l.y);
-        gy += sg[a] * (dx * l.y + dy * l.x);
+        gy += sg[a] * fma(dy, l.x, dx * l.y);
         lx -= sg[a] * l.x;
         ly -= sg[a] * l.y;
         rx[a] = dx * w;   // L_q / (a - z_q)
