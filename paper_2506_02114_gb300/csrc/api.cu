@@ -174,7 +174,8 @@ struct mm_map {
   int64_t col_lo = 0, col_hi = 0;  // cell columns [col_lo, col_hi)
   int rows_per_item = 64;
   cudaStream_t plan_stream = nullptr;
-  cudaStream_t last_stream = nullptr;
+  cudaStream_t last_stream = nullptr;  // where work on the handle's buffers was last queued
+  bool queued = false;                 // by a run (the stream may be NULL, the default one)
 
   // stars
   DBuf<double> pos_in, m_in, sx, sy, sm;
@@ -986,6 +987,8 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
   const CellRect R = rect ? *rect : all;
   h->launches = 0;
   h->led_batch = false;
+  h->last_stream = st;
+  h->queued = true;
   CKS(record(h, 0, st));
   CKS(clear_map(h, st));
   if (h->mode == MM_PLAIN_FP64) {
@@ -1031,7 +1034,6 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
       LCH(launch_normalize(h->acc, h->span, P.npix, P.npix_y, map_scale(h), h->map.p, st));
       CKS(record(h, 4, st));
       h->ev_recorded = h->opt.time_stages != 0;
-      h->last_stream = st;
       h->ran = true;
       return MM_OK;
     }
@@ -1065,7 +1067,6 @@ static mm_status run_one(mm_map *h, cudaStream_t st, const CellRect *rect = null
   LCH(launch_normalize(h->acc, h->span, P.npix, P.npix_y, map_scale(h), h->map.p, st));
   CKS(record(h, 4, st));
   h->ev_recorded = h->opt.time_stages != 0;
-  h->last_stream = st;
   h->ran = true;
   return MM_OK;
 }
@@ -1533,16 +1534,8 @@ mm_status mm_normalize_fixed(const mm_map *hc, const uint64_t *acc, float *out, 
   return MM_OK;
 }
 
-mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
-  if (!hs || n <= 0) return fail(MM_EINVAL, "empty batch");
-  cudaStream_t st = (cudaStream_t)stream;
-  for (int i = 0; i < n; i++) {
-    if (!hs[i]) return fail(MM_EINVAL, "handle %d is NULL", i);
-    if (hs[i]->mode != MM_FMM_FP32) return fail(MM_EINVAL, "batch needs MM_FMM_FP32 handles");
-    if (hs[i]->device != hs[0]->device) return fail(MM_EINVAL, "batch spans devices");
-    if (hs[i]->timed_out) return fail(MM_ESTATE, "handle %d timed out earlier", i);
-  }
-  CK(cudaSetDevice(hs[0]->device));
+// A batch of checked handles (mm_run_batch).
+static mm_status queue_batch(mm_map *const *hs, int32_t n, cudaStream_t st) {
   const LaunchApart apart;
   mm_map *lead = hs[0];
   // the lead's fan-out streams (created by its first batch call)
@@ -1568,6 +1561,8 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     mm_map *h = hs[i];
     cudaStream_t si = lead->fan[i % nfan];
     h->launches = 0;
+    h->last_stream = st;
+    h->queued = true;
     CKS(record(h, 0, si));
     CKS(clear_map(h, si));
     if (h->fresh) {
@@ -1620,7 +1615,6 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     LCH(launch_normalize(h->acc, h->span, h->P.npix, h->P.npix_y, map_scale(h), h->map.p, si));
     CKS(record(h, 4, si));
     h->ev_recorded = h->opt.time_stages != 0;
-    h->last_stream = st;
     h->ran = true;
   }
   for (int k = 0; k < nfan; k++) {
@@ -1628,6 +1622,23 @@ mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
     CK(cudaStreamWaitEvent(st, lead->fan_join[k], 0));
   }
   return MM_OK;
+}
+
+mm_status mm_run_batch(mm_map *const *hs, int32_t n, void *stream) {
+  if (!hs || n <= 0) return fail(MM_EINVAL, "empty batch");
+  for (int i = 0; i < n; i++) {
+    if (!hs[i]) return fail(MM_EINVAL, "handle %d is NULL", i);
+    if (hs[i]->mode != MM_FMM_FP32) return fail(MM_EINVAL, "batch needs MM_FMM_FP32 handles");
+    if (hs[i]->device != hs[0]->device) return fail(MM_EINVAL, "batch spans devices");
+    if (hs[i]->timed_out) return fail(MM_ESTATE, "handle %d timed out earlier", i);
+  }
+  CK(cudaSetDevice(hs[0]->device));
+  const mm_status s = queue_batch(hs, n, (cudaStream_t)stream);
+  // (a batch that failed half-way has not joined its streams: what they hold
+  // ends before any of the handles can be destroyed)
+  if (s != MM_OK)
+    for (cudaStream_t f : hs[0]->fan) cudaStreamSynchronize(f);
+  return s;
 }
 
 mm_status mm_get_map(const mm_map *hc, float *out, int32_t on_device) {
@@ -1825,7 +1836,9 @@ mm_status mm_get_stats(const mm_map *hc, mm_stats *out) {
 void mm_destroy(mm_map *h) {
   if (!h) return;
   cudaSetDevice(h->device);
-  if (h->last_stream) cudaStreamSynchronize(h->last_stream);
+  // The buffers go back in the plan stream's order, which a run's stream is no
+  // part of: the last run, on whatever stream (NULL too), ends first.
+  if (h->last_stream || h->queued) cudaStreamSynchronize(h->last_stream);
   // frees in stream order on the plan stream (synchronised below)
   AllocStream free_on(h->plan_stream);
   DBuf<double> *dbs[] = {&h->pos_in, &h->m_in, &h->sx, &h->sy, &h->sm};
