@@ -326,7 +326,7 @@ static __host__ __device__ __forceinline__ size_t local_smem(int p) {
 __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
     k_local(TreeDev T, int level, int64_t n, int p, const int32_t *node_act,
             const double2 *__restrict__ MLop, const double2 *__restrict__ LLop,
-            const double2 *__restrict__ mp, double2 *loc, unsigned *err) {
+            const double2 *mp, double2 *loc, unsigned *err) {
   grid_begin();
   extern __shared__ __align__(16) double2 s_loc[];
   __shared__ LocalSources S;
@@ -742,7 +742,7 @@ struct RecSmem {
 template <int NB>
 __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     TreeDev T, FmmConst C, int64_t n_rec, const int32_t *active_list, SubTables tb,
-    const double2 *__restrict__ loc, LeafRec *leaf, NearPos *near_pos, float *near_m,
+    const double2 *loc, LeafRec *leaf, NearPos *near_pos, float *near_m,
     float2 *coef, unsigned *near_total, unsigned near_cap, unsigned *err) {
   grid_begin();
   extern __shared__ __align__(16) unsigned char s_rec[];

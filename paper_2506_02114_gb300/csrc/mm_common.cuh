@@ -24,7 +24,9 @@ namespace mm {
 
 // First thing in a kernel that launch_next launches: the stream's next kernel
 // may be set up from now on, and this one begins when the kernels before it
-// are complete and their writes visible.
+// are complete and their writes visible.  (What those write is no
+// `const __restrict__` parameter here: it is not constant while this kernel
+// lives, and its loads must not move ahead of the wait.)
 __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

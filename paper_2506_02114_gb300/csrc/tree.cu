@@ -44,7 +44,7 @@ __global__ void k_star_keys(const double *__restrict__ pos, int64_t n, double R0
 }
 
 __global__ void k_gather_stars(const double *__restrict__ pos, const double *__restrict__ m,
-                               const int32_t *__restrict__ idx, int64_t n, double *sx,
+                               const int32_t *idx, int64_t n, double *sx,
                                double *sy, double *sm) {
   grid_begin();
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
