@@ -243,7 +243,9 @@ typedef struct {
                                invariant, 2 a vertex outside every active leaf,
                                4 a star-rectangle corner near a sub-cell, 8 a
                                map index out of range (only the MM_DEBUG build
-                               checks, and skips the access) */
+                               checks, and skips the access), 16 direct stars
+                               beyond the slots the plan counted (internal; the
+                               map is not valid) */
   int32_t queue_slots;      /* capacity of the second-pass queue, in triangles
                                (0: none; see mm_options.big_queue_slots) */
 } mm_stats;

@@ -1242,6 +1242,7 @@ static mm_status create_impl(mm_map *h, double kappa_tot, double shear, double s
   unsigned e = 0;
   CK(cudaMemcpy(&e, h->err.p, sizeof e, cudaMemcpyDeviceToHost));
   if (e & ERR_TREE_INVARIANT) return fail(MM_ECUDA, "internal: quadtree invariant violated");
+  if (e & ERR_NEAR_SLOTS) return fail(MM_ECUDA, "internal: direct stars beyond the slots counted");
   if (e & ERR_RECT_CORNER)
     return fail(MM_EINVAL,
                 "a corner of star_rect lies within two half-diagonals of a ray-grid sub-cell: "

@@ -845,8 +845,9 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   }
   __syncthreads();
   const unsigned off = S.base + (unsigned)S.cnt[rec];
-  // (never exceeded: the plan counted the same stars)
+  // (the plan counted the same stars: a record without room is an error)
   const bool room = off + (unsigned)n_dir <= near_cap;
+  if (!room && j == 0) atomicOr(err, ERR_NEAR_SLOTS);
 
   // near-field stars, eight at a time: into the expansion, or noted as direct
   double d1 = j < 2 ? S.d1[j][rec] : 0.0;

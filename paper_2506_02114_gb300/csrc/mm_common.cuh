@@ -40,6 +40,8 @@ enum : unsigned int {
                               // slowly (a star-rectangle corner is near it)
   ERR_BOUNDS = 8u,            // MM_DEBUG builds: a map or row-difference index out of
                               // range (the access was skipped)
+  ERR_NEAR_SLOTS = 16u,       // a record's direct stars exceed the slots the plan counted
+                              // (they are in no sum: the map is not valid)
 };
 
 // Per sub-cell of an active leaf: everything a ray vertex in it needs (64
