@@ -701,11 +701,12 @@ struct RecSmem {
   NearRanges N;
   double c[2][MM_REC], r[2][MM_REC], Lq[MM_REC], d1[2][MM_REC];
   float fs[MM_REC];                         // 1 / (L_q delta)
-  double star[MM_REC][8][3];                // far stars of a round: mass, 1/w
+  double star[MM_REC][8][3];                // far stars of a round: mass, 1/w; at the end
+                                            // [2]: a lane's share of the direct mass
   float2 v[MM_REC][8 * (NB - 1) + 2];       // their terms m w^-n / n
-  float F[MM_REC], md[MM_REC];
+  float F[MM_REC];
   int cnt[MM_REC];
-  unsigned base;
+  unsigned off[MM_REC], base;
   double2 lg[MM_REC][4];                    // corner logarithms (rectangular region)
 };
 
@@ -736,7 +737,7 @@ struct RecSmem {
 // tables; 32 threads form the 16 records' centres, d_1 and images, one axis
 // each.  Records reserve their direct stars' slots themselves.  67 000 records
 // of 50 000 stars: 307 us with a thread a record (after a count and a scan of
-// 32 us), 162 us like this (171 with IEEE divisions by the grid steps and the
+// 32 us), 167 us like this (176 with IEEE divisions by the grid steps and the
 // pixel, and the near stars tested twice); a 48^2 map's 848 records 160 and 24 us.
 // NB >= p_eval.
 template <int NB>
@@ -902,8 +903,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
     __syncwarp();
   }
   // the direct stars in the record's grid frame, and their mass (for the
-  // culling bound alone)
-  float md = 0.f;
+  // culling bound alone, in FP64: a bound has to hold for any number of stars)
+  double md = 0.0;
   if (room) {
     const double xr = S.r[0][rec], yr = S.r[1][rec];
     for (int t = j; t < n_dir; t += 8) {
@@ -917,12 +918,12 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
       np.Ky = (float)Ky;
       np.fy = (float)(syg - Ky);
       near_pos[off + t] = np;
-      const float m = (float)T.sm[i];
-      near_m[off + t] = m;
-      md += m;
+      const double m = T.sm[i];
+      near_m[off + t] = (float)m;
+      md = t < 8 ? m : md + m;
     }
   }
-  for (int b = 1; b < 8; b <<= 1) md += __shfl_xor_sync(0xffffffffu, md, b);
+  S.star[rec][j][2] = md;
 
   // Rectangular star region: the sheet's part beyond -kappa_star z is the
   // conjugate of At, analytic inside the rectangle, so its potential joins
@@ -1026,9 +1027,8 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
       out[0] = out[2] = 0.f;
     }
     S.F[rec] = F;
-    S.md[rec] = md;
     S.cnt[rec] = room ? n_dir : 0;
-    S.star[rec][1][2] = __hiloint2double(0, (int)off);
+    S.off[rec] = off;
   }
   if (valid && j < 2) S.d1[j][rec] = d1;
   __syncthreads();
@@ -1056,7 +1056,7 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   // |series| <= F.  If that box lies D pixels beyond a map edge, a vertex
   // whose direct stars are all farther than M_direct / (delta (D - margin))
   // is deflected by them less than D - margin, so it lands beyond that edge
-  // too.  (F and M_direct are FP32 sums: 1 % covers their rounding.)
+  // too.  (F is a sum of at most 63 FP32 terms: 1 % covers its rounding.)
   const double margin = 2.0;
   const double B = div_near(fabs(a) * (Lq2 + fmax(C.hx, C.hy)), C.delta, C.inv_delta) +
                    1.01 * (double)S.F[r2];
@@ -1065,6 +1065,10 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   int side = ax ? MM_CULL_BOTTOM : MM_CULL_LEFT;
   if (Dhi > D) D = Dhi, side = ax ? MM_CULL_TOP : MM_CULL_RIGHT;
   const bool in = U > -1.9e8 && U < 1.9e8;
+  // the direct stars' mass: half of the lanes' shares by each axis' thread
+  const double *m8 = &S.star[r2][4 * ax][2];
+  double md2 = ((m8[0] + m8[3]) + m8[6]) + m8[9];
+  md2 += __shfl_xor_sync(0xffffffffu, md2, 1);
   // axis 1's numbers to axis 0's thread, which writes the record
   const double D1 = __shfl_down_sync(0xffffffffu, D, 1);
   const int side1 = __shfl_down_sync(0xffffffffu, side, 1);
@@ -1087,14 +1091,14 @@ __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(
   R.Vf = fU1;
   R.zsx = zs;
   R.zsy = zs1;
-  R.near_off = __double2loint(S.star[rec2][1][2]);
+  R.near_off = (int32_t)S.off[rec2];
   R.near_cnt = S.cnt[rec2];
   R.coef_off = (int32_t)((g0 + rec2) * cs);
   R.node = node2;
   R.cull_side = MM_CULL_NONE;
   R.cull_r2 = -1.f;
   if (C.cull && D > 2.0 * margin && in && in1) {
-    const double rc = 1.001 * (double)S.md[rec2] / (C.delta * (D - margin) * C.hx);  // of h_x
+    const double rc = md2 / (C.delta * (D - margin) * C.hx);  // of h_x
     R.cull_side = side;
     R.cull_r2 = (float)(rc * rc * 1.01);
   }

@@ -57,3 +57,20 @@ def test_direct_stars_without_a_slot_are_reported(records, n, sub):
     recs, total, written, err = records(x, y, m, sub, -2)
     assert err == ERR_NEAR_SLOTS and written[1] == 0
     assert recs["near_cnt"].sum() < total
+
+
+@pytest.mark.parametrize("n,mass", [(1, 0.7), (300, 0.3), (4000000, 1.0155)])
+def test_culling_radius_covers_the_direct_mass(records, n, mass):
+    """Beyond the radius the direct stars' whole mass moves a vertex by less
+    than the record's distance from the map (1000 - 8 - 16 pixels: the centre's
+    image, the macro term over the leaf, the map) less the margin of 2.  Millions
+    of stars in one place: in FP32 each would add its mass rounded to the sum's
+    last bit (1/32 here, a loss of 1.5 % a star)."""
+    recs, total, _, err = records(np.full(n, 0.3), np.full(n, -0.2), np.full(n, mass), 0, -1)
+    assert err == 0 and total == n and recs["near_cnt"][0] == n
+    side = recs["cull_side"][0]
+    assert side == 2   # beyond the right edge
+    # |1 - kappa + kappa_* + gamma| (L + h) / delta, with h = 0.5 and L = 8
+    D = 1000.0 - 1.3 * 8.5 - 16.0
+    r2 = (n * mass / (D - 2.0) / 0.5) ** 2
+    assert r2 <= recs["cull_r2"][0] <= 1.02 * r2
