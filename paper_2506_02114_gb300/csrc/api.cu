@@ -515,7 +515,10 @@ static mm_status run_tree(mm_map *h, cudaStream_t st, bool plan) {
       CKS(ensure_nodes(h, h->level_off[l + 1] + nxt));
       CKS(upload_level_off(h, st));
     }
-    LCH(launch_level_children(tree_dev(h), tree_out(h), l, n, h->split.p, h->group.p, st));
+    const int64_t groups = (n + MM_SPLIT_GROUP - 1) / MM_SPLIT_GROUP;
+    const bool scan = groups > MM_SUM_GROUPS;
+    if (scan) LCH(launch_group_scan(h->group.p, groups, st));
+    LCH(launch_level_children(tree_dev(h), tree_out(h), l, n, h->split.p, h->group.p, scan, st));
     if (plan && h->level_cnt[l + 1] == 0) {
       h->depth = l;
       h->n_nodes = h->level_off[l + 1];
@@ -560,7 +563,10 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
                         h->row_cell.p, st));
   LCH(launch_active_flags(T, nn, h->col_cell.p, h->col_lo, h->col_hi, h->row_cell.p, h->row_lo,
                           h->row_hi, h->node_act.p, h->leaf_flag.p, h->leaf_group.p, st));
-  LCH(launch_compact_leaves(nn, h->leaf_flag.p, h->leaf_group.p, h->node_active.p,
+  const int64_t groups = (nn + MM_ACTIVE_GROUP - 1) / MM_ACTIVE_GROUP;
+  const bool scan = groups > MM_SUM_GROUPS;
+  if (scan) LCH(launch_group_scan(h->leaf_group.p, groups, st));
+  LCH(launch_compact_leaves(nn, h->leaf_flag.p, h->leaf_group.p, scan, h->node_active.p,
                             h->active_list.p, h->top_info.p, st));
   if (plan) {
     const int32_t *src[1] = {h->top_info.p};

@@ -131,20 +131,93 @@ __global__ void __launch_bounds__(256) k_level_split(TreeDev T, TreeOut O, int l
   }
 }
 
+// Split nodes (active leaves) before group g, from the groups' counts or, where
+// those are many, from their running sum (k_group_scan).  Adding up the counts
+// in every block is quadratic in a level's nodes, but spares a launch (see
+// MM_SUM_GROUPS).  Call with all threads of a block of 256; the sum is in *s_base
+// after the block's next __syncthreads.
+__device__ __forceinline__ void before_group(const int32_t *group, int64_t g, bool scanned,
+                                             int *s_base) {
+  int before = 0;
+  if (scanned) {
+    if (threadIdx.x == 0) *s_base = group[g];
+    return;
+  }
+  for (int64_t k = threadIdx.x; k < g; k += 256) before += group[k];
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (threadIdx.x == 0) *s_base = 0;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && before) atomicAdd(s_base, before);
+}
+
+// group[k] <- group[0] + .. + group[k - 1], one block.  16 counts a thread and
+// round; the array is 16-byte aligned.
+#define MM_SCAN_EACH 16
+__global__ void __launch_bounds__(1024) k_group_scan(int32_t *group, int64_t n) {
+  grid_begin();
+  __shared__ int s_w[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int carry = 0;
+  for (int64_t base = 0; base < n; base += 1024 * MM_SCAN_EACH) {
+    const int64_t k0 = base + (int64_t)threadIdx.x * MM_SCAN_EACH;
+    const bool whole = k0 + MM_SCAN_EACH <= n;
+    int v[MM_SCAN_EACH], sum = 0;
+#pragma unroll
+    for (int k = 0; k < MM_SCAN_EACH; k += 4) {
+      int4 a = make_int4(0, 0, 0, 0);
+      if (whole) {
+        a = *reinterpret_cast<const int4 *>(group + k0 + k);
+      } else {
+        if (k0 + k < n) a.x = group[k0 + k];
+        if (k0 + k + 1 < n) a.y = group[k0 + k + 1];
+        if (k0 + k + 2 < n) a.z = group[k0 + k + 2];
+        if (k0 + k + 3 < n) a.w = group[k0 + k + 3];
+      }
+      v[k] = a.x;
+      v[k + 1] = a.y;
+      v[k + 2] = a.z;
+      v[k + 3] = a.w;
+      sum += a.x + a.y + a.z + a.w;
+    }
+    int incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += u;
+    }
+    if (lane == 31) s_w[w] = incl;
+    __syncthreads();
+    int before = carry + incl - sum;
+    for (int k = 0; k < 32; k++) {
+      if (k < w) before += s_w[k];
+      carry += s_w[k];
+    }
+#pragma unroll
+    for (int k = 0; k < MM_SCAN_EACH; k += 4) {
+      const int4 a = make_int4(before, before + v[k], before + v[k] + v[k + 1],
+                               before + v[k] + v[k + 1] + v[k + 2]);
+      before = a.w + v[k + 3];
+      if (whole) {
+        *reinterpret_cast<int4 *>(group + k0 + k) = a;
+      } else {
+        if (k0 + k < n) group[k0 + k] = a.x;
+        if (k0 + k + 1 < n) group[k0 + k + 1] = a.y;
+        if (k0 + k + 2 < n) group[k0 + k + 2] = a.z;
+        if (k0 + k + 3 < n) group[k0 + k + 3] = a.w;
+      }
+    }
+    __syncthreads();  // (s_w is written anew)
+  }
+}
+
 // Four lanes per node, 64 nodes (two groups) per block.
 __global__ void __launch_bounds__(256) k_level_children(TreeDev T, TreeOut O, int level, int64_t n,
-                                                        const int32_t *split,
-                                                        const int32_t *group) {
+                                                        const int32_t *split, const int32_t *group,
+                                                        bool scanned) {
   grid_begin();
   __shared__ int s_w[8], s_base;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = threadIdx.x & 3;
-  // split nodes of the groups before this block's
-  int before = 0;
-  for (int64_t k = threadIdx.x; k < 2 * (int64_t)blockIdx.x; k += 256) before += group[k];
-  before = __reduce_add_sync(0xffffffffu, before);
-  if (threadIdx.x == 0) s_base = 0;
-  __syncthreads();
-  if (lane == 0 && before) atomicAdd(&s_base, before);
+  before_group(group, 2 * (int64_t)blockIdx.x, scanned, &s_base);
   const int64_t t = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2);
   const int64_t node = T.level_off[level] + t;
   const bool f = t < n && split[t];
@@ -305,28 +378,26 @@ __global__ void k_active_flags(TreeDev T, int64_t n_nodes, const int32_t *col_ce
 // Numbers the active leaves in the order of their nodes, block by block of
 // k_active_flags; the last block stores how many there are.
 __global__ void __launch_bounds__(256) k_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag,
-                                                        const int32_t *group,
+                                                        const int32_t *group, bool scanned,
                                                         int32_t *node_active,
                                                         int32_t *active_list, int32_t *total) {
   grid_begin();
   __shared__ int s_w[8], s_base;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int before = 0;
-  for (int64_t k = threadIdx.x; k < blockIdx.x; k += 256) before += group[k];
-  before = __reduce_add_sync(0xffffffffu, before);
-  if (threadIdx.x == 0) s_base = 0;
-  __syncthreads();
-  if (lane == 0 && before) atomicAdd(&s_base, before);
+  before_group(group, blockIdx.x, scanned, &s_base);
   const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const bool f = t < n_nodes && leaf_flag[t];
   const unsigned m = __ballot_sync(0xffffffffu, f);
   if (lane == 0) s_w[w] = __popc(m);
   __syncthreads();
-  int rank = s_base + __popc(m & ((1u << lane) - 1u));
-  for (int k = 0; k < w; k++) rank += s_w[k];
+  int rank = s_base + __popc(m & ((1u << lane) - 1u)), all = s_base;
+  for (int k = 0; k < 8; k++) {
+    if (k < w) rank += s_w[k];
+    all += s_w[k];
+  }
   if (t < n_nodes) node_active[t] = f ? rank : -1;
   if (f) active_list[rank] = (int32_t)t;
-  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) *total = s_base + group[blockIdx.x];
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) *total = all;
 }
 
 // Lookup grid over the active region at level glevel: the active leaf
@@ -388,10 +459,16 @@ cudaError_t launch_level_split(const TreeDev &T, const TreeOut &O, int level, in
   return cudaGetLastError();
 }
 
+cudaError_t launch_group_scan(int32_t *group, int64_t n, cudaStream_t st) {
+  launch_next(k_group_scan, 1, 1024, 0, st, group, n);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_level_children(const TreeDev &T, const TreeOut &O, int level, int64_t n,
-                                  const int32_t *split, const int32_t *group, cudaStream_t st) {
+                                  const int32_t *split, const int32_t *group, bool scanned,
+                                  cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  launch_next(k_level_children, blocks_for(n, 64), 256, 0, st, T, O, level, n, split, group);
+  launch_next(k_level_children, blocks_for(n, 64), 256, 0, st, T, O, level, n, split, group, scanned);
   return cudaGetLastError();
 }
 
@@ -413,12 +490,12 @@ cudaError_t launch_active_flags(const TreeDev &T, int64_t n_nodes, const int32_t
 }
 
 cudaError_t launch_compact_leaves(int64_t n_nodes, const int32_t *leaf_flag, const int32_t *group,
-                                  int32_t *node_active, int32_t *active_list, int32_t *total,
-                                  cudaStream_t st) {
+                                  bool scanned, int32_t *node_active, int32_t *active_list,
+                                  int32_t *total, cudaStream_t st) {
   static_assert(MM_ACTIVE_GROUP == 256, "one thread per node of a group");
   if (n_nodes <= 0) return cudaSuccess;
-  launch_next(k_compact_leaves, blocks_for(n_nodes, 256), 256, 0, st, n_nodes, leaf_flag, group,
-                                                             node_active, active_list, total);
+  launch_next(k_compact_leaves, blocks_for(n_nodes, 256), 256, 0, st, n_nodes, leaf_flag, group, scanned,
+              node_active, active_list, total);
   return cudaGetLastError();
 }
 

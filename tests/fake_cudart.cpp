@@ -75,7 +75,7 @@ void kernel(const void *f, void **args) {
     int32_t *info = word(3);
     info[0] = info[1] = info[2] = 1;
   } else if (n.find("k_compact_leaves") != std::string::npos) {
-    *word(5) = 1;
+    *word(6) = 1;
   }
 }
 
