@@ -31,6 +31,10 @@
  *     Its buffers come from the device's default memory pool (stream-ordered
  *     allocation); the library raises that pool's release threshold, so the
  *     memory of a destroyed handle stays with the process for the next one.
+ *     Destroying a handle whose second-pass queue went by bands (see
+ *     big_queue_slots; up to 5.6 GB by default) gives back what the pool then
+ *     holds unused beyond 1/32 of the device's memory.  A handle keeps up to
+ *     32 MB for mm_shoot_points once that has been called.
  *   - "stream" arguments are cudaStream_t values passed as void*; NULL is the
  *     legacy default stream.
  */

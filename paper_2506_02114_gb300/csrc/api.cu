@@ -157,6 +157,31 @@ static void keep_pool_memory(int dev) {
   done[dev] = true;
 }
 
+// Memory that the pool holds and nobody uses.
+static uint64_t pool_idle(cudaMemPool_t pool, uint64_t &used) {
+  uint64_t held = 0;
+  if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return 0;
+  return held > used ? held - used : 0;
+}
+
+// Gives the driver back what the pool holds unused beyond 1/32 of the device's
+// memory, which is one handle's largest default queue (leaves_room): after a
+// handle with a queue of gigabytes, so that other allocators of the process
+// are not left without what many such handles took.  Handles made one after
+// the other still find the queue in the pool (5.6 GB: 0.006 ms, 4.2 ms to take
+// from the driver and 7.0 to give back).
+static void trim_pool(int device) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemPool_t pool;
+  uint64_t used = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+      cudaDeviceGetDefaultMemPool(&pool, device) != cudaSuccess)
+    return;
+  if (pool_idle(pool, used) > total_b / 32) cudaMemPoolTrimTo(pool, used + total_b / 32);
+}
+
 // ---------------------------------------------------------------------------
 // the handle
 // ---------------------------------------------------------------------------
@@ -845,11 +870,8 @@ static bool leaves_room(int device, int64_t bytes) {
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
   cudaMemPool_t pool;
-  uint64_t held = 0, used = 0;
-  if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess &&
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
-    free_b += held - used;
+  uint64_t used = 0;
+  if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) free_b += pool_idle(pool, used);
   return (uint64_t)bytes <= free_b / 32;
 }
 
@@ -1897,6 +1919,7 @@ void mm_destroy(mm_map *h) {
   if (h->plan_stream) {
     cudaStreamSynchronize(h->plan_stream);
     cudaStreamDestroy(h->plan_stream);
+    if (h->band_shift >= 0 && h->bigq_cap > 0) trim_pool(h->device);
   }
   if (h->pin) cudaFreeHost(h->pin);
   delete h;

@@ -5,6 +5,8 @@
 // stream may still use it is noticed.  Not a GPU model: maps stay zero.
 #include <cuda_runtime_api.h>
 
+#include <sys/mman.h>
+
 #include <algorithm>
 #include <cstdint>
 #include <cstdlib>
@@ -25,6 +27,7 @@ Clock host;                                              // what the host has wa
 long ops = 0, unordered = 0, mallocs = 0, fail_malloc = -1, launches = 0, fail_launch = -1;
 cudaError_t pending = cudaSuccess;
 size_t pool_used = 0, pool_held = 0;
+const size_t total_mem = 280ull << 30;
 long next_stream = 1, next_event = 1;
 
 int id(cudaStream_t s) { return (int)(intptr_t)s; }
@@ -48,8 +51,10 @@ void check_free(int s) {
 cudaError_t get(void **p, size_t n, bool pooled) {
   std::lock_guard<std::mutex> l(mu);
   if (mallocs++ == fail_malloc) return cudaErrorMemoryAllocation;
-  *p = calloc(n ? n : 1, 1);
-  if (!*p) return cudaErrorMemoryAllocation;
+  // (never touched pages cost nothing: a queue of gigabytes is only an address range)
+  *p = mmap(nullptr, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE,
+            -1, 0);
+  if (*p == MAP_FAILED) return cudaErrorMemoryAllocation;
   blocks[*p] = n;
   if (pooled) {
     pool_used += n;
@@ -61,8 +66,8 @@ void put(void *p, bool pooled) {
   const auto it = blocks.find(p);
   if (it == blocks.end()) return;
   if (pooled) pool_used -= it->second;
+  munmap(p, it->second ? it->second : 1);
   blocks.erase(it);
-  free(p);
 }
 void copy(void *d, const void *s, size_t n) {
   if (n <= (size_t)64 << 20) memcpy(d, s, n);
@@ -84,6 +89,8 @@ void kernel(const void *f, void **args) {
 extern "C" {
 
 long fake_unordered() { return unordered; }
+long fake_pool_idle() { return (long)(pool_held - pool_used); }
+long fake_total_memory() { return (long)total_mem; }
 long fake_mallocs() { return mallocs; }
 long fake_launches() { return launches; }
 // the n-th allocation or launch from fake_reset on fails
@@ -178,8 +185,8 @@ cudaError_t cudaGetLastError() {
 cudaError_t cudaPeekAtLastError() { return cudaSuccess; }
 const char *cudaGetErrorString(cudaError_t) { return "fake runtime"; }
 cudaError_t cudaMemGetInfo(size_t *f, size_t *t) {
-  *f = 270ull << 30;
-  *t = 280ull << 30;
+  *f = total_mem - (10ull << 30) - pool_held;
+  *t = total_mem;
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void **, const void *) { return cudaErrorInvalidSymbol; }
@@ -237,6 +244,11 @@ cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t *p, int) {
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t keep) {
+  std::lock_guard<std::mutex> l(mu);
+  pool_held = std::max(pool_used, std::min(pool_held, keep));
+  return cudaSuccess;
+}
 cudaError_t cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr a, void *v) {
   std::lock_guard<std::mutex> l(mu);
   *static_cast<uint64_t *>(v) = a == cudaMemPoolAttrUsedMemCurrent ? pool_used : pool_held;

@@ -1,5 +1,6 @@
 """The library's host code on a stand-in for the CUDA runtime (fake_cudart.cpp,
-no GPU): buffers are given back only after every stream that may use them."""
+no GPU): buffers are given back only after every stream that may use them, and
+the pool does not keep the queues of many large maps."""
 import ctypes
 import glob
 import os
@@ -26,7 +27,8 @@ def fake(tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(out)
     L.fake_fail_malloc.argtypes = L.fake_fail_launch.argtypes = [ctypes.c_long]
-    for f in ("fake_unordered", "fake_mallocs", "fake_launches"):
+    for f in ("fake_unordered", "fake_mallocs", "fake_launches", "fake_pool_idle",
+              "fake_total_memory"):
         getattr(L, f).restype = ctypes.c_long
     path, real = build.LIB, mm._lib
     mm._lib, build.LIB = None, out
@@ -97,3 +99,22 @@ def test_destroy_waits_for_what_a_failed_batch_queued(fake):
     for h in hs[::-1]:
         mm.destroy(h)
     assert fake.fake_unordered() == 0
+
+
+def test_large_queues_do_not_stay_with_the_pool(fake):
+    """One handle's queue of gigabytes may wait in the pool for the next
+    handle; those of several alive at once go back to the driver."""
+    fake.fake_reset()
+    bound = fake.fake_total_memory() // 32
+    hs = [make(npix=2200, big_queue_slots=1 << 27) for _ in range(4)]   # 5.6 GB each
+    assert all(mm.get_stats(h)["queue_slots"] == 1 << 27 for h in hs)
+    for h in hs[1:]:
+        mm.destroy(h)
+        assert fake.fake_pool_idle() <= bound
+    assert fake.fake_pool_idle() > 5e9
+    mm.destroy(hs[0])
+    assert fake.fake_pool_idle() <= bound
+    # an ordinary handle's memory stays for the next one
+    idle = fake.fake_pool_idle()
+    mm.destroy(make())
+    assert fake.fake_pool_idle() == idle
