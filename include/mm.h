@@ -117,8 +117,11 @@ typedef struct {
                                accumulators (16 B per pixel) exceed half the
                                GPU's L2: else 2 per cell, at most the most of 1
                                per 5 cells and 64 per pixel; none below 2^22 or
-                               beyond 1/32 of the memory to be had, or with
-                               kappa_star < 0.001.
+                               beyond 1/32 of the memory to be had, with
+                               kappa_star < 0.001, or where the first pass is
+                               the faster one: a cell more than a pixel wide
+                               without stars, sqrt(kappa_star <m^2>/<m>) below
+                               7 pixels and 6 work items for each of its warps.
                                -1 -> none (the first pass deals every larger
                                triangle); n > 0 -> n.  When the expected larger
                                triangles exceed it the first pass runs in

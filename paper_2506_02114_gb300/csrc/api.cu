@@ -875,6 +875,28 @@ static bool leaves_room(int device, int64_t bytes) {
   return (uint64_t)bytes <= free_b / 32;
 }
 
+// Whether the first pass had better deal a large map's larger triangles where
+// it finds them, by default: where the macro model alone stretches a cell over
+// more than a pixel, so that nearly every triangle is a larger one, and the
+// stars scatter neighbours by so few pixels that a warp's lines stay in the L2
+// all the same.  A slot written, sorted and read again then costs more than the
+// order gains.  Items enough to keep the warps even are needed, too (the queue
+// deals its triangles evenly whatever the items).
+// Both sides at 277 points (2100^2 to 5000^2 pixels, 2 to 100 rays landing on
+// one, kappa_star 0.05 to 0.8, scatter 1 to 47 pixels): at the 72 inside these
+// limits bands took 2 to 60 % longer (3000^2: 9.3 -> 10.9 ms, 4500^2: 20.4 ->
+// 25.6).  Between 7 and 8 pixels 4 % less to 38 % longer, between 0.8 and 1 pixel
+// a cell 23 % less to 17 % longer; with half an item a warp (rows_per_item 512,
+// 0.93 pixels a cell) half as long.
+static bool better_in_place(const mm_map *h, int64_t cells) {
+  const mm_params &P = h->P;
+  const double scatter = std::sqrt(P.kappa_star * P.m2_over_m) / P.delta;
+  const double cell = std::max(std::fabs(P.a1) * P.h[0], std::fabs(P.a2) * P.h[1]) / P.delta;
+  const int64_t rows = h->opt.rows_per_item > 0 ? h->rows_per_item : 32;
+  const double items = (double)cells / (MM_STRIP * (double)rows);
+  return h->mode == MM_FMM_FP32 && scatter < 7.0 && cell > 1.0 && items >= 6.0 * 8 * shoot_grid();
+}
+
 static mm_status alloc_map_buffers(mm_map *h) {
   const size_t np = (size_t)h->P.npix * h->P.npix_y;
   const size_t nspan = (size_t)h->P.npix_y * (h->P.npix + 1);
@@ -908,8 +930,8 @@ static mm_status alloc_map_buffers(mm_map *h) {
   // Measured, no queue -> by bands: 3001^2 near the critical line 128 -> 96 ms,
   // 5000^2 1557 -> 665 (1500 cells a pixel), 5000^2 and 10000^2 far from it
   // 128 -> 110 and 656 -> 470, 2060^2 30.7 -> 24.5, a quarter of the rays 33 ->
-  // 24 (3000^2), 6 cells a pixel 51 -> 32 and 9.4 -> 10.8; by kappa_star (4000^2)
-  // 168 -> 119 at 0.25, 71 -> 58 at 0.05, 52 -> 44 at 0.01.  Next to no stars
+  // 24 (3000^2), 6 cells a pixel 51 -> 32 (where they lose: better_in_place); by
+  // kappa_star (4000^2) 168 -> 119 at 0.25, 71 -> 58 at 0.05, 52 -> 44 at 0.01.  Next to no stars
   // (3e-5, 10000 x 1000): 70 -> 125 ms, the macro model maps neighbours onto the
   // same few pixels and every triangle is a larger one, so below 1e-3 no bands.
   // 2^26 / 2^27 / 2^28 slots: 99 / 97 / 96 ms and, on the second 5000^2 map,
@@ -928,6 +950,7 @@ static mm_status alloc_map_buffers(mm_map *h) {
                         ? shift
                         : -1;
     const int32_t want = h->mode == MM_FMM_IRS ? -1 : h->opt.big_queue_slots;
+    if (want == 0 && better_in_place(h, cells)) h->band_shift = -1;
     const int64_t est = est_jobs(h, cells);
     int64_t slots = h->jobs_pm >= 0 ? est + est / 4 + 4096 : est;
     const int64_t ample = std::min(2 * cells, 32 * (int64_t)h->P.npix * h->P.npix_y);

@@ -28,6 +28,7 @@ long ops = 0, unordered = 0, mallocs = 0, fail_malloc = -1, launches = 0, fail_l
 cudaError_t pending = cudaSuccess;
 size_t pool_used = 0, pool_held = 0;
 const size_t total_mem = 280ull << 30;
+size_t others = 10ull << 30;  // taken by other processes and libraries
 long next_stream = 1, next_event = 1;
 
 int id(cudaStream_t s) { return (int)(intptr_t)s; }
@@ -93,6 +94,7 @@ long fake_pool_idle() { return (long)(pool_held - pool_used); }
 long fake_total_memory() { return (long)total_mem; }
 long fake_mallocs() { return mallocs; }
 long fake_launches() { return launches; }
+void fake_others(size_t bytes) { others = bytes; }
 // the n-th allocation or launch from fake_reset on fails
 void fake_fail_malloc(long n) { fail_malloc = n; }
 void fake_fail_launch(long n) { fail_launch = n; }
@@ -102,6 +104,7 @@ void fake_reset() {
   unordered = mallocs = launches = 0;
   fail_malloc = fail_launch = -1;
   pool_held = pool_used;
+  others = 10ull << 30;
 }
 
 // registration and launches
@@ -185,7 +188,7 @@ cudaError_t cudaGetLastError() {
 cudaError_t cudaPeekAtLastError() { return cudaSuccess; }
 const char *cudaGetErrorString(cudaError_t) { return "fake runtime"; }
 cudaError_t cudaMemGetInfo(size_t *f, size_t *t) {
-  *f = total_mem - (10ull << 30) - pool_held;
+  *f = total_mem - others - pool_held;
   *t = total_mem;
   return cudaSuccess;
 }
