@@ -401,7 +401,6 @@ static TreeDev tree_dev(const mm_map *h) {
   T.parent = h->parent.p;
   T.nb = h->nb.p;
   T.level_off = h->d_level_off.p;
-  T.depth = h->depth;
   return T;
 }
 
@@ -552,6 +551,16 @@ static mm_status run_tree(mm_map *h, cudaStream_t st, bool plan) {
   return MM_OK;
 }
 
+// SMs of the current device, and the blocks of a first pass (256 threads each,
+// MM_SHOOT_MINB resident per SM).
+static int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return std::max(1, sms);
+}
+static int shoot_grid() { return sm_count() * MM_SHOOT_MINB; }
+
 // Terms of a sub-cell's re-centred local expansion evaluated per ray.  The
 // far-field stars of a leaf of half-length L lie outside its 3 x 3 block
 // (L-inf distance >= 3L from the centre), so truncating the expansion about
@@ -642,7 +651,7 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
     CK(h->sub_bin.ensure(P1 * P1));
     LCH(launch_sub_tables(h->sub, h->p, h->sub_up.p, h->sub_fp.p, h->sub_bin.p, st));
   }
-  const int p = h->p, P1 = p + 1;
+  const int p = h->p, P1 = p + 1, sms = sm_count();
   // the error word, and the direct stars' slots reserved so far
   CK(cudaMemsetAsync(h->err.p, 0, 2 * sizeof(unsigned), st));
 
@@ -650,13 +659,13 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   // (M2L reads multipoles of levels >= 2 only)
   LCH(launch_p2m(T, nn, p, h->MLop.p, h->mp.p, st));
   for (int l = h->depth - 1; l >= 2; l--)
-    LCH(launch_m2m(T, l, h->level_cnt[l], p, h->MMop.p, h->mp.p, st));
+    LCH(launch_m2m(T, l, h->level_cnt[l], p, h->MMop.p, h->mp.p, sms, st));
   // down-sweep: levels 0 and 1 have no well-separated nodes, so their locals
   // (at most five) are zero; every active node below gets its own
   CK(cudaMemsetAsync(h->loc.p, 0, (size_t)std::min<int64_t>(nn, 5) * P1 * sizeof(double2), st));
   for (int l = 2; l <= h->depth; l++)
     LCH(launch_local(T, l, h->level_cnt[l], p, h->node_act.p, h->MLop.p, h->LLop.p, h->mp.p,
-                    h->loc.p, h->err.p, st));
+                    h->loc.p, h->err.p, sms, st));
 
   // near-field lists and leaf records, per sub-cell record
   FmmConst C;
@@ -730,20 +739,10 @@ static mm_status run_fmm(mm_map *h, cudaStream_t st, bool plan) {
   return MM_OK;
 }
 
-static int shoot_grid() {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  per_sm = MM_SHOOT_MINB;  // resident 256-thread blocks per SM
-  return std::max(1, sms * per_sm);
-}
-
 static void fill_mapdev(mm_map *h) {
   const mm_params &P = h->P;
   MapDev &M = h->md;
   memset(&M, 0, sizeof M);
-  M.n0 = P.n[0];
-  M.n1 = P.n[1];
   M.row_begin = h->row_lo;
   M.row_end = h->row_hi;
   M.col_begin = h->col_lo;

@@ -27,16 +27,6 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
   return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
-// z^k by repeated squaring (k >= 0)
-__device__ __forceinline__ double2 cpow(double2 z, int k) {
-  double2 r = make_double2(1.0, 0.0);
-  while (k > 0) {
-    if (k & 1) r = cmul(r, z);
-    z = cmul(z, z);
-    k >>= 1;
-  }
-  return r;
-}
 
 // 2^e as a double, -1022 <= e <= 1023.
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
@@ -491,7 +481,7 @@ __global__ void __launch_bounds__(MM_LOCAL_THREADS, 8)
         }
     }
   }
-  if (on) (im ? &loc[node * P1 + row].y : &loc[node * P1 + row].x)[0] = acc;  // (c_0 stays zero)
+  if (on) (im ? &loc[node * P1 + row].y : &loc[node * P1 + row].x)[0] = acc;  // (c_0 has no reader)
 }
 
 // ---------------------------------------------------------------------------
@@ -1214,13 +1204,14 @@ cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *
 }
 
 cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const double2 *MMop,
-                       double2 *mp, cudaStream_t st) {
+                       double2 *mp, int sms, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   // 8 nodes a block fill its warps (4 children x p/2 rows each); fewer where
   // their coefficients would not fit 48 KB, and where a level's nodes would
-  // leave SMs idle (a node's work is 2 us of one SM's FP64 pipe)
+  // leave less than two blocks an SM (a node's work is 2 us of one SM's FP64
+  // pipe)
   int per_block = p <= 32 ? 8 : 4;
-  while (per_block > 1 && n < 304 * (int64_t)per_block) per_block >>= 1;
+  while (per_block > 1 && n < 2 * (int64_t)sms * per_block) per_block >>= 1;
   const int threads = 32 * ((per_block * 4 * ((p + 1) / 2) + 31) / 32);
   const size_t smem = sizeof(double2) * 2 * per_block * 4 * (size_t)(p + 1);
   launch_next(k_m2m, blocks_for(n, per_block), threads, smem, st, T, level, n, p, per_block, MMop, mp);
@@ -1229,19 +1220,19 @@ cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const doub
 
 cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const int32_t *node_act,
                          const double2 *MLop, const double2 *LLop, const double2 *mp,
-                         double2 *loc, unsigned *err, cudaStream_t st) {
+                         double2 *loc, unsigned *err, int sms, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const size_t smem = local_smem(p);
-  if (smem > 48 * 1024) {
+  if (smem + sizeof(LocalSources) > 48 * 1024) {  // (the sources lie in the block's own)
     cudaError_t e = cudaFuncSetAttribute(k_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
   }
   // parts per node where a level's nodes (most of them inactive when the grid
   // is a small part of the star region) leave SMs idle: the levels of 16 and 64
-  // nodes took 24 and 36 us in one part, 14 and 22 in four; above 3000 nodes
+  // nodes took 24 and 36 us in one part, 14 and 22 in four; above 20 nodes an SM
   // the pipe is busy anyway and a part costs 6 % more of it
-  const unsigned parts = n <= 304 ? 4 : n <= 3000 ? 2 : 1;
+  const unsigned parts = n <= 2 * (int64_t)sms ? 4 : n <= 20 * (int64_t)sms ? 2 : 1;
   launch_next(k_local, dim3((unsigned)n, parts), MM_LOCAL_THREADS, smem, st, T, level, n, p, node_act, MLop, LLop, mp,
                                                        loc, err);
   return cudaGetLastError();

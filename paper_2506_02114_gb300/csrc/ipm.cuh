@@ -549,13 +549,13 @@ __device__ __forceinline__ void pixel_task(const MapAcc &M, const RowRecs *rr, i
   }
 }
 
-// Instruction-bound: per 32 pixels ~75 instructions (deal, four loads of the
-// row's record, three piece means, one reduction), per 32 rows ~200.  The
-// first two pieces' means in packed pairs, the pixel's address and the run's
-// gap prepared once a row, the row's run from its two sides, and owners found
-// from one reduction took the second pass of the 2000^2 map from 12.25 to
-// 10.44 ms, bit for bit the same.  Its L2 reductions then run at 1.8e11/s,
-// 85 % of the measured scattered rate.
+// Instruction-bound: per 32 pixels 88 instructions (deal, four loads of the
+// row's record, three piece means, one reduction), per 32 rows 228, and 169 to
+// set up 32 triangles.  The first two pieces' means in packed pairs, the pixel's
+// address and the run's gap prepared once a row, the row's run from its two
+// sides, and owners found from one reduction took the second pass of the 2000^2
+// map from 12.25 to 10.44 ms, bit for bit the same.  Its L2 reductions run at
+// 1.3e11/s (that map at one ray a pixel), 60 % of the measured scattered rate.
 //
 // The nb (<= 32) triangles q[0..nb) (warp shared memory) spanning more than
 // 2 x 2 pixels.  Their pixel rows within the map are dealt out to the lanes,

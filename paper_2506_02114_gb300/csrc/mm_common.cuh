@@ -92,7 +92,6 @@ struct RawTri;  // a triangle larger than 2 x 2 pixels (ipm.cuh)
 // item's bounds come from,
 struct MapItems {
   // ray grid
-  int64_t n0, n1;             // vertices per axis
   int64_t row_begin, row_end; // cell rows [row_begin, row_end)
   int64_t col_begin, col_end; // cell columns [col_begin, col_end)
   int32_t strips, rows_per_item;
@@ -133,7 +132,7 @@ struct MapCore {
   unsigned long long *acc;    // npix_y*npix fixed point, 2^32 = one triangle
   unsigned long long *span;   // npix_y*(npix+1) row difference array
   // statistics (per map)
-  unsigned long long *stat;   // triangle counters, see IpmCounters
+  unsigned long long *stat;   // triangle counters, ST_* (ipm.cuh)
   // larger triangles handed to the second kernel (capacity 0: none)
   RawTri *bigq;
   unsigned long long *bigq_n; // [0] triangles queued, [1] the second kernel's batch counter,

@@ -59,7 +59,6 @@ struct TreeDev {
   const int32_t *nb;          // per node: the nine same-level cells around it (row-major,
                               // itself in the middle), -1 where the cell is no node
   const int64_t *level_off;   // [MM_DMAX + 2]
-  int32_t depth;
 };
 
 cudaError_t launch_star_keys(const double *pos, int64_t n, double R0, uint64_t *keys,
@@ -132,10 +131,10 @@ struct FmmConst {
 cudaError_t launch_p2m(const TreeDev &T, int64_t n_nodes, int p, const double2 *MLop, double2 *mp,
                        cudaStream_t st);
 cudaError_t launch_m2m(const TreeDev &T, int level, int64_t n, int p, const double2 *MMop,
-                       double2 *mp, cudaStream_t st);
+                       double2 *mp, int sms, cudaStream_t st);
 cudaError_t launch_local(const TreeDev &T, int level, int64_t n, int p, const int32_t *node_act,
                          const double2 *MLop, const double2 *LLop, const double2 *mp,
-                         double2 *loc, unsigned *err, cudaStream_t st);
+                         double2 *loc, unsigned *err, int sms, cudaStream_t st);
 // *total += direct-sum stars of all records (the plan sizes their arrays)
 cudaError_t launch_near_count(const TreeDev &T, const FmmConst &C, int64_t n_active,
                               const int32_t *active_list, unsigned *total, unsigned *err,

@@ -158,8 +158,6 @@ extern "C" mm_status mm_map_plain_fp64_noalloc(
 
   MapDev md;
   memset(&md, 0, sizeof md);
-  md.n0 = n0;
-  md.n1 = n1;
   md.row_begin = 0;
   md.row_end = n1 - 1;
   md.col_begin = 0;
