@@ -992,7 +992,9 @@ static mm_status alloc_map_buffers(mm_map *h) {
     }
   }
   CK(h->err.ensure(2));
-  CK(cudaMemset(h->err.p, 0, 2 * sizeof(unsigned)));  // read after the plan in every mode
+  // (read after the plan in every mode; in the order it was taken in, before
+  // which the block may still be another handle's)
+  CK(cudaMemsetAsync(h->err.p, 0, 2 * sizeof(unsigned), h->plan_stream));
   CK(h->d_md.ensure(1));
   return MM_OK;
 }

@@ -2,7 +2,8 @@
 // its host code runs without a GPU: device memory is host memory, kernels do
 // nothing but fill the few counters the plan reads back (a tree of one leaf),
 // and every stream's work is counted, so that a buffer given back while some
-// stream may still use it is noticed.  Not a GPU model: maps stay zero.
+// stream may still use it, or used before it is there, is noticed.  Not a GPU
+// model: maps stay zero.
 #include <cuda_runtime_api.h>
 
 #include <sys/mman.h>
@@ -19,7 +20,12 @@ namespace {
 
 std::mutex mu;
 std::map<const void *, std::string> names;               // kernels by host function
-std::map<const void *, size_t> blocks;                   // live device memory
+struct Block {
+  size_t n;
+  int stream;  // pooled memory: whose order it was taken in, and after which operation
+  long op;
+};
+std::map<const char *, Block> blocks;                    // live device memory
 typedef std::map<int, long> Clock;                       // stream -> operations known done
 std::map<int, Clock> streams;                            // what each stream is ordered after
 std::map<cudaEvent_t, Clock> events;
@@ -49,25 +55,37 @@ void check_free(int s) {
     }
   }
 }
-cudaError_t get(void **p, size_t n, bool pooled) {
+// Use of an address in the order of stream s: pooled memory is there only
+// after the operation that took it from the pool.
+void check_use(const void *p, int s) {
+  auto it = blocks.upper_bound(static_cast<const char *>(p));
+  if (it == blocks.begin()) return;
+  --it;
+  if (static_cast<const char *>(p) >= it->first + it->second.n || it->second.op == 0) return;
+  Clock known = host;
+  merge(known, streams[s]);
+  if (known[it->second.stream] < it->second.op) unordered++;
+}
+cudaError_t get(void **p, size_t n, bool pooled, cudaStream_t s) {
   std::lock_guard<std::mutex> l(mu);
   if (mallocs++ == fail_malloc) return cudaErrorMemoryAllocation;
   // (never touched pages cost nothing: a queue of gigabytes is only an address range)
   *p = mmap(nullptr, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE,
             -1, 0);
   if (*p == MAP_FAILED) return cudaErrorMemoryAllocation;
-  blocks[*p] = n;
+  if (pooled) enqueue(s);
+  blocks[static_cast<char *>(*p)] = Block{n ? n : 1, id(s), pooled ? ops : 0};
   if (pooled) {
-    pool_used += n;
+    pool_used += n ? n : 1;
     pool_held = std::max(pool_held, pool_used);
   }
   return cudaSuccess;
 }
 void put(void *p, bool pooled) {
-  const auto it = blocks.find(p);
+  const auto it = blocks.find(static_cast<char *>(p));
   if (it == blocks.end()) return;
-  if (pooled) pool_used -= it->second;
-  munmap(p, it->second ? it->second : 1);
+  if (pooled) pool_used -= it->second.n;
+  munmap(p, it->second.n);
   blocks.erase(it);
 }
 void copy(void *d, const void *s, size_t n) {
@@ -198,8 +216,8 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *, const void *) {
 }
 
 // memory
-cudaError_t cudaMalloc(void **p, size_t n) { return get(p, n, false); }
-cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return get(p, n, true); }
+cudaError_t cudaMalloc(void **p, size_t n) { return get(p, n, false, nullptr); }
+cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t s) { return get(p, n, true, s); }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) {
   *p = calloc(n, 1);
   return cudaSuccess;
@@ -222,22 +240,28 @@ cudaError_t cudaFreeAsync(void *p, cudaStream_t s) {
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t st) {
   std::lock_guard<std::mutex> l(mu);
+  check_use(d, id(st));
+  check_use(s, id(st));
   copy(d, s, n);
   enqueue(st);
   return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) {
   std::lock_guard<std::mutex> l(mu);
+  check_use(d, 0);
+  check_use(s, 0);
   copy(d, s, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void *d, int v, size_t n) {
   std::lock_guard<std::mutex> l(mu);
+  check_use(d, 0);
   if (n <= (size_t)1 << 20) memset(d, v, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t st) {
   std::lock_guard<std::mutex> l(mu);
+  check_use(d, id(st));
   if (n <= (size_t)1 << 20) memset(d, v, n);
   enqueue(st);
   return cudaSuccess;

@@ -69,6 +69,21 @@ def test_destroy_waits_for_the_last_run(fake, mode, stream):
     assert fake.fake_unordered() == 0
 
 
+@pytest.mark.parametrize("mode", MODES)
+def test_buffers_are_used_in_the_order_they_were_taken(fake, mode):
+    """A block of the pool is there in the order of the stream it was taken
+    on: until then it may be another handle's, created on another thread."""
+    fake.fake_reset()
+    h = make(mode)
+    assert fake.fake_unordered() == 0
+    mm.run(h, 0)
+    mm.get_map_fixed(h)
+    mm.shoot_points(h, np.zeros((3, 2)))
+    mm.get_stats(h)
+    assert fake.fake_unordered() == 0
+    mm.destroy(h)
+
+
 @pytest.mark.parametrize("stream", [0, 77])
 def test_destroy_waits_for_a_batch(fake, stream):
     fake.fake_reset()
