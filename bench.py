@@ -64,14 +64,24 @@ TUNE_CACHE = os.path.join(ROOT, "paper_2506_02114_gb300", "tune", "sm_103.jsonl"
 # (profiles/counters_fmm_fp32_salpeter_2000_rpp1.md): valid only for the kernel
 # sources they were taken on (hash below), reported beside the live roofline.
 NCU_COUNTERS = {
-    "sources_sha1": "80cfb1b8280ba260da4a0304e21ea6bba0d63497",
+    "sources_sha1": "9f1a93a454bb6fabf18f6cc565b8bf90fa4a5286",
     "case": "fmm_fp32_salpeter_2000 at 1 ray per pixel (1.64e8 rays), ncu --clock-control none",
-    "k_shoot_ipm": {"issue_active": 0.641, "warps_active": 0.370, "alu_active": 0.470,
-                    "fma_active": 0.268, "l2_red_requests_per_s": 3.41e10},
-    "k_big_ipm": {"issue_active": 0.835, "warps_active": 0.573, "alu_active": 0.581,
-                  "fma_active": 0.393, "l2_red_requests_per_s": 1.27e11},
+    "k_shoot_ipm": {"issue_active": 0.637, "warps_active": 0.369, "alu_active": 0.471,
+                    "fma_active": 0.268, "l2_red_requests_per_s": 3.40e10},
+    "k_big_ipm": {"issue_active": 0.835, "warps_active": 0.571, "alu_active": 0.579,
+                  "fma_active": 0.391, "l2_red_requests_per_s": 1.26e11},
     "k_direct64_vertices": {"fp64_pipe_active": 0.914},
 }
+
+
+def queue_bytes(st):
+    """Bytes of a handle's second-pass queue: 32 a slot, 10 more for the order
+    of a map taken by bands (accumulators above half the L2, 2^22 slots)."""
+    import torch
+    p = st["params"]
+    half_l2 = torch.cuda.get_device_properties(0).L2_cache_size / 2
+    banded = st["queue_slots"] >= 1 << 22 and 16 * p["npix"] * p["npix_y"] > half_l2
+    return st["queue_slots"] * (42 if banded else 32)
 
 
 def kernel_sources_sha1():
@@ -786,7 +796,7 @@ def run_native(args):
                    "sub_levels": sorted({st["sub_levels"] for st in stats}),
                    "rows_per_item": sorted({st["rows_per_item"] for st in stats}),
                    "tuned_from_cache": tuned.count(2), "tuned_by_timing": tuned.count(1),
-                   "queue_gb": sum(st["queue_slots"] for st in stats) * 32 / 1e9,
+                   "queue_gb": sum(queue_bytes(st) for st in stats) / 1e9,
                    "mapping": "irs" if args.irs else "ipm",
                    "band_rows": list(band[:2]) if band else None,
                    "l2": "flushed before every step (256 MiB write)",

@@ -84,8 +84,9 @@ typedef struct {
   int64_t row_begin;        /* shoot only cell rows [row_begin, row_end) of the */
   int64_t row_end;          /*   ray grid; both 0 -> every row */
   int32_t rows_per_item;    /* rows of cells per warp work item, 1..4096; 0 ->
-                               the largest of 256, 128, ..., 16 that leaves every
-                               resident warp >= 16 items */
+                               the largest of 256, 128, 64 that leaves every
+                               resident warp >= 16 items, else of 32, 16 that
+                               leaves it >= 2, else 8 */
   int32_t sub_levels;       /* FMM mode: each leaf's local expansion is re-centred
                                exactly on its 4^s sub-cells (s levels below the
                                leaf); a sub-cell sums directly only the leaf's

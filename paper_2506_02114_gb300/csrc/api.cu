@@ -166,12 +166,12 @@ static uint64_t pool_idle(cudaMemPool_t pool, uint64_t &used) {
   return held > used ? held - used : 0;
 }
 
-// Gives the driver back what the pool holds unused beyond 1/32 of the device's
+// Gives the CUDA driver back what the pool holds unused beyond 1/32 of the device's
 // memory, which is one handle's largest default queue (leaves_room): after a
 // handle with a queue of gigabytes, so that other allocators of the process
 // are not left without what many such handles took.  Handles made one after
 // the other still find the queue in the pool (5.6 GB: 0.006 ms, 4.2 ms to take
-// from the driver and 7.0 to give back).
+// from the CUDA driver and 7.0 to give back).
 static void trim_pool(int device) {
   size_t free_b = 0, total_b = 0;
   cudaMemPool_t pool;

@@ -727,8 +727,8 @@ struct RecSmem {
 // tables; 32 threads form the 16 records' centres, d_1 and images, one axis
 // each.  Records reserve their direct stars' slots themselves.  67 000 records
 // of 50 000 stars: 307 us with a thread a record (after a count and a scan of
-// 32 us), 167 us like this (176 with IEEE divisions by the grid steps and the
-// pixel, and the near stars tested twice); a 48^2 map's 848 records 160 and 24 us.
+// 32 us), 162 us like this (171 with IEEE divisions by the grid steps and the
+// pixel, and the near stars tested twice), 167 with the direct masses' FP64 sum; a 48^2 map's 848 records 160 and 24 us.
 // NB >= p_eval.
 template <int NB>
 __global__ void __launch_bounds__(MM_REC_THREADS) k_leaf_finalize(

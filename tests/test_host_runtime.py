@@ -120,7 +120,7 @@ def test_destroy_waits_for_what_a_failed_batch_queued(fake):
 
 def test_large_queues_do_not_stay_with_the_pool(fake):
     """One handle's queue of gigabytes may wait in the pool for the next
-    handle; those of several alive at once go back to the driver."""
+    handle; those of several alive at once go back."""
     fake.fake_reset()
     bound = fake.fake_total_memory() // 32
     hs = [make(npix=2200, big_queue_slots=1 << 27) for _ in range(4)]   # 5.6 GB each
